@@ -67,7 +67,7 @@ typedef struct dbg_graph *dbg_handle;
  * The built graph does not depend on these values: only the speed does. */
 typedef struct dbg_tuning {
   int block_threads;  /* threads per CTA, a multiple of 32 in [64, 1024] (default 256) */
-  int tile_reads;     /* reads staged per tile, in [1, block_threads] (default block_threads) */
+  int tile_reads;     /* reads staged per tile, in [1, block_threads] (default: by the number of reads) */
   int grid_ctas;      /* CTAs in the persistent grid (default: SMs x resident CTAs per SM) */
   int warp_aggregate; /* direct insert: 1 merges a warp's equal keys with __match_any_sync,
                          0 does not, -1: default (1) */

@@ -1657,15 +1657,13 @@ struct Marks {
 // One tiled chain over items[0..n) (N >= n): their tables are cut into
 // regions of 2^shift slots (`parts` of them, `tiles` tiles), item i's first
 // region is items[i].region0, and items[i].tile_begin numbers the walk's
-// tiles of kScatterTileReads reads.  `direct` holds the same items numbered
-// for the direct kernel (`direct_tiles` tiles), which does the call instead
+// tiles of kScatterTileReads reads.  The direct kernel does the call instead
 // when the events do not fit the scratch.  The scratch's event buffer, second
 // buffer and aux area must exist.  `status` receives a timeout of the split.
 template <int N>
 int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int parts,
-                uint64_t tiles, uint64_t walk_tiles, const ItemDesc *direct,
-                uint64_t direct_tiles, const dbg_tuning &tuning, int sms, cudaStream_t s,
-                bool fresh, const Marks &mark, const InputParts *input = nullptr) {
+                uint64_t tiles, uint64_t walk_tiles, const dbg_tuning &tuning, int sms,
+                cudaStream_t s, bool fresh, const Marks &mark, const InputParts *input = nullptr) {
   const int scatter_reads = scatter_tile_reads(tuning);
   const MetaView mv = meta_view(sc);
   const int tpr = 1 << (shift - kTileLog2);
@@ -1792,7 +1790,7 @@ int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int par
     k_tables_init<N><<<dim3(std::max(1, sms * 8 / n), n), 256, 0, s>>>(ip, mv.flag);
     DBG_CK(cudaGetLastError());
   }
-  const int st = launch_insert(direct, n, direct_tiles, tuning, sms, s, mv.flag);
+  const int st = launch_insert(items, n, tuning, sms, s, mv.flag);
   if (st != DBG_OK) return st;
   mark(8, s);
   return DBG_OK;
@@ -1806,8 +1804,8 @@ int wait_input(const InputParts *input, cudaStream_t s) {
   return DBG_OK;
 }
 
-int launch_binned(dbg_handle h, const ItemDesc &it, uint64_t tiles, const dbg_tuning &tuning,
-                  cudaStream_t s, int call, bool fresh, const InputParts *input) {
+int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cudaStream_t s,
+                  int call, bool fresh, const InputParts *input) {
   constexpr int B = 256;
   const dbg_tuning t = resolve_tuning(tuning);
   // the tiled apply re-partitions each region by tile, so its first pass can
@@ -1840,10 +1838,8 @@ int launch_binned(dbg_handle h, const ItemDesc &it, uint64_t tiles, const dbg_tu
     walk.region0 = 0;
     const uint64_t sr = (uint64_t)scatter_tile_reads(tuning);
     const uint64_t walk_tiles = (it.n_reads + sr - 1) / sr;
-    ItemDesc direct = it;
-    direct.tile_begin = 0;
-    DBG_TRY(tiled_chain<1>(h->bin, &walk, 1, geo.shift, geo.parts, n_tiles, walk_tiles, &direct,
-                           tiles, tuning, sms, s, fresh, mark, input));
+    DBG_TRY(tiled_chain<1>(h->bin, &walk, 1, geo.shift, geo.parts, n_tiles, walk_tiles, tuning,
+                           sms, s, fresh, mark, input));
     h->built_counts = fresh;  // a rebuild counted its vertices and edges (unless it fell back)
     if (!capturing) DBG_CK(cudaEventRecord(h->bin.done, s));
     return DBG_OK;
@@ -1903,7 +1899,7 @@ int launch_binned(dbg_handle h, const ItemDesc &it, uint64_t tiles, const dbg_tu
   }
   // the direct insert runs only if the events did not fit the buffer
   mark(7, s);
-  const int st = launch_insert(&it, 1, tiles, tuning, h->sm_count, s, mv.flag);
+  const int st = launch_insert(&it, 1, tuning, h->sm_count, s, mv.flag);
   if (st != DBG_OK) return st;
   mark(8, s);
   if (!capturing) DBG_CK(cudaEventRecord(h->bin.done, s));
@@ -1991,24 +1987,22 @@ int launch_binned_batch(const ItemDesc *items, const uint64_t *want, int n,
   const uint64_t sr = (uint64_t)scatter_tile_reads(tuning);
   for (const Chain &c : chains) {
     const int m = c.i1 - c.i0;
-    std::vector<ItemDesc> walk(items + c.i0, items + c.i1), direct(items + c.i0, items + c.i1);
-    uint64_t walk_tiles = 0, direct_tiles = 0;
+    std::vector<ItemDesc> walk(items + c.i0, items + c.i1);
+    uint64_t walk_tiles = 0;
     int region0 = 0;
     for (int i = 0; i < m; ++i) {
       walk[i].tile_begin = walk_tiles;
       walk[i].region0 = region0;
       walk_tiles += (walk[i].n_reads + sr - 1) / sr;
       region0 += regions_of(walk[i].n_slots, shift);
-      direct[i].tile_begin = direct_tiles;
-      direct_tiles += (direct[i].n_reads + (uint64_t)t.tile_reads - 1) / (uint64_t)t.tile_reads;
     }
     if (!ready) {  // no scratch inside this capture: the direct insert does it
-      if (fresh) DBG_TRY(launch_tables_init(direct.data(), m, sms, s));
-      DBG_TRY(launch_insert(direct.data(), m, direct_tiles, tuning, sms, s));
+      if (fresh) DBG_TRY(launch_tables_init(walk.data(), m, sms, s));
+      DBG_TRY(launch_insert(walk.data(), m, tuning, sms, s));
       continue;
     }
     DBG_TRY(tiled_chain<kBatchItems>(sc, walk.data(), m, shift, c.parts, c.tiles, walk_tiles,
-                                     direct.data(), direct_tiles, tuning, sms, s, fresh, Marks{}));
+                                     tuning, sms, s, fresh, Marks{}));
   }
   if (!capturing) DBG_CK(cudaEventRecord(sc.done, s));
   return DBG_OK;

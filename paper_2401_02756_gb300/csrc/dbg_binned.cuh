@@ -63,15 +63,14 @@ int wait_input(const InputParts *input, cudaStream_t s);
 // instead of reading it, which empties the table without a pass of its own.
 // `input`: the reads arrive in parts; the tiled chain's scatter takes each
 // part as it arrives, every other path waits for all of them first.
-int launch_binned(dbg_handle h, const ItemDesc &it, uint64_t tiles, const dbg_tuning &tuning,
-                  cudaStream_t s, int call, bool fresh = false,
+int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cudaStream_t s,
+                  int call, bool fresh = false,
                   const InputParts *input = nullptr);
 
 // Insert many read sets, each into its own table (k <= 31), through binned
 // chains: every chain is one launch of each binned kernel over all of its
-// items (up to kBatchItems of them and kBinMaxParts regions).  items[i]
-// carries the direct kernel's tile numbering (tile_begin over `tile_reads`
-// reads per tile); `want[i]` is the event capacity item i asks for.  The
+// items (up to kBatchItems of them and kBinMaxParts regions).  `want[i]` is
+// the event capacity item i asks for.  The
 // scratch is the library's own, per device.  Items of a chain whose events
 // do not fit the scratch (a call captured into a CUDA graph before the
 // scratch was large enough) take the direct insert instead.

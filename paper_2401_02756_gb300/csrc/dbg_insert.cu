@@ -48,7 +48,7 @@ struct InsertVisitor {
       if (valid) {
         uint64_t slot;
         if (find_or_claim(c.table, c.n_slots, c.max_probes, key, slot)) {
-          if (edge) atomicAdd(&c.table[slot].cnt[label], 1u);
+          if (edge) red_add_u32(&c.table[slot].cnt[label], 1u);
         } else if (spill_or_fail(c.spill, c.spill_cap, c.spill_count, c.status, key, edge, label)) {
           *s_cap_hit = 1u;
         }
@@ -82,8 +82,14 @@ struct InsertVisitor {
   }
 };
 
+// Bound by the latency of dependent L2 round trips: a warp waits for its
+// longest probe chain (about four loads and a CAS over its 32 positions), so
+// the kernel is held to 32 registers for 64 warps an SM (a few words spill):
+// 9.2 M positions into a 56 MB table 270 us at 48 registers -> 231 us.  A run
+// of four positions per thread with their probes in flight together took
+// 335 us: twice the instructions, at 13 active lanes instead of 19.
 template <int BLOCK, bool AGG, int N>
-__global__ void __launch_bounds__(BLOCK)
+__global__ void __launch_bounds__(BLOCK, 2048 / BLOCK)
     k_insert(const __grid_constant__ ItemPack<N> pk, int tile_reads, const uint32_t *gate) {
   if (gate != nullptr && ld_volatile_u32(gate) != 0u) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -93,20 +99,46 @@ __global__ void __launch_bounds__(BLOCK)
                                gridDim.x);
 }
 
+// Reads per tile when the tuning leaves it open.  A tile is a CTA's unit of
+// work, and a thread holds one position in flight, so a read set of few tiles
+// leaves the chip idle: 1,000 reads in tiles of 256 ran on 4 CTAs (276 us;
+// now 17).  The reads are cut into whole waves of the resident CTAs with at
+// most kAutoTileReads reads a tile (20,000 reads on 1,216 CTAs: 94 us as one
+// wave of 17, 109 as a wave of 16 and its rest), and at least kMinTileReads:
+// a tile of one read would leave most of a CTA's threads idle.
+constexpr int kMinTileReads = 2, kAutoTileReads = 20;
+
+int auto_tile_reads(uint64_t reads, uint64_t resident) {
+  const uint64_t waves = std::max<uint64_t>(1, (reads + resident * kAutoTileReads - 1) /
+                                                   (resident * kAutoTileReads));
+  const uint64_t ctas = resident * waves;
+  return (int)std::max<uint64_t>(kMinTileReads, (reads + ctas - 1) / ctas);
+}
+
+// Number the items' tiles and launch.
 template <int BLOCK, bool AGG, int N>
-int launch_one(const ItemPack<N> &pk, int tile_reads, int grid_ctas, int sm_count,
-               cudaStream_t stream, const uint32_t *gate) {
+int launch_one(ItemPack<N> &pk, int tile_reads, int grid_ctas, int sm_count, cudaStream_t stream,
+               const uint32_t *gate) {
   auto kern = k_insert<BLOCK, AGG, N>;
-  const size_t smem = tile_smem_bytes(tile_reads);
-  if (smem > 48 * 1024) {
+  int per_sm = 0;
+  size_t smem = tile_smem_bytes(tile_reads > 0 ? tile_reads : kAutoTileReads);
+  if (smem > 48 * 1024)
     DBG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BLOCK, smem));
+  const int resident = std::max(1, per_sm) * std::max(1, sm_count);
+  if (tile_reads <= 0) {
+    uint64_t reads = 0;
+    for (int i = 0; i < pk.n_items; ++i) reads += pk.d[i].n_reads;
+    tile_reads = auto_tile_reads(reads, (uint64_t)resident);
+    smem = tile_smem_bytes(tile_reads);
   }
-  int grid = grid_ctas;
-  if (grid <= 0) {
-    int per_sm = 0;
-    DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BLOCK, smem));
-    grid = std::max(1, per_sm) * std::max(1, sm_count);
+  pk.total_tiles = 0;
+  for (int i = 0; i < pk.n_items; ++i) {
+    pk.d[i].tile_begin = pk.total_tiles;
+    pk.total_tiles += (pk.d[i].n_reads + (uint64_t)tile_reads - 1) / (uint64_t)tile_reads;
   }
+  if (pk.total_tiles == 0) return DBG_OK;
+  int grid = grid_ctas > 0 ? grid_ctas : resident;
   if ((uint64_t)grid > pk.total_tiles) grid = (int)pk.total_tiles;
   kern<<<grid, BLOCK, smem, stream>>>(pk, tile_reads, gate);
   DBG_CK(cudaGetLastError());
@@ -114,12 +146,15 @@ int launch_one(const ItemPack<N> &pk, int tile_reads, int grid_ctas, int sm_coun
 }
 
 template <int N>
-int launch_pack(const ItemPack<N> &pk, const dbg_tuning &t, int sm_count, cudaStream_t stream,
-                const uint32_t *gate) {
+int launch_pack(const ItemDesc *items, int n_items, int tile_reads, const dbg_tuning &t,
+                int sm_count, cudaStream_t stream, const uint32_t *gate) {
+  ItemPack<N> pk{};
+  pk.n_items = n_items;
+  for (int i = 0; i < n_items; ++i) pk.d[i] = items[i];
   const bool agg = t.warp_aggregate != 0;
-#define DBG_LAUNCH(B)                                                                           \
-  return agg ? launch_one<B, true, N>(pk, t.tile_reads, t.grid_ctas, sm_count, stream, gate)   \
-             : launch_one<B, false, N>(pk, t.tile_reads, t.grid_ctas, sm_count, stream, gate)
+#define DBG_LAUNCH(B)                                                                    \
+  return agg ? launch_one<B, true, N>(pk, tile_reads, t.grid_ctas, sm_count, stream, gate) \
+             : launch_one<B, false, N>(pk, tile_reads, t.grid_ctas, sm_count, stream, gate)
   switch (t.block_threads) {
     case 128: DBG_LAUNCH(128);
     case 256: DBG_LAUNCH(256);
@@ -145,24 +180,16 @@ dbg_tuning resolve_tuning(const dbg_tuning &t) {
   return r;
 }
 
-int launch_insert(const ItemDesc *items, int n_items, uint64_t total_tiles,
-                  const dbg_tuning &tuning, int sm_count, cudaStream_t stream,
-                  const uint32_t *gate) {
-  if (total_tiles == 0 || n_items <= 0) return DBG_OK;
+int launch_insert(const ItemDesc *items, int n_items, const dbg_tuning &tuning, int sm_count,
+                  cudaStream_t stream, const uint32_t *gate) {
+  if (n_items <= 0) return DBG_OK;
   if (n_items > kBatchItems) return DBG_ERR_INVALID_ARG;
   const dbg_tuning t = resolve_tuning(tuning);
-  if (n_items == 1) {
-    ItemPack<1> pk{};
-    pk.n_items = 1;
-    pk.total_tiles = total_tiles;
-    pk.d[0] = items[0];
-    return launch_pack(pk, t, sm_count, stream, gate);
-  }
-  ItemPack<kBatchItems> pk{};
-  pk.n_items = n_items;
-  pk.total_tiles = total_tiles;
-  for (int i = 0; i < n_items; ++i) pk.d[i] = items[i];
-  return launch_pack(pk, t, sm_count, stream, gate);
+  // (0: chosen by the launch; resolve_tuning's default is the streaming walk's)
+  const int tile_reads = tuning.tile_reads > 0 ? t.tile_reads : 0;
+  return n_items == 1
+             ? launch_pack<1>(items, n_items, tile_reads, t, sm_count, stream, gate)
+             : launch_pack<kBatchItems>(items, n_items, tile_reads, t, sm_count, stream, gate);
 }
 
 }  // namespace dbg

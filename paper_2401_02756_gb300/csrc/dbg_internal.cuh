@@ -117,6 +117,10 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64_hint(const unsigned
   return v;
 }
 
+__device__ __forceinline__ void red_add_u32(uint32_t *p, uint32_t v) {
+  asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 __device__ __forceinline__ void red_add_u32_hint(uint32_t *p, uint32_t v, uint64_t pol) {
   asm volatile("red.relaxed.gpu.global.add.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(p), "r"(v),
                "l"(pol)
@@ -314,12 +318,12 @@ struct ItemPack {
 };
 
 // Launch the insert kernel over host-side descriptors items[0..n_items)
-// (tile_begin already set, total_tiles their sum); n_items <= kBatchItems.
+// (their tile_begin is not read: the launch cuts the reads into tiles itself);
+// n_items <= kBatchItems.
 // `gate`: if not null, the kernel does nothing when *gate != 0 (read on the
 // device when it runs).
-int launch_insert(const ItemDesc *items, int n_items, uint64_t total_tiles,
-                  const dbg_tuning &tuning, int sm_count, cudaStream_t stream,
-                  const uint32_t *gate = nullptr);
+int launch_insert(const ItemDesc *items, int n_items, const dbg_tuning &tuning, int sm_count,
+                  cudaStream_t stream, const uint32_t *gate = nullptr);
 
 // Resolved tuning (defaults filled in).
 dbg_tuning resolve_tuning(const dbg_tuning &t);

@@ -543,14 +543,14 @@ bool want_binned(dbg_handle h) {
 // with the init kernel before they insert.
 // `input`: the read set's bases arrive in parts (see dbg::InputParts); only
 // the binned scatter takes them part by part, every other kernel waits for all.
-int insert_one(dbg_handle h, const dbg::ItemDesc &it, uint64_t tiles, cudaStream_t s,
-               bool fresh = false, const dbg::InputParts *input = nullptr) {
+int insert_one(dbg_handle h, const dbg::ItemDesc &it, cudaStream_t s, bool fresh = false,
+               const dbg::InputParts *input = nullptr) {
   h->built_counts = false;  // (set again by a rebuild on the tiled binned path)
   const int call = dbg::timer_begin_call(h);
   const bool binned = h->k <= 32 && want_binned(h) &&
                       (h->bin.cap == dbg::bin_events_wanted(h) ||
                        dbg::ensure_bin_scratch(h, 0) == DBG_OK);
-  if (binned) return dbg::launch_binned(h, it, tiles, h->tuning, s, call, fresh, input);
+  if (binned) return dbg::launch_binned(h, it, h->tuning, s, call, fresh, input);
   DBG_TRY(dbg::wait_input(input, s));
   if (fresh) DBG_TRY(dbg::launch_table_init(h->table, h->n_slots, s));
   if (h->k > 32) {  // 128-bit keys: their own kernel
@@ -560,7 +560,7 @@ int insert_one(dbg_handle h, const dbg::ItemDesc &it, uint64_t tiles, cudaStream
     return st;
   }
   dbg::timer_mark(h, call, 0, s);
-  const int st = dbg::launch_insert(&it, 1, tiles, h->tuning, h->sm_count, s);
+  const int st = dbg::launch_insert(&it, 1, h->tuning, h->sm_count, s);
   dbg::timer_mark(h, call, 1, s);  // direct call: kernel 0 spans marks 0..1
   return st;
 }
@@ -578,10 +578,8 @@ extern "C" int dbg_insert_reads(dbg_handle h, const uint8_t *packed, const uint6
   if (!packed || !offsets) return DBG_ERR_INVALID_ARG;
   DeviceGuard g(h->device);
   if (g.err != cudaSuccess) return dbg::cuda_fail(g.err, "cudaSetDevice");
-  const dbg_tuning t = dbg::resolve_tuning(h->tuning);
-  const uint64_t tiles = (n_reads + (uint64_t)t.tile_reads - 1) / (uint64_t)t.tile_reads;
   const dbg::ItemDesc it = dbg::make_item(h, packed, offsets, n_reads, 0);
-  return insert_one(h, it, tiles, static_cast<cudaStream_t>(stream));
+  return insert_one(h, it, static_cast<cudaStream_t>(stream));
 }
 
 namespace {
@@ -607,10 +605,8 @@ extern "C" int dbg_build_reads(dbg_handle h, const uint8_t *packed, const uint64
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   DBG_TRY(clear_status(h, s));
   if (n_reads == 0) return dbg::launch_table_init(h->table, h->n_slots, s);
-  const dbg_tuning t = dbg::resolve_tuning(h->tuning);
-  const uint64_t tiles = (n_reads + (uint64_t)t.tile_reads - 1) / (uint64_t)t.tile_reads;
   const dbg::ItemDesc it = dbg::make_item(h, packed, offsets, n_reads, 0);
-  return insert_one(h, it, tiles, s, /*fresh=*/true);
+  return insert_one(h, it, s, /*fresh=*/true);
 }
 
 namespace {
@@ -687,7 +683,7 @@ static bool offsets_non_decreasing(const uint64_t *offsets, uint64_t n_reads) {
 // passes (a refused call waits for its copies, so that the caller may reuse
 // its buffers).
 static int insert_whole(dbg_handle h, const uint8_t *packed, const uint64_t *offsets, uint64_t n_reads,
-                        uint64_t all_bytes, const dbg_tuning &t, cudaStream_t s, bool fresh) {
+                        uint64_t all_bytes, cudaStream_t s, bool fresh) {
   DBG_TRY(grow_stage(h, std::max<uint64_t>(16, (all_bytes + 15) & ~15ull), n_reads));
   const uint64_t byte0 = offsets[0] >> 2, end = (offsets[n_reads] + 3) >> 2;
   DBG_CK(cudaStreamWaitEvent(h->copy_stream, h->ev_consumed[0], 0));
@@ -732,13 +728,12 @@ static int insert_whole(dbg_handle h, const uint8_t *packed, const uint64_t *off
   DBG_CK(cudaStreamWaitEvent(s, h->ev_copied[0], 0));
   const dbg::ItemDesc it =
       dbg::make_item(h, h->stage_packed[0], h->stage_offsets[0], n_reads, byte0 * 4);
-  const uint64_t tiles = (n_reads + (uint64_t)t.tile_reads - 1) / (uint64_t)t.tile_reads;
   dbg::InputParts input;
   input.n = n_parts;
   input.read_cut = read_cut;
   input.ready = h->ev_part;
   if (n_parts == 1) DBG_CK(cudaStreamWaitEvent(s, h->ev_part[0], 0));
-  DBG_TRY(insert_one(h, it, tiles, s, fresh, n_parts > 1 ? &input : nullptr));
+  DBG_TRY(insert_one(h, it, s, fresh, n_parts > 1 ? &input : nullptr));
   DBG_CK(cudaEventRecord(h->ev_consumed[0], s));
   return DBG_OK;
 }
@@ -757,7 +752,6 @@ static int insert_reads_host(dbg_handle h, const uint8_t *packed, const uint64_t
     DBG_TRY(clear_status(h, s));
     return dbg::launch_table_init(h->table, h->n_slots, s);
   }
-  const dbg_tuning t = dbg::resolve_tuning(h->tuning);
 
   // the whole input when it is small enough (one insert, which the binned
   // path needs to see the whole read set at once), else chunks of at most
@@ -765,7 +759,7 @@ static int insert_reads_host(dbg_handle h, const uint8_t *packed, const uint64_t
   if (offsets[n_reads] >= offsets[0]) {
     const uint64_t all_bytes = ((offsets[n_reads] + 3) >> 2) - (offsets[0] >> 2);
     if (all_bytes + (n_reads + 1) * sizeof(uint64_t) <= kStageAllBytes)
-      return insert_whole(h, packed, offsets, n_reads, all_bytes, t, s, fresh);
+      return insert_whole(h, packed, offsets, n_reads, all_bytes, s, fresh);
   }
   if (!offsets_non_decreasing(offsets, n_reads)) return DBG_ERR_INVALID_ARG;
   if (fresh) DBG_TRY(clear_status(h, s));
@@ -807,8 +801,7 @@ static int insert_reads_host(dbg_handle h, const uint8_t *packed, const uint64_t
     DBG_CK(cudaStreamWaitEvent(s, h->ev_copied[b], 0));
     const dbg::ItemDesc it =
         dbg::make_item(h, h->stage_packed[b], h->stage_offsets[b], r1 - r0, byte0 * 4);
-    const uint64_t tiles = (r1 - r0 + (uint64_t)t.tile_reads - 1) / (uint64_t)t.tile_reads;
-    st = insert_one(h, it, tiles, s, fresh && c == 0);
+    st = insert_one(h, it, s, fresh && c == 0);
     if (st != DBG_OK) return st;
     DBG_CK(cudaEventRecord(h->ev_consumed[b], s));
   }
@@ -845,19 +838,17 @@ static int insert_batch(const dbg_batch_item *items, int n_items, void *stream, 
   DeviceGuard g(dev);
   if (g.err != cudaSuccess) return dbg::cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const dbg_tuning t = dbg::resolve_tuning(items[0].graph->tuning);
+  const dbg_tuning t = items[0].graph->tuning;  // (resolved by the launches)
   const int sms = items[0].graph->sm_count;
   std::vector<dbg::ItemDesc> group, binned;
   std::vector<uint64_t> wants;
   group.reserve(dbg::kBatchItems);
-  uint64_t tiles = 0;
   for (int i = 0; i <= n_items; ++i) {
     const bool flush = (i == n_items) || (int)group.size() == dbg::kBatchItems;
     if (flush && !group.empty()) {
       if (fresh) DBG_TRY(dbg::launch_tables_init(group.data(), (int)group.size(), sms, s));
-      DBG_TRY(dbg::launch_insert(group.data(), (int)group.size(), tiles, t, sms, s));
+      DBG_TRY(dbg::launch_insert(group.data(), (int)group.size(), t, sms, s));
       group.clear();
-      tiles = 0;
     }
     if (i == n_items) break;
     dbg_handle h = items[i].graph;
@@ -868,8 +859,7 @@ static int insert_batch(const dbg_batch_item *items, int n_items, void *stream, 
         DBG_TRY(dbg::launch_table_init(h->table, h->n_slots, s));
       }
       if (items[i].n_reads == 0) continue;
-      const dbg_tuning th = dbg::resolve_tuning(h->tuning);
-      DBG_TRY(insert_one(h, it, (items[i].n_reads + th.tile_reads - 1) / th.tile_reads, s));
+      DBG_TRY(insert_one(h, it, s));
       continue;
     }
     if (h->k <= 31 && h->tuning.insert_path != 1) {  // binned chains below (an empty read
@@ -879,8 +869,6 @@ static int insert_batch(const dbg_batch_item *items, int n_items, void *stream, 
       continue;
     }
     if (items[i].n_reads == 0 && !fresh) continue;
-    it.tile_begin = tiles;
-    tiles += (items[i].n_reads + (uint64_t)t.tile_reads - 1) / (uint64_t)t.tile_reads;
     group.push_back(it);
   }
   return dbg::launch_binned_batch(binned.data(), wants.data(), (int)binned.size(), t, sms, s,
