@@ -9,25 +9,44 @@
 //
 // Contigs.  An outgoing edge of a vertex is a label with a nonzero counter.
 // The first flag of the paper (no edge points to the vertex) is recomputed
-// from the counters as they are: every slot clears the mark word in its
-// padding, then every edge marks its target.  A vertex starts contigs when
-// its first flag is set or it has not exactly one outgoing edge, one contig
-// per outgoing edge; a contig follows edges while the vertex it reaches has
-// exactly one outgoing edge, and stops on reaching a vertex it has already
-// visited (keeping the edge into it).  Contigs are listed by (start key,
-// label): the start edges are emitted in any order and radix-sorted.
+// from the counters as they are.  A vertex starts contigs when its first flag
+// is set or it has not exactly one outgoing edge, one contig per outgoing
+// edge; a contig follows edges while the vertex it reaches has exactly one
+// outgoing edge, and stops on reaching a vertex it has already visited
+// (keeping the edge into it).  Contigs are listed by (start key, label): the
+// start edges are emitted in any order and radix-sorted.
 //
-// One thread walks one contig.  The walk first measures the contig: Brent's
-// cycle detection (R. P. Brent, "An improved Monte Carlo factorization
-// algorithm", BIT 20, 1980) over the single-exit successor map finds the
-// first repeated vertex, if any, with O(1) state; a second walk writes the
-// bases at the offset an exclusive scan of the lengths gives.
+// One pass over the table finds every edge's target once: the target is
+// marked in a bit per slot, and a vertex with one outgoing edge keeps its
+// successor's slot in the slot's padding, so that a step of a walk is one
+// 32-byte load.  A second pass over the bits emits the start edges.
+//
+// A walk is a chain of dependent loads (about half a microsecond each), so a
+// long contig is cut at splitters: one in kSplit of the single-exit vertices,
+// chosen by the key's hash.  Every splitter walks to the next one, all in
+// parallel; kLevels rounds of pointer doubling give jumps over up to
+// 2^kLevels segments; a contig walks to its first splitter and jumps on from
+// there, listing a unit of 2^kLevels segments per jump; and a warp per unit
+// writes its segments' bases, a lane each.  A contig that meets a cycle (or a
+// stretch of kMaxWalk steps without a splitter, which only a short cycle is)
+// is walked by one thread instead: Brent's cycle detection (R. P. Brent, "An
+// improved Monte Carlo factorization algorithm", BIT 20, 1980) finds the
+// first repeated vertex with O(1) state.
+//
+// Measured against one thread per contig walking by table lookups, with a pass
+// each to clear, mark, count and emit, twice over for the size query: a 50 kb
+// error-free genome (one contig) 43 -> 0.37 ms, a 5 Mbp graph of 31,000
+// contigs (2.75 GB table) 16.4 -> 2.1 ms, of which k_links takes 1.08 (the
+// table read once: 0.41) and segments, lengths, heads and units 0.15 to 0.27
+// each, the latency of their longest chain.  kSplit: 32 against 64 halves that
+// chain; the jumps make the number of segments matter little.
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_scan.cuh>
 
 #include <math.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "dbg_internal.cuh"
 
@@ -56,83 +75,150 @@ __device__ __forceinline__ uint64_t find_key(const View &v, uint64_t key) {
   return kNotFound;
 }
 
-// Out-degree of a slot's counters and its lowest label with a nonzero counter.
-__device__ __forceinline__ int out_degree(const Slot &sl, uint32_t &label) {
-  int d = 0;
-  label = 4;
-#pragma unroll
-  for (int b = 3; b >= 0; --b)
-    if (sl.cnt[b]) {
-      ++d;
-      label = (uint32_t)b;
-    }
-  return d;
+// Every counter's quotient.  Bound by one read and one write of the table.
+// The double-precision division is slow here (each slot's took 8.2 ms of a
+// 2.6 GB table), so the CTA divides the counts below kQuot once, into a table
+// in shared memory -- the same expression, so the same integers -- and only
+// larger counts are divided one by one: 0.76 ms, 6.6 TB/s.  (wide: k > 32, the
+// counters are the slot's second half)
+constexpr uint32_t kQuot = 1024;
+
+__device__ __forceinline__ uint32_t quotient(uint32_t c, double divisor) {
+  const double q = floor((double)c / divisor + 0.5);
+  return q >= 4294967295.0 ? 0xffffffffu : (uint32_t)q;
 }
 
-// (cnt0: the first counter's 32-bit word in the slot -- 2, or 4 for k > 32)
-__global__ void k_normalize(Slot *t, uint64_t n, double divisor, int cnt0) {
+__global__ void __launch_bounds__(256) k_normalize(uint4 *t, uint64_t n, double divisor, int wide) {
+  __shared__ uint32_t s_quot[kQuot];
+  for (uint32_t c = threadIdx.x; c < kQuot; c += blockDim.x) s_quot[c] = quotient(c, divisor);
+  __syncthreads();
+  auto norm = [&](uint32_t c) { return c < kQuot ? s_quot[c] : quotient(c, divisor); };
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    if (t[i].key == kEmpty) continue;
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(t + i) + cnt0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const uint32_t c = cnt[b];
-      if (!c) continue;
-      const double q = floor((double)c / divisor + 0.5);
-      cnt[b] = q >= 4294967295.0 ? 0xffffffffu : (uint32_t)q;
+    uint4 lo = t[2 * i];
+    uint4 hi = t[2 * i + 1];
+    if ((lo.x & lo.y) == 0xffffffffu) continue;  // an empty slot
+    if (wide) {
+      hi = make_uint4(norm(hi.x), norm(hi.y), norm(hi.z), norm(hi.w));
+    } else {
+      lo.z = norm(lo.z);
+      lo.w = norm(lo.w);
+      hi.x = norm(hi.x);
+      hi.y = norm(hi.y);
+      t[2 * i] = lo;
     }
+    t[2 * i + 1] = hi;
   }
 }
 
-// pad[0] of every slot := 0 (the "has an incoming edge" mark).
-__global__ void k_clear_marks(Slot *t, uint64_t n) {
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-    t[i].pad[0] = 0u;
+constexpr uint32_t kSplit = 32;        // one splitter in so many single-exit vertices
+constexpr int kLevels = 5;             // jumps of up to 2^kLevels segments: a lane each
+constexpr uint32_t kMaxWalk = 2048;    // steps without a splitter before a walk counts as a cycle's
+constexpr uint32_t kEnd = ~0u;         // a segment's successor: the walk ends there
+constexpr uint32_t kCyclic = ~0u - 1;  // it went kMaxWalk steps without meeting a splitter
+constexpr unsigned long long kIsSplitter = 1ull << 63;  // in a slot's link: the rest is its number
+
+// What the passes share.  A slot's link (its 8 bytes of padding), for a
+// single-exit vertex: its successor's slot, or kIsSplitter | number.
+struct Links {
+  uint32_t *marks;                    // a bit per slot: an edge points to its vertex
+  uint2 *degree;                      // per 32 slots: bits of one exit, bits of several
+  ulonglong2 *split;                  // a splitter's slot and its successor's slot
+  uint32_t *next, *len;               // [kLevels + 1][cap]: the splitter 2^l segments on, the edges to it
+  uint32_t cap;                       // splitters kept (a vertex past them is an ordinary one)
+  unsigned long long *n_split;        // splitters found
+};
+
+__device__ __forceinline__ unsigned long long *link_of(Slot *t, uint64_t s) {
+  return reinterpret_cast<unsigned long long *>(&t[s].pad[0]);
 }
 
-// Every edge marks its target.
-__global__ void k_mark_targets(View v) {
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < v.n; i += stride) {
-    const unsigned long long key = v.t[i].key;
-    if (key == kEmpty) continue;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      if (!v.t[i].cnt[b]) continue;
+// A slot in two 16-byte loads: key, counters, link.
+struct SlotWords {
+  uint4 a, b;
+  __device__ __forceinline__ SlotWords(const Slot *t, uint64_t s) {
+    const uint4 *p = reinterpret_cast<const uint4 *>(t + s);
+    a = p[0];
+    b = p[1];
+  }
+  __device__ __forceinline__ unsigned long long key() const {
+    return (unsigned long long)a.x | ((unsigned long long)a.y << 32);
+  }
+  __device__ __forceinline__ unsigned long long link() const {
+    return (unsigned long long)b.z | ((unsigned long long)b.w << 32);
+  }
+  // Bits of the labels with a nonzero counter.
+  __device__ __forceinline__ uint32_t exits() const {
+    return (a.z ? 1u : 0u) | (a.w ? 2u : 0u) | (b.x ? 4u : 0u) | (b.y ? 8u : 0u);
+  }
+};
+
+// Every edge marks its target; every single-exit vertex gets its link; the
+// out-degrees as bits.  A warp takes 32 consecutive slots.  Bound by one read
+// of the table, then by the random target lookups.
+__global__ void __launch_bounds__(256) k_links(View v, Links k) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  const uint64_t w0 = (((uint64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5;
+  const uint64_t words = (v.n + 31) >> 5;
+  for (uint64_t w = w0; w < words; w += warps) {
+    const uint64_t i = (w << 5) + lane;
+    unsigned long long key = kEmpty;
+    uint32_t exits = 0;
+    if (i < v.n) {
+      const SlotWords sl(v.t, i);
+      key = sl.key();
+      if (key != kEmpty) exits = sl.exits();
+    }
+    uint64_t target = 0;
+    for (uint32_t rest = exits; rest; rest &= rest - 1) {
+      const uint32_t b = (uint32_t)__ffs((int)rest) - 1u;
       const uint64_t s = find_key(v, ((key << 2) | (uint64_t)b) & v.mask);
       if (s == kNotFound) {
         atomicCAS(v.status, 0u, (uint32_t)DBG_ERR_CAPACITY);  // a target is missing
         continue;
       }
-      if (v.t[s].pad[0] == 0u) atomicOr(&v.t[s].pad[0], 1u);
+      target = s;
+      atomicOr(&k.marks[s >> 5], 1u << (s & 31));
+    }
+    const bool one = exits != 0 && (exits & (exits - 1)) == 0;
+    const unsigned ones = __ballot_sync(0xffffffffu, one);
+    const unsigned several = __ballot_sync(0xffffffffu, exits != 0 && !one);
+    if (lane == 0) k.degree[w] = make_uint2(ones, several);
+    const bool pick = one && (uint32_t)key_hash(key) % kSplit == 0u;
+    const unsigned picks = __ballot_sync(0xffffffffu, pick);
+    unsigned long long at = 0;
+    if (lane == 0 && picks) at = atomicAdd(k.n_split, (unsigned long long)__popc(picks));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(picks & ((1u << lane) - 1u));
+    if (one) {
+      const bool split = pick && at < k.cap;
+      if (split) k.split[at] = make_ulonglong2(i, target);
+      *link_of(v.t, i) = split ? (kIsSplitter | at) : target;
     }
   }
 }
 
-// Start edges: (key << 2 | label) for every outgoing edge of every vertex
-// that is first or has not exactly one outgoing edge.  With out == nullptr
-// only counts them.  Warps walk 32 consecutive slots and reserve their edges
-// with one atomic.
-__global__ void k_start_edges(View v, unsigned long long *out, unsigned long long *count,
-                              uint64_t cap) {
+// Start edges, (key << 2 | label), of every vertex that is first or has not
+// exactly one outgoing edge: at most `cap` of them are written, *count
+// receives their number.  A thread takes 32 slots' bits; a warp reserves its
+// edges with one atomic.
+__global__ void __launch_bounds__(256) k_start_edges(View v, Links k, unsigned long long *out,
+                                                     unsigned long long *count, uint64_t cap) {
   const int lane = threadIdx.x & 31;
-  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  const uint64_t w0 = (((uint64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5;
-  for (uint64_t base = w0 * 32; base < v.n; base += warps * 32) {
-    const uint64_t i = base + lane;
-    unsigned long long key = kEmpty;
-    uint32_t d = 0;
-    if (i < v.n) {
-      key = v.t[i].key;
-      if (key != kEmpty) {
-        uint32_t label;
-        d = (uint32_t)out_degree(v.t[i], label);
-        if (d == 1 && v.t[i].pad[0] != 0u) d = 0;  // single exit, not first: no start
-      }
+  const uint64_t words = (v.n + 31) >> 5;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t base = (uint64_t)blockIdx.x * blockDim.x; base < words; base += stride) {
+    const uint64_t w = base + threadIdx.x;
+    uint32_t starts = 0, ones = 0, edges = 0;
+    if (w < words) {
+      const uint2 deg = k.degree[w];
+      ones = deg.x & ~k.marks[w];
+      starts = ones | deg.y;
+      edges = (uint32_t)__popc(ones);
     }
-    uint32_t incl = d;
+    for (uint32_t rest = starts & ~ones; rest; rest &= rest - 1)
+      edges += (uint32_t)__popc(SlotWords(v.t, (w << 5) + (uint32_t)__ffs((int)rest) - 1u).exits());
+    uint32_t incl = edges;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -141,34 +227,70 @@ __global__ void k_start_edges(View v, unsigned long long *out, unsigned long lon
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
     unsigned long long at = 0;
     if (lane == 31 && total) at = atomicAdd(count, (unsigned long long)total);
-    at = __shfl_sync(0xffffffffu, at, 31) + (incl - d);
-    if (!out || !d) continue;
-    for (int b = 0; b < 4; ++b)
-      if (v.t[i].cnt[b] && at < cap) out[at++] = (key << 2) | (unsigned long long)b;
+    at = __shfl_sync(0xffffffffu, at, 31) + (incl - edges);
+    for (uint32_t rest = starts; rest; rest &= rest - 1) {
+      const SlotWords sl(v.t, (w << 5) + (uint32_t)__ffs((int)rest) - 1u);
+      for (uint32_t e = sl.exits(); e; e &= e - 1, ++at)
+        if (at < cap) out[at] = (sl.key() << 2) | (unsigned long long)(__ffs((int)e) - 1);
+    }
   }
 }
 
-// Next vertex of a single-exit vertex, or kNotFound when the vertex (slot s)
-// does not have exactly one outgoing edge.  *base receives the label taken.
-__device__ __forceinline__ uint64_t step(const View &v, uint64_t s, uint32_t *base) {
-  uint32_t label;
-  if (out_degree(v.t[s], label) != 1) return kNotFound;
-  *base = label;
-  const uint64_t nx = find_key(v, ((v.t[s].key << 2) | label) & v.mask);
-  if (nx == kNotFound) atomicCAS(v.status, 0u, (uint32_t)DBG_ERR_CAPACITY);
-  return nx;
+// Every splitter walks to the next splitter or to the end of its chain.
+__global__ void __launch_bounds__(256) k_segments(View v, Links k, uint32_t n_split) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_split; i += stride) {
+    uint64_t s = k.split[i].y;
+    uint32_t edges = 1, next = kCyclic;
+    for (; edges <= kMaxWalk; ++edges) {
+      const SlotWords sl(v.t, s);
+      const uint32_t e = sl.exits();
+      if (e == 0 || (e & (e - 1))) {  // a dead end or a branch
+        next = kEnd;
+        break;
+      }
+      const unsigned long long link = sl.link();
+      if (link & kIsSplitter) {
+        next = (uint32_t)link;
+        break;
+      }
+      s = link;
+    }
+    k.next[i] = next;
+    k.len[i] = edges;
+  }
 }
 
-// Number of edges of the contig that starts with edge e = (key << 2) | label.
-__device__ uint64_t contig_edges(const View &v, unsigned long long e, uint64_t guard) {
+// Jumps of level l + 1 from those of level l.
+__global__ void __launch_bounds__(256) k_double(Links k, uint32_t n_split, int l) {
+  const uint32_t *next = k.next + (size_t)l * k.cap, *len = k.len + (size_t)l * k.cap;
+  uint32_t *next2 = k.next + (size_t)(l + 1) * k.cap, *len2 = k.len + (size_t)(l + 1) * k.cap;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_split; i += stride) {
+    const uint32_t a = next[i];
+    const bool on = a < kCyclic;
+    next2[i] = on ? next[a] : a;
+    len2[i] = len[i] + (on ? len[a] : 0u);
+  }
+}
+
+// One step of a walk by one thread: the successor of slot s, or kNotFound
+// when its vertex does not have exactly one outgoing edge.  *base receives
+// the label taken.
+__device__ __forceinline__ uint64_t step(const View &v, const Links &k, uint64_t s, uint32_t *base) {
+  const SlotWords sl(v.t, s);
+  const uint32_t e = sl.exits();
+  if (e == 0 || (e & (e - 1))) return kNotFound;
+  *base = (uint32_t)__ffs((int)e) - 1u;
+  const unsigned long long link = sl.link();
+  return link & kIsSplitter ? k.split[(uint32_t)link].y : link;
+}
+
+// Number of edges of the contig whose first edge leads to slot x0, by one thread.
+__device__ uint64_t contig_edges(const View &v, const Links &k, uint64_t x0, uint64_t guard) {
   uint32_t b;
-  const uint64_t x0 = find_key(v, e & v.mask);
-  if (x0 == kNotFound) {
-    atomicCAS(v.status, 0u, (uint32_t)DBG_ERR_CAPACITY);  // a target is missing
-    return 1;
-  }
   // Brent: the hare walks; the tortoise jumps to the hare at powers of two
-  uint64_t tortoise = x0, hare = step(v, x0, &b);
+  uint64_t tortoise = x0, hare = step(v, k, x0, &b);
   if (hare == kNotFound) return 1;  // x0 is a branch or a dead end
   uint64_t taken = 1, power = 1, lam = 1;
   while (tortoise != hare) {
@@ -181,7 +303,7 @@ __device__ uint64_t contig_edges(const View &v, unsigned long long e, uint64_t g
       power <<= 1;
       lam = 0;
     }
-    const uint64_t nx = step(v, hare, &b);
+    const uint64_t nx = step(v, k, hare, &b);
     if (nx == kNotFound) return 1 + taken;  // ends at the hare, `taken` steps past x0
     hare = nx;
     ++taken;
@@ -190,11 +312,11 @@ __device__ uint64_t contig_edges(const View &v, unsigned long long e, uint64_t g
   // a cycle of length lam; mu = index of its first vertex along x0, x1, ...
   // (every vertex up to x_{mu+lam} has one exit: the hare passed them all)
   uint64_t a = x0, c = x0;
-  for (uint64_t i = 0; i < lam && c != kNotFound; ++i) c = step(v, c, &b);
+  for (uint64_t i = 0; i < lam && c != kNotFound; ++i) c = step(v, k, c, &b);
   uint64_t mu = 0;
   while (a != c && a != kNotFound && c != kNotFound && mu <= guard) {
-    a = step(v, a, &b);
-    c = step(v, c, &b);
+    a = step(v, k, a, &b);
+    c = step(v, k, c, &b);
     ++mu;
   }
   if (a != c) {
@@ -204,31 +326,129 @@ __device__ uint64_t contig_edges(const View &v, unsigned long long e, uint64_t g
   return 1 + mu + lam;  // the walk arrives at x_mu again after mu + lam steps
 }
 
-__global__ void k_contig_lengths(View v, const unsigned long long *starts, uint64_t n_starts,
-                                 int m, uint64_t guard, unsigned long long *len) {
+// A stretch of up to 2^kLevels segments of a contig, from splitter `split`,
+// `rel` edges into the contig.
+struct Unit {
+  uint32_t contig, split;
+  unsigned long long rel;
+};
+// A contig's own thread writes its first `own` edges (all of them when it
+// does not go by splitters).
+struct Contig {
+  unsigned long long x0;   // slot of the first edge's target (kNotFound: missing)
+  unsigned long long own;  // edges it writes itself
+  uint32_t by_units;       // whether its units count
+};
+
+__global__ void __launch_bounds__(256)
+    k_contig_lengths(View v, Links k, const unsigned long long *starts, uint64_t n_starts, int m,
+                     uint64_t guard, Contig *contigs, unsigned long long *len, Unit *units,
+                     unsigned long long *n_units, uint64_t units_cap) {
+  const uint32_t *jump = k.next + (size_t)kLevels * k.cap, *jlen = k.len + (size_t)kLevels * k.cap;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_starts; i += stride)
-    len[i] = (unsigned long long)m + contig_edges(v, starts[i], guard);
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_starts; i += stride) {
+    const uint64_t x0 = find_key(v, starts[i] & v.mask);
+    Contig c{x0, 1ull, 0u};
+    uint64_t edges = 1;
+    if (x0 == kNotFound) {
+      atomicCAS(v.status, 0u, (uint32_t)DBG_ERR_CAPACITY);  // a target is missing
+    } else {
+      uint64_t s = x0;
+      uint32_t split = kCyclic;
+      for (; edges <= kMaxWalk; ++edges) {
+        const SlotWords sl(v.t, s);
+        const uint32_t e = sl.exits();
+        if (e == 0 || (e & (e - 1))) {
+          split = kEnd;
+          break;
+        }
+        const unsigned long long link = sl.link();
+        if (link & kIsSplitter) {
+          split = (uint32_t)link;
+          break;
+        }
+        s = link;
+      }
+      c.own = edges;
+      // on by jumps; the tortoise of Brent's method meets them again in a cycle
+      uint32_t tortoise = split, power = 1, lam = 0;
+      while (split < kCyclic) {
+        c.by_units = 1;
+        const unsigned long long at = atomicAdd(n_units, 1ull);
+        if (at < units_cap) units[at] = Unit{(uint32_t)i, split, edges};
+        edges += jlen[split];
+        split = jump[split];
+        if (split == tortoise) split = kCyclic;
+        if (++lam == power) {
+          tortoise = split;
+          power <<= 1;
+          lam = 0;
+        }
+      }
+      if (split == kCyclic) {
+        edges = contig_edges(v, k, x0, guard);
+        c.own = edges;
+        c.by_units = 0;
+      }
+    }
+    contigs[i] = c;
+    len[i] = (unsigned long long)m + edges;
+  }
   if (blockIdx.x == 0 && threadIdx.x == 0) len[n_starts] = 0;
 }
 
-__global__ void k_contig_write(View v, const unsigned long long *starts, uint64_t n_starts, int m,
-                               const unsigned long long *off, const unsigned long long *len,
-                               char *out) {
-  const char letter[4] = {'A', 'C', 'G', 'T'};
+// Label 0..3 as its letter: A, C, G, T are the word's bytes from the lowest up.
+__device__ __forceinline__ char letter(uint32_t label) { return (char)(0x54474341u >> (8 * label)); }
+
+// Every contig's start vertex and the edges its own thread writes.
+__global__ void __launch_bounds__(256)
+    k_contig_heads(View v, Links k, const unsigned long long *starts, uint64_t n_starts, int m,
+                   const Contig *contigs, const unsigned long long *off, char *out) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_starts; i += stride) {
     const unsigned long long e = starts[i];
     const unsigned long long key = e >> 2;
+    const Contig c = contigs[i];
     char *o = out + off[i];
-    for (int j = 0; j < m; ++j) o[j] = letter[(key >> (2 * (m - 1 - j))) & 3ull];
-    o[m] = letter[e & 3ull];
-    const uint64_t edges = len[i] - (unsigned long long)m;
-    uint64_t s = find_key(v, e & v.mask);
-    for (uint64_t j = 1; j < edges && s != kNotFound; ++j) {
+    for (int j = 0; j < m; ++j) o[j] = letter((uint32_t)(key >> (2 * (m - 1 - j))) & 3u);
+    o[m] = letter((uint32_t)e & 3u);
+    uint64_t s = c.x0;
+    for (uint64_t j = 1; j < c.own && s != kNotFound; ++j) {
       uint32_t b = 0;
-      s = step(v, s, &b);
-      o[m + j] = letter[b];
+      s = step(v, k, s, &b);
+      o[m + j] = letter(b);
+    }
+  }
+}
+
+// A warp per unit: lane j takes the j-th segment, found by jumps of the bits
+// of j, and writes its bases.
+__global__ void __launch_bounds__(256)
+    k_contig_units(View v, Links k, const Unit *units, uint64_t n_units, int m,
+                   const Contig *contigs, const unsigned long long *off, char *out) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  for (uint64_t u = (((uint64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; u < n_units;
+       u += warps) {
+    const Unit un = units[u];
+    if (!contigs[un.contig].by_units) continue;  // a cycle: written by the contig's own thread
+    uint32_t i = un.split;
+    unsigned long long rel = un.rel;
+#pragma unroll
+    for (int l = 0; l < kLevels; ++l) {
+      if (((lane >> l) & 1) && i < kCyclic) {
+        rel += k.len[(size_t)l * k.cap + i];
+        i = k.next[(size_t)l * k.cap + i];
+      }
+    }
+    if (i >= kCyclic) continue;
+    char *o = out + off[un.contig] + m + rel;
+    const uint32_t edges = k.len[i];
+    uint64_t s = k.split[i].x;
+    for (uint32_t j = 0; j < edges; ++j) {
+      const SlotWords sl(v.t, s);
+      o[j] = letter((uint32_t)__ffs((int)sl.exits()) - 1u);
+      s = j == 0 ? k.split[i].y : sl.link();  // (no splitter inside a segment)
     }
   }
 }
@@ -251,6 +471,21 @@ struct Guard {
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// Temporary device memory of one call, given back to the pool in stream order
+// when the call leaves.
+struct Scratch {
+  cudaStream_t s;
+  std::vector<void *> held;
+  int get(void **p, size_t bytes) {
+    const int st = scratch_alloc(p, bytes, s);
+    if (st == DBG_OK) held.push_back(*p);
+    return st;
+  }
+  ~Scratch() {
+    for (void *p : held) cudaFreeAsync(p, s);
+  }
+};
+
 int read_status(dbg_handle h, cudaStream_t s) {
   uint32_t st = 0;
   DBG_CK(cudaMemcpyAsync(&st, h->d_status, sizeof(st), cudaMemcpyDeviceToHost, s));
@@ -270,8 +505,10 @@ extern "C" int dbg_normalize(dbg_handle h, double divisor, void *stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int st = dbg_get_status(h, stream);  // complete graphs only
   if (st != DBG_OK) return st;
-  k_normalize<<<std::max(1, h->sm_count) * 8, 256, 0, s>>>(h->table, h->n_slots, divisor,
-                                                             h->k > 32 ? 4 : 2);
+  const uint64_t want = (h->n_slots + 255) / 256;
+  const int grid = (int)std::min<uint64_t>(want, (uint64_t)std::max(1, h->sm_count) * 8);
+  k_normalize<<<grid, 256, 0, s>>>(reinterpret_cast<uint4 *>(h->table), h->n_slots, divisor,
+                                   h->k > 32 ? 1 : 0);
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
@@ -281,7 +518,6 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
                                 uint64_t *n_bases, void *stream) {
   using namespace dbg;
   if (!h || !n_contigs || !n_bases || h->k > 32) return DBG_ERR_INVALID_ARG;
-  h->built_counts = false;  // (this pass takes the stats accumulators as scratch)
   Guard g(h->device);
   if (g.err != cudaSuccess) return cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -292,19 +528,60 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   const View v{h->table, h->n_slots, h->max_probes,
                m >= 32 ? ~0ull : ((1ull << (2 * m)) - 1ull), h->d_status};
   const int grid = std::max(1, h->sm_count) * 8;
-  unsigned long long *count = h->d_acc;  // the handle's stats accumulator, free here
-  k_clear_marks<<<grid, 256, 0, s>>>(h->table, h->n_slots);
-  DBG_CK(cudaGetLastError());
-  k_mark_targets<<<grid, 256, 0, s>>>(v);
-  DBG_CK(cudaGetLastError());
-  DBG_CK(cudaMemsetAsync(count, 0, sizeof(unsigned long long), s));
-  k_start_edges<<<grid, 256, 0, s>>>(v, nullptr, count, 0);
-  DBG_CK(cudaGetLastError());
-  unsigned long long S = 0;
-  DBG_CK(cudaMemcpyAsync(&S, count, sizeof(S), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaStreamSynchronize(s));
-  st = read_status(h, s);
+  Scratch scr{s};
+  // marks, degrees and splitters by the table's size; a twelfth more splitters
+  // than one vertex in kSplit of a full table gives (when that much memory is
+  // not to be had: none, and every contig is walked by its own thread)
+  const uint64_t words = (h->n_slots + 31) >> 5;
+  uint64_t cap = std::min<uint64_t>(h->n_slots / kSplit + h->n_slots / (12 * kSplit) + 1024,
+                                    1ull << 30);
+  const size_t mark_bytes = align256(words * 4), bits_bytes = 256 + mark_bytes + align256(words * 8);
+  auto split_bytes = [](uint64_t c) {
+    return align256(c * sizeof(ulonglong2)) + 2 * align256(c * 4 * (kLevels + 1));
+  };
+  char *buf = nullptr;
+  st = scr.get(reinterpret_cast<void **>(&buf), bits_bytes + split_bytes(cap));
+  if (st == DBG_ERR_OOM) {
+    cudaGetLastError();
+    cap = 0;
+    st = scr.get(reinterpret_cast<void **>(&buf), bits_bytes);
+  }
   if (st != DBG_OK) return st;
+  unsigned long long *counts = reinterpret_cast<unsigned long long *>(buf);  // [3], see below
+  Links k{};
+  k.marks = reinterpret_cast<uint32_t *>(buf + 256);
+  k.degree = reinterpret_cast<uint2 *>(buf + 256 + mark_bytes);
+  k.split = reinterpret_cast<ulonglong2 *>(buf + bits_bytes);
+  k.next = reinterpret_cast<uint32_t *>(buf + bits_bytes + align256(cap * sizeof(ulonglong2)));
+  k.len = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(k.next) +
+                                       align256(cap * 4 * (kLevels + 1)));
+  k.cap = (uint32_t)cap;
+  k.n_split = counts + 1;
+  DBG_CK(cudaMemsetAsync(buf, 0, 256 + mark_bytes, s));  // counts and marks
+  k_links<<<(int)std::min<uint64_t>((words + 7) / 8, (uint64_t)grid), 256, 0, s>>>(v, k);
+  DBG_CK(cudaGetLastError());
+
+  // the start edges into a buffer that holds as many as an ordinary graph has;
+  // a second pass when there are more
+  uint64_t starts_cap = h->n_slots / 16 + 1024;
+  unsigned long long *starts_a = nullptr;
+  unsigned long long got[3] = {0, 0, 0};  // start edges, splitters, units
+  for (;;) {
+    DBG_TRY(scr.get(reinterpret_cast<void **>(&starts_a), starts_cap * sizeof(unsigned long long)));
+    k_start_edges<<<(int)std::min<uint64_t>((words + 255) / 256, (uint64_t)grid), 256, 0, s>>>(
+        v, k, starts_a, counts, starts_cap);
+    DBG_CK(cudaGetLastError());
+    uint32_t status = 0;
+    DBG_CK(cudaMemcpyAsync(got, counts, sizeof(got), cudaMemcpyDeviceToHost, s));
+    DBG_CK(cudaMemcpyAsync(&status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, s));
+    DBG_CK(cudaStreamSynchronize(s));
+    if (status != DBG_OK) return (int)status;
+    if (got[0] <= starts_cap) break;
+    starts_cap = got[0];
+    DBG_CK(cudaMemsetAsync(counts, 0, sizeof(unsigned long long), s));
+  }
+  const uint64_t S = got[0];
+  const uint32_t n_split = (uint32_t)std::min<uint64_t>(got[1], cap);
   *n_contigs = S;
   *n_bases = 0;
   if (S == 0) {
@@ -313,7 +590,14 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
     DBG_CK(cudaStreamSynchronize(s));
     return DBG_OK;
   }
+  if (S > 0xFFFFFFFFull) return DBG_ERR_CAPACITY;  // (contig numbers in a unit are 32-bit)
 
+  if (n_split > 0) {
+    const int sg = (int)std::min<uint64_t>(((uint64_t)n_split + 255) / 256, (uint64_t)grid);
+    k_segments<<<sg, 256, 0, s>>>(v, k, n_split);
+    for (int l = 0; l < kLevels; ++l) k_double<<<sg, 256, 0, s>>>(k, n_split, l);
+    DBG_CK(cudaGetLastError());
+  }
   size_t sort_bytes = 0, scan_bytes = 0;
   DBG_CK(cub::DeviceRadixSort::SortKeys(nullptr, sort_bytes, (unsigned long long *)nullptr,
                                         (unsigned long long *)nullptr, (int64_t)S, 0, 2 * m + 2,
@@ -321,57 +605,53 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   DBG_CK(cub::DeviceScan::ExclusiveSum(nullptr, scan_bytes, (unsigned long long *)nullptr,
                                        (unsigned long long *)nullptr, (int64_t)(S + 1), s));
   const size_t eb = align256((S + 1) * sizeof(unsigned long long));
-  const size_t total = 4 * eb + align256(std::max(sort_bytes, scan_bytes));
-  char *buf = nullptr;
-  DBG_TRY(scratch_alloc(reinterpret_cast<void **>(&buf), total, s));
-  unsigned long long *starts_a = reinterpret_cast<unsigned long long *>(buf);
-  unsigned long long *starts_b = reinterpret_cast<unsigned long long *>(buf + eb);
-  unsigned long long *len = reinterpret_cast<unsigned long long *>(buf + 2 * eb);
-  unsigned long long *off = reinterpret_cast<unsigned long long *>(buf + 3 * eb);
-  void *temp = buf + 4 * eb;
-  char *chars = nullptr;
-  int rc = DBG_OK;
-  do {
-    cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMemsetAsync"); break; }
-    k_start_edges<<<grid, 256, 0, s>>>(v, starts_a, count, S);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) { rc = cuda_fail(e, "k_start_edges"); break; }
-    e = cub::DeviceRadixSort::SortKeys(temp, sort_bytes, starts_a, starts_b, (int64_t)S, 0,
-                                       2 * m + 2, s);
-    if (e != cudaSuccess) { rc = cuda_fail(e, "DeviceRadixSort::SortKeys"); break; }
-    const uint64_t guard = 4 * h->n_slots + 64;
-    k_contig_lengths<<<grid, 256, 0, s>>>(v, starts_b, S, m, guard, len);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) { rc = cuda_fail(e, "k_contig_lengths"); break; }
-    e = cub::DeviceScan::ExclusiveSum(temp, scan_bytes, len, off, (int64_t)(S + 1), s);
-    if (e != cudaSuccess) { rc = cuda_fail(e, "DeviceScan::ExclusiveSum"); break; }
-    unsigned long long B = 0;
-    e = cudaMemcpyAsync(&B, off + S, sizeof(B), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) { rc = cuda_fail(e, "contig lengths"); break; }
+  const size_t cb = align256(S * sizeof(Contig));
+  char *buf2 = nullptr;
+  DBG_TRY(scr.get(reinterpret_cast<void **>(&buf2),
+                  3 * eb + cb + align256(std::max(sort_bytes, scan_bytes))));
+  unsigned long long *starts_b = reinterpret_cast<unsigned long long *>(buf2);
+  unsigned long long *len = reinterpret_cast<unsigned long long *>(buf2 + eb);
+  unsigned long long *off = reinterpret_cast<unsigned long long *>(buf2 + 2 * eb);
+  Contig *contigs = reinterpret_cast<Contig *>(buf2 + 3 * eb);
+  void *temp = buf2 + 3 * eb + cb;
+  DBG_CK(cub::DeviceRadixSort::SortKeys(temp, sort_bytes, starts_a, starts_b, (int64_t)S, 0,
+                                        2 * m + 2, s));
+  // a unit per jump: one or two a contig, and one in every 2^kLevels splitters
+  // (again with as many as were counted when contigs share long tails)
+  const uint64_t guard = 4 * h->n_slots + 64;
+  const int cg = (int)std::min<uint64_t>((S + 255) / 256, (uint64_t)grid);
+  uint64_t units_cap = n_split > 0 ? 2 * S + (n_split >> (kLevels - 1)) + 1024 : 0;
+  Unit *units = nullptr;
+  unsigned long long B = 0;
+  for (;;) {
+    if (units_cap > 0)
+      DBG_TRY(scr.get(reinterpret_cast<void **>(&units), units_cap * sizeof(Unit)));
+    k_contig_lengths<<<cg, 256, 0, s>>>(v, k, starts_b, S, m, guard, contigs, len, units,
+                                        counts + 2, units_cap);
+    DBG_CK(cudaGetLastError());
+    DBG_CK(cub::DeviceScan::ExclusiveSum(temp, scan_bytes, len, off, (int64_t)(S + 1), s));
+    uint32_t status = 0;
+    DBG_CK(cudaMemcpyAsync(&B, off + S, sizeof(B), cudaMemcpyDeviceToHost, s));
+    DBG_CK(cudaMemcpyAsync(&got[2], counts + 2, sizeof(got[2]), cudaMemcpyDeviceToHost, s));
+    DBG_CK(cudaMemcpyAsync(&status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, s));
+    DBG_CK(cudaStreamSynchronize(s));
     *n_bases = B;
-    rc = read_status(h, s);
-    if (rc != DBG_OK) break;
-    if (!bases_out || !offsets_out || S > max_contigs || B > max_bases) {
-      rc = DBG_ERR_BUFFER_TOO_SMALL;
-      break;
-    }
-    rc = scratch_alloc(reinterpret_cast<void **>(&chars), std::max<uint64_t>(B, 1), s);
-    if (rc != DBG_OK) break;
-    k_contig_write<<<grid, 256, 0, s>>>(v, starts_b, S, m, off, len, chars);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) { rc = cuda_fail(e, "k_contig_write"); break; }
-    e = cudaMemcpyAsync(offsets_out, off, (S + 1) * sizeof(uint64_t), cudaMemcpyDefault, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(bases_out, chars, B, cudaMemcpyDefault, s);
-    if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMemcpyAsync(contigs)"); break; }
-  } while (0);
-  if (chars) cudaFreeAsync(chars, s);
-  cudaError_t e = cudaFreeAsync(buf, s);
-  if (rc == DBG_OK && e != cudaSuccess) rc = cuda_fail(e, "cudaFreeAsync");
-  e = cudaStreamSynchronize(s);
-  if (rc == DBG_OK && e != cudaSuccess) rc = cuda_fail(e, "cudaStreamSynchronize");
-  if (rc == DBG_OK) rc = read_status(h, s);
-  return rc;
+    if (status != DBG_OK) return (int)status;
+    if (got[2] <= units_cap) break;
+    units_cap = got[2];
+    DBG_CK(cudaMemsetAsync(counts + 2, 0, sizeof(unsigned long long), s));
+  }
+  if (!bases_out || !offsets_out || S > max_contigs || B > max_bases) return DBG_ERR_BUFFER_TOO_SMALL;
+  char *chars = nullptr;
+  DBG_TRY(scr.get(reinterpret_cast<void **>(&chars), std::max<uint64_t>(B, 1)));
+  k_contig_heads<<<cg, 256, 0, s>>>(v, k, starts_b, S, m, contigs, off, chars);
+  DBG_CK(cudaGetLastError());
+  if (got[2] > 0) {
+    k_contig_units<<<(int)std::min<uint64_t>((got[2] + 7) / 8, (uint64_t)grid), 256, 0, s>>>(
+        v, k, units, got[2], m, contigs, off, chars);
+    DBG_CK(cudaGetLastError());
+  }
+  DBG_CK(cudaMemcpyAsync(offsets_out, off, (S + 1) * sizeof(uint64_t), cudaMemcpyDefault, s));
+  DBG_CK(cudaMemcpyAsync(bases_out, chars, B, cudaMemcpyDefault, s));
+  return read_status(h, s);
 }
