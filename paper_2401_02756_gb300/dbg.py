@@ -398,19 +398,25 @@ class Graph:
         """The graph's contigs (Alg. 5), ordered by (start vertex, label)."""
         L = load()
         n, b = ctypes.c_uint64(), ctypes.c_uint64()
-        st = L.dbg_find_contigs(self.handle, None, 0, None, 0, ctypes.byref(n), ctypes.byref(b),
-                                _stream(stream))
-        if st not in (OK, ERR_BUFFER_TOO_SMALL):
-            raise DbgError(st, "dbg_find_contigs")
+        # buffers that an ordinary graph's contigs fit (untouched pages cost
+        # nothing), and exact ones when they do not: one call instead of a
+        # sizing call and a second one
+        slots = self.info()["n_slots"]
+        max_n, max_b = slots // 64 + 1024, slots // 4 + 65536
+        while True:
+            bases = np.empty(max_b, dtype=np.uint8)
+            offs = np.empty(max_n + 1, dtype=np.uint64)
+            st = L.dbg_find_contigs(self.handle, bases.ctypes.data, max_b, offs.ctypes.data, max_n,
+                                    ctypes.byref(n), ctypes.byref(b), _stream(stream))
+            if st != ERR_BUFFER_TOO_SMALL:
+                break
+            max_n, max_b = n.value, b.value
+        _check(st, "dbg_find_contigs")
         if n.value == 0:
             return []
-        bases = np.empty(b.value, dtype=np.uint8)
-        offs = np.empty(n.value + 1, dtype=np.uint64)
-        _check(L.dbg_find_contigs(self.handle, bases.ctypes.data, bases.size, offs.ctypes.data,
-                                  n.value, ctypes.byref(n), ctypes.byref(b), _stream(stream)),
-               "dbg_find_contigs")
-        raw = bases.tobytes().decode("ascii")
-        return [raw[int(offs[i]):int(offs[i + 1])] for i in range(n.value)]
+        raw = bases[:b.value].tobytes().decode("ascii")
+        ends = offs[:n.value + 1].tolist()
+        return [raw[i:j] for i, j in zip(ends, ends[1:])]
 
     def export_into(self, keys, counts, stream=None) -> int:
         """One dbg_export_sorted call into caller-owned CUDA tensors (keys
