@@ -344,22 +344,24 @@ int dbg_stats(dbg_handle h, uint64_t *n_vertices, uint64_t *n_edges, void *strea
  * in-place device outputs (below) may have served as scratch.  Temporary
  * device memory comes from a stream-ordered pool the library keeps per
  * device (up to 4 GiB of it stays cached between calls) and is released to
- * it before return: about 6 bytes per vertex (the sorted slot indices and the
- * lists of runs of keys that share their first 16 bases) when both outputs
- * are 16-byte aligned device buffers and k <= 32 -- the sort then runs
- * inside keys_out and counts_out, whose max_n rows it uses, and the
- * compaction that fills them counts the vertices, so no separate counting
- * pass over the table is made -- otherwise about 40 bytes per vertex (80 for
- * k > 32).  Errors: INVALID_ARG, OOM, CUDA, BUFFER_TOO_SMALL, and the sticky
- * status (nothing exported when it is set). */
+ * it before return.  When both outputs are 16-byte aligned device buffers
+ * the records are sorted inside them, and the temporary memory is the sort's
+ * bins (up to about 8 MB, or a byte for every 25 vertices if that is more);
+ * a graph built on the binned path places its records in the handle's event
+ * buffer first, and one with k > 32 in up to 4 GiB of the pool (32 bytes a
+ * vertex).  Other outputs go through temporary ones (24 bytes a row, 32 for
+ * k > 32).  Keys crowded into a few prefixes are left to a radix sort (about
+ * 6 bytes a vertex in place, otherwise 40, 80 for k > 32).  Errors:
+ * INVALID_ARG, OOM, CUDA, BUFFER_TOO_SMALL, and the sticky status (nothing
+ * exported when it is set). */
 int dbg_export_sorted(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t max_n,
                       uint64_t *n_out, void *stream);
 
 /* Device bytes of scratch dbg_export_sorted_with needs for a graph of
  * n_vertices vertices (k <= 32, a table of at most 2^32 slots): the sort's
- * histograms, one slot index per vertex and the lists of runs of keys that
- * share a prefix.  0 for arguments it does not take.  Needs a device (the
- * sort sizes its work for it). */
+ * bins, and for the radix sort behind it its histograms, one slot index per
+ * vertex and the lists of runs of keys that share a prefix.  0 for arguments
+ * it does not take.  Needs a device (the sort sizes its work for it). */
 uint64_t dbg_export_scratch_bytes(int k, uint64_t n_vertices, uint64_t n_slots);
 
 /* dbg_export_sorted with every byte of device memory from the caller: for a

@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "dbg_binned.cuh"
+#include "dbg_export.cuh"
 #include "dbg_tiles.cuh"
 #include "dbg_tma.cuh"
 
@@ -2006,6 +2007,10 @@ int launch_binned_batch(const ItemDesc *items, const uint64_t *want, int n,
   }
   if (!capturing) DBG_CK(cudaEventRecord(sc.done, s));
   return DBG_OK;
+}
+
+uint64_t bin_ev2_bytes(dbg_handle h) {
+  return h->bin.ev2 ? ev2_capacity(h->bin.cap) * sizeof(uint64_t) : 0;
 }
 
 uint64_t batch_scratch_bytes(int dev) {

@@ -18,6 +18,7 @@
 
 #include <algorithm>
 
+#include "dbg_export.cuh"
 #include "dbg_internal.cuh"
 
 namespace dbg {
@@ -606,52 +607,21 @@ bool in_place_outputs(const uint64_t *keys_out, const uint32_t *counts_out) {
          ((uintptr_t)keys_out & 15u) == 0 && ((uintptr_t)counts_out & 15u) == 0;
 }
 
-// Compaction of the prefix export into in-place outputs of `stride` rows,
-// counting the occupied slots as it goes (no separate counting pass): at most
-// `stride` (prefix, index) pairs are written -- prefixes at keys_out as 32-bit
-// words, indices after them -- and *D_out receives the count.  Returns the
-// sticky status (or NEEDS_GROW) instead when the graph has one.
-int compact_counted(dbg_handle h, uint64_t *keys_out, uint64_t stride, uint64_t *D_out,
-                    cudaStream_t s) {
-  const int bits = 2 * (h->k - 1);
-  const int pshift = bits > 32 ? bits - 32 : 0;
-  uint32_t *pa = reinterpret_cast<uint32_t *>(keys_out);
-  DBG_CK(cudaMemsetAsync(h->d_acc, 0, sizeof(unsigned long long), s));
-  const int sms = std::max(1, h->sm_count);
-  k_compact_prefix<<<sms * 8, kCompactBlock, 0, s>>>(h->table, h->n_slots, pshift, pa, pa + stride,
-                                                     h->d_acc, stride);
-  DBG_CK(cudaGetLastError());
-  unsigned long long D = 0, spilled = 0;
-  uint32_t status = 0;
-  DBG_CK(cudaMemcpyAsync(&D, h->d_acc, sizeof(D), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaMemcpyAsync(&status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaMemcpyAsync(&spilled, h->d_spill_count, sizeof(spilled), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaStreamSynchronize(s));
-  if (status != DBG_OK) return (int)status;
-  if (spilled > 0) return DBG_ERR_NEEDS_GROW;
-  *D_out = D;
-  return DBG_OK;
-}
-
 // The prefix-sort export of D vertices (tables of at most 2^32 slots).
 // Buffers: two (prefix, index) pairs for the sort, the sorted indices, the
 // sort's temporary space, a counter, the long-run flag and the run lists.  In
 // place (both outputs 16-byte aligned device buffers) the pairs live in
 // keys_out (8 bytes a row) and counts_out, and the gather writes the outputs
-// directly; otherwise everything is temporary.  `stride` (in place): the rows
-// the pair layout assumes (D when 0); `compacted`: compact_counted has
-// already written the pairs with that stride.  Returns DBG_ERR_CAPACITY (not
+// directly; otherwise everything is temporary.  Returns DBG_ERR_CAPACITY (not
 // a graph error: the caller falls back to the full-width sort) when a run of
 // equal prefixes is too long.
 int export_prefix(dbg_handle h, uint64_t D, uint64_t *keys_out, uint32_t *counts_out,
-                  cudaStream_t s, void *caller, uint64_t caller_bytes, uint64_t stride = 0,
-                  bool compacted = false) {
+                  cudaStream_t s, void *caller, uint64_t caller_bytes) {
   const int bits = 2 * (h->k - 1);
   const int pshift = bits > 32 ? bits - 32 : 0;
   const int pbits = bits > 32 ? 32 : bits;
   const bool in_place = in_place_outputs(keys_out, counts_out);
-  if ((caller || compacted) && !in_place) return DBG_ERR_INVALID_ARG;
-  if (stride == 0) stride = D;
+  if (caller && !in_place) return DBG_ERR_INVALID_ARG;
   PrefixScratch ps{};
   DBG_TRY(prefix_scratch(h->k, D, in_place, ps));
   // one wave of the run pass: as many CTAs as fit on the device at once
@@ -680,9 +650,9 @@ int export_prefix(dbg_handle h, uint64_t D, uint64_t *keys_out, uint32_t *counts
   uint4 *counts;
   if (in_place) {
     pa = reinterpret_cast<uint32_t *>(keys_out);
-    ia = pa + stride;
+    ia = pa + D;
     pb = reinterpret_cast<uint32_t *>(counts_out);
-    ib = pb + stride;
+    ib = pb + D;
     keys = reinterpret_cast<unsigned long long *>(keys_out);
     counts = reinterpret_cast<uint4 *>(counts_out);
   } else {
@@ -701,12 +671,10 @@ int export_prefix(dbg_handle h, uint64_t D, uint64_t *keys_out, uint32_t *counts
     cudaError_t e = cudaMemsetAsync(buf, 0, 16, s);  // count, flag
     if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMemsetAsync"); break; }
     const int sms = std::max(1, h->sm_count);
-    if (!compacted) {
-      k_compact_prefix<<<sms * 8, kCompactBlock, 0, s>>>(h->table, h->n_slots, pshift, pa, ia,
-                                                         count, D);
-      e = cudaGetLastError();
-      if (e != cudaSuccess) { rc = cuda_fail(e, "k_compact_prefix"); break; }
-    }
+    k_compact_prefix<<<sms * 8, kCompactBlock, 0, s>>>(h->table, h->n_slots, pshift, pa, ia, count,
+                                                       D);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) { rc = cuda_fail(e, "k_compact_prefix"); break; }
     cub::DoubleBuffer<uint32_t> dk(pa, pb), dv(ia, ib);
     size_t temp_bytes = ps.temp;
     e = cub::DeviceRadixSort::SortPairs(temp, temp_bytes, dk, dv, (int64_t)D, 0, pbits, s);
@@ -765,6 +733,49 @@ int prefix_scratch_bytes(int k, uint64_t D, uint64_t &bytes) {
 }  // namespace
 }  // namespace dbg
 
+namespace dbg {
+namespace {
+
+// The radix sorts, for graphs the sort by bins leaves: keys crowded into few
+// bins, tables of 2^32 slots and more.  (D vertices, counted before.)
+int export_radix(dbg_handle h, uint64_t D, uint64_t *keys_out, uint32_t *counts_out,
+                 cudaStream_t s) {
+  if (h->k > 32) return export_sorted_wide(h, D, keys_out, counts_out, s);
+  if (h->n_slots <= 0xFFFFFFFFull) {
+    const int st = export_prefix(h, D, keys_out, counts_out, s, nullptr, 0);
+    if (st != DBG_ERR_CAPACITY) return st;  // (a long run of equal prefixes: full width)
+    return export_pairs<uint32_t>(h, D, keys_out, counts_out, s);
+  }
+  return export_pairs<unsigned long long>(h, D, keys_out, counts_out, s);
+}
+
+// The sort by bins into outputs that are not aligned device buffers (host
+// memory, or one of the two not asked for): into temporary ones, then copied.
+int export_bins_copied(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t max_n,
+                       uint64_t *D, cudaStream_t s, bool *too_dense) {
+  const uint64_t rows = std::min(max_n, h->n_slots);
+  const size_t key_bytes = h->k > 32 ? 16 : 8, kb = align256(rows * key_bytes);
+  char *buf = nullptr;
+  DBG_TRY(scratch_alloc(reinterpret_cast<void **>(&buf), kb + align256(rows * 16), s));
+  int rc = export_bins(h, reinterpret_cast<uint64_t *>(buf), reinterpret_cast<uint32_t *>(buf + kb),
+                       rows, D, s, nullptr, 0, too_dense);
+  if (rc == DBG_OK && !*too_dense && *D <= rows && *D > 0) {
+    cudaError_t e = cudaSuccess;
+    if (keys_out) e = cudaMemcpyAsync(keys_out, buf, *D * key_bytes, cudaMemcpyDefault, s);
+    if (e == cudaSuccess && counts_out)
+      e = cudaMemcpyAsync(counts_out, buf + kb, *D * 16, cudaMemcpyDefault, s);
+    if (e != cudaSuccess) rc = cuda_fail(e, "cudaMemcpyAsync(export)");
+  }
+  cudaError_t e = cudaFreeAsync(buf, s);
+  if (rc == DBG_OK && e != cudaSuccess) rc = cuda_fail(e, "cudaFreeAsync");
+  e = cudaStreamSynchronize(s);
+  if (rc == DBG_OK && e != cudaSuccess) rc = cuda_fail(e, "cudaStreamSynchronize");
+  return rc;
+}
+
+}  // namespace
+}  // namespace dbg
+
 extern "C" int dbg_export_sorted(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out,
                                  uint64_t max_n, uint64_t *n_out, void *stream) {
   using namespace dbg;
@@ -775,40 +786,34 @@ extern "C" int dbg_export_sorted(dbg_handle h, uint64_t *keys_out, uint32_t *cou
 
   uint64_t D = 0;
   int st;
-  if (h->k <= 32 && h->n_slots <= 0xFFFFFFFFull && max_n > 0 &&
-      in_place_outputs(keys_out, counts_out)) {
-    // in place: the compaction into the outputs counts the vertices itself
-    st = compact_counted(h, keys_out, max_n, &D, s);
+  if (h->n_slots <= 0xFFFFFFFFull && max_n > 0 && (keys_out || counts_out)) {
+    bool too_dense = false;
+    st = in_place_outputs(keys_out, counts_out)
+             ? export_bins(h, keys_out, counts_out, max_n, &D, s, nullptr, 0, &too_dense)
+             : export_bins_copied(h, keys_out, counts_out, max_n, &D, s, &too_dense);
     if (st != DBG_OK) return st;
     *n_out = D;
     if (D > max_n) return DBG_ERR_BUFFER_TOO_SMALL;
-    if (D == 0) return DBG_OK;
-    st = export_prefix(h, D, keys_out, counts_out, s, nullptr, 0, max_n, true);
-    if (st != DBG_ERR_CAPACITY) return st;  // (a long run of equal prefixes: full width)
-    return export_pairs<uint32_t>(h, D, keys_out, counts_out, s);
+    return too_dense ? export_radix(h, D, keys_out, counts_out, s) : DBG_OK;
   }
   st = dbg_stats(h, &D, nullptr, stream);
   if (st != DBG_OK) return st;
   *n_out = D;
   if (D > max_n) return DBG_ERR_BUFFER_TOO_SMALL;
   if (D == 0) return DBG_OK;
-  if (h->k > 32) return export_sorted_wide(h, D, keys_out, counts_out, s);
-  if (h->n_slots <= 0xFFFFFFFFull) {
-    st = export_prefix(h, D, keys_out, counts_out, s, nullptr, 0);
-    if (st != DBG_ERR_CAPACITY) return st;  // (a long run of equal prefixes: full width)
-    return export_pairs<uint32_t>(h, D, keys_out, counts_out, s);
-  }
-  return export_pairs<unsigned long long>(h, D, keys_out, counts_out, s);
+  return export_radix(h, D, keys_out, counts_out, s);
 }
 
 extern "C" uint64_t dbg_export_scratch_bytes(int k, uint64_t n_vertices, uint64_t n_slots) {
   using namespace dbg;
   if (k < 2 || k > 32 || n_slots > 0xFFFFFFFFull) return 0;
   const uint64_t D = std::max<uint64_t>(n_vertices, 1);
-  uint64_t a = 0, b = 0;  // the prefix sort's, and the full-width fall-back's
+  // the sort by bins', and the prefix sort's and the full-width sort's behind it
+  uint64_t a = 0, b = 0, c = 0;
   if (prefix_scratch_bytes(k, D, a) != DBG_OK) return 0;
   if (in_place_scratch_bytes<uint32_t>(D, 2 * (k - 1), b) != DBG_OK) return 0;
-  return std::max(a, b);
+  if (export_bins_scratch(k, D, c) != DBG_OK) return 0;
+  return std::max(a, std::max(b, c));
 }
 
 extern "C" int dbg_export_sorted_with(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out,
@@ -819,16 +824,24 @@ extern "C" int dbg_export_sorted_with(dbg_handle h, uint64_t *keys_out, uint32_t
   Guard g(h->device);
   if (g.err != cudaSuccess) return cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  uint64_t D = 0;
-  const bool counted = max_n > 0 && scratch && in_place_outputs(keys_out, counts_out);
-  int st = counted ? compact_counted(h, keys_out, max_n, &D, s) : dbg_stats(h, &D, nullptr, stream);
-  if (st != DBG_OK) return st;
+  uint64_t D = 0, need = 0;
+  DBG_TRY(export_bins_scratch(h->k, std::min(max_n, h->n_slots), need));
+  bool too_dense = true;
+  if (max_n > 0 && scratch && ((uintptr_t)scratch & 255u) == 0 && scratch_bytes >= need &&
+      in_place_outputs(keys_out, counts_out)) {
+    DBG_TRY(export_bins(h, keys_out, counts_out, max_n, &D, s, scratch, scratch_bytes, &too_dense));
+  } else {
+    DBG_TRY(dbg_stats(h, &D, nullptr, stream));
+  }
   *n_out = D;
   if (D > max_n) return DBG_ERR_BUFFER_TOO_SMALL;
   if (D == 0) return DBG_OK;
+  if (!too_dense) {  // (scratch below what the size query asks for is refused, used or not)
+    DBG_TRY(prefix_scratch_bytes(h->k, D, need));
+    return scratch_bytes < need ? DBG_ERR_INVALID_ARG : DBG_OK;
+  }
   if (!keys_out || !counts_out || !scratch) return DBG_ERR_INVALID_ARG;
-  st = export_prefix(h, D, keys_out, counts_out, s, scratch, scratch_bytes, counted ? max_n : 0,
-                     counted);
+  const int st = export_prefix(h, D, keys_out, counts_out, s, scratch, scratch_bytes);
   if (st != DBG_ERR_CAPACITY) return st;  // (a long run of equal prefixes: full width)
   return export_pairs<uint32_t>(h, D, keys_out, counts_out, s, scratch, scratch_bytes);
 }
