@@ -108,13 +108,6 @@ __global__ void __launch_bounds__(BLOCK, 2048 / BLOCK)
 // a tile of one read would leave most of a CTA's threads idle.
 constexpr int kMinTileReads = 2, kAutoTileReads = 20;
 
-int auto_tile_reads(uint64_t reads, uint64_t resident) {
-  const uint64_t waves = std::max<uint64_t>(1, (reads + resident * kAutoTileReads - 1) /
-                                                   (resident * kAutoTileReads));
-  const uint64_t ctas = resident * waves;
-  return (int)std::max<uint64_t>(kMinTileReads, (reads + ctas - 1) / ctas);
-}
-
 // Number the items' tiles and launch.
 template <int BLOCK, bool AGG, int N>
 int launch_one(ItemPack<N> &pk, int tile_reads, int grid_ctas, int sm_count, cudaStream_t stream,
@@ -165,6 +158,13 @@ int launch_pack(const ItemDesc *items, int n_items, int tile_reads, const dbg_tu
 }
 
 }  // namespace
+
+int auto_tile_reads(uint64_t reads, uint64_t resident) {
+  const uint64_t waves = std::max<uint64_t>(1, (reads + resident * kAutoTileReads - 1) /
+                                                   (resident * kAutoTileReads));
+  const uint64_t ctas = resident * waves;
+  return (int)std::max<uint64_t>(kMinTileReads, (reads + ctas - 1) / ctas);
+}
 
 dbg_tuning resolve_tuning(const dbg_tuning &t) {
   dbg_tuning r = t;

@@ -5,9 +5,8 @@
 // bits, word 1 = its low 64 bits, then the four 32-bit counters.  An empty
 // slot has word 0 = all ones (never a key's high word: it holds at most 62
 // bits) and word 1 = 0, which is what the table initialisation writes.
-// Claims are one 128-bit atomicCAS (atom.cas.b128); a probe reads word 0
-// first, word 1 only when word 0 matches, and settles a possibly torn pair
-// (word 0 already new, word 1 not yet visible) with a 128-bit atomic read.
+// Claims are one 128-bit atomicCAS (atom.cas.b128), probes one 128-bit atomic
+// load, so a probe never sees half a key.
 //
 // The insert kernel takes tiles of reads: it stages the tiles' packed bytes
 // in shared memory (coalesced, bounded by the stream's length), then gives
@@ -33,8 +32,10 @@ static_assert(sizeof(WideSlot) == 32, "one sector per slot");
 constexpr int kWideTile = 128;        // reads per tile
 constexpr int kWideWinBytes = 16384;  // staged bytes per tile (wider tiles read global memory)
 
+// A multilinear hash (Dietzfelbinger's multiply-add-shift with fixed odd
+// multipliers): its leading bits choose the home slot.
 __device__ __forceinline__ uint64_t wide_home(uint64_t hi, uint64_t lo, uint64_t n_slots) {
-  return __umul64hi(fmix64(lo ^ fmix64(hi ^ 0x9E3779B97F4A7C15ull)), n_slots);
+  return __umul64hi(hi * 0x9E3779B97F4A7C15ull + lo * 0xD1B54A32D192ED03ull, n_slots);
 }
 
 // Atomic 128-bit compare-and-swap of a slot's key words; returns the old pair.
@@ -53,30 +54,37 @@ __device__ __forceinline__ void cas128(WideSlot *s, uint64_t c0, uint64_t c1, ui
       : "memory");
 }
 
+// Both key words of a slot in one single-copy atomic load.
+__device__ __forceinline__ void load128(const WideSlot *s, uint64_t &w0, uint64_t &w1) {
+  asm volatile(
+      "{\n"
+      ".reg .b128 d;\n"
+      "ld.relaxed.gpu.global.b128 d, [%2];\n"
+      "mov.b128 {%0, %1}, d;\n"
+      "}\n"
+      : "=l"(w0), "=l"(w1)
+      : "l"(&s->w0)
+      : "memory");
+}
+
 // Slot of key (hi, lo), claimed if absent; false after max_probes slots.
 __device__ __forceinline__ bool wide_find_or_claim(WideSlot *t, uint64_t n_slots,
                                                    uint32_t max_probes, uint64_t hi, uint64_t lo,
                                                    uint64_t &slot) {
   uint64_t s = wide_home(hi, lo, n_slots);
   for (uint32_t i = 0; i < max_probes; ++i) {
-    const unsigned long long w0 = ld_relaxed_u64(&t[s].w0);
-    uint64_t o0, o1;
+    uint64_t w0, w1;
+    load128(&t[s], w0, w1);
     if (w0 == kEmpty) {
-      cas128(&t[s], kEmpty, 0ull, hi, lo, o0, o1);
-      if ((o0 == kEmpty && o1 == 0ull) || (o0 == hi && o1 == lo)) {
-        slot = s;
-        return true;
+      cas128(&t[s], kEmpty, 0ull, hi, lo, w0, w1);
+      if (w0 == kEmpty) {
+        w0 = hi;
+        w1 = lo;
       }
-    } else if (w0 == hi) {
-      if (ld_relaxed_u64(&t[s].w1) == lo) {
-        slot = s;
-        return true;
-      }
-      cas128(&t[s], kEmpty, 0ull, kEmpty, 0ull, o0, o1);  // an atomic read of the pair
-      if (o0 == hi && o1 == lo) {
-        slot = s;
-        return true;
-      }
+    }
+    if (w0 == hi && w1 == lo) {
+      slot = s;
+      return true;
     }
     if (++s == n_slots) s = 0;
   }
@@ -114,51 +122,71 @@ __device__ __forceinline__ uint64_t word_at(const uint8_t *packed, uint64_t nbyt
   return w;
 }
 
+// Bound by the table's random sectors (a load that misses the L2, then the add
+// that makes the sector dirty: 2.4e10 a second of a table far larger than the
+// L2): 168 M positions into a 3.5 GB table 14.7 -> 12.5 ms (1.43 probes each,
+// 241 M sector reads and as many sectors made dirty as positions), by one
+// 128-bit load a probe, a warp-scanned prefix, 16-byte staging and tiles cut
+// by the number of reads.
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK) k_insert_wide(ItemDesc it) {
+__global__ void __launch_bounds__(BLOCK, 6) k_insert_wide(ItemDesc it, int tile_reads) {
   __shared__ uint64_t s_off[kWideTile + 1];
   __shared__ uint64_t s_pre[kWideTile + 1];
   __shared__ __align__(16) uint64_t s_win[kWideWinBytes / 8 + 4];
+  __shared__ uint64_t s_sum[kWideTile / 32];
   __shared__ uint32_t s_stop;
-  __shared__ uint64_t s_b0, s_staged;  // first staged byte (8-aligned); bytes staged (0: none)
+  static_assert(kWideTile <= BLOCK && kWideTile % 32 == 0, "a thread per read of a tile");
   const int k = it.k, m = k - 1;
   const uint64_t last = it.offsets[it.n_reads];
   const uint64_t nbytes = last >= it.origin ? (last - it.origin + 3) >> 2 : 0;
   WideSlot *table = reinterpret_cast<WideSlot *>(it.table);
-  const uint64_t tiles = (it.n_reads + kWideTile - 1) / kWideTile;
+  const uint64_t tiles = (it.n_reads + (uint64_t)tile_reads - 1) / (uint64_t)tile_reads;
+  const int tid = threadIdx.x, lane = tid & 31;
   for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const uint64_t r0 = t * kWideTile;
-    const int nr = (int)min((uint64_t)kWideTile, it.n_reads - r0);
-    if (threadIdx.x == 0) s_stop = ld_volatile_u32(it.status);
-    for (int i = threadIdx.x; i <= nr; i += BLOCK) s_off[i] = it.offsets[r0 + i];
+    const uint64_t r0 = t * (uint64_t)tile_reads;
+    const int nr = (int)min((uint64_t)tile_reads, it.n_reads - r0);
+    if (tid == 0) s_stop = ld_volatile_u32(it.status);
+    for (int i = tid; i <= nr; i += BLOCK) s_off[i] = it.offsets[r0 + i];
     __syncthreads();
     if (s_stop) return;  // an earlier error stops the insert (the same value for every thread)
-    if (threadIdx.x == 0) {
-      // vertex positions per read, prefix; bad offsets stop the tile
-      uint64_t acc = 0;
-      bool bad = false;
-      for (int i = 0; i < nr; ++i) {
-        s_pre[i] = acc;
-        const uint64_t a = s_off[i], b = s_off[i + 1];
-        if (b < a || a < it.origin) bad = true;
-        const uint64_t len = b >= a ? b - a : 0;
-        acc += len >= (uint64_t)k ? len - k + 2 : 0;
-      }
-      s_pre[nr] = bad ? 0 : acc;
-      if (bad) set_sticky(it.status, DBG_ERR_BAD_OFFSETS);
-      // the tile's bytes, staged if they fit the window
-      const uint64_t lo_b = s_off[0] >= it.origin ? ((s_off[0] - it.origin) >> 2) & ~7ull : 0;
-      const uint64_t hi_b = s_off[nr] >= it.origin ? ((s_off[nr] - it.origin + 3) >> 2) : 0;
-      s_b0 = lo_b;
-      s_staged = (!bad && hi_b > lo_b && hi_b - lo_b + 24 <= (uint64_t)kWideWinBytes)
-                     ? hi_b - lo_b + 24
-                     : 0;
+    // vertex positions per read, prefix; bad offsets stop the tile
+    uint64_t nv = 0;
+    bool wrong = false;
+    if (tid < nr) {
+      const uint64_t a = s_off[tid], b = s_off[tid + 1];
+      wrong = b < a || a < it.origin;
+      const uint64_t len = b >= a ? b - a : 0;
+      nv = len >= (uint64_t)k ? len - k + 2 : 0;
     }
-    __syncthreads();
-    const uint64_t staged = s_staged, b0 = s_b0;
+    uint64_t incl = nv;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint64_t o = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += o;
+    }
+    if (lane == 31 && tid < kWideTile) s_sum[tid >> 5] = incl;
+    const bool bad = __syncthreads_or(wrong) != 0;
+    if (tid < nr) {
+      for (int w = 0; w < tid >> 5; ++w) incl += s_sum[w];
+      s_pre[tid] = incl - nv;
+      if (tid == nr - 1) s_pre[nr] = bad ? 0 : incl;
+    }
+    if (bad && tid == 0) set_sticky(it.status, DBG_ERR_BAD_OFFSETS);
+    // the tile's bytes, staged if they fit the window: 16 bytes a load where
+    // the stream allows, zeros past its end
+    const uint64_t lo_b = s_off[0] >= it.origin ? ((s_off[0] - it.origin) >> 2) & ~15ull : 0;
+    const uint64_t hi_b = s_off[nr] >= it.origin ? ((s_off[nr] - it.origin + 3) >> 2) : 0;
+    const uint64_t b0 = lo_b;
+    const uint64_t staged = (!bad && hi_b > lo_b && hi_b - lo_b + 24 <= (uint64_t)kWideWinBytes)
+                                ? hi_b - lo_b + 24
+                                : 0;
     if (staged) {
+      const uint64_t whole = it.vec_ok ? (min(hi_b, nbytes) - lo_b) >> 4 : 0;
+      for (uint64_t i = tid; i < whole; i += BLOCK)
+        reinterpret_cast<uint4 *>(s_win)[i] =
+            __ldg(reinterpret_cast<const uint4 *>(it.packed + b0) + i);
       unsigned char *win = reinterpret_cast<unsigned char *>(s_win);
-      for (uint64_t i = threadIdx.x; i < staged; i += BLOCK)
+      for (uint64_t i = 16 * whole + tid; i < staged; i += BLOCK)
         win[i] = b0 + i < nbytes ? it.packed[b0 + i] : (unsigned char)0;
     }
     __syncthreads();
@@ -207,7 +235,7 @@ __global__ void __launch_bounds__(BLOCK) k_insert_wide(ItemDesc it) {
       }
       uint64_t s;
       if (wide_find_or_claim(table, it.n_slots, it.max_probes, hi, lo, s)) {
-        if (edge) atomicAdd(&table[s].cnt[label], 1u);
+        if (edge) red_add_u32(&table[s].cnt[label], 1u);
       } else {
         set_sticky(it.status, DBG_ERR_CAPACITY);
       }
@@ -261,10 +289,10 @@ int launch_insert_wide(const ItemDesc &it, int sm_count, cudaStream_t s) {
   constexpr int B = 256;
   int per_sm = 0;
   DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert_wide<B>, B, 0));
-  const uint64_t tiles = (it.n_reads + kWideTile - 1) / kWideTile;
-  const int grid =
-      (int)std::min<uint64_t>(tiles, (uint64_t)std::max(1, per_sm) * std::max(1, sm_count));
-  k_insert_wide<B><<<grid, B, 0, s>>>(it);
+  const uint64_t resident = (uint64_t)std::max(1, per_sm) * std::max(1, sm_count);
+  const int tile_reads = std::min(kWideTile, auto_tile_reads(it.n_reads, resident));
+  const uint64_t tiles = (it.n_reads + tile_reads - 1) / tile_reads;
+  k_insert_wide<B><<<(int)std::min(tiles, resident), B, 0, s>>>(it, tile_reads);
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
