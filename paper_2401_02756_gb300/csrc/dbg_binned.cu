@@ -360,7 +360,7 @@ __device__ __forceinline__ uint32_t cta_exclusive_prefix(uint32_t local, uint32_
 // count pass (the tiled path), one atomic on the region's bucket cursor per
 // round; after a count pass, the slice's run start in the region (reserved
 // at the start of the slice) + the events of the region already placed.
-template <int BLOCK>
+template <int BLOCK, bool SMALL>
 struct ScatterVisitor {
   static constexpr bool kUniformRounds = true;
   static constexpr int kRound = BLOCK * kRun;  // events of one round = one flush
@@ -385,7 +385,8 @@ struct ScatterVisitor {
   __device__ void vertex(bool valid, uint64_t key, bool edge, uint32_t label, int, int sub,
                          const VertexCtx &c) {
     if (valid) {
-      const uint32_t p = (uint32_t)c.region0 + (uint32_t)(home_slot(key, c.n_slots) >> shift);
+      const uint32_t p = (uint32_t)c.region0 +
+                         (uint32_t)(home_of_hash<SMALL>(key_hash(key), c.n_slots) >> shift);
       ev[sub] = make_event(key, edge, label);
       where[sub] = (p << 16) | atomicAdd(&hist[p], 1u);
     } else {
@@ -456,7 +457,7 @@ constexpr size_t scatter_smem(int tile_reads, int parts) {
          (size_t)parts * (4 + 4 + 8 + 8) + 64;
 }
 
-template <int BLOCK, int N>
+template <int BLOCK, int N, bool SMALL>
 __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
     k_bin_scatter(const __grid_constant__ ItemPack<N> pk, int tile_reads, int shift, int parts,
                   uint64_t t0, uint64_t t1, uint64_t slices, const uint32_t *hist,
@@ -466,9 +467,9 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
   if (ld_volatile_u32(use_binned) == 0u) return;
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned char *p = smem + tile_smem_bytes(tile_reads);
-  ScatterVisitor<BLOCK> vis;
+  ScatterVisitor<BLOCK, SMALL> vis;
   vis.sorted = reinterpret_cast<uint64_t *>(p);
-  p += (size_t)ScatterVisitor<BLOCK>::kRound * 8;
+  p += (size_t)ScatterVisitor<BLOCK, SMALL>::kRound * 8;
   vis.gbase = reinterpret_cast<unsigned long long *>(p);
   p += (size_t)parts * 8;
   vis.cur = reinterpret_cast<unsigned long long *>(p);
@@ -790,9 +791,10 @@ __device__ __forceinline__ int unit_region(const unsigned long long *unit_base, 
 
 // Tile of an event inside its region: its home slot in the region's table
 // (n_slots slots), relative to the region's first tile.
+template <bool SMALL>
 __device__ __forceinline__ uint32_t tile_in_region(uint64_t ev, uint64_t n_slots,
                                                    uint64_t first_tile) {
-  const uint64_t home = home_slot(ev >> 3, n_slots);
+  const uint64_t home = home_of_hash<SMALL>(key_hash(ev >> 3), n_slots);
   return (uint32_t)((home >> kTileLog2) - first_tile);
 }
 
@@ -822,7 +824,7 @@ constexpr int kMaxBinsPerThread = 4;  // tiles per region / tile scatter threads
 template <int BLOCK, bool STAGED>
 constexpr size_t tile_scatter_smem(int tpr) {
   return (size_t)BLOCK * kBatch * (8 + 4) + (STAGED ? ((size_t)BLOCK * kBatch + 2) * 8 : 0) +
-         (size_t)tpr * 20;
+         (size_t)tpr * 24;
 }
 
 // A CTA's chunks, in order: its units blockIdx.x, + gridDim.x, ..., each cut
@@ -861,7 +863,7 @@ __device__ __forceinline__ void stage_chunk(uint64_t *stage, const uint64_t *ev,
   if (bytes) bulk_load(stage, ev + x0, bytes, bar);
 }
 
-template <int BLOCK, bool STAGED>
+template <int BLOCK, bool STAGED, bool SMALL>
 __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)  // two CTAs of 512 threads per SM
     k_tile_scatter(const uint64_t *__restrict__ ev, uint64_t *__restrict__ ev2, uint64_t ev2_cap,
                    const unsigned long long *begin, const unsigned long long *counts, TileAux aux,
@@ -877,6 +879,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)  // two CTAs of 512 threa
   uint32_t *s_fit = s_off + tpr;   // tpr: events of the run that fit the bucket
   uint32_t *s_at = s_fit + tpr;    // tpr: their place, relative to the region's first bucket
   uint32_t *s_ovf = s_at + tpr;    // tpr: the rest's place in the overflow area (~0: none)
+  uint32_t *s_dst = s_ovf + tpr;   // tpr: place minus chunk position when all of it fits, else ~0
   __shared__ uint32_t s_warp[BLOCK / 32];
   __shared__ __align__(8) uint64_t s_bar;
   __shared__ uint32_t s_failed;
@@ -925,7 +928,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)  // two CTAs of 512 threa
 #pragma unroll
     for (int r = 0; r < kBatch; ++r) {
       if (e[r] != kEmpty) {
-        const uint32_t t = tile_in_region(e[r], ns, first_tile);
+        const uint32_t t = tile_in_region<SMALL>(e[r], ns, first_tile);
         where[r] = (t << 16) | atomicAdd(&s_hist[t], 1u);
       }
     }
@@ -976,6 +979,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)  // two CTAs of 512 threa
         const uint32_t fit = at >= cap ? 0u : min(h, cap - at);
         s_fit[j] = fit;
         s_at[j] = (uint32_t)((uint64_t)j * cap + at);
+        s_dst[j] = fit == h ? s_at[j] - s_off[j] : ~0u;
         if (fit < h) {
           const unsigned long long o = atomicAdd(aux.overflow, (unsigned long long)(h - fit));
           if (o + (h - fit) > over_cap) {  // the area is full: the direct insert takes over
@@ -1001,6 +1005,12 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)  // two CTAs of 512 threa
     const uint32_t n = (uint32_t)(c.y - c.x);
     for (uint32_t i = tid; i < n; i += BLOCK) {
       const uint32_t t = s_tile[i];
+      const uint32_t dst = s_dst[t];
+      if (dst != ~0u) {  // (one look-up instead of three: split 13.56 -> 13.16 ms at 100 Mbp;
+                         // below, also the rare place whose difference is ~0)
+        out[dst + i] = s_ev[i];
+        continue;
+      }
       const uint32_t r = i - s_off[t];
       const uint32_t fit = s_fit[t];
       if (r < fit) {
@@ -1064,7 +1074,7 @@ constexpr size_t kSoaTileBytes = (size_t)kTileSlots * (8 + 16);
 // failed (max_probes inside the tile), or deferred (the probe left the tile).
 // Slots are examined in probe order exactly as one at a time would: the first
 // slot from home that holds the key or is empty decides.
-template <class Tile>
+template <bool SMALL, class Tile>
 __device__ __forceinline__ void tile_event(uint64_t e, const Tile &tile, uint8_t *fp, uint64_t first,
                                            int len, uint64_t n_slots, uint32_t max_probes,
                                            uint32_t *status, SpillRecord *spill,
@@ -1074,7 +1084,7 @@ __device__ __forceinline__ void tile_event(uint64_t e, const Tile &tile, uint8_t
                                            unsigned long long *deferred_n) {
   const unsigned long long key = e >> 3;
   const uint64_t h = key_hash(key);
-  const int home = (int)(__umul64hi(h, n_slots) - first);  // = home_slot(key) - first
+  const int home = (int)(home_of_hash<SMALL>(h, n_slots) - first);  // = home_slot(key) - first
   const uint32_t f = slot_fp(h), f4 = f * 0x01010101u;
   // the key can only sit in [home, limit): max_probes slots, or up to the tile's end
   const bool capped = max_probes <= (uint32_t)(len - home);
@@ -1142,7 +1152,7 @@ __device__ __forceinline__ void empty_soa_tile(const SoaTile &tile, uint32_t *fp
   for (int i = threadIdx.x; i < kFpBytes / 4; i += blockDim.x) fp32[i] = 0u;
 }
 
-template <int BLOCK, bool FRESH, int N>
+template <int BLOCK, bool FRESH, int N, bool SMALL>
 __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 threads per SM
     k_tile_apply(const __grid_constant__ ItemPack<N> pk, const uint64_t *__restrict__ ev2,
                  uint64_t *ev, const unsigned long long *begin, TileAux aux, int parts,
@@ -1260,10 +1270,10 @@ __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 thr
         for (int r = 0; r < kBatch; ++r) {
           if (e[r] == kEmpty) continue;
           if constexpr (FRESH)
-            tile_event(e[r], soa, fp, first, len, n_slots, it.max_probes, status, it.spill,
+            tile_event<SMALL>(e[r], soa, fp, first, len, n_slots, it.max_probes, status, it.spill,
                        it.spill_cap, it.spill_count, p, ev, begin, aux.deferred_n);
           else
-            tile_event(e[r], aos, fp, first, len, n_slots, it.max_probes, status, it.spill,
+            tile_event<SMALL>(e[r], aos, fp, first, len, n_slots, it.max_probes, status, it.spill,
                        it.spill_cap, it.spill_count, p, ev, begin, aux.deferred_n);
         }
         base += (uint64_t)BLOCK * kBatch;
@@ -1626,18 +1636,18 @@ int launch_apply_m(dbg_handle h, const MetaView &mv, const BinGeometry &geo, int
   }
 }
 
-template <int BT, bool STAGED>
+template <int BT, bool STAGED, bool SMALL>
 int launch_tile_scatter(const BinScratch &sc, const MetaView &mv, const TileAux &aux, int parts,
                         uint64_t unit, int tpr, int sms, cudaStream_t s, uint32_t *status) {
   if (tpr > kMaxBinsPerThread * BT) return DBG_ERR_INVALID_ARG;  // (the launch sizes BT by tpr)
   const size_t smem = tile_scatter_smem<BT, STAGED>(tpr);
   // (set even below 48 KB: the kernel's static shared memory counts too)
-  DBG_CK(cudaFuncSetAttribute(k_tile_scatter<BT, STAGED>,
+  DBG_CK(cudaFuncSetAttribute(k_tile_scatter<BT, STAGED, SMALL>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_scatter<BT, STAGED>, BT,
+  DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_scatter<BT, STAGED, SMALL>, BT,
                                                        smem));
-  k_tile_scatter<BT, STAGED><<<std::max(1, per_sm) * sms, BT, smem, s>>>(
+  k_tile_scatter<BT, STAGED, SMALL><<<std::max(1, per_sm) * sms, BT, smem, s>>>(
       sc.ev, sc.ev2, ev2_capacity(sc.cap), mv.begin, mv.counts, aux, parts, unit, tpr, status,
       mv.flag);
   DBG_CK(cudaGetLastError());
@@ -1661,10 +1671,10 @@ struct Marks {
 // tiles of kScatterTileReads reads.  The direct kernel does the call instead
 // when the events do not fit the scratch.  The scratch's event buffer, second
 // buffer and aux area must exist.  `status` receives a timeout of the split.
-template <int N>
-int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int parts,
+template <int N, bool SMALL>
+int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int parts,
                 uint64_t tiles, uint64_t walk_tiles, const dbg_tuning &tuning, int sms,
-                cudaStream_t s, bool fresh, const Marks &mark, const InputParts *input = nullptr) {
+                cudaStream_t s, bool fresh, const Marks &mark, const InputParts *input) {
   const int scatter_reads = scatter_tile_reads(tuning);
   const MetaView mv = meta_view(sc);
   const int tpr = 1 << (shift - kTileLog2);
@@ -1709,10 +1719,10 @@ int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int par
     // read-modify-write of partly written sectors)
     constexpr int BS = 512;
     const size_t smem = scatter_smem<BS>(scatter_reads, parts);
-    DBG_CK(cudaFuncSetAttribute(k_bin_scatter<BS, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    DBG_CK(cudaFuncSetAttribute(k_bin_scatter<BS, N, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem));
     int per_sm = 0;
-    DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bin_scatter<BS, N>, BS, smem));
+    DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bin_scatter<BS, N, SMALL>, BS, smem));
     // one launch over every read tile, or (input arriving in parts) one per
     // part, each after its part's copy: tiles [cut[c], cut[c + 1]) hold reads
     // that have all arrived (a tile split by a cut goes to the later part)
@@ -1731,7 +1741,7 @@ int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int par
       const uint64_t sl = std::min<uint64_t>(b - a, kBinSlices);
       const int grid = (int)std::max<uint64_t>(
           1, std::min<uint64_t>(sl, (uint64_t)std::max(1, per_sm) * sms));
-      k_bin_scatter<BS, N><<<grid, BS, smem, s>>>(pk, scatter_reads, shift, parts, a, b, sl,
+      k_bin_scatter<BS, N, SMALL><<<grid, BS, smem, s>>>(pk, scatter_reads, shift, parts, a, b, sl,
                                                   mv.hist, mv.cursor, sc.ev, sc.cap, mv.ctr,
                                                   mv.flag, mv.begin + 1);
       DBG_CK(cudaGetLastError());
@@ -1751,13 +1761,13 @@ int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int par
   if (tuning.split_threads > 0 && tpr <= kMaxBinsPerThread * tuning.split_threads)
     bt = tuning.split_threads;
   if (bt == 256) {
-    DBG_TRY((launch_tile_scatter<256, true>(sc, mv, aux, parts, unit, tpr, sms, s,
+    DBG_TRY((launch_tile_scatter<256, true, SMALL>(sc, mv, aux, parts, unit, tpr, sms, s,
                                             items[0].status)));
   } else if (bt == 512) {  // (1024 tiles: two bins per thread; measured faster than 1024 threads)
-    DBG_TRY((launch_tile_scatter<512, true>(sc, mv, aux, parts, unit, tpr, sms, s,
+    DBG_TRY((launch_tile_scatter<512, true, SMALL>(sc, mv, aux, parts, unit, tpr, sms, s,
                                             items[0].status)));
   } else {
-    DBG_TRY((launch_tile_scatter<1024, false>(sc, mv, aux, parts, unit, tpr, sms, s,
+    DBG_TRY((launch_tile_scatter<1024, false, SMALL>(sc, mv, aux, parts, unit, tpr, sms, s,
                                               items[0].status)));
   }
   mark(5, s);
@@ -1768,7 +1778,7 @@ int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int par
     // probe latencies
     constexpr int BA = 512;
     const size_t smem = (fresh ? kSoaTileBytes : (size_t)kTileSlots * sizeof(Slot)) + kFpBytes;
-    auto kern = fresh ? k_tile_apply<BA, true, N> : k_tile_apply<BA, false, N>;
+    auto kern = fresh ? k_tile_apply<BA, true, N, SMALL> : k_tile_apply<BA, false, N, SMALL>;
     DBG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BA, smem));
@@ -1795,6 +1805,19 @@ int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int par
   if (st != DBG_OK) return st;
   mark(8, s);
   return DBG_OK;
+}
+
+// tables of 2^32 slots and more (137 GB) take the general home slot
+template <int N>
+int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int parts, uint64_t tiles,
+                uint64_t walk_tiles, const dbg_tuning &tuning, int sms, cudaStream_t s, bool fresh,
+                const Marks &mark, const InputParts *input = nullptr) {
+  bool small = true;
+  for (int i = 0; i < n; ++i) small = small && items[i].n_slots <= 0xFFFFFFFFull;
+  return small ? tiled_chain_of<N, true>(sc, items, n, shift, parts, tiles, walk_tiles, tuning, sms,
+                                         s, fresh, mark, input)
+               : tiled_chain_of<N, false>(sc, items, n, shift, parts, tiles, walk_tiles, tuning, sms,
+                                          s, fresh, mark, input);
 }
 
 }  // namespace
@@ -1882,12 +1905,12 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
   {
     constexpr int BS = 512;
     const size_t smem = scatter_smem<BS>(tile_reads, geo.parts);
-    DBG_CK(cudaFuncSetAttribute(k_bin_scatter<BS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    DBG_CK(cudaFuncSetAttribute(k_bin_scatter<BS, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem));
     int per_sm = 0;
-    DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bin_scatter<BS, 1>, BS, smem));
+    DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bin_scatter<BS, 1, false>, BS, smem));
     const int grid = (int)std::min<uint64_t>(slices, (uint64_t)std::max(1, per_sm) * sms);
-    k_bin_scatter<BS, 1><<<grid, BS, smem, s>>>(pk, tile_reads, geo.shift, geo.parts, 0,
+    k_bin_scatter<BS, 1, false><<<grid, BS, smem, s>>>(pk, tile_reads, geo.shift, geo.parts, 0,
                                                 walk_tiles, slices, mv.hist, mv.cursor, h->bin.ev,
                                                 h->bin.cap, mv.ctr, mv.flag, nullptr);
     DBG_CK(cudaGetLastError());
