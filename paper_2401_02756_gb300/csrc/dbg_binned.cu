@@ -50,7 +50,17 @@ constexpr int kRun = 8;             // consecutive vertex positions per thread (
 constexpr int kTileLog2 = 11;
 constexpr int kTileSlots = 1 << kTileLog2;  // 2048 slots: 64 KB as 32-byte slots, 48 KB split
 constexpr int kMaxTilesPerRegion = 4096;    // beyond this the streaming apply is used
-constexpr int kTiledShift = 21;             // automatic regions of the tiled path: 1024 tiles
+
+// Automatic regions of the tiled path: 2^18 to 2^21 slots, so that a table has
+// at most 256 of them (few regions: long runs in the scatter) and no larger
+// ones than that takes (few tiles per region: long runs in the split).  A
+// build at 2^18 / 2^19 / 2^20 / 2^21 slots: 9.9 M slots 0.72 / 0.73 / 0.75 /
+// 0.80 ms, 86 M 3.65 / 3.61 / 3.66 / 3.77, 131 M 7.93 / 7.82 / 7.88 / 8.15,
+// 657 M (more parts than fit below 2^19) - / 63 / 41.6 / 40.7.  A chain of
+// tables scatters one table's reads at a time, so it takes four times the
+// regions: 24 tables of 50 kb to 2 Mbp 7.32 / 7.36 / 7.54 / 7.90 ms.
+constexpr int kTiledShiftMin = 18, kTiledShiftMax = 21;
+constexpr uint64_t kTableRegions = 256, kChainRegions = 1024;
 
 // The tiled path's bookkeeping for one chain of items (one or many tables).
 // Regions never span two tables: item i's table is cut into regions
@@ -197,13 +207,17 @@ __global__ void __launch_bounds__(1024)
 // totals[i] = vertex positions of item i's reads, sum of max(0, len - k + 2),
 // and edges[i] = its k-mers, sum of max(0, len - k + 1) (grid: x strides over
 // the item's reads, y = item).
-// clear: also zero every item's sticky status and spill count (a rebuild
-// from empty; this is the chain's first kernel, so every later one sees it).
+// The chain's first kernel: it also zeroes the tiles' fill counts and, with
+// `clear`, every item's sticky status and spill count (a rebuild from empty).
 template <int N>
 __global__ void k_bin_totals(const __grid_constant__ ItemPack<N> pk, unsigned long long *totals,
-                             unsigned long long *edges, int clear) {
+                             unsigned long long *edges, int clear, uint32_t *fill, uint64_t tiles) {
   const int i = blockIdx.y;
   if (i >= pk.n_items) return;
+  // the tiles' fill counts, for the split
+  for (uint64_t t = ((uint64_t)i * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; t < tiles;
+       t += (uint64_t)gridDim.x * gridDim.y * blockDim.x)
+    fill[t] = 0u;
   if (clear && blockIdx.x == 0 && threadIdx.x == 0) {
     *pk.d[i].status = 0u;
     *pk.d[i].spill_count = 0ull;
@@ -1413,6 +1427,15 @@ int ceil_log2(uint64_t x) {
 
 }  // namespace
 
+namespace {
+
+int tiled_shift(uint64_t n_slots, uint64_t regions) {
+  return std::min(kTiledShiftMax,
+                  std::max(kTiledShiftMin, ceil_log2((n_slots + regions - 1) / regions)));
+}
+
+}  // namespace
+
 BinGeometry bin_geometry(uint64_t n_slots, int region_log2) {
   BinGeometry g;
   g.shift = std::max(region_log2 > 0 ? region_log2 : kBinMinShift,
@@ -1428,9 +1451,9 @@ struct MetaView {
   unsigned long long *cursor;  // kBinMaxParts
   unsigned long long *ctr;     // 4 counters; ctr[3] holds the use-binned flag
   uint32_t *flag;
-  unsigned long long *apply_ctr;  // kBinApplyCounters
   unsigned long long *totals;  // kBatchItems: vertex positions per item
   unsigned long long *edges;   // kBatchItems: edges (k-mers) per item
+  unsigned long long *apply_ctr;  // kBinApplyCounters
   uint32_t *hist;              // kBinSlices * kBinMaxParts
 };
 
@@ -1442,10 +1465,10 @@ MetaView meta_view(const BinScratch &sc) {
   v.cursor = v.counts + kBinMaxParts;
   v.ctr = v.cursor + kBinMaxParts;
   v.flag = reinterpret_cast<uint32_t *>(v.ctr + 3);
-  v.apply_ctr = v.ctr + 4;
-  v.totals = v.apply_ctr + (size_t)kBinMaxParts * kBinApplyCounters;
+  v.totals = v.ctr + 4;
   v.edges = v.totals + kBatchItems;
-  v.hist = reinterpret_cast<uint32_t *>(v.edges + kBatchItems);
+  v.apply_ctr = v.edges + kBatchItems;
+  v.hist = reinterpret_cast<uint32_t *>(v.apply_ctr + (size_t)kBinMaxParts * kBinApplyCounters);
   return v;
 }
 
@@ -1684,11 +1707,7 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
   pk.total_tiles = walk_tiles;
   for (int i = 0; i < n; ++i) pk.d[i] = items[i];
   const uint64_t slices = std::min<uint64_t>(walk_tiles, kBinSlices);
-  DBG_CK(cudaMemsetAsync(mv.ctr, 0, 4 * sizeof(unsigned long long), s));
-  DBG_CK(cudaMemsetAsync(mv.counts, 0, parts * sizeof(unsigned long long), s));
-  DBG_CK(cudaMemsetAsync(mv.totals, 0, n * sizeof(unsigned long long), s));
-  DBG_CK(cudaMemsetAsync(mv.edges, 0, n * sizeof(unsigned long long), s));
-  DBG_CK(cudaMemsetAsync(aux.fill, 0, tiles * sizeof(uint32_t), s));
+  DBG_CK(cudaMemsetAsync(mv.ctr, 0, kBinClearedBytes, s));  // counters, totals, edges
   sc.counters = aux.overflow;
   mark(1, s);
   // bucket sizing: positions per item, then buckets and the region table
@@ -1702,7 +1721,8 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
     const uint64_t want = std::min<uint64_t>((max_reads + 256 * 32 - 1) / (256 * 32),
                                              (uint64_t)std::max(1, 16384 / n));
     const int gx = (int)std::max<uint64_t>(want, (uint64_t)std::max(1, (sms * 4 + n - 1) / n));
-    k_bin_totals<N><<<dim3(gx, n), 256, 0, s>>>(pk, mv.totals, mv.edges, fresh ? 1 : 0);
+    k_bin_totals<N><<<dim3(gx, n), 256, 0, s>>>(pk, mv.totals, mv.edges, fresh ? 1 : 0, aux.fill,
+                                                tiles);
     DBG_CK(cudaGetLastError());
     k_bin_buckets<N><<<1, 1024, 0, s>>>(pk, mv.totals, mv.edges, fresh ? 1 : 0, shift, parts,
                                         mv.begin, mv.cursor, sc.cap, mv.ctr, mv.flag, aux);
@@ -1833,12 +1853,12 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
   constexpr int B = 256;
   const dbg_tuning t = resolve_tuning(tuning);
   // the tiled apply re-partitions each region by tile, so its first pass can
-  // use coarser regions (fewer of them: a cheaper scatter); measured best at
-  // 1024 tiles per region on the 100 Mbp workload (2^20-slot regions:
-  // 47.6 ms a build, 2^21: 46.9 ms, 2^22: 51.3 ms)
+  // use coarser regions than the streaming one
   const bool want_tiled = t.apply_mode != 1 && h->bin.cap < kMaxChainEvents;
   const BinGeometry geo =
-      bin_geometry(h->n_slots, t.region_log2 > 0 ? t.region_log2 : (want_tiled ? kTiledShift : 0));
+      bin_geometry(h->n_slots, t.region_log2 > 0 ? t.region_log2
+                               : want_tiled      ? tiled_shift(h->n_slots, kTableRegions)
+                                                 : 0);
   const int sms = std::max(1, h->sm_count);
   const Marks mark{h, call};
 
@@ -1873,7 +1893,7 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
   // gap-free region ranges, then the apply (a rebuild empties the table
   // first: this apply reads it)
   DBG_TRY(wait_input(input, s));
-  if (fresh) DBG_TRY(launch_table_init(h->table, h->n_slots, s));
+  if (fresh) DBG_TRY(launch_empty(h, s));
   const MetaView mv = meta_view(h->bin);
   const int tile_reads = std::min(t.tile_reads, B);
   const uint64_t walk_tiles = (it.n_reads + (uint64_t)tile_reads - 1) / (uint64_t)tile_reads;
@@ -1958,7 +1978,11 @@ int launch_binned_batch(const ItemDesc *items, const uint64_t *want, int n,
                         const dbg_tuning &tuning, int sm_count, cudaStream_t s, bool fresh) {
   if (n <= 0) return DBG_OK;
   const dbg_tuning t = resolve_tuning(tuning);
-  const int shift = t.region_log2 > 0 ? std::max(t.region_log2, kTileLog2) : kTiledShift;
+  uint64_t slots = 0;  // (of a chain's worth of tables)
+  for (int i = 0; i < n; ++i) slots += items[i].n_slots;
+  if (n > kBatchItems) slots = slots / (uint64_t)n * kBatchItems;
+  const int shift = t.region_log2 > 0 ? std::max(t.region_log2, kTileLog2)
+                                      : tiled_shift(slots, kChainRegions);
   const int sms = std::max(1, sm_count);
   int dev = 0;
   DBG_CK(cudaGetDevice(&dev));

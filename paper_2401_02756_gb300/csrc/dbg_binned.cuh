@@ -17,9 +17,9 @@ constexpr int kBinMinShift = 18;                     // automatic: regions of at
 constexpr int kBinApplyCounters = 64;                // apply: chunk counters per launch, at most
 
 // meta area: begin[kBinMaxParts + 1] | counts[kBinMaxParts] | cursor[kBinMaxParts] |
-// counters[4] (the last holds the flag) | apply counters[kBinMaxParts][kBinApplyCounters] |
-// item totals[kBatchItems] | item edges[kBatchItems] | slice histograms
-// u32[kBinSlices][kBinMaxParts]
+// counters[4] (the last holds the flag) | item totals[kBatchItems] |
+// item edges[kBatchItems] | apply counters[kBinMaxParts][kBinApplyCounters] |
+// slice histograms u32[kBinSlices][kBinMaxParts]
 constexpr size_t kBinMetaBytes =
     ((size_t)kBinMaxParts + 1) * 8 + 2 * (size_t)kBinMaxParts * 8 + 4 * 8 +
     (size_t)kBinMaxParts * kBinApplyCounters * 8 + 2 * (size_t)kBatchItems * 8 +
@@ -29,6 +29,9 @@ struct BinGeometry {
   int shift;  // region = slots [p << shift, (p + 1) << shift)
   int parts;
 };
+
+// What a tiled chain clears of it: the counters, totals and edges.
+constexpr size_t kBinClearedBytes = (4 + 2 * (size_t)kBatchItems) * 8;
 
 // Regions of 2^region_log2 slots (0: automatic), widened until there are at
 // most kBinMaxParts of them.

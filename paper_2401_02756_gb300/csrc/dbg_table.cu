@@ -99,8 +99,13 @@ struct DeviceGuard {
 };
 
 // K2: every slot EMPTY with zero counters; two 16-byte stores per slot.
-__global__ void k_table_init(uint4 *t, uint64_t n_vec, const uint32_t *gate) {
-  if (gate != nullptr && ld_volatile_u32(gate) != 0u) return;
+// (status, spilled: if not null, cleared too)
+__global__ void k_table_init(uint4 *t, uint64_t n_vec, uint32_t *status,
+                             unsigned long long *spilled) {
+  if (status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
+    *status = 0u;
+    *spilled = 0ull;
+  }
   const uint4 head = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);
   const uint4 tail = make_uint4(0u, 0u, 0u, 0u);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -137,7 +142,8 @@ int stream_grid(int sm_count, int per_sm) { return std::max(1, sm_count) * per_s
 
 }  // namespace
 
-int launch_table_init(Slot *table, uint64_t n_slots, cudaStream_t stream, const uint32_t *gate) {
+static int table_init(Slot *table, uint64_t n_slots, uint32_t *status, unsigned long long *spilled,
+                      cudaStream_t stream) {
   int dev = 0, sms = 0;
   DBG_CK(cudaGetDevice(&dev));
   DBG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -145,9 +151,18 @@ int launch_table_init(Slot *table, uint64_t n_slots, cudaStream_t stream, const 
   uint64_t want = (n_vec + 255) / 256;
   const int grid = (int)std::min<uint64_t>(want, (uint64_t)stream_grid(sms, 8));
   k_table_init<<<std::max(grid, 1), 256, 0, stream>>>(reinterpret_cast<uint4 *>(table), n_vec,
-                                                      gate);
+                                                      status, spilled);
   DBG_CK(cudaGetLastError());
   return DBG_OK;
+}
+
+int launch_table_init(Slot *table, uint64_t n_slots, cudaStream_t stream) {
+  return table_init(table, n_slots, nullptr, nullptr, stream);
+}
+
+int launch_empty(dbg_handle h, cudaStream_t stream) {
+  h->built_counts = false;
+  return table_init(h->table, h->n_slots, h->d_status, h->d_spill_count, stream);
 }
 
 int launch_stats(const Slot *table, uint64_t n_slots, unsigned long long *acc, cudaStream_t stream,
@@ -367,12 +382,7 @@ extern "C" int dbg_reset(dbg_handle h, void *stream) {
   h->built_counts = false;
   DeviceGuard g(h->device);
   if (g.err != cudaSuccess) return dbg::cuda_fail(g.err, "cudaSetDevice");
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int st = dbg::launch_table_init(h->table, h->n_slots, s);
-  if (st != DBG_OK) return st;
-  DBG_CK(cudaMemsetAsync(h->d_status, 0, sizeof(uint32_t), s));
-  DBG_CK(cudaMemsetAsync(h->d_spill_count, 0, sizeof(unsigned long long), s));
-  return DBG_OK;
+  return dbg::launch_empty(h, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int dbg_set_tuning(dbg_handle h, const dbg_tuning *t) {
@@ -538,9 +548,10 @@ bool want_binned(dbg_handle h) {
   return h->n_slots * sizeof(dbg::Slot) >= dbg::kBinMinTableBytes;
 }
 
-// fresh: the table's contents are discarded first (dbg_build_reads); the
-// binned path folds that into its tiled apply, the others empty the table
-// with the init kernel before they insert.
+// fresh: the graph's contents, sticky status and spill count are discarded
+// first (dbg_build_reads); the binned path folds that into its first kernel
+// and its tiled apply, the others empty the graph with the init kernel before
+// they insert.
 // `input`: the read set's bases arrive in parts (see dbg::InputParts); only
 // the binned scatter takes them part by part, every other kernel waits for all.
 int insert_one(dbg_handle h, const dbg::ItemDesc &it, cudaStream_t s, bool fresh = false,
@@ -552,7 +563,7 @@ int insert_one(dbg_handle h, const dbg::ItemDesc &it, cudaStream_t s, bool fresh
                        dbg::ensure_bin_scratch(h, 0) == DBG_OK);
   if (binned) return dbg::launch_binned(h, it, h->tuning, s, call, fresh, input);
   DBG_TRY(dbg::wait_input(input, s));
-  if (fresh) DBG_TRY(dbg::launch_table_init(h->table, h->n_slots, s));
+  if (fresh) DBG_TRY(dbg::launch_empty(h, s));
   if (h->k > 32) {  // 128-bit keys: their own kernel
     dbg::timer_mark(h, call, 0, s);
     const int st = dbg::launch_insert_wide(it, h->sm_count, s);
@@ -582,20 +593,6 @@ extern "C" int dbg_insert_reads(dbg_handle h, const uint8_t *packed, const uint6
   return insert_one(h, it, static_cast<cudaStream_t>(stream));
 }
 
-namespace {
-
-// The sticky status and the spill count back to zero, stream-ordered (the
-// part of dbg_reset that is not the table).
-// (the start of every rebuild: its counts, if any, are set by its insert)
-int clear_status(dbg_handle h, cudaStream_t s) {
-  h->built_counts = false;
-  DBG_CK(cudaMemsetAsync(h->d_status, 0, sizeof(uint32_t), s));
-  DBG_CK(cudaMemsetAsync(h->d_spill_count, 0, sizeof(unsigned long long), s));
-  return DBG_OK;
-}
-
-}  // namespace
-
 extern "C" int dbg_build_reads(dbg_handle h, const uint8_t *packed, const uint64_t *offsets,
                                uint64_t n_reads, void *stream) {
   if (!h) return DBG_ERR_INVALID_ARG;
@@ -603,8 +600,7 @@ extern "C" int dbg_build_reads(dbg_handle h, const uint8_t *packed, const uint64
   DeviceGuard g(h->device);
   if (g.err != cudaSuccess) return dbg::cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  DBG_TRY(clear_status(h, s));
-  if (n_reads == 0) return dbg::launch_table_init(h->table, h->n_slots, s);
+  if (n_reads == 0) return dbg::launch_empty(h, s);
   const dbg::ItemDesc it = dbg::make_item(h, packed, offsets, n_reads, 0);
   return insert_one(h, it, s, /*fresh=*/true);
 }
@@ -724,7 +720,6 @@ static int insert_whole(dbg_handle h, const uint8_t *packed, const uint64_t *off
     DBG_CK(cudaStreamSynchronize(h->copy_stream));
     return DBG_ERR_INVALID_ARG;
   }
-  if (fresh) DBG_TRY(clear_status(h, s));
   DBG_CK(cudaStreamWaitEvent(s, h->ev_copied[0], 0));
   const dbg::ItemDesc it =
       dbg::make_item(h, h->stage_packed[0], h->stage_offsets[0], n_reads, byte0 * 4);
@@ -748,9 +743,7 @@ static int insert_reads_host(dbg_handle h, const uint8_t *packed, const uint64_t
   if (g.err != cudaSuccess) return dbg::cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (n_reads == 0) {
-    if (!fresh) return DBG_OK;
-    DBG_TRY(clear_status(h, s));
-    return dbg::launch_table_init(h->table, h->n_slots, s);
+    return fresh ? dbg::launch_empty(h, s) : DBG_OK;
   }
 
   // the whole input when it is small enough (one insert, which the binned
@@ -762,7 +755,6 @@ static int insert_reads_host(dbg_handle h, const uint8_t *packed, const uint64_t
       return insert_whole(h, packed, offsets, n_reads, all_bytes, s, fresh);
   }
   if (!offsets_non_decreasing(offsets, n_reads)) return DBG_ERR_INVALID_ARG;
-  if (fresh) DBG_TRY(clear_status(h, s));
   std::vector<uint64_t> cuts{0};
   uint64_t max_bytes = 0, max_reads = 0;
   for (uint64_t r0 = 0; cuts.back() != n_reads && r0 < n_reads;) {
@@ -854,10 +846,7 @@ static int insert_batch(const dbg_batch_item *items, int n_items, void *stream, 
     dbg_handle h = items[i].graph;
     dbg::ItemDesc it = dbg::make_item(h, items[i].packed, items[i].offsets, items[i].n_reads, 0);
     if (h->k > 32) {  // 128-bit keys: their own kernel, one item at a time
-      if (fresh) {
-        DBG_TRY(clear_status(h, s));
-        DBG_TRY(dbg::launch_table_init(h->table, h->n_slots, s));
-      }
+      if (fresh) DBG_TRY(dbg::launch_empty(h, s));
       if (items[i].n_reads == 0) continue;
       DBG_TRY(insert_one(h, it, s));
       continue;
