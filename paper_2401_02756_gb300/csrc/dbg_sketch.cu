@@ -30,20 +30,33 @@ constexpr int kSketchItems = 2 * kBatchItems;
 // grows, and after the first few thousand keys almost no key raises it: a key
 // whose rho cannot exceed the smallest register (a lower bound the CTA
 // refreshes at every tile start) is dropped after one compare, the others
-// read their register first and take the atomic only to raise it.  The
+// read their register first and take the atomic only to raise it.  At a tile
+// start the CTA also exchanges registers with the item's global ones, which
+// its other CTAs fill: the bound is then that of all keys seen so far, not of
+// the CTA's share (64 samples on 1,052 CTAs: 1.61 -> 1.46 ms; with the
+// CTA's own bound almost every step had a lane whose key passed it).  The
 // registers are the same as without the bound.
 struct SketchVisitor {
   static constexpr bool kUniformRounds = false;
   uint32_t *s_reg;
+  uint32_t *g_reg;  // the item's registers in global memory
   volatile uint32_t *s_floor;  // every register is at least this (any value it held stays true)
-  // a key whose rest (the hash's 54 low bits, left-aligned) has its high word
-  // above lim_hi has rho <= floor: rest >= 2^(64 - floor) for floor <= 32;
-  // for a floor above 32, rest >= 2^32 suffices; a floor of 0 drops nothing
-  uint32_t lim_hi = ~0u;
+  // The bits of the hash from 53 down to 32 are the leading bits of the 54 that
+  // rho counts zeros in: a key for which they are above `lim` has rho <= floor
+  // (a floor of 0 drops nothing; from 22 on, any set bit among them does).
+  uint32_t lim = kLead;
+  static constexpr uint32_t kLead = (1u << 22) - 1u;
   __device__ void tile_begin() {
     const uint32_t f = *s_floor;
-    lim_hi = f == 0u ? ~0u : (f <= 32u ? (1u << (32u - f)) - 1u : 0u);
-    if (threadIdx.x < 32) {  // the next tile's bound
+    lim = f < 22u ? kLead >> f : 0u;
+    for (int j = threadIdx.x; j < kSketchRegs; j += blockDim.x) {
+      const uint32_t own = s_reg[j], all = ld_volatile_u32(g_reg + j);
+      if (own > all)
+        atomicMax(&g_reg[j], own);
+      else
+        s_reg[j] = all;  // (between tiles: no other thread touches it)
+    }
+    if (threadIdx.x < 32) {  // the next tile's bound (registers only grow: any moment's will do)
       uint32_t m = ~0u;
       for (int j = threadIdx.x; j < kSketchRegs; j += 32)
         m = min(m, *reinterpret_cast<volatile uint32_t *>(&s_reg[j]));
@@ -56,9 +69,17 @@ struct SketchVisitor {
   __device__ void round_end() {}
   __device__ void vertex(bool valid, uint64_t key, bool, uint32_t, int, int, const VertexCtx &) {
     if (!valid) return;
-    const uint64_t h = fmix64(key ^ kSketchSalt);
-    const uint32_t rest_hi = (uint32_t)(h >> 22);  // bits 53..22 of the hash
-    if (rest_hi > lim_hi) return;  // 1 + clz(rest) <= floor: no register can rise
+    // fmix64(key ^ salt) up to its second product, whose high word is the
+    // hash's (the last shift by 33 leaves it alone): the low word is only
+    // needed for the few keys that the test lets through
+    uint64_t x = key ^ kSketchSalt;
+    x = (x ^ (x >> 33)) * 0xff51afd7ed558ccdull;
+    x ^= x >> 33;
+    const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
+    const uint32_t h_hi = __umulhi(lo, 0x1a85ec53u) + lo * 0xc4ceb9feu + hi * 0x1a85ec53u;
+    if ((h_hi & kLead) > lim) return;  // 1 + clz(rest) <= floor: no register can rise
+    uint64_t h = x * 0xc4ceb9fe1a85ec53ull;
+    h ^= h >> 33;
     const uint64_t rest = h << 10;
     const uint32_t idx = (uint32_t)(h >> 54);
     const uint32_t rho = rest ? (uint32_t)__clzll(rest) + 1u : 55u;
@@ -75,7 +96,7 @@ __global__ void __launch_bounds__(BLOCK, kSketchCtas)
   for (int j = threadIdx.x; j < kSketchRegs; j += BLOCK) s_reg[j] = 0u;
   if (threadIdx.x == 0) s_floor = 0u;
   __syncthreads();
-  SketchVisitor vis{s_reg, &s_floor};
+  SketchVisitor vis{s_reg, regs, &s_floor};
   for_each_vertex<BLOCK, 1, kSketchRun>(pk, tile_reads, smem, vis, blockIdx.x, pk.total_tiles,
                                         gridDim.x);
   __syncthreads();
@@ -97,15 +118,16 @@ __global__ void __launch_bounds__(BLOCK, kSketchCtas)
   for (int j = threadIdx.x; j < kSketchRegs; j += BLOCK) s_reg[j] = 0u;
   if (threadIdx.x == 0) s_floor = 0u;
   __syncthreads();
-  SketchVisitor vis{s_reg, &s_floor};
+  SketchVisitor vis{s_reg, nullptr, &s_floor};
   const uint64_t t1 = min(pk.total_tiles, (blockIdx.x + 1) * chunk);
   for (uint64_t t = blockIdx.x * chunk; t < t1;) {
     const int it = find_item(pk, t);
     const uint64_t end = it + 1 < pk.n_items ? pk.d[it + 1].tile_begin : pk.total_tiles;
     const uint64_t tb = min(t1, end);
+    uint32_t *g = reinterpret_cast<uint32_t *>(pk.d[it].table);
+    vis.g_reg = g;
     for_each_vertex<BLOCK, kSketchItems, kSketchRun>(pk, tile_reads, smem, vis, t, tb, 1);
     __syncthreads();
-    uint32_t *g = reinterpret_cast<uint32_t *>(pk.d[it].table);
     for (int j = threadIdx.x; j < kSketchRegs; j += BLOCK)
       if (s_reg[j]) {
         atomicMax(&g[j], s_reg[j]);
