@@ -32,8 +32,9 @@
  *     word (at most 62 bits); for k > 32 (the paper's default is k = 51,
  *     Section "Code organization") it is a 128-bit integer of at most 126
  *     bits, exported as two words per vertex, high word first.  Graphs with
- *     k > 32 support create, insert (direct path), batch, stats, export and
- *     normalize; spill, grow, the no-alloc export and contigs take k <= 32.
+ *     k > 32 support create, insert (direct path), build (binned for large
+ *     tables and k <= 63), batch, stats, export and normalize; spill, grow,
+ *     the no-alloc export and contigs take k <= 32.
  *   - Counters: 32-bit unsigned, one per label in the order A, C, G, T,
  *     wrapping modulo 2^32 (the paper's are 8-bit, Section "Graph data
  *     structure"; the wider width keeps high-coverage repeats exact).
@@ -71,7 +72,8 @@ typedef struct dbg_tuning {
   int grid_ctas;      /* CTAs in the persistent grid (default: SMs x resident CTAs per SM) */
   int warp_aggregate; /* direct insert: 1 merges a warp's equal keys with __match_any_sync,
                          0 does not, -1: default (1) */
-  int insert_path;    /* 0: automatic; 1: direct; 2: binned (k <= 31; see dbg_insert_reads) */
+  int insert_path;    /* 0: automatic; 1: direct; 2: binned (k <= 31, and rebuilds with
+                         k from 33 to 63; see dbg_insert_reads) */
   int apply_unroll;   /* binned apply: probe slots per thread, 2, 4 or 8 (0: default 4) */
   int apply_chunk;    /* binned apply: events per thread per work chunk, 4, 8 or 16 (0: 8) */
   int apply_ctas;     /* binned apply: CTAs per SM (0: as many as fit) */
@@ -234,7 +236,11 @@ int dbg_insert_reads_host(dbg_handle h, const uint8_t *packed, const uint64_t *o
  * once.  So the table is not valid until the stream has passed the call:
  * no other call may use the handle from another stream meanwhile.  The
  * sticky status and pending spill records are cleared first.  n_reads == 0
- * only empties the table.  Errors: as dbg_insert_reads. */
+ * only empties the table.  A rebuild with k from 33 to 63 is binned too, with
+ * 16-byte events (tables of 256 MiB or more; default 3 events per slot, 34
+ * bytes per event across the two buffers; the direct insert when they would
+ * take more than half of the device's free memory).  Errors: as
+ * dbg_insert_reads. */
 int dbg_build_reads(dbg_handle h, const uint8_t *packed, const uint64_t *offsets,
                     uint64_t n_reads, void *stream);
 
@@ -270,7 +276,7 @@ typedef struct dbg_batch_item {
  * dbg_release_scratch; batched calls on one device run one after another on
  * the GPU.  Graphs on the direct path (and k = 32) share launches: one
  * kernel for up to 128 of them, its CTAs taking (item, read tile) work units
- * from one index space.  Graphs with k > 32 take their own kernel one by
+ * from one index space.  Graphs with k > 32 take their own kernels one by
  * one.  Every graph
  * must live on the current device; all work is on `stream`.  The call may be
  * captured into a CUDA graph (cudaStreamBeginCapture on `stream`) after one

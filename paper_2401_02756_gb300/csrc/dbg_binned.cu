@@ -40,6 +40,7 @@
 #include "dbg_export.cuh"
 #include "dbg_tiles.cuh"
 #include "dbg_tma.cuh"
+#include "dbg_wide.cuh"
 
 namespace dbg {
 namespace {
@@ -1516,6 +1517,9 @@ int ensure_events(BinScratch &sc, uint64_t events) {
 }  // namespace
 
 uint64_t bin_events_wanted(dbg_handle h) {
+  if (h->k > 32)
+    return 2 * (h->bin_want ? h->bin_want
+                            : std::max(kBinMinEvents, kBinWideEventsPerSlot * h->n_slots));
   return h->bin_want ? h->bin_want : default_events(h->n_slots);
 }
 
@@ -1949,6 +1953,8 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
   if (!capturing) DBG_CK(cudaEventRecord(h->bin.done, s));
   return DBG_OK;
 }
+
+#include "dbg_binned_wide.cuh"
 
 // ---------------------------------------------------------------------------
 // batches: chains of many tables, with the library's own scratch

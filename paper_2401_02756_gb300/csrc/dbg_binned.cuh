@@ -12,6 +12,7 @@ constexpr uint64_t kBinEventsPerSlot = 4;             // default event buffer: 4
                                                       // (4 + 1/4, the buckets' margin included)
 
 constexpr uint64_t kBinSlices = 4096;                // count/scatter work units, at most
+constexpr uint64_t kBinWideEventsPerSlot = 3;         // default of 16-byte events (k > 32)
 constexpr int kBinMinShift = 18;                     // automatic: regions of at least 2^18 slots (8 MiB)
 
 constexpr int kBinApplyCounters = 64;                // apply: chunk counters per launch, at most
@@ -37,8 +38,9 @@ constexpr size_t kBinClearedBytes = (4 + 2 * (size_t)kBatchItems) * 8;
 // most kBinMaxParts of them.
 BinGeometry bin_geometry(uint64_t n_slots, int region_log2);
 
-// The event capacity a handle's binned inserts use: what dbg_reserve_events
-// asked for, else the default of 4.25 per table slot.
+// The event capacity a handle's binned inserts use, in 8-byte units: what
+// dbg_reserve_events asked for, else the default of 4.25 per table slot (k > 32:
+// two units an event, 3 events per slot by default).
 uint64_t bin_events_wanted(dbg_handle h);
 
 // Make sure the handle holds an event buffer of at least `events` events
@@ -69,6 +71,15 @@ int wait_input(const InputParts *input, cudaStream_t s);
 int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cudaStream_t s,
                   int call, bool fresh = false,
                   const InputParts *input = nullptr);
+
+// Rebuild a graph with k from 33 to 63 through 16-byte events (dbg_binned_wide.cuh);
+// the scratch must be there (wide_scratch_ready).
+int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int call);
+
+// Whether a wide rebuild on `s` can have its scratch: made now if it is not
+// there yet, unless the stream is being captured or the device is short of
+// memory.
+bool wide_scratch_ready(dbg_handle h, cudaStream_t s);
 
 // Insert many read sets, each into its own table (k <= 31), through binned
 // chains: every chain is one launch of each binned kernel over all of its

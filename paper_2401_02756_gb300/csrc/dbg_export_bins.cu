@@ -530,7 +530,7 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
   if (scratch && scratch_bytes < sh.total) return DBG_ERR_INVALID_ARG;
   // room for 32-byte records: the graph's own event buffer (idle between its
   // inserts; its event orders the two) when the graph has one that fits, or
-  // for k > 32, which has none, the pool
+  // for k > 32 the pool
   Slot *rec = nullptr;
   uint64_t rec_rows = 0;
   bool own = false;
@@ -540,7 +540,7 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
     own = rec_rows >= rows / 2;  // (a table is rarely more than two thirds full)
     if (!own) rec = nullptr;
   }
-  const bool pooled = h->k > 32 && !scratch && rows * sizeof(Slot) <= kMaxPooledRecords;
+  const bool pooled = !rec && h->k > 32 && !scratch && rows * sizeof(Slot) <= kMaxPooledRecords;
   if (pooled) {
     rec_rows = rows;
     const int st = scratch_alloc(reinterpret_cast<void **>(&rec), rows * sizeof(Slot), s);

@@ -352,7 +352,8 @@ int launch_empty(dbg_handle h, cudaStream_t stream);
 int launch_stats(const Slot *table, uint64_t n_slots, unsigned long long *acc, cudaStream_t stream,
                  bool wide);
 // Graphs with k > 32 (128-bit keys, dbg_wide.cu).
-int launch_insert_wide(const ItemDesc &it, int sm_count, cudaStream_t s);
+int launch_insert_wide(const ItemDesc &it, int sm_count, cudaStream_t s,
+                       const uint32_t *gate = nullptr);
 int export_sorted_wide(dbg_handle h, uint64_t D, uint64_t *keys_out, uint32_t *counts_out,
                        cudaStream_t s);
 

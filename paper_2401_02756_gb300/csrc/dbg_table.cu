@@ -425,7 +425,7 @@ extern "C" int dbg_get_info(dbg_handle h, dbg_info *out) {
   out->table_bytes = h->n_slots * sizeof(dbg::Slot);
   out->max_probes = h->max_probes;
   out->device = h->device;
-  out->event_capacity = h->bin.cap ? h->bin.cap : h->bin_want;
+  out->event_capacity = h->bin.cap ? h->bin.cap / (h->k > 32 ? 2 : 1) : h->bin_want;
   out->spill_capacity = h->spill_cap;
   return DBG_OK;
 }
@@ -539,9 +539,10 @@ extern "C" int dbg_reserve_events(dbg_handle h, uint64_t events) {
 namespace {
 
 // Path for one read set into h: binned when asked for, or automatically for
-// large tables; never for k = 32 (keys of 62 bits do not fit an event).
+// large tables; never for k = 32 and k = 64 (keys of 62 and 126 bits do not fit
+// an event).
 bool want_binned(dbg_handle h) {
-  if (h->k > 31) return false;
+  if (h->k == 32 || h->k == 64) return false;
   const int path = h->tuning.insert_path;
   if (path == 1) return false;
   if (path == 2) return true;
@@ -558,6 +559,10 @@ int insert_one(dbg_handle h, const dbg::ItemDesc &it, cudaStream_t s, bool fresh
                const dbg::InputParts *input = nullptr) {
   h->built_counts = false;  // (set again by a rebuild on the tiled binned path)
   const int call = dbg::timer_begin_call(h);
+  if (h->k > 32 && fresh && want_binned(h) && dbg::wide_scratch_ready(h, s)) {
+    DBG_TRY(dbg::wait_input(input, s));
+    return dbg::launch_binned_wide(h, it, s, call);
+  }
   const bool binned = h->k <= 32 && want_binned(h) &&
                       (h->bin.cap == dbg::bin_events_wanted(h) ||
                        dbg::ensure_bin_scratch(h, 0) == DBG_OK);
@@ -845,10 +850,11 @@ static int insert_batch(const dbg_batch_item *items, int n_items, void *stream, 
     if (i == n_items) break;
     dbg_handle h = items[i].graph;
     dbg::ItemDesc it = dbg::make_item(h, items[i].packed, items[i].offsets, items[i].n_reads, 0);
-    if (h->k > 32) {  // 128-bit keys: their own kernel, one item at a time
-      if (fresh) DBG_TRY(dbg::launch_empty(h, s));
-      if (items[i].n_reads == 0) continue;
-      DBG_TRY(insert_one(h, it, s));
+    if (h->k > 32) {  // 128-bit keys: their own kernels, one item at a time
+      if (items[i].n_reads > 0)
+        DBG_TRY(insert_one(h, it, s, fresh));
+      else if (fresh)
+        DBG_TRY(dbg::launch_empty(h, s));
       continue;
     }
     if (h->k <= 31 && h->tuning.insert_path != 1) {  // binned chains below (an empty read
