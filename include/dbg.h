@@ -355,8 +355,9 @@ int dbg_stats(dbg_handle h, uint64_t *n_vertices, uint64_t *n_edges, void *strea
  * bins (up to about 8 MB, or a byte for every 25 vertices if that is more);
  * a graph built on the binned path places its records in the handle's event
  * buffer first, and one with k > 32 in up to 4 GiB of the pool (32 bytes a
- * vertex).  Other outputs go through temporary ones (24 bytes a row, 32 for
- * k > 32).  Keys crowded into a few prefixes are left to a radix sort (about
+ * vertex).  Pinned host outputs (both, 16-byte aligned) are written by the
+ * sort itself, from records in one of those places; others go through
+ * temporary outputs (24 bytes a row, 32 for k > 32).  Keys crowded into a few prefixes are left to a radix sort (about
  * 6 bytes a vertex in place, otherwise 40, 80 for k > 32).  Errors:
  * INVALID_ARG, OOM, CUDA, BUFFER_TOO_SMALL, and the sticky status (nothing
  * exported when it is set). */

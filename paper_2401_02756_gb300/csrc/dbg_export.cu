@@ -749,8 +749,43 @@ int export_radix(dbg_handle h, uint64_t D, uint64_t *keys_out, uint32_t *counts_
   return export_pairs<unsigned long long>(h, D, keys_out, counts_out, s);
 }
 
-// The sort by bins into outputs that are not aligned device buffers (host
-// memory, or one of the two not asked for): into temporary ones, then copied.
+// The device's view of pinned host memory [p, p + bytes), 16-byte aligned, or
+// null.
+void *mapped_host(void *p, uint64_t bytes) {
+  if (!p || bytes == 0 || ((uintptr_t)p & 15u)) return nullptr;
+  cudaPointerAttributes a{}, z{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
+      cudaPointerGetAttributes(&z, static_cast<char *>(p) + bytes - 1) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  const bool host = a.type == cudaMemoryTypeHost && z.type == cudaMemoryTypeHost &&
+                    a.devicePointer && z.devicePointer;
+  // (both ends in one mapping)
+  return host && static_cast<char *>(z.devicePointer) - static_cast<char *>(a.devicePointer) ==
+                     (int64_t)(bytes - 1)
+             ? a.devicePointer
+             : nullptr;
+}
+
+// The sort by bins into pinned host memory: the bucket sort writes its rows
+// there itself, at the link's rate (192 GB/s, as a copy's), so that the copy
+// of 4.3 M rows (0.54 ms) and the sort (0.09) are one pass.
+// `*no_records`: it cannot be done that way.
+int export_bins_mapped(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t max_n,
+                       uint64_t *D, cudaStream_t s, bool *too_dense, bool *no_records) {
+  *no_records = true;
+  const uint64_t key_bytes = h->k > 32 ? 16 : 8;
+  if (max_n > (1ull << 40)) return DBG_OK;
+  void *keys = mapped_host(keys_out, max_n * key_bytes);
+  void *counts = keys ? mapped_host(counts_out, max_n * 16) : nullptr;
+  if (!counts) return DBG_OK;
+  return export_bins(h, static_cast<uint64_t *>(keys), static_cast<uint32_t *>(counts), max_n, D, s,
+                     nullptr, 0, too_dense, no_records);
+}
+
+// The sort by bins into other outputs (pageable or unaligned memory, or one of
+// the two not asked for): into temporary ones, then copied.
 int export_bins_copied(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t max_n,
                        uint64_t *D, cudaStream_t s, bool *too_dense) {
   const uint64_t rows = std::min(max_n, h->n_slots);
@@ -787,10 +822,14 @@ extern "C" int dbg_export_sorted(dbg_handle h, uint64_t *keys_out, uint32_t *cou
   uint64_t D = 0;
   int st;
   if (h->n_slots <= 0xFFFFFFFFull && max_n > 0 && (keys_out || counts_out)) {
-    bool too_dense = false;
-    st = in_place_outputs(keys_out, counts_out)
-             ? export_bins(h, keys_out, counts_out, max_n, &D, s, nullptr, 0, &too_dense)
-             : export_bins_copied(h, keys_out, counts_out, max_n, &D, s, &too_dense);
+    bool too_dense = false, copied = false;
+    if (in_place_outputs(keys_out, counts_out)) {
+      st = export_bins(h, keys_out, counts_out, max_n, &D, s, nullptr, 0, &too_dense);
+    } else {
+      st = export_bins_mapped(h, keys_out, counts_out, max_n, &D, s, &too_dense, &copied);
+      if (st == DBG_OK && copied)
+        st = export_bins_copied(h, keys_out, counts_out, max_n, &D, s, &too_dense);
+    }
     if (st != DBG_OK) return st;
     *n_out = D;
     if (D > max_n) return DBG_ERR_BUFFER_TOO_SMALL;

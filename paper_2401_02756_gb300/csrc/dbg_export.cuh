@@ -14,10 +14,13 @@ int export_bins_scratch(int k, uint64_t rows, uint64_t &bytes);
 // nothing is written).  `scratch`: caller's device memory (256-byte aligned),
 // or null to take it from the library's pool.  *too_dense: the keys crowd into
 // bins too large for this sort and nothing is written.  Waits for `s`.
-// Returns the graph's sticky status (or NEEDS_GROW) when it has one.
+// `no_records` (if not null): the outputs are to be written once, in order --
+// pinned host memory --, so the records must have a place of their own; set,
+// with nothing else done, when there is none.  Returns the graph's sticky
+// status (or NEEDS_GROW) when it has one.
 int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t max_rows,
                 uint64_t *D, cudaStream_t s, void *scratch, uint64_t scratch_bytes,
-                bool *too_dense);
+                bool *too_dense, bool *no_records = nullptr);
 
 // Bytes of the handle's second event buffer (dbg_binned.cu).
 uint64_t bin_ev2_bytes(dbg_handle h);

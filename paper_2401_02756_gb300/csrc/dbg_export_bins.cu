@@ -15,8 +15,9 @@
 // (32-bit prefix, slot index) pairs this replaces moved 16 bytes a record four
 // times, gathered a random slot per vertex and put runs of equal prefixes in
 // order in two more passes.  Export of 422.6 M vertices of a 20.8 GB table
-// 35.4 -> 22.5 ms (histogram 4.1, place 10.8, sort 7.7), of 57 M 5.1 -> 2.9
-// ms; k = 51, 75 M vertices (two 64-bit radix sorts before) 19.7 -> 4.3 ms.
+// 35.4 -> 22 ms (histogram 4.0, place 10.8 to 12.3 from card to card, sort 6.5;
+// 7.7 with the counters at the slot's byte 8, two loads a row), of 57 M 5.1 ->
+// 2.8 ms; k = 51, 75 M vertices (two 64-bit radix sorts before) 19.7 -> 4.2 ms.
 //
 // The place pass is at the rate of its stores.  A store to a sector that is
 // not in the L2 costs one of about 4.1e10 misses a second however many of its
@@ -134,6 +135,22 @@ template <bool WIDE>
 __device__ __forceinline__ uint4 row_of(const Words &v) {
   return WIDE ? make_uint4(v.w[4], v.w[5], v.w[6], v.w[7])
               : make_uint4(v.w[2], v.w[3], v.w[4], v.w[5]);
+}
+// A placed record: a one-word slot's counters come first, so that its row is
+// one aligned 16-byte load in the sort (a two-word slot's row already is).
+template <bool WIDE>
+__device__ __forceinline__ Words record_of(const Words &v) {
+  if constexpr (WIDE) return v;
+  return Words{{v.w[2], v.w[3], v.w[4], v.w[5], v.w[0], v.w[1], 0u, 0u}};
+}
+template <bool WIDE>
+__device__ __forceinline__ Key<WIDE> ld_record_key(const Slot *p) {
+  if constexpr (WIDE) {
+    const uint4 a = *reinterpret_cast<const uint4 *>(p);
+    return Key<true>{word64(a.x, a.y), word64(a.z, a.w)};
+  } else {
+    return Key<false>{*(reinterpret_cast<const unsigned long long *>(p) + 2)};
+  }
 }
 template <bool WIDE>
 __device__ __forceinline__ Key<WIDE> ld_key(const Slot *p) {
@@ -281,7 +298,7 @@ __global__ void __launch_bounds__(256) k_place(const Slot *t, uint64_t n, Plan p
     for (int u = 0; u < kSlotsPerThread; ++u) {
       if (at[u] == ~0u) continue;
       if constexpr (RECORDS) {
-        st_record(rec + at[u], v[u]);
+        st_record(rec + at[u], record_of<WIDE>(v[u]));
       } else {
         keys[at[u]] = key_of<WIDE>(v[u]);
         counts[at[u]] = row_of<WIDE>(v[u]);
@@ -332,7 +349,7 @@ __global__ void __launch_bounds__(kSortBlock, RECORDS && !WIDE ? 6 : 4)
     const uint32_t i = q * kSortBlock + tid;
     if (i < n) {
       if constexpr (RECORDS)
-        k[q] = ld_key<WIDE>(rec + s0 + i);
+        k[q] = ld_record_key<WIDE>(rec + s0 + i);
       else
         k[q] = keys[s0 + i];
     }
@@ -406,14 +423,7 @@ __global__ void __launch_bounds__(kSortBlock, RECORDS && !WIDE ? 6 : 4)
     keys[s0 + i] = s_key[i];
     uint4 row;
     if constexpr (RECORDS) {  // (its sector was read with the key: an L2 hit)
-      const uint32_t *r = reinterpret_cast<const uint32_t *>(rec + s0 + s_src[i]);
-      if constexpr (WIDE) {
-        row = *reinterpret_cast<const uint4 *>(r + 4);
-      } else {
-        const uint2 lo = *reinterpret_cast<const uint2 *>(r + 2);
-        const uint2 hi = *reinterpret_cast<const uint2 *>(r + 4);
-        row = make_uint4(lo.x, lo.y, hi.x, hi.y);
-      }
+      row = *(reinterpret_cast<const uint4 *>(rec + s0 + s_src[i]) + (WIDE ? 1 : 0));
     } else {
       row = s_row[i];
     }
@@ -520,8 +530,9 @@ int export_bins_scratch(int k, uint64_t rows, uint64_t &bytes) {
 
 int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t max_rows,
                 uint64_t *D, cudaStream_t s, void *scratch, uint64_t scratch_bytes,
-                bool *too_dense) {
+                bool *too_dense, bool *no_records) {
   *too_dense = false;
+  if (no_records) *no_records = false;
   const uint64_t rows = std::min(max_rows, h->n_slots);
   Shape sh{};
   DBG_TRY(export_shape(h->k, rows, sh));
@@ -530,7 +541,7 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
   if (scratch && scratch_bytes < sh.total) return DBG_ERR_INVALID_ARG;
   // room for 32-byte records: the graph's own event buffer (idle between its
   // inserts; its event orders the two) when the graph has one that fits, or
-  // for k > 32 the pool
+  // the pool (k > 32, and outputs that only the sort may write)
   Slot *rec = nullptr;
   uint64_t rec_rows = 0;
   bool own = false;
@@ -540,7 +551,8 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
     own = rec_rows >= rows / 2;  // (a table is rarely more than two thirds full)
     if (!own) rec = nullptr;
   }
-  const bool pooled = !rec && h->k > 32 && !scratch && rows * sizeof(Slot) <= kMaxPooledRecords;
+  const bool pooled = !rec && (h->k > 32 || no_records) && !scratch &&
+                      rows * sizeof(Slot) <= kMaxPooledRecords;
   if (pooled) {
     rec_rows = rows;
     const int st = scratch_alloc(reinterpret_cast<void **>(&rec), rows * sizeof(Slot), s);
@@ -553,6 +565,10 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
   int rc = DBG_OK;
   ExportMeta m{};
   for (;;) {
+    if (no_records && !rec) {
+      *no_records = true;
+      break;
+    }
     if (own) {
       const cudaError_t e = cudaStreamWaitEvent(s, h->bin.done, 0);
       if (e != cudaSuccess) { rc = cuda_fail(e, "cudaStreamWaitEvent"); break; }
@@ -572,7 +588,7 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
     const cudaError_t e = cudaFreeAsync(buf, s);
     if (rc == DBG_OK && e != cudaSuccess) rc = cuda_fail(e, "cudaFreeAsync");
   }
-  if (rc != DBG_OK) return rc;
+  if (rc != DBG_OK || (no_records && *no_records)) return rc;
   if (m.status != DBG_OK) return (int)m.status;
   if (m.spilled > 0) return DBG_ERR_NEEDS_GROW;
   *D = m.vertices;

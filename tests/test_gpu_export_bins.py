@@ -120,3 +120,34 @@ def test_keys_crowded_into_one_bin(k, shared, n):
     assert g.export_into(keys, counts) == D
     same(keys, counts, ref, D)
     g.close()
+
+
+@pytest.mark.parametrize("k", [21, 51])
+@pytest.mark.parametrize("reads,crowd", [(1, 0), (4000, 0), (300, 5000)])
+def test_pinned_host_outputs(k, reads, crowd):
+    # written by the sort itself; keys crowded into one bin go the copied way
+    import torch
+    rng = np.random.default_rng(k)
+    head = synth.codes_to_ascii(synth.random_genome(k // 2, 9))
+    base = synth.ragged_reads(reads, 120, k, 5)
+    texts = [head + synth.codes_to_ascii(rng.integers(0, 4, k - k // 2)) for _ in range(crowd)]
+    rs = synth.from_strings(texts + [base.read_ascii(i) for i in range(reads)] + ["ACGT" * 30], k)
+    ref = expected(rs)
+    D = len(ref.keys)
+    g = dbg.Graph(k, 2 * D + 8)
+    g.insert(*to_device(rs))
+    for rows in (D, 2 * D + 3):
+        keys = torch.full((rows, 2) if k > 32 else (rows,), -7, dtype=torch.int64, pin_memory=True)
+        counts = torch.full((rows, 4), -7, dtype=torch.int32, pin_memory=True)
+        got = g.export(out=(keys.numpy(), counts.numpy()))
+        assert len(got[0]) == D
+        same(keys, counts, ref, D)
+        assert bool((keys[D:] == -7).all()) and bool((counts[D:] == -7).all())
+    keys = torch.full((1, 2) if k > 32 else (1,), -7, dtype=torch.int64, pin_memory=True)
+    counts = torch.full((1, 4), -7, dtype=torch.int32, pin_memory=True)
+    import ctypes
+    n = ctypes.c_uint64()
+    st = dbg.load().dbg_export_sorted(g.handle, keys.data_ptr(), counts.data_ptr(), 1,
+                                      ctypes.byref(n), None)
+    assert st == dbg.ERR_BUFFER_TOO_SMALL and n.value == D and bool((keys == -7).all())
+    g.close()
