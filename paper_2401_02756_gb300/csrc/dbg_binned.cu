@@ -312,8 +312,10 @@ __global__ void __launch_bounds__(1024)
     const uint64_t ns = pk.d[lo].n_slots;
     const uint64_t first = (uint64_t)(p - pk.d[lo].region0) << shift;
     const uint64_t slots = min((uint64_t)1 << shift, ns - first);
-    const double expected = (double)totals[lo] * (double)slots / (double)ns;
-    bk[j] = (unsigned long long)ceil(expected * 1.03 + 16.0 * sqrt(expected) + 256.0);
+    // (single precision: double-precision roots and quotients held this one CTA
+    // up; the rounding, 1e-6 of the events, is nothing to a margin of 3 %)
+    const float expected = (float)totals[lo] * ((float)slots / (float)ns);
+    bk[j] = (unsigned long long)ceilf(expected * 1.03f + 16.0f * sqrtf(expected) + 256.0f);
     nt[j] = (slots + kTileSlots - 1) >> kTileLog2;
     aux.region_item[p] = (uint32_t)lo;
     aux.region_first[p] = first;
@@ -717,52 +719,54 @@ __global__ void __launch_bounds__(1024)
                  const unsigned long long *cursor, int parts, uint64_t unit, uint64_t ev2_cap,
                  TileAux aux, const uint32_t *use_binned) {
   if (ld_volatile_u32(use_binned) == 0u) return;
-  __shared__ double s_red[3][32];
+  // (single precision throughout, see k_bin_buckets: the sizes need not be exact,
+  // only their sum within the buffer, and `avail` leaves a 64th of it free)
+  __shared__ float s_red[3][32];
   __shared__ unsigned long long s_warp[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned long long n[2];
   uint32_t rt[2];
-  double mean[2], slack[2];
-  double sums[3] = {0.0, 0.0, 0.0};  // events, slack over all buckets, buckets
+  float mean[2], slack[2];
+  float sums[3] = {0.0f, 0.0f, 0.0f};  // events, slack over all buckets, buckets
   for (int i = 0; i < 2; ++i) {
     const int p = 2 * tid + i;
     n[i] = 0ull;
     rt[i] = 0u;
-    mean[i] = slack[i] = 0.0;
+    mean[i] = slack[i] = 0.0f;
     if (p < parts) {
       n[i] = cursor[p] - begin[p];
       counts[p] = n[i];
       rt[i] = aux.region_tile0[p + 1] - aux.region_tile0[p];
       if (n[i]) {
-        mean[i] = (double)n[i] / (double)rt[i];
-        slack[i] = 0.03 * mean[i] + 16.0 * sqrt(mean[i]) + 64.0;
-        sums[0] += (double)n[i];
-        sums[1] += slack[i] * (double)rt[i];
-        sums[2] += (double)rt[i];
+        mean[i] = (float)n[i] / (float)rt[i];
+        slack[i] = 0.03f * mean[i] + 16.0f * sqrtf(mean[i]) + 64.0f;
+        sums[0] += (float)n[i];
+        sums[1] += slack[i] * (float)rt[i];
+        sums[2] += (float)rt[i];
       }
     }
   }
   for (int j = 0; j < 3; ++j) {
-    double v = sums[j];
+    float v = sums[j];
     for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(kFull, v, d);
     if (lane == 0) s_red[j][warp] = v;
   }
   __syncthreads();
   if (warp == 0) {
     for (int j = 0; j < 3; ++j) {
-      double v = s_red[j][lane];
+      float v = s_red[j][lane];
       for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(kFull, v, d);
       if (lane == 0) s_red[j][0] = v;
     }
   }
   __syncthreads();
-  const double N = s_red[0][0], D = s_red[1][0], R = s_red[2][0];
-  const double avail = (double)(ev2_cap - ev2_cap / 64);
-  const double f = D > 0.0 ? fmin(1.0, fmax(0.0, (avail - N - R) / D)) : 0.0;
-  const double want = N + f * D;
-  const double g = want > avail ? avail / want : 1.0;
+  const float N = s_red[0][0], D = s_red[1][0], R = s_red[2][0];
+  const float avail = (float)(ev2_cap - ev2_cap / 64);
+  const float f = D > 0.0f ? fminf(1.0f, fmaxf(0.0f, (avail - N - R) / D)) : 0.0f;
+  const float want = N + f * D;
+  const float g = want > avail ? avail / want : 1.0f;
   uint32_t cap[2];
-  for (int i = 0; i < 2; ++i) cap[i] = n[i] ? (uint32_t)floor((mean[i] + f * slack[i]) * g) : 0u;
+  for (int i = 0; i < 2; ++i) cap[i] = n[i] ? (uint32_t)floorf((mean[i] + f * slack[i]) * g) : 0u;
 
   const unsigned long long ua = (n[0] + unit - 1) / unit, ub = (n[1] + unit - 1) / unit;
   unsigned long long units_total, buckets_total;
@@ -1337,14 +1341,21 @@ __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 thr
   if (!FRESH && threadIdx.x == 0) bulk_wait_all();
 }
 
-// One event, from its home slot, with the global find-or-claim (its tile is
-// final by now).
+// One event with the global find-or-claim (its tile is final by now): from its
+// home slot, or (left_tile: its probe found every slot from home to the tile's
+// end taken by other keys, and no slot empties again) from the next tile on.
 // Returns 1 when the event claimed a new slot (a new vertex), else 0.
-__device__ __forceinline__ uint32_t global_event(uint64_t e, const ItemDesc &it) {
+__device__ __forceinline__ uint32_t global_event(uint64_t e, const ItemDesc &it, bool left_tile) {
   const unsigned long long key = e >> 3;
-  uint64_t s;
+  uint64_t s = home_slot(key, it.n_slots);
+  uint32_t probed = 0;
+  if (left_tile) {
+    const uint64_t end = min((s | (uint64_t)(kTileSlots - 1)) + 1, it.n_slots);
+    probed = (uint32_t)(end - s);
+    s = end == it.n_slots ? 0 : end;
+  }
   bool claimed = false;
-  if (find_or_claim(it.table, it.n_slots, it.max_probes, key, s, &claimed)) {
+  if (find_or_claim_from(it.table, it.n_slots, it.max_probes, key, s, probed, s, &claimed)) {
     if (e & 4ull) atomicAdd(&it.table[s].cnt[e & 3ull], 1u);
   } else {
     spill_or_fail(it.spill, it.spill_cap, it.spill_count, it.status, key, (e & 4ull) != 0,
@@ -1354,7 +1365,7 @@ __device__ __forceinline__ uint32_t global_event(uint64_t e, const ItemDesc &it)
 }
 
 // The events that left their tile (each region's list), then those of the
-// overflow area ((event, region) pairs), from their home slots.  New
+// overflow area ((event, region) pairs).  New
 // vertices are added to their graph's built counts (meaningful only on a
 // rebuild, which zeroed them): one atomic per warp and region, and for the
 // overflow area one per warp of a single table, else one per new vertex.
@@ -1371,7 +1382,7 @@ __global__ void k_tile_deferred(const __grid_constant__ ItemPack<N> pk,
     const ItemDesc &it = pk.d[aux.region_item[p]];
     const uint64_t *list = ev + begin[p];
     uint32_t claimed = 0;
-    for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) claimed += global_event(list[i], it);
+    for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) claimed += global_event(list[i], it, true);
     claimed = __reduce_add_sync(kFull, claimed);
     if ((threadIdx.x & 31) == 0 && claimed)
       atomicAdd(small_built(it.status), (unsigned long long)claimed);
@@ -1382,7 +1393,7 @@ __global__ void k_tile_deferred(const __grid_constant__ ItemPack<N> pk,
   uint32_t claimed = 0;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < no; i += stride) {
     const ItemDesc &it = pk.d[aux.region_item[over[2 * i + 1]]];
-    const uint32_t c = global_event(over[2 * i], it);
+    const uint32_t c = global_event(over[2 * i], it, false);
     if (N == 1)
       claimed += c;
     else if (c)

@@ -82,3 +82,21 @@ def test_a_failed_build_is_cleared_by_the_next():
     g.reset()
     assert g.status() == dbg.OK and g.stats() == (0, 0)
     g.close()
+
+
+@pytest.mark.parametrize("slots_over", [0, 3, 5000])
+@pytest.mark.parametrize("max_probes", [0, 1 << 30])
+def test_probes_that_leave_their_tile(slots_over, max_probes):
+    # tables at a load near one: many events are applied past their tile's end,
+    # and wrap past the table's
+    rs = reads(7)
+    keys, counts = direct(rs)
+    g = dbg.Graph(31, keys.size + slots_over, max_probes=max_probes)
+    g.set_tuning(insert_path=2, region_log2=16)
+    g.set_spill(100_000)
+    g.build(*to_device(rs))
+    if g.status() == dbg.ERR_NEEDS_GROW:
+        g.grow(2 * keys.size)
+    got = g.export()
+    assert np.array_equal(got[0], keys) and np.array_equal(got[1], counts)
+    g.close()
