@@ -363,11 +363,9 @@ __global__ void __launch_bounds__(kWideBlock, 3)
     const uint32_t n = min(aux.fill[t], cap);
     const uint64_t first = aux.region_first[p] + (j << kTileLog2);
     const int len = (int)min((uint64_t)kTileSlots, n_slots - first);
-    uint4 *dst = reinterpret_cast<uint4 *>(it.table + first);
     if (n == 0) {
-      const uint4 head = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);
-      const uint4 tail = make_uint4(0u, 0u, 0u, 0u);
-      for (int i = tid; i < 2 * len; i += kWideBlock) __stcs(dst + i, (i & 1) ? tail : head);
+      for (int sl = tid; sl < len; sl += kWideBlock)
+        st_sector(it.table + first + sl, ~0u, ~0u, 0u, 0u, 0u, 0u, 0u, 0u);
       continue;  // (shared memory untouched: still the EMPTY tile)
     }
     if (tid == 0) s_stop = ld_volatile_u32(it.status);
@@ -395,7 +393,7 @@ __global__ void __launch_bounds__(kWideBlock, 3)
           bool done = false;
           while (q < limit) {
             const uint32_t w = __funnelshift_r(fp32[q >> 2], fp32[(q >> 2) + 1], 8 * (q & 3));
-            uint32_t cand = zero_bytes(w ^ f4) | zero_bytes(w);
+            uint32_t cand = candidate_bytes(w, f4);
             if (limit - q < 4) cand &= (1u << (8 * (limit - q))) - 1u;
             if (cand == 0u) {
               q += 4;
@@ -424,21 +422,15 @@ __global__ void __launch_bounds__(kWideBlock, 3)
       }
     }
     __syncthreads();
-    for (int i = tid; i < 2 * len; i += kWideBlock) {
-      const uint32_t sl = (uint32_t)i >> 1;
-      uint4 v;
-      if ((i & 1) == 0) {
-        const unsigned long long wa = ka[sl], wb = kb[sl];
-        const unsigned long long hi = wa == kEmpty ? kEmpty : wide_hi(wa);
-        const unsigned long long lo = wa == kEmpty ? 0ull : wide_lo(wa, wb);
-        v = make_uint4((uint32_t)hi, (uint32_t)(hi >> 32), (uint32_t)lo, (uint32_t)(lo >> 32));
-        ka[sl] = kb[sl] = kEmpty;
-      } else {
-        v = make_uint4(cnt[sl], cnt[kTileSlots + sl], cnt[2 * kTileSlots + sl],
-                       cnt[3 * kTileSlots + sl]);
-        cnt[sl] = cnt[kTileSlots + sl] = cnt[2 * kTileSlots + sl] = cnt[3 * kTileSlots + sl] = 0u;
-      }
-      __stcs(dst + i, v);
+    for (int sl = tid; sl < len; sl += kWideBlock) {
+      const unsigned long long wa = ka[sl], wb = kb[sl];
+      const unsigned long long hi = wa == kEmpty ? kEmpty : wide_hi(wa);
+      const unsigned long long lo = wa == kEmpty ? 0ull : wide_lo(wa, wb);
+      uint32_t *c = cnt + sl;
+      st_sector(it.table + first + sl, (uint32_t)hi, (uint32_t)(hi >> 32), (uint32_t)lo,
+                (uint32_t)(lo >> 32), c[0], c[kTileSlots], c[2 * kTileSlots], c[3 * kTileSlots]);
+      ka[sl] = kb[sl] = kEmpty;
+      c[0] = c[kTileSlots] = c[2 * kTileSlots] = c[3 * kTileSlots] = 0u;
     }
     for (int i = tid; i < kFpBytes / 4; i += kWideBlock) {
       const uint32_t w = fp32[i];  // four fingerprints: non-zero for a key

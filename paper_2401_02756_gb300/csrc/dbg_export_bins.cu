@@ -115,10 +115,7 @@ __device__ __forceinline__ Words ld_slot(const Slot *p) {
   return v;
 }
 __device__ __forceinline__ void st_record(Slot *p, const Words &v) {
-  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v.w[0]),
-               "r"(v.w[1]), "r"(v.w[2]), "r"(v.w[3]), "r"(v.w[4]), "r"(v.w[5]), "r"(v.w[6]),
-               "r"(v.w[7])
-               : "memory");
+  st_sector(p, v.w[0], v.w[1], v.w[2], v.w[3], v.w[4], v.w[5], v.w[6], v.w[7]);
 }
 
 __device__ __forceinline__ unsigned long long word64(uint32_t lo, uint32_t hi) {

@@ -112,6 +112,14 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
   return v;
 }
 
+// 32 bytes in one store (32-byte aligned): a full sector in one request.
+__device__ __forceinline__ void st_sector(void *p, uint32_t a, uint32_t b, uint32_t c, uint32_t d,
+                                          uint32_t e, uint32_t f, uint32_t g, uint32_t h) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(a), "r"(b), "r"(c),
+               "r"(d), "r"(e), "r"(f), "r"(g), "r"(h)
+               : "memory");
+}
+
 // An L2 cache policy that keeps the lines it touches ahead of others
 // (evict_last) for the whole access.
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {

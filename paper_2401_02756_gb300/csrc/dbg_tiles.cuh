@@ -295,6 +295,9 @@ __device__ __forceinline__ void for_each_vertex(const ItemPack<N> &pk, int tile_
             // runs of up to R positions of one read: run u of the sub-tile
             // belongs to the last read whose first run is at or before u
             const uint32_t n_runs = s_urel[rb];
+            // (reads of one length: the run's read is its share of the runs, without
+            // the nine steps of a search; the 100 Mbp scatter 12.8 -> 12.0 ms)
+            const float per_run = (float)(rb - ra) / (float)n_runs;
             for (uint32_t ub = 0; ub < n_runs; ub += (uint32_t)BLOCK) {
               if (!Visitor::kUniformRounds && vis.stop(lane)) break;
               const uint32_t u = ub + (uint32_t)tid;
@@ -302,13 +305,17 @@ __device__ __forceinline__ void for_each_vertex(const ItemPack<N> &pk, int tile_
               LabelWord labels = 0;
               uint32_t cnt = 0, cnt_edge = 0;
               if (u < n_runs) {
-                int lo = ra, hi = rb - 1;
-                while (lo < hi) {
-                  const int mid = (lo + hi + 1) >> 1;
-                  if (s_urel[mid] <= u)
-                    lo = mid;
-                  else
-                    hi = mid - 1;
+                int lo = min(ra + (int)(((float)u + 0.5f) * per_run), rb - 1);
+                if (s_urel[lo] > u || s_urel[lo + 1] <= u) {  // reads of uneven length
+                  int hi = rb - 1;
+                  lo = ra;
+                  while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (s_urel[mid] <= u)
+                      lo = mid;
+                    else
+                      hi = mid - 1;
+                  }
                 }
                 const uint32_t j0 = (u - s_urel[lo]) * (uint32_t)R;  // first position in the read
                 const uint32_t nvr = s_vrel[lo + 1] - s_vrel[lo];     // > j0
