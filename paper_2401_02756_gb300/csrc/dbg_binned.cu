@@ -1354,6 +1354,11 @@ __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 thr
       for (uint32_t base = 0;;) {
 #pragma unroll
         for (int r = 0; r < kBatch; ++r) {
+          if constexpr (!FRESH) {  // (a held graph's lot leaves a tile few events:
+            // 0.18 ms a lot of 12 M events, 0.187 with the queue)
+            if (is_event(e[r])) probe.finish(e[r], it, p, ev, begin, aux.deferred_n);
+            continue;
+          }
           const bool keep = is_event(e[r]) && (!step || probe.first_step(e[r]));
           const unsigned m = __ballot_sync(kFull, keep);
           if (m == 0u) continue;
@@ -1372,7 +1377,7 @@ __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 thr
         load_bucket<BLOCK>(bucket, base, n, e);
       }
       __syncwarp();
-      if (lane < (int)open) probe.finish(queue[lane], it, p, ev, begin, aux.deferred_n);
+      if (FRESH && lane < (int)open) probe.finish(queue[lane], it, p, ev, begin, aux.deferred_n);
     }
     __syncthreads();
     if constexpr (FRESH) {
@@ -1876,8 +1881,9 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
     // three) fill an SM with 48 warps, enough to hide the dependent hash and
     // probe latencies
     constexpr int BA = 512;
-    const size_t smem = (fresh ? kSoaTileBytes : (size_t)kTileSlots * sizeof(Slot)) + kFpBytes +
-                        (BA / 32) * kTileQueue * sizeof(uint64_t);
+    const size_t smem = (fresh ? kSoaTileBytes + (BA / 32) * kTileQueue * sizeof(uint64_t)
+                               : (size_t)kTileSlots * sizeof(Slot)) +
+                        kFpBytes;
     auto kern = fresh ? k_tile_apply<BA, true, N, SMALL> : k_tile_apply<BA, false, N, SMALL>;
     DBG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;

@@ -151,3 +151,22 @@ def test_pinned_host_outputs(k, reads, crowd):
                                       ctypes.byref(n), None)
     assert st == dbg.ERR_BUFFER_TOO_SMALL and n.value == D and bool((keys == -7).all())
     g.close()
+
+
+@pytest.mark.parametrize("k", [11, 31])
+@pytest.mark.parametrize("reads", [1, 400, 30_000])
+def test_large_outputs_placed_by_bucket(k, reads):
+    # a direct insert has no event buffer to sort records in; above 2^21 rows
+    # the keys and rows are placed by their bucket
+    rs = synth.ragged_reads(reads, 160, k, 13 * reads + k)
+    ref = expected(rs)
+    D = len(ref.keys)
+    rows = (1 << 21) + 4099
+    g = dbg.Graph(k, rows)
+    g.set_tuning(insert_path=1)
+    g.insert(*to_device(rs))
+    keys, counts = outputs(rows, k)
+    assert g.export_into(keys, counts) == D
+    same(keys, counts, ref, D)
+    assert bool((keys[D:] == -7).all()) and bool((counts[D:] == -7).all())
+    g.close()
