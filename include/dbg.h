@@ -81,7 +81,8 @@ typedef struct dbg_tuning {
   int region_log2;    /* binned: table region of 2^region_log2 slots, 16..26 (0: automatic) */
   int apply_group;    /* binned apply (streaming): regions per launch (0: all in one launch) */
   int apply_mode;     /* binned apply: 0 automatic (tiled), 1 streaming, 2 tiled */
-  int scatter_reads;  /* binned scatter (tiled apply): reads per read tile, 32..512 (0: 416) */
+  int scatter_reads;  /* binned scatter (tiled apply): reads per read tile, 32..512 (0: 416,
+                         fewer for read sets that leave CTAs without a tile) */
   int split_threads;  /* binned split: threads per CTA, 256, 512 or 1024, at least a quarter
                          of the tiles per region (0: automatic) */
 } dbg_tuning;

@@ -474,8 +474,19 @@ struct ScatterVisitor {
 
 constexpr int kScatterTileReads = 416;  // reads per scatter tile without a count pass (<= 512)
 
-int scatter_tile_reads(const dbg_tuning &t) {
-  return t.scatter_reads > 0 ? t.scatter_reads : kScatterTileReads;
+// Reads per scatter tile for `reads` reads: kScatterTileReads, or with fewer
+// than kFullWaves of such tiles for every resident CTA as many as give each CTA
+// the same number of tiles: 70,000 reads of 150 bases in 416s are 169 tiles for
+// 304 CTAs, 3,600 reads of 5,000 are 9 (0.225 -> 0.199 ms and 2.46 -> 0.58 ms a
+// build).  Past kFullWaves the last wave is a small part, and 416 keeps the rounds
+// within a tile whole.
+int scatter_tile_reads(const dbg_tuning &t, uint64_t reads, int sms) {
+  constexpr uint64_t kFullWaves = 8, kMinReads = 8;
+  if (t.scatter_reads > 0) return t.scatter_reads;
+  const uint64_t ctas = 2 * (uint64_t)sms;  // (resident: the kernel's launch bounds)
+  const uint64_t waves = (reads + ctas * kScatterTileReads - 1) / (ctas * kScatterTileReads);
+  if (waves == 0 || waves > kFullWaves) return kScatterTileReads;
+  return (int)std::max(kMinReads, (reads + ctas * waves - 1) / (ctas * waves));
 }
 
 template <int BLOCK>
@@ -1775,14 +1786,13 @@ struct Marks {
 // One tiled chain over items[0..n) (N >= n): their tables are cut into
 // regions of 2^shift slots (`parts` of them, `tiles` tiles), item i's first
 // region is items[i].region0, and items[i].tile_begin numbers the walk's
-// tiles of kScatterTileReads reads.  The direct kernel does the call instead
+// tiles of `scatter_reads` reads.  The direct kernel does the call instead
 // when the events do not fit the scratch.  The scratch's event buffer, second
 // buffer and aux area must exist.  `status` receives a timeout of the split.
 template <int N, bool SMALL>
 int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int parts,
-                uint64_t tiles, uint64_t walk_tiles, const dbg_tuning &tuning, int sms,
-                cudaStream_t s, bool fresh, const Marks &mark, const InputParts *input) {
-  const int scatter_reads = scatter_tile_reads(tuning);
+                uint64_t tiles, uint64_t walk_tiles, int scatter_reads, const dbg_tuning &tuning,
+                int sms, cudaStream_t s, bool fresh, const Marks &mark, const InputParts *input) {
   const MetaView mv = meta_view(sc);
   const int tpr = 1 << (shift - kTileLog2);
   const TileAux aux = tile_aux(sc, parts, tiles);
@@ -1916,14 +1926,14 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
 // tables of 2^32 slots and more (137 GB) take the general home slot
 template <int N>
 int tiled_chain(BinScratch &sc, const ItemDesc *items, int n, int shift, int parts, uint64_t tiles,
-                uint64_t walk_tiles, const dbg_tuning &tuning, int sms, cudaStream_t s, bool fresh,
-                const Marks &mark, const InputParts *input = nullptr) {
+                uint64_t walk_tiles, int scatter_reads, const dbg_tuning &tuning, int sms,
+                cudaStream_t s, bool fresh, const Marks &mark, const InputParts *input = nullptr) {
   bool small = true;
   for (int i = 0; i < n; ++i) small = small && items[i].n_slots <= 0xFFFFFFFFull;
-  return small ? tiled_chain_of<N, true>(sc, items, n, shift, parts, tiles, walk_tiles, tuning, sms,
-                                         s, fresh, mark, input)
-               : tiled_chain_of<N, false>(sc, items, n, shift, parts, tiles, walk_tiles, tuning, sms,
-                                          s, fresh, mark, input);
+  return small ? tiled_chain_of<N, true>(sc, items, n, shift, parts, tiles, walk_tiles,
+                                         scatter_reads, tuning, sms, s, fresh, mark, input)
+               : tiled_chain_of<N, false>(sc, items, n, shift, parts, tiles, walk_tiles,
+                                          scatter_reads, tuning, sms, s, fresh, mark, input);
 }
 
 }  // namespace
@@ -1966,9 +1976,9 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
     ItemDesc walk = it;  // the scatter's read tiles (larger than the direct kernel's)
     walk.tile_begin = 0;
     walk.region0 = 0;
-    const uint64_t sr = (uint64_t)scatter_tile_reads(tuning);
-    const uint64_t walk_tiles = (it.n_reads + sr - 1) / sr;
-    DBG_TRY(tiled_chain<1>(h->bin, &walk, 1, geo.shift, geo.parts, n_tiles, walk_tiles, tuning,
+    const int sr = scatter_tile_reads(tuning, it.n_reads, sms);
+    const uint64_t walk_tiles = (it.n_reads + (uint64_t)sr - 1) / (uint64_t)sr;
+    DBG_TRY(tiled_chain<1>(h->bin, &walk, 1, geo.shift, geo.parts, n_tiles, walk_tiles, sr, tuning,
                            sms, s, fresh, mark, input));
     h->built_counts = fresh;  // a rebuild counted its vertices and edges (unless it fell back)
     if (!capturing) DBG_CK(cudaEventRecord(h->bin.done, s));
@@ -2120,10 +2130,12 @@ int launch_binned_batch(const ItemDesc *items, const uint64_t *want, int n,
     ready = ensure_tile_scratch(sc, need_parts, need_tiles, false);
   }
   if (!capturing) DBG_CK(cudaStreamWaitEvent(s, sc.done, 0));
-  const uint64_t sr = (uint64_t)scatter_tile_reads(tuning);
   for (const Chain &c : chains) {
     const int m = c.i1 - c.i0;
     std::vector<ItemDesc> walk(items + c.i0, items + c.i1);
+    uint64_t reads = 0;
+    for (const ItemDesc &it : walk) reads += it.n_reads;
+    const uint64_t sr = (uint64_t)scatter_tile_reads(tuning, reads, sms);
     uint64_t walk_tiles = 0;
     int region0 = 0;
     for (int i = 0; i < m; ++i) {
@@ -2138,7 +2150,7 @@ int launch_binned_batch(const ItemDesc *items, const uint64_t *want, int n,
       continue;
     }
     DBG_TRY(tiled_chain<kBatchItems>(sc, walk.data(), m, shift, c.parts, c.tiles, walk_tiles,
-                                     tuning, sms, s, fresh, Marks{}));
+                                     (int)sr, tuning, sms, s, fresh, Marks{}));
   }
   if (!capturing) DBG_CK(cudaEventRecord(sc.done, s));
   return DBG_OK;
