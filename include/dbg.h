@@ -237,7 +237,14 @@ int dbg_insert_reads_host(dbg_handle h, const uint8_t *packed, const uint64_t *o
  * once.  So the table is not valid until the stream has passed the call:
  * no other call may use the handle from another stream meanwhile.  The
  * sticky status and pending spill records are cleared first.  n_reads == 0
- * only empties the table.  A rebuild with k from 33 to 63 is binned too, with
+ * only empties the table.  A rebuild (k <= 31) of a table of 16 MiB to 256 MiB
+ * is binned too when about 4 million events or more are to be expected -- the
+ * size dbg_reserve_events gave, else 64 a read -- with buffers that the
+ * library's pool lends for the call (17 bytes per event for the reserved size,
+ * else for 4.25 events per slot or 160 per read, up to 2.3 GB); inside a
+ * stream capture, without that memory or with more events than it holds the
+ * direct insert does it.  dbg_binned_counters does not tell of such a call.  A
+ * rebuild with k from 33 to 63 is binned too, with
  * 16-byte events (tables of 256 MiB or more; default 3 events per slot, 34
  * bytes per event across the two buffers; the direct insert when they would
  * take more than half of the device's free memory).  Errors: as
@@ -296,13 +303,13 @@ int dbg_insert_batch(const dbg_batch_item *items, int n_items, void *stream);
 int dbg_build_batch(const dbg_batch_item *items, int n_items, void *stream);
 
 /* Give back the device memory the library keeps between calls: the batched
- * inserts' buffers and the export's cached temporary memory, on every device
+ * inserts' buffers and the pool of the exports and of mid-size rebuilds, on every device
  * (each is synchronised first).  Later calls allocate again as needed.
  * Errors: CUDA. */
 int dbg_release_scratch(void);
 
 /* Device bytes the library holds between calls on the current device: the
- * batched inserts' buffers and the export's cached temporary memory (what
+ * batched inserts' buffers and the pool of the exports and of mid-size rebuilds (what
  * dbg_release_scratch gives back).  A caller that keeps a device-memory
  * budget counts them; 0 when there is no device. */
 uint64_t dbg_scratch_bytes(void);

@@ -2046,6 +2046,69 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
   return DBG_OK;
 }
 
+// A rebuild of a table that the held scratch is too much for (2.8 times the
+// table, and the graph may be one of many).  The direct insert is bound by its
+// requests to L2 (a probe and a counter add an event, 2.6e10 events/s); the
+// binned kernels take a third of that time an event and 0.15 ms for themselves.
+// Reads of 150 bases, direct and binned: 3.6 M events 0.18 / 0.14 ms, 8.5 M 0.34 /
+// 0.20, 24 M 0.92 / 0.45; 2.4 M are even, and below kBinPooledMinEvents the kernels'
+// own time decides.  Under 16 MiB (256 tiles for 456 CTAs of the apply) the gain
+// is a third (48 M events 2.1 / 1.4 ms), not worth a scratch 50 times the table.
+// The events the scratch has room for: what was reserved, else as for a held buffer
+// 4.25 a slot, or 160 a read (what reads of 150 bases and their buckets' margins
+// need, whatever their coverage); more than that and the direct insert does it.
+int launch_binned_pooled(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cudaStream_t s,
+                         int call, const InputParts *input, bool *done) {
+  *done = false;
+  constexpr uint64_t kMaxPooledEvents = 128ull << 20;  // (2.3 GB: the pool keeps as much)
+  const dbg_tuning t = resolve_tuning(tuning);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  DBG_CK(cudaStreamIsCapturing(s, &capture));
+  if (capture != cudaStreamCaptureStatusNone || t.apply_mode == 1) return DBG_OK;
+  if ((h->bin_want ? h->bin_want : 64 * it.n_reads) < kBinPooledMinEvents ||
+      h->bin_want > kMaxPooledEvents)
+    return DBG_OK;
+  const BinGeometry geo = bin_geometry(
+      h->n_slots, t.region_log2 > 0 ? t.region_log2 : tiled_shift(h->n_slots, kTableRegions));
+  if (geo.shift < kTileLog2 || (1 << (geo.shift - kTileLog2)) > kMaxTilesPerRegion) return DBG_OK;
+  const uint64_t tiles = table_tiles(h->n_slots, geo.shift);
+  uint64_t events = h->bin_want;
+  if (events == 0) {
+    events = std::max(kBinEventsPerSlot * h->n_slots + h->n_slots / 4,
+                      160 * std::min(it.n_reads, kMaxPooledEvents));
+    events = std::min(events, kMaxPooledEvents) + 65536 + 2048 * (uint64_t)geo.parts;
+  }
+
+  // one block: the meta area without its slice histograms, the aux area, the two buffers
+  auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
+  const size_t off_aux = al(kBinMetaBytes - (size_t)kBinSlices * kBinMaxParts * 4);
+  const size_t off_ev = off_aux + al(tile_aux_layout(geo.parts, tiles).total);
+  const size_t off_ev2 = off_ev + al(events * sizeof(uint64_t));
+  void *block = nullptr;
+  if (scratch_alloc(&block, off_ev2 + ev2_capacity(events) * sizeof(uint64_t), s) != DBG_OK) {
+    cudaGetLastError();  // clear the allocation failure
+    return DBG_OK;
+  }
+  char *b = static_cast<char *>(block);
+  BinScratch sc;
+  sc.meta = reinterpret_cast<unsigned long long *>(b);
+  sc.aux = b + off_aux;
+  sc.ev = reinterpret_cast<uint64_t *>(b + off_ev);
+  sc.ev2 = reinterpret_cast<uint64_t *>(b + off_ev2);
+  sc.cap = events;
+  ItemDesc walk = it;  // the scatter's read tiles (larger than the direct kernel's)
+  walk.tile_begin = 0;
+  walk.region0 = 0;
+  const int sms = std::max(1, h->sm_count), sr = scatter_tile_reads(tuning, it.n_reads, sms);
+  const uint64_t walk_tiles = (it.n_reads + (uint64_t)sr - 1) / (uint64_t)sr;
+  const int st = tiled_chain<1>(sc, &walk, 1, geo.shift, geo.parts, tiles, walk_tiles, sr, tuning,
+                                sms, s, true, Marks{h, call}, input);
+  cudaFreeAsync(block, s);
+  h->built_counts = st == DBG_OK;
+  *done = true;
+  return st;
+}
+
 #include "dbg_binned_wide.cuh"
 
 // ---------------------------------------------------------------------------

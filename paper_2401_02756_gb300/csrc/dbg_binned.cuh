@@ -7,6 +7,8 @@ namespace dbg {
 
 constexpr int kBinMaxParts = 2048;           // regions of one chain (one or many tables), at most
 constexpr uint64_t kBinMinTableBytes = 256ull << 20;  // auto mode: tables at least this big
+constexpr uint64_t kBinPooledMinTableBytes = 16ull << 20;  // auto mode, rebuilds: with scratch from
+constexpr uint64_t kBinPooledMinEvents = 4000000;          // the pool (see launch_binned_pooled)
 constexpr uint64_t kBinMinEvents = 16ull << 20;       // smallest event buffer
 constexpr uint64_t kBinEventsPerSlot = 4;             // default event buffer: 4.25 events per slot
                                                       // (4 + 1/4, the buckets' margin included)
@@ -71,6 +73,13 @@ int wait_input(const InputParts *input, cudaStream_t s);
 int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cudaStream_t s,
                   int call, bool fresh = false,
                   const InputParts *input = nullptr);
+
+// Rebuild a graph of fewer than kBinMinTableBytes through the binned kernels, with
+// scratch from the library's pool for the call.  False in *done: the scratch
+// is not to be had (a captured stream, the device out of memory, a scratch of the
+// caller's size, a tuning the tiled kernels do not take), nothing was launched.
+int launch_binned_pooled(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cudaStream_t s,
+                         int call, const InputParts *input, bool *done);
 
 // Rebuild a graph with k from 33 to 63 through 16-byte events (dbg_binned_wide.cuh);
 // the scratch must be there (wide_scratch_ready).

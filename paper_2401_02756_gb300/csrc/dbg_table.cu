@@ -567,6 +567,12 @@ int insert_one(dbg_handle h, const dbg::ItemDesc &it, cudaStream_t s, bool fresh
                       (h->bin.cap == dbg::bin_events_wanted(h) ||
                        dbg::ensure_bin_scratch(h, 0) == DBG_OK);
   if (binned) return dbg::launch_binned(h, it, h->tuning, s, call, fresh, input);
+  if (fresh && h->k < 32 && h->tuning.insert_path == 0 &&
+      h->n_slots * sizeof(dbg::Slot) >= dbg::kBinPooledMinTableBytes) {
+    bool done = false;
+    const int st = dbg::launch_binned_pooled(h, it, h->tuning, s, call, input, &done);
+    if (done || st != DBG_OK) return st;
+  }
   DBG_TRY(dbg::wait_input(input, s));
   if (fresh) DBG_TRY(dbg::launch_empty(h, s));
   if (h->k > 32) {  // 128-bit keys: their own kernel
