@@ -1421,6 +1421,43 @@ __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 thr
   if (!FRESH && threadIdx.x == 0) bulk_wait_all();
 }
 
+// find_or_claim from slot s, `probed` slots past the home that are known to hold
+// other keys, with the keys of kAhead slots loaded at a time: the events
+// that are left for the global pass are those with long probes, and each step
+// was a trip to memory (29,000 events of a 5 Mbp build: 39 -> 25 us).  (A slot seen taken by another key stays that key's; one
+// seen empty is claimed or refused by the CAS.)
+__device__ __forceinline__ bool find_or_claim_ahead(Slot *table, uint64_t n_slots,
+                                                    uint32_t max_probes, uint64_t key, uint64_t s,
+                                                    uint32_t probed, uint64_t &slot_out,
+                                                    bool *claimed) {
+  constexpr uint32_t kAhead = 8;
+  while (probed < max_probes) {
+    unsigned long long cur[kAhead];
+    uint64_t at[kAhead];
+#pragma unroll
+    for (uint32_t j = 0; j < kAhead; ++j) {
+      at[j] = s;
+      cur[j] = ld_relaxed_u64(&table[s].key);
+      if (++s == n_slots) s = 0;
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < kAhead; ++j) {
+      if (probed >= max_probes) return false;
+      ++probed;
+      if (cur[j] == kEmpty) {
+        cur[j] = atomicCAS(&table[at[j]].key, kEmpty, (unsigned long long)key);
+        *claimed = cur[j] == kEmpty;
+        if (*claimed) cur[j] = key;
+      }
+      if (cur[j] == key) {
+        slot_out = at[j];
+        return true;
+      }
+    }
+  }
+  return false;
+}
+
 // One event with the global find-or-claim (its tile is final by now): from its
 // home slot, or (left_tile: its probe found every slot from home to the tile's
 // end taken by other keys, and no slot empties again) from the next tile on.
@@ -1435,7 +1472,7 @@ __device__ __forceinline__ uint32_t global_event(uint64_t e, const ItemDesc &it,
     s = end == it.n_slots ? 0 : end;
   }
   bool claimed = false;
-  if (find_or_claim_from(it.table, it.n_slots, it.max_probes, key, s, probed, s, &claimed)) {
+  if (find_or_claim_ahead(it.table, it.n_slots, it.max_probes, key, s, probed, s, &claimed)) {
     if (e & 4ull) atomicAdd(&it.table[s].cnt[e & 3ull], 1u);
   } else {
     spill_or_fail(it.spill, it.spill_cap, it.spill_count, it.status, key, (e & 4ull) != 0,
@@ -1444,29 +1481,69 @@ __device__ __forceinline__ uint32_t global_event(uint64_t e, const ItemDesc &it,
   return claimed ? 1u : 0u;
 }
 
+// Empty an item's table with `ctas` CTAs, this one the cta-th.
+__device__ __forceinline__ void empty_table(const ItemDesc &it, uint64_t cta, uint64_t ctas) {
+  uint4 *t = reinterpret_cast<uint4 *>(it.table);
+  const uint64_t n_vec = 2 * it.n_slots;
+  const uint4 head = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);
+  const uint4 tail = make_uint4(0u, 0u, 0u, 0u);
+  for (uint64_t v = cta * blockDim.x + threadIdx.x; v < n_vec; v += ctas * blockDim.x)
+    t[v] = (v & 1) ? tail : head;
+}
+
+// What the chain leaves to the direct insert, which counts nothing: the tables
+// of a rebuild, emptied.
+template <int N>
+__device__ __forceinline__ void hand_over(const ItemPack<N> &pk) {
+  for (int i = 0; i < pk.n_items; ++i) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *small_counted(pk.d[i].status) = 0u;
+    empty_table(pk.d[i], blockIdx.x, gridDim.x);
+  }
+}
+
+// Part of a list of n that this CTA takes: CTAs share a region's list when
+// there are fewer regions than CTAs (a table of 1.6 M slots
+// has seven: 23 us of its 0.2 ms build with a CTA each, 13 shared and with the
+// look-ahead above).
+struct ListShare {
+  int per_list, lists;
+  __device__ __forceinline__ ListShare(int parts)
+      : per_list(max(1, (int)gridDim.x / parts)), lists(parts) {}
+  template <class F>
+  __device__ __forceinline__ void each_list(F &&f) const {
+    for (int w = blockIdx.x; w < lists * per_list; w += gridDim.x)
+      f(w / per_list, (uint64_t)(w % per_list) * blockDim.x + threadIdx.x,
+        (uint64_t)per_list * blockDim.x);
+  }
+};
+
 // The events that left their tile (each region's list), then those of the
 // overflow area ((event, region) pairs).  New
 // vertices are added to their graph's built counts (meaningful only on a
 // rebuild, which zeroed them): one atomic per warp and region, and for the
 // overflow area one per warp of a single table, else one per new vertex.
+// fresh: a rebuild; without the binned path the tables are emptied here.
 template <int N>
 __global__ void k_tile_deferred(const __grid_constant__ ItemPack<N> pk,
                                 const uint64_t *__restrict__ ev,
                                 const uint64_t *__restrict__ ev2, const unsigned long long *begin,
-                                TileAux aux, int parts, const uint32_t *use_binned) {
-  if (ld_volatile_u32(use_binned) == 0u) return;
-  for (int p = blockIdx.x; p < parts; p += gridDim.x) {
+                                TileAux aux, int parts, bool fresh, const uint32_t *use_binned) {
+  if (ld_volatile_u32(use_binned) == 0u) {
+    if (fresh) hand_over(pk);
+    return;
+  }
+  ListShare(parts).each_list([&](int p, uint64_t i, uint64_t step) {
     const uint64_t n = aux.deferred_n[p];
-    if (n == 0) continue;
-    if (threadIdx.x == 0) atomicAdd(aux.deferred, (unsigned long long)n);
+    if (n == 0) return;
+    if (i == 0) atomicAdd(aux.deferred, (unsigned long long)n);
     const ItemDesc &it = pk.d[aux.region_item[p]];
     const uint64_t *list = ev + begin[p];
     uint32_t claimed = 0;
-    for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) claimed += global_event(list[i], it, true);
+    for (; i < n; i += step) claimed += global_event(list[i], it, true);
     claimed = __reduce_add_sync(kFull, claimed);
     if ((threadIdx.x & 31) == 0 && claimed)
       atomicAdd(small_built(it.status), (unsigned long long)claimed);
-  }
+  });
   const uint64_t no = *aux.overflow;  // (all of it written: the flag is still set)
   const uint64_t *over = ev2 + aux.region_base[parts];
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -1486,29 +1563,17 @@ __global__ void k_tile_deferred(const __grid_constant__ ItemPack<N> pk,
   }
 }
 
-// Empty every item's table (grid: x strides over the slots, y = item); with
-// a gate, nothing happens when *gate != 0 (the binned kernels did the work: a
-// rebuild's tiled apply has emptied the tables itself); without one, the
-// items' sticky statuses and spill counts are cleared too.
+// Empty every item's table (grid: x strides over the slots, y = item) and clear
+// its sticky status and spill count.
 template <int N>
-__global__ void k_tables_init(const __grid_constant__ ItemPack<N> pk, const uint32_t *gate) {
-  if (gate != nullptr && ld_volatile_u32(gate) != 0u) return;
+__global__ void k_tables_init(const __grid_constant__ ItemPack<N> pk) {
   const int i = blockIdx.y;
   if (i >= pk.n_items) return;
-  if (gate == nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     *pk.d[i].status = 0u;
     *pk.d[i].spill_count = 0ull;
   }
-  // (the gated form runs when a binned chain gave its call to the direct
-  // insert, which counts nothing)
-  if (gate != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *small_counted(pk.d[i].status) = 0u;
-  uint4 *t = reinterpret_cast<uint4 *>(pk.d[i].table);
-  const uint64_t n_vec = 2 * pk.d[i].n_slots;
-  const uint4 head = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);
-  const uint4 tail = make_uint4(0u, 0u, 0u, 0u);
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n_vec; v += stride)
-    t[v] = (v & 1) ? tail : head;
+  empty_table(pk.d[i], blockIdx.x, gridDim.x);
 }
 
 int ceil_log2(uint64_t x) {
@@ -1905,18 +1970,12 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
     DBG_CK(cudaGetLastError());
   }
   mark(6, s);
-  k_tile_deferred<N><<<sms * 4, 256, 0, s>>>(pk, sc.ev, sc.ev2, mv.begin, aux, parts, mv.flag);
+  k_tile_deferred<N><<<sms * 8, 256, 0, s>>>(pk, sc.ev, sc.ev2, mv.begin, aux, parts, fresh,
+                                             mv.flag);
   DBG_CK(cudaGetLastError());
   // the direct insert runs only if the events did not fit the buffer (then no
-  // binned kernel touched the tables: a rebuild from empty empties them first)
+  // binned kernel touched the tables: the last one has emptied a rebuild's)
   mark(7, s);
-  if (fresh) {
-    ItemPack<N> ip{};
-    ip.n_items = n;
-    for (int i = 0; i < n; ++i) ip.d[i] = items[i];
-    k_tables_init<N><<<dim3(std::max(1, sms * 8 / n), n), 256, 0, s>>>(ip, mv.flag);
-    DBG_CK(cudaGetLastError());
-  }
   const int st = launch_insert(items, n, tuning, sms, s, mv.flag);
   if (st != DBG_OK) return st;
   mark(8, s);
@@ -2130,7 +2189,7 @@ int launch_tables_init(const ItemDesc *items, int n, int sm_count, cudaStream_t 
   ip.n_items = n;
   for (int i = 0; i < n; ++i) ip.d[i] = items[i];
   k_tables_init<kBatchItems><<<dim3(std::max(1, std::max(1, sm_count) * 8 / n), n), 256, 0, s>>>(
-      ip, nullptr);
+      ip);
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }

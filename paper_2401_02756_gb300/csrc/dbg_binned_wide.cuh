@@ -446,10 +446,14 @@ __global__ void __launch_bounds__(kWideBlock, 3)
 
 // As k_tile_deferred: the events that left their tile, then the overflow area,
 // from their home slots.
-__global__ void k_wide_deferred(ItemDesc it, const WideEvent *__restrict__ ev,
+__global__ void k_wide_deferred(const __grid_constant__ ItemPack<1> pk, const WideEvent *__restrict__ ev,
                                 const WideEvent *__restrict__ ev2, const unsigned long long *begin,
                                 TileAux aux, int parts, const uint32_t *use_binned) {
-  if (ld_volatile_u32(use_binned) == 0u) return;
+  if (ld_volatile_u32(use_binned) == 0u) {
+    hand_over(pk);
+    return;
+  }
+  const ItemDesc &it = pk.d[0];
   WideSlot *table = reinterpret_cast<WideSlot *>(it.table);
   uint32_t claimed = 0;
   auto apply = [&](const WideEvent &e) {
@@ -463,11 +467,11 @@ __global__ void k_wide_deferred(ItemDesc it, const WideEvent *__restrict__ ev,
     }
     claimed += fresh ? 1u : 0u;
   };
-  for (int p = blockIdx.x; p < parts; p += gridDim.x) {
+  ListShare(parts).each_list([&](int p, uint64_t i, uint64_t step) {
     const uint64_t n = aux.deferred_n[p];
-    if (n && threadIdx.x == 0) atomicAdd(aux.deferred, (unsigned long long)n);
-    for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) apply(ev[begin[p] + i]);
-  }
+    if (n && i == 0) atomicAdd(aux.deferred, (unsigned long long)n);
+    for (; i < n; i += step) apply(ev[begin[p] + i]);
+  });
   const uint64_t no = *aux.overflow;  // (all of it written: the flag is still set)
   const WideEvent *over = ev2 + aux.region_base[parts];
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -573,13 +577,11 @@ int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int cal
     DBG_CK(cudaGetLastError());
   }
   mark(6, s);
-  k_wide_deferred<<<sms * 4, 256, 0, s>>>(pk.d[0], ev, ev2, mv.begin, aux, parts, mv.flag);
+  k_wide_deferred<<<sms * 8, 256, 0, s>>>(pk, ev, ev2, mv.begin, aux, parts, mv.flag);
   DBG_CK(cudaGetLastError());
   // the direct insert runs only if the events did not fit (then nothing has
-  // touched the table: it is emptied first)
+  // touched the table: the last kernel has emptied it)
   mark(7, s);
-  k_tables_init<1><<<dim3(sms * 8, 1), 256, 0, s>>>(pk, mv.flag);
-  DBG_CK(cudaGetLastError());
   DBG_TRY(launch_insert_wide(it, h->sm_count, s, mv.flag));
   mark(8, s);
   h->built_counts = true;  // (unless it fell back: see small_counted)

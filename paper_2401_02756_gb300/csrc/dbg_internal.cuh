@@ -185,13 +185,11 @@ __device__ __forceinline__ uint64_t key_from_words(uint64_t lo, uint64_t hi, uin
 // probing from the home slot, a relaxed load first, atomicCAS only on EMPTY).
 // Returns false after max_probes slots without success.
 // `claimed` (optional): set when this call claimed the slot (a new vertex).
-// find_or_claim_from starts at slot s, `probed` slots past the key's home, all
-// of them known to hold other keys.
-__device__ __forceinline__ bool find_or_claim_from(Slot *table, uint64_t n_slots,
-                                                   uint32_t max_probes, uint64_t key, uint64_t s,
-                                                   uint32_t probed, uint64_t &slot_out,
-                                                   bool *claimed = nullptr) {
-  for (uint32_t i = probed; i < max_probes; ++i) {
+__device__ __forceinline__ bool find_or_claim(Slot *table, uint64_t n_slots, uint32_t max_probes,
+                                              uint64_t key, uint64_t &slot_out,
+                                              bool *claimed = nullptr) {
+  uint64_t s = home_slot(key, n_slots);
+  for (uint32_t i = 0; i < max_probes; ++i) {
     unsigned long long cur = ld_relaxed_u64(&table[s].key);
     if (cur == key) {
       slot_out = s;
@@ -208,13 +206,6 @@ __device__ __forceinline__ bool find_or_claim_from(Slot *table, uint64_t n_slots
     if (++s == n_slots) s = 0;
   }
   return false;
-}
-
-__device__ __forceinline__ bool find_or_claim(Slot *table, uint64_t n_slots, uint32_t max_probes,
-                                              uint64_t key, uint64_t &slot_out,
-                                              bool *claimed = nullptr) {
-  return find_or_claim_from(table, n_slots, max_probes, key, home_slot(key, n_slots), 0u, slot_out,
-                            claimed);
 }
 
 // Every graph's small block of device memory (64 bytes beside its table):
