@@ -216,6 +216,7 @@ __global__ void __launch_bounds__(1024)
 template <int N>
 __global__ void k_bin_totals(const __grid_constant__ ItemPack<N> pk, unsigned long long *totals,
                              unsigned long long *edges, int clear, uint32_t *fill, uint64_t tiles) {
+  after_previous();
   const int i = blockIdx.y;
   if (i >= pk.n_items) return;
   // the tiles' fill counts, for the split
@@ -289,6 +290,7 @@ __global__ void __launch_bounds__(1024)
                   const unsigned long long *edges, int fresh, int shift, int parts,
                   unsigned long long *begin, unsigned long long *cursor, uint64_t cap,
                   unsigned long long *ctr, uint32_t *use_binned, TileAux aux) {
+  after_previous();
   __shared__ unsigned long long s_warp[32];
   const int tid = threadIdx.x;
   if (tid < pk.n_items) {  // a rebuild counts its vertices (its claims) and its edges
@@ -502,6 +504,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
                   unsigned long long *cursor, uint64_t *out, uint64_t cap,
                   unsigned long long *ctr, uint32_t *use_binned,
                   const unsigned long long *bucket_end) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) return;
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned char *p = smem + tile_smem_bytes(tile_reads);
@@ -740,6 +743,7 @@ __global__ void __launch_bounds__(1024)
     k_tile_units(unsigned long long *counts, const unsigned long long *begin,
                  const unsigned long long *cursor, int parts, uint64_t unit, uint64_t ev2_cap,
                  TileAux aux, const uint32_t *use_binned) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) return;
   // (single precision throughout, see k_bin_buckets: the sizes need not be exact,
   // only their sum within the buffer, and `avail` leaves a 64th of it free)
@@ -909,6 +913,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)  // two CTAs of 512 threa
     k_tile_scatter(const uint64_t *__restrict__ ev, uint64_t *__restrict__ ev2, uint64_t ev2_cap,
                    const unsigned long long *begin, const unsigned long long *counts, TileAux aux,
                    int parts, uint64_t unit, int tpr, uint32_t *status, uint32_t *use_binned) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) return;
   constexpr int C = BLOCK * kBatch;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1209,6 +1214,7 @@ __device__ __forceinline__ void load_bucket(const uint64_t *__restrict__ bucket,
 
 // tile_region[t] = the region of every tile t (one CTA per region).
 __global__ void k_tile_map(TileAux aux, int parts, const uint32_t *use_binned) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) return;
   const int p = blockIdx.x;
   if (p >= parts) return;
@@ -1243,6 +1249,7 @@ __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 thr
     k_tile_apply(const __grid_constant__ ItemPack<N> pk, const uint64_t *__restrict__ ev2,
                  uint64_t *ev, const unsigned long long *begin, TileAux aux, int parts,
                  int tpr_log2, const uint32_t *use_binned) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) return;
   extern __shared__ __align__(16) unsigned char smem[];  // (bulk copies need 16 bytes)
   // !FRESH: kTileSlots slots (AoS); FRESH: keys and label-major counters (SoA)
@@ -1528,6 +1535,7 @@ __global__ void k_tile_deferred(const __grid_constant__ ItemPack<N> pk,
                                 const uint64_t *__restrict__ ev,
                                 const uint64_t *__restrict__ ev2, const unsigned long long *begin,
                                 TileAux aux, int parts, bool fresh, const uint32_t *use_binned) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) {
     if (fresh) hand_over(pk);
     return;
@@ -1567,6 +1575,7 @@ __global__ void k_tile_deferred(const __grid_constant__ ItemPack<N> pk,
 // its sticky status and spill count.
 template <int N>
 __global__ void k_tables_init(const __grid_constant__ ItemPack<N> pk) {
+  after_previous();
   const int i = blockIdx.y;
   if (i >= pk.n_items) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1819,9 +1828,14 @@ int launch_apply_m(dbg_handle h, const MetaView &mv, const BinGeometry &geo, int
   }
 }
 
+// Launches of a chain overlap (launch_next) up to so many tiles of all its
+// tables: 8 M slots (at 86 M slots they no longer gain).
+constexpr uint64_t kOverlapTiles = 4096;
+
 template <int BT, bool STAGED, bool SMALL>
-int launch_tile_scatter(const BinScratch &sc, const MetaView &mv, const TileAux &aux, int parts,
-                        uint64_t unit, int tpr, int sms, cudaStream_t s, uint32_t *status) {
+int launch_tile_scatter(bool overlap, const BinScratch &sc, const MetaView &mv,
+                        const TileAux &aux, int parts, uint64_t unit, int tpr, int sms,
+                        cudaStream_t s, uint32_t *status) {
   if (tpr > kMaxBinsPerThread * BT) return DBG_ERR_INVALID_ARG;  // (the launch sizes BT by tpr)
   const size_t smem = tile_scatter_smem<BT, STAGED>(tpr);
   // (set even below 48 KB: the kernel's static shared memory counts too)
@@ -1830,9 +1844,9 @@ int launch_tile_scatter(const BinScratch &sc, const MetaView &mv, const TileAux 
   int per_sm = 0;
   DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_scatter<BT, STAGED, SMALL>, BT,
                                                        smem));
-  k_tile_scatter<BT, STAGED, SMALL><<<std::max(1, per_sm) * sms, BT, smem, s>>>(
-      sc.ev, sc.ev2, ev2_capacity(sc.cap), mv.begin, mv.counts, aux, parts, unit, tpr, status,
-      mv.flag);
+  DBG_TRY(launch_next(overlap, k_tile_scatter<BT, STAGED, SMALL>, std::max(1, per_sm) * sms, BT,
+                      smem, s, sc.ev, sc.ev2, ev2_capacity(sc.cap), mv.begin, mv.counts, aux, parts,
+                      unit, tpr, status, mv.flag));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
@@ -1860,6 +1874,7 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
                 int sms, cudaStream_t s, bool fresh, const Marks &mark, const InputParts *input) {
   const MetaView mv = meta_view(sc);
   const int tpr = 1 << (shift - kTileLog2);
+  const bool overlap = tiles <= kOverlapTiles;
   const TileAux aux = tile_aux(sc, parts, tiles);
   ItemPack<N> pk{};
   pk.n_items = n;
@@ -1880,14 +1895,14 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
     const uint64_t want = std::min<uint64_t>((max_reads + 256 * 32 - 1) / (256 * 32),
                                              (uint64_t)std::max(1, 16384 / n));
     const int gx = (int)std::max<uint64_t>(want, (uint64_t)std::max(1, (sms * 4 + n - 1) / n));
-    k_bin_totals<N><<<dim3(gx, n), 256, 0, s>>>(pk, mv.totals, mv.edges, fresh ? 1 : 0, aux.fill,
-                                                tiles);
+    DBG_TRY(launch_next(overlap, k_bin_totals<N>, dim3(gx, n), 256, 0, s, pk, mv.totals, mv.edges,
+                        fresh ? 1 : 0, aux.fill, tiles));
     DBG_CK(cudaGetLastError());
-    k_bin_buckets<N><<<1, 1024, 0, s>>>(pk, mv.totals, mv.edges, fresh ? 1 : 0, shift, parts,
-                                        mv.begin, mv.cursor, sc.cap, mv.ctr, mv.flag, aux);
+    DBG_TRY(launch_next(overlap, k_bin_buckets<N>, 1, 1024, 0, s, pk, mv.totals, mv.edges, fresh ? 1
+                        : 0, shift, parts, mv.begin, mv.cursor, sc.cap, mv.ctr, mv.flag, aux));
     DBG_CK(cudaGetLastError());
     if (N > 1) {
-      k_tile_map<<<parts, 256, 0, s>>>(aux, parts, mv.flag);
+      DBG_TRY(launch_next(overlap, k_tile_map, parts, 256, 0, s, aux, parts, mv.flag));
       DBG_CK(cudaGetLastError());
     }
   }
@@ -1920,16 +1935,16 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
       const uint64_t sl = std::min<uint64_t>(b - a, kBinSlices);
       const int grid = (int)std::max<uint64_t>(
           1, std::min<uint64_t>(sl, (uint64_t)std::max(1, per_sm) * sms));
-      k_bin_scatter<BS, N, SMALL, true><<<grid, BS, smem, s>>>(pk, scatter_reads, shift, parts, a, b, sl,
-                                                  mv.hist, mv.cursor, sc.ev, sc.cap, mv.ctr,
-                                                  mv.flag, mv.begin + 1);
+      DBG_TRY(launch_next(overlap, k_bin_scatter<BS, N, SMALL, true>, grid, BS, smem, s, pk,
+                          scatter_reads, shift, parts, a, b, sl, mv.hist, mv.cursor, sc.ev, sc.cap,
+                          mv.ctr, mv.flag, mv.begin + 1));
       DBG_CK(cudaGetLastError());
     }
   }
   const uint64_t unit = tile_unit(tpr);
   mark(4, s);
-  k_tile_units<<<1, 1024, 0, s>>>(mv.counts, mv.begin, mv.cursor, parts, unit,
-                                  ev2_capacity(sc.cap), aux, mv.flag);
+  DBG_TRY(launch_next(overlap, k_tile_units, 1, 1024, 0, s, mv.counts, mv.begin, mv.cursor, parts,
+                      unit, ev2_capacity(sc.cap), aux, mv.flag));
   DBG_CK(cudaGetLastError());
   // chunks of 8 events per thread: larger blocks for more tiles per region,
   // so that each tile's run in a chunk stays several events long (a timeout of
@@ -1940,13 +1955,13 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
   if (tuning.split_threads > 0 && tpr <= kMaxBinsPerThread * tuning.split_threads)
     bt = tuning.split_threads;
   if (bt == 256) {
-    DBG_TRY((launch_tile_scatter<256, true, SMALL>(sc, mv, aux, parts, unit, tpr, sms, s,
+    DBG_TRY((launch_tile_scatter<256, true, SMALL>(overlap, sc, mv, aux, parts, unit, tpr, sms, s,
                                             items[0].status)));
   } else if (bt == 512) {  // (1024 tiles: two bins per thread; measured faster than 1024 threads)
-    DBG_TRY((launch_tile_scatter<512, true, SMALL>(sc, mv, aux, parts, unit, tpr, sms, s,
+    DBG_TRY((launch_tile_scatter<512, true, SMALL>(overlap, sc, mv, aux, parts, unit, tpr, sms, s,
                                             items[0].status)));
   } else {
-    DBG_TRY((launch_tile_scatter<1024, false, SMALL>(sc, mv, aux, parts, unit, tpr, sms, s,
+    DBG_TRY((launch_tile_scatter<1024, false, SMALL>(overlap, sc, mv, aux, parts, unit, tpr, sms, s,
                                               items[0].status)));
   }
   mark(5, s);
@@ -1965,13 +1980,13 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
     DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BA, smem));
     const uint64_t grid = std::max<uint64_t>(
         1, std::min<uint64_t>(tiles, (uint64_t)std::max(1, per_sm) * sms));
-    kern<<<(int)grid, BA, smem, s>>>(pk, sc.ev2, sc.ev, mv.begin, aux, parts, shift - kTileLog2,
-                                     mv.flag);
+    DBG_TRY(launch_next(overlap, kern, (int)grid, BA, smem, s, pk, sc.ev2, sc.ev, mv.begin, aux,
+                        parts, shift - kTileLog2, mv.flag));
     DBG_CK(cudaGetLastError());
   }
   mark(6, s);
-  k_tile_deferred<N><<<sms * 8, 256, 0, s>>>(pk, sc.ev, sc.ev2, mv.begin, aux, parts, fresh,
-                                             mv.flag);
+  DBG_TRY(launch_next(overlap, k_tile_deferred<N>, sms * 8, 256, 0, s, pk, sc.ev, sc.ev2, mv.begin,
+                      aux, parts, fresh, mv.flag));
   DBG_CK(cudaGetLastError());
   // the direct insert runs only if the events did not fit the buffer (then no
   // binned kernel touched the tables: the last one has emptied a rebuild's)
@@ -2188,8 +2203,8 @@ int launch_tables_init(const ItemDesc *items, int n, int sm_count, cudaStream_t 
   ItemPack<kBatchItems> ip{};
   ip.n_items = n;
   for (int i = 0; i < n; ++i) ip.d[i] = items[i];
-  k_tables_init<kBatchItems><<<dim3(std::max(1, std::max(1, sm_count) * 8 / n), n), 256, 0, s>>>(
-      ip);
+  DBG_TRY(launch_after(k_tables_init<kBatchItems>, dim3(std::max(1, std::max(1, sm_count) * 8 / n),
+                       n), 256, 0, s, ip));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }

@@ -53,6 +53,7 @@ size_t wide_scatter_smem(int parts) {
 __global__ void __launch_bounds__(kWideBlock, 2)
     k_wide_scatter(ItemDesc it, int shift, int parts, unsigned long long *cursor,
                    const unsigned long long *bucket_end, WideEvent *out, uint32_t *use_binned) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) return;
   extern __shared__ __align__(16) unsigned char smem[];
   WideEvent *sorted = reinterpret_cast<WideEvent *>(smem);
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(kWideBlock, 2)
     k_wide_split(const WideEvent *__restrict__ ev, WideEvent *__restrict__ ev2, uint64_t ev2_cap,
                  const unsigned long long *begin, const unsigned long long *counts, TileAux aux,
                  int parts, uint64_t unit, int tpr, uint32_t *use_binned) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) return;
   extern __shared__ __align__(16) unsigned char smem[];
   WideEvent *s_ev = reinterpret_cast<WideEvent *>(smem);                  // kWideFlush, in tile order
@@ -340,6 +342,7 @@ __global__ void __launch_bounds__(kWideBlock, 3)
     k_wide_apply(ItemDesc it, const WideEvent *__restrict__ ev2, WideEvent *ev,
                  const unsigned long long *begin, TileAux aux, int parts, int tpr_log2,
                  const uint32_t *use_binned) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) return;
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned long long *ka = reinterpret_cast<unsigned long long *>(smem);
@@ -449,6 +452,7 @@ __global__ void __launch_bounds__(kWideBlock, 3)
 __global__ void k_wide_deferred(const __grid_constant__ ItemPack<1> pk, const WideEvent *__restrict__ ev,
                                 const WideEvent *__restrict__ ev2, const unsigned long long *begin,
                                 TileAux aux, int parts, const uint32_t *use_binned) {
+  after_previous();
   if (ld_volatile_u32(use_binned) == 0u) {
     hand_over(pk);
     return;
@@ -518,6 +522,7 @@ int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int cal
   const int shift = wide_shift(h), parts = regions_of(h->n_slots, shift);
   const int tpr = 1 << (shift - kTileLog2), sms = std::max(1, h->sm_count);
   const uint64_t tiles = table_tiles(h->n_slots, shift);
+  const bool overlap = tiles <= kOverlapTiles;
   const uint64_t cap = sc.cap / 2, cap2 = ev2_capacity(sc.cap) / 2;  // events
   const Marks mark{h, call};
   const MetaView mv = meta_view(sc);
@@ -537,9 +542,10 @@ int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int cal
   mark(1, s);
   const int gx = (int)std::max<uint64_t>((uint64_t)sms * 4,
                                          std::min<uint64_t>(16384, (it.n_reads + 8191) / 8192));
-  k_bin_totals<1><<<dim3(gx, 1), 256, 0, s>>>(pk, mv.totals, mv.edges, 1, aux.fill, tiles);
-  k_bin_buckets<1><<<1, 1024, 0, s>>>(pk, mv.totals, mv.edges, 1, shift, parts, mv.begin, mv.cursor,
-                                      cap, mv.ctr, mv.flag, aux);
+  DBG_TRY(launch_next(overlap, k_bin_totals<1>, dim3(gx, 1), 256, 0, s, pk, mv.totals, mv.edges, 1,
+                      aux.fill, tiles));
+  DBG_TRY(launch_next(overlap, k_bin_buckets<1>, 1, 1024, 0, s, pk, mv.totals, mv.edges, 1, shift,
+                      parts, mv.begin, mv.cursor, cap, mv.ctr, mv.flag, aux));
   DBG_CK(cudaGetLastError());
   mark(3, s);
   {
@@ -548,20 +554,22 @@ int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int cal
     int per_sm = 0;
     DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wide_scatter, kWideBlock, smem));
     const uint64_t walk = (it.n_reads + kWideTile - 1) / kWideTile;
-    k_wide_scatter<<<(int)std::min<uint64_t>(walk, (uint64_t)std::max(1, per_sm) * sms), kWideBlock,
-                     smem, s>>>(pk.d[0], shift, parts, mv.cursor, mv.begin + 1, ev, mv.flag);
+    DBG_TRY(launch_next(overlap, k_wide_scatter, (int)std::min<uint64_t>(walk, (uint64_t)std::max(1,
+                        per_sm) * sms), kWideBlock, smem, s, pk.d[0], shift, parts, mv.cursor,
+                        mv.begin + 1, ev, mv.flag));
     DBG_CK(cudaGetLastError());
   }
   mark(4, s);
   const uint64_t unit = tile_unit(tpr);
-  k_tile_units<<<1, 1024, 0, s>>>(mv.counts, mv.begin, mv.cursor, parts, unit, cap2, aux, mv.flag);
+  DBG_TRY(launch_next(overlap, k_tile_units, 1, 1024, 0, s, mv.counts, mv.begin, mv.cursor, parts,
+                      unit, cap2, aux, mv.flag));
   {
     const size_t smem = wide_split_smem(tpr);
     DBG_CK(cudaFuncSetAttribute(k_wide_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wide_split, kWideBlock, smem));
-    k_wide_split<<<std::max(1, per_sm) * sms, kWideBlock, smem, s>>>(
-        ev, ev2, cap2, mv.begin, mv.counts, aux, parts, unit, tpr, mv.flag);
+    DBG_TRY(launch_next(overlap, k_wide_split, std::max(1, per_sm) * sms, kWideBlock, smem, s, ev,
+                        ev2, cap2, mv.begin, mv.counts, aux, parts, unit, tpr, mv.flag));
     DBG_CK(cudaGetLastError());
   }
   mark(5, s);
@@ -571,13 +579,14 @@ int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int cal
     int per_sm = 0;
     DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wide_apply, kWideBlock,
                                                          kWideTileBytes));
-    k_wide_apply<<<(int)std::min<uint64_t>(tiles, (uint64_t)std::max(1, per_sm) * sms), kWideBlock,
-                   kWideTileBytes, s>>>(pk.d[0], ev2, ev, mv.begin, aux, parts, shift - kTileLog2,
-                                        mv.flag);
+    DBG_TRY(launch_next(overlap, k_wide_apply, (int)std::min<uint64_t>(tiles, (uint64_t)std::max(1,
+                        per_sm) * sms), kWideBlock, kWideTileBytes, s, pk.d[0], ev2, ev, mv.begin,
+                        aux, parts, shift - kTileLog2, mv.flag));
     DBG_CK(cudaGetLastError());
   }
   mark(6, s);
-  k_wide_deferred<<<sms * 8, 256, 0, s>>>(pk, ev, ev2, mv.begin, aux, parts, mv.flag);
+  DBG_TRY(launch_next(overlap, k_wide_deferred, sms * 8, 256, 0, s, pk, ev, ev2, mv.begin, aux,
+                      parts, mv.flag));
   DBG_CK(cudaGetLastError());
   // the direct insert runs only if the events did not fit (then nothing has
   // touched the table: the last kernel has emptied it)

@@ -89,6 +89,7 @@ __device__ __forceinline__ uint32_t quotient(uint32_t c, double divisor) {
 }
 
 __global__ void __launch_bounds__(256) k_normalize(uint4 *t, uint64_t n, double divisor, int wide) {
+  after_previous();
   __shared__ uint32_t s_quot[kQuot];
   for (uint32_t c = threadIdx.x; c < kQuot; c += blockDim.x) s_quot[c] = quotient(c, divisor);
   __syncthreads();
@@ -157,6 +158,7 @@ struct SlotWords {
 // out-degrees as bits.  A warp takes 32 consecutive slots.  Bound by one read
 // of the table, then by the random target lookups.
 __global__ void __launch_bounds__(256) k_links(View v, Links k) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t w0 = (((uint64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5;
@@ -204,6 +206,7 @@ __global__ void __launch_bounds__(256) k_links(View v, Links k) {
 // edges with one atomic.
 __global__ void __launch_bounds__(256) k_start_edges(View v, Links k, unsigned long long *out,
                                                      unsigned long long *count, uint64_t cap) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const uint64_t words = (v.n + 31) >> 5;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -238,6 +241,7 @@ __global__ void __launch_bounds__(256) k_start_edges(View v, Links k, unsigned l
 
 // Every splitter walks to the next splitter or to the end of its chain.
 __global__ void __launch_bounds__(256) k_segments(View v, Links k, uint32_t n_split) {
+  after_previous();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_split; i += stride) {
     uint64_t s = k.split[i].y;
@@ -263,6 +267,7 @@ __global__ void __launch_bounds__(256) k_segments(View v, Links k, uint32_t n_sp
 
 // Jumps of level l + 1 from those of level l.
 __global__ void __launch_bounds__(256) k_double(Links k, uint32_t n_split, int l) {
+  after_previous();
   const uint32_t *next = k.next + (size_t)l * k.cap, *len = k.len + (size_t)l * k.cap;
   uint32_t *next2 = k.next + (size_t)(l + 1) * k.cap, *len2 = k.len + (size_t)(l + 1) * k.cap;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -344,6 +349,7 @@ __global__ void __launch_bounds__(256)
     k_contig_lengths(View v, Links k, const unsigned long long *starts, uint64_t n_starts, int m,
                      uint64_t guard, Contig *contigs, unsigned long long *len, Unit *units,
                      unsigned long long *n_units, uint64_t units_cap) {
+  after_previous();
   const uint32_t *jump = k.next + (size_t)kLevels * k.cap, *jlen = k.len + (size_t)kLevels * k.cap;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_starts; i += stride) {
@@ -404,6 +410,7 @@ __device__ __forceinline__ char letter(uint32_t label) { return (char)(0x5447434
 __global__ void __launch_bounds__(256)
     k_contig_heads(View v, Links k, const unsigned long long *starts, uint64_t n_starts, int m,
                    const Contig *contigs, const unsigned long long *off, char *out) {
+  after_previous();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_starts; i += stride) {
     const unsigned long long e = starts[i];
@@ -426,6 +433,7 @@ __global__ void __launch_bounds__(256)
 __global__ void __launch_bounds__(256)
     k_contig_units(View v, Links k, const Unit *units, uint64_t n_units, int m,
                    const Contig *contigs, const unsigned long long *off, char *out) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   for (uint64_t u = (((uint64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; u < n_units;
@@ -507,8 +515,8 @@ extern "C" int dbg_normalize(dbg_handle h, double divisor, void *stream) {
   if (st != DBG_OK) return st;
   const uint64_t want = (h->n_slots + 255) / 256;
   const int grid = (int)std::min<uint64_t>(want, (uint64_t)std::max(1, h->sm_count) * 8);
-  k_normalize<<<grid, 256, 0, s>>>(reinterpret_cast<uint4 *>(h->table), h->n_slots, divisor,
-                                   h->k > 32 ? 1 : 0);
+  DBG_TRY(launch_after(k_normalize, grid, 256, 0, s, reinterpret_cast<uint4 *>(h->table),
+                       h->n_slots, divisor, h->k > 32 ? 1 : 0));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
@@ -558,7 +566,8 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   k.cap = (uint32_t)cap;
   k.n_split = counts + 1;
   DBG_CK(cudaMemsetAsync(buf, 0, 256 + mark_bytes, s));  // counts and marks
-  k_links<<<(int)std::min<uint64_t>((words + 7) / 8, (uint64_t)grid), 256, 0, s>>>(v, k);
+  DBG_TRY(launch_after(k_links, (int)std::min<uint64_t>((words + 7) / 8, (uint64_t)grid), 256, 0, s,
+                       v, k));
   DBG_CK(cudaGetLastError());
 
   // the start edges into a buffer that holds as many as an ordinary graph has;
@@ -568,8 +577,8 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   unsigned long long got[3] = {0, 0, 0};  // start edges, splitters, units
   for (;;) {
     DBG_TRY(scr.get(reinterpret_cast<void **>(&starts_a), starts_cap * sizeof(unsigned long long)));
-    k_start_edges<<<(int)std::min<uint64_t>((words + 255) / 256, (uint64_t)grid), 256, 0, s>>>(
-        v, k, starts_a, counts, starts_cap);
+    DBG_TRY(launch_after(k_start_edges, (int)std::min<uint64_t>((words + 255) / 256,
+                         (uint64_t)grid), 256, 0, s, v, k, starts_a, counts, starts_cap));
     DBG_CK(cudaGetLastError());
     uint32_t status = 0;
     DBG_CK(cudaMemcpyAsync(got, counts, sizeof(got), cudaMemcpyDeviceToHost, s));
@@ -594,8 +603,8 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
 
   if (n_split > 0) {
     const int sg = (int)std::min<uint64_t>(((uint64_t)n_split + 255) / 256, (uint64_t)grid);
-    k_segments<<<sg, 256, 0, s>>>(v, k, n_split);
-    for (int l = 0; l < kLevels; ++l) k_double<<<sg, 256, 0, s>>>(k, n_split, l);
+    DBG_TRY(launch_after(k_segments, sg, 256, 0, s, v, k, n_split));
+    for (int l = 0; l < kLevels; ++l) DBG_TRY(launch_after(k_double, sg, 256, 0, s, k, n_split, l));
     DBG_CK(cudaGetLastError());
   }
   size_t sort_bytes = 0, scan_bytes = 0;
@@ -626,8 +635,8 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   for (;;) {
     if (units_cap > 0)
       DBG_TRY(scr.get(reinterpret_cast<void **>(&units), units_cap * sizeof(Unit)));
-    k_contig_lengths<<<cg, 256, 0, s>>>(v, k, starts_b, S, m, guard, contigs, len, units,
-                                        counts + 2, units_cap);
+    DBG_TRY(launch_after(k_contig_lengths, cg, 256, 0, s, v, k, starts_b, S, m, guard, contigs, len,
+                         units, counts + 2, units_cap));
     DBG_CK(cudaGetLastError());
     DBG_CK(cub::DeviceScan::ExclusiveSum(temp, scan_bytes, len, off, (int64_t)(S + 1), s));
     uint32_t status = 0;
@@ -644,11 +653,11 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   if (!bases_out || !offsets_out || S > max_contigs || B > max_bases) return DBG_ERR_BUFFER_TOO_SMALL;
   char *chars = nullptr;
   DBG_TRY(scr.get(reinterpret_cast<void **>(&chars), std::max<uint64_t>(B, 1)));
-  k_contig_heads<<<cg, 256, 0, s>>>(v, k, starts_b, S, m, contigs, off, chars);
+  DBG_TRY(launch_after(k_contig_heads, cg, 256, 0, s, v, k, starts_b, S, m, contigs, off, chars));
   DBG_CK(cudaGetLastError());
   if (got[2] > 0) {
-    k_contig_units<<<(int)std::min<uint64_t>((got[2] + 7) / 8, (uint64_t)grid), 256, 0, s>>>(
-        v, k, units, got[2], m, contigs, off, chars);
+    DBG_TRY(launch_after(k_contig_units, (int)std::min<uint64_t>((got[2] + 7) / 8, (uint64_t)grid),
+                         256, 0, s, v, k, units, got[2], m, contigs, off, chars));
     DBG_CK(cudaGetLastError());
   }
   DBG_CK(cudaMemcpyAsync(offsets_out, off, (S + 1) * sizeof(uint64_t), cudaMemcpyDefault, s));

@@ -165,6 +165,7 @@ __device__ __forceinline__ Key<WIDE> ld_key(const Slot *p) {
 // Vertices per bin.  Bound by one read of the table.
 template <bool WIDE>
 __global__ void __launch_bounds__(256) k_histogram(const Slot *t, uint64_t n, Plan p) {
+  after_previous();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += stride * kSlotsPerThread) {
@@ -206,6 +207,7 @@ __device__ __forceinline__ void fill_meta(const Plan &p, uint32_t vertices, cons
 // The plan of up to kPlanBins bins in one CTA: prefix, buckets, largest bin.
 __global__ void __launch_bounds__(kPlanBlock)
     k_plan(Plan p, const uint32_t *status, const unsigned long long *spilled) {
+  after_previous();
   constexpr int kPer = kPlanBins / kPlanBlock;
   __shared__ uint32_t s_warp[32], s_last[kPlanBlock + 1];
   const uint32_t nbins = 1u << p.bin_bits;
@@ -257,6 +259,7 @@ __global__ void __launch_bounds__(kPlanBlock)
 // The same from a finished prefix (more bins).
 __global__ void __launch_bounds__(256)
     k_buckets(Plan p, const uint32_t *status, const unsigned long long *spilled) {
+  after_previous();
   const uint32_t nbins = 1u << p.bin_bits;
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t n = 0;
@@ -280,6 +283,7 @@ __global__ void __launch_bounds__(256)
 template <bool WIDE, bool RECORDS>
 __global__ void __launch_bounds__(256) k_place(const Slot *t, uint64_t n, Plan p, Slot *rec,
                                                Key<WIDE> *keys, uint4 *counts) {
+  after_previous();
   if (!may_run(p)) return;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -330,6 +334,7 @@ constexpr size_t sort_smem() {
 template <bool WIDE, bool RECORDS>
 __global__ void __launch_bounds__(kSortBlock, RECORDS && !WIDE ? 6 : 4)
     k_bucket_sort(Plan p, const Slot *rec, Key<WIDE> *keys, uint4 *counts) {
+  after_previous();
   constexpr int kPer = kBucketCap / kSortBlock;
   constexpr int kBinsPer = kLocalBins / kSortBlock;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -502,29 +507,32 @@ int run(dbg_handle h, const Shape &sh, uint64_t max_rows, void *buf, Slot *rec, 
   const int grid = (int)std::min<uint64_t>((n + 256 * kSlotsPerThread - 1) / (256 * kSlotsPerThread),
                                            (uint64_t)sms * 8);
   DBG_CK(cudaMemsetAsync(b, 0, sh.off_start, s));  // meta and histogram
-  k_histogram<WIDE><<<grid, 256, 0, s>>>(h->table, n, p);
+  DBG_TRY(launch_after(k_histogram<WIDE>, grid, 256, 0, s, h->table, n, p));
   DBG_CK(cudaGetLastError());
   if (sh.nbins <= (uint32_t)kPlanBins) {
-    k_plan<<<1, kPlanBlock, 0, s>>>(p, h->d_status, h->d_spill_count);
+    DBG_TRY(launch_after(k_plan, 1, kPlanBlock, 0, s, p, h->d_status, h->d_spill_count));
   } else {
     size_t temp = sh.temp;
     DBG_CK(cub::DeviceScan::ExclusiveSum(b + sh.off_temp, temp, p.bins, p.bins,
                                          (int)sh.nbins + 1, s));
-    k_buckets<<<(sh.nbins + 256) / 256, 256, 0, s>>>(p, h->d_status, h->d_spill_count);
+    DBG_TRY(launch_after(k_buckets, (sh.nbins + 256) / 256, 256, 0, s, p, h->d_status,
+                         h->d_spill_count));
   }
   DBG_CK(cudaGetLastError());
   if (rec) {
     constexpr size_t smem = sort_smem<WIDE, true>();
-    k_place<WIDE, true><<<grid, 256, 0, s>>>(h->table, n, p, rec, keys, counts);
+    DBG_TRY(launch_after(k_place<WIDE, true>, grid, 256, 0, s, h->table, n, p, rec, keys, counts));
     DBG_CK(cudaFuncSetAttribute(k_bucket_sort<WIDE, true>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_bucket_sort<WIDE, true><<<sh.buckets, kSortBlock, smem, s>>>(p, rec, keys, counts);
+    DBG_TRY(launch_after(k_bucket_sort<WIDE, true>, sh.buckets, kSortBlock, smem, s, p, rec, keys,
+                         counts));
   } else {
     constexpr size_t smem = sort_smem<WIDE, false>();
-    k_place<WIDE, false><<<grid, 256, 0, s>>>(h->table, n, p, rec, keys, counts);
+    DBG_TRY(launch_after(k_place<WIDE, false>, grid, 256, 0, s, h->table, n, p, rec, keys, counts));
     DBG_CK(cudaFuncSetAttribute(k_bucket_sort<WIDE, false>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_bucket_sort<WIDE, false><<<sh.buckets, kSortBlock, smem, s>>>(p, rec, keys, counts);
+    DBG_TRY(launch_after(k_bucket_sort<WIDE, false>, sh.buckets, kSortBlock, smem, s, p, rec, keys,
+                         counts));
   }
   DBG_CK(cudaGetLastError());
   DBG_CK(cudaMemcpyAsync(&m, p.meta, sizeof(m), cudaMemcpyDeviceToHost, s));

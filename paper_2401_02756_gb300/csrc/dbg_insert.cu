@@ -91,6 +91,7 @@ struct InsertVisitor {
 template <int BLOCK, bool AGG, int N>
 __global__ void __launch_bounds__(BLOCK, 2048 / BLOCK)
     k_insert(const __grid_constant__ ItemPack<N> pk, int tile_reads, const uint32_t *gate) {
+  after_previous();
   if (gate != nullptr && ld_volatile_u32(gate) != 0u) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ volatile uint32_t s_cap_hit;
@@ -133,7 +134,7 @@ int launch_one(ItemPack<N> &pk, int tile_reads, int grid_ctas, int sm_count, cud
   if (pk.total_tiles == 0) return DBG_OK;
   int grid = grid_ctas > 0 ? grid_ctas : resident;
   if ((uint64_t)grid > pk.total_tiles) grid = (int)pk.total_tiles;
-  kern<<<grid, BLOCK, smem, stream>>>(pk, tile_reads, gate);
+  DBG_TRY(launch_after(kern, grid, BLOCK, smem, stream, pk, tile_reads, gate));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }

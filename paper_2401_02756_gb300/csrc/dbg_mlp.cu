@@ -48,6 +48,7 @@ template <bool TRAIN>
 __global__ void __launch_bounds__(32 * kWarps)
     k_rows(const float *__restrict__ P, const float *__restrict__ x,
            const float *__restrict__ target, int B, float *y, Work w) {
+  after_previous();
   __shared__ float s_h1[kRows][kHid], s_h2[kRows][kHid], s_dh2[kRows][kHid];
   __shared__ float s_part[kRows][kHid], s_dy[kRows];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -158,6 +159,7 @@ constexpr int kGradRows = 256;                  // rows staged at a time
 // its biases too.
 __global__ void __launch_bounds__(256, 2)
     k_grads(const float *__restrict__ x, const float *__restrict__ target, int B, Work w, Adam ad) {
+  after_previous();
   __shared__ __align__(16) float s_x[kGradRows][kCols];
   __shared__ float s_red[4][kHid][kCols + 1];
   const int j = threadIdx.x & (kHid - 1), group = threadIdx.x >> 6;
@@ -253,6 +255,7 @@ __global__ void k_init(float *p, uint64_t seed) {
 
 // x[b][j] = registers[b * stride + j] / 64: sketch registers as network inputs.
 __global__ void k_features(const uint32_t *regs, int64_t stride, int B, float *x) {
+  after_previous();
   const int64_t n = (int64_t)B * kIn;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -283,7 +286,8 @@ extern "C" uint64_t dbg_mlp_work_floats(int batch) {
 extern "C" int dbg_mlp_features(const uint32_t *registers, int64_t stride, int batch, float *x,
                                 void *stream) {
   if (!registers || !x || batch <= 0 || stride < DBG_MLP_INPUTS) return DBG_ERR_INVALID_ARG;
-  k_features<<<256, 256, 0, static_cast<cudaStream_t>(stream)>>>(registers, stride, batch, x);
+  DBG_TRY(launch_after(k_features, 256, 256, 0, static_cast<cudaStream_t>(stream), registers,
+                       stride, batch, x));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
@@ -298,8 +302,8 @@ extern "C" int dbg_mlp_init(float *params, uint64_t seed, void *stream) {
 extern "C" int dbg_mlp_forward(const float *params, const float *x, int batch, float *y,
                                float *work, void *stream) {
   if (!params || !x || !y || !work || batch <= 0) return DBG_ERR_INVALID_ARG;
-  k_rows<false><<<(batch + kRows - 1) / kRows, 32 * kWarps, 0, static_cast<cudaStream_t>(stream)>>>(
-      params, x, nullptr, batch, y, Work{});
+  DBG_TRY(launch_after(k_rows<false>, (batch + kRows - 1) / kRows, 32 * kWarps, 0,
+                       static_cast<cudaStream_t>(stream), params, x, nullptr, batch, y, Work{}));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
@@ -312,12 +316,13 @@ extern "C" int dbg_mlp_train_step(float *params, float *grads, float *adam_m, fl
     return DBG_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const Work w = carve(work, batch);
-  k_rows<true><<<(batch + kRows - 1) / kRows, 32 * kWarps, 0, s>>>(params, x, target, batch, w.y, w);
+  DBG_TRY(launch_after(k_rows<true>, (batch + kRows - 1) / kRows, 32 * kWarps, 0, s, params, x,
+                       target, batch, w.y, w));
   DBG_CK(cudaGetLastError());
   const float b1 = 0.9f, b2 = 0.999f;
   const Adam ad{params, grads, adam_m, adam_v, lr,
                 b1,     b2,    1e-8f,  1.f - powf(b1, (float)step), 1.f - powf(b2, (float)step)};
-  k_grads<<<kGradCtas, 256, 0, s>>>(x, target, batch, w, ad);
+  DBG_TRY(launch_after(k_grads, kGradCtas, 256, 0, s, x, target, batch, w, ad));
   DBG_CK(cudaGetLastError());
   if (loss_out) DBG_CK(cudaMemcpyAsync(loss_out, w.loss, sizeof(float), cudaMemcpyDefault, s));
   return DBG_OK;

@@ -105,6 +105,7 @@ struct SketchVisitor {
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, kSketchCtas)
     k_sketch(const __grid_constant__ ItemPack<1> pk, int tile_reads, uint64_t chunk, uint32_t *regs) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t *s_reg = reinterpret_cast<uint32_t *>(smem + tile_smem_bytes(tile_reads));
   __shared__ uint32_t s_floor;
@@ -123,6 +124,7 @@ template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, kSketchCtas)
     k_sketch_batch(const __grid_constant__ ItemPack<kSketchItems> pk, int tile_reads,
                    uint64_t chunk) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t *s_reg = reinterpret_cast<uint32_t *>(smem + tile_smem_bytes(tile_reads));
   __shared__ uint32_t s_floor;
@@ -151,6 +153,7 @@ uint64_t sketch_chunk(uint64_t tiles, uint64_t resident) {
 
 // Every item's registers and status word := 0.
 __global__ void k_zero_registers(const __grid_constant__ ItemPack<kSketchItems> pk) {
+  after_previous();
   const int i = blockIdx.x;
   uint32_t *r = reinterpret_cast<uint32_t *>(pk.d[i].table);
   for (int j = threadIdx.x; j <= kSketchRegs; j += blockDim.x) r[j] = 0u;
@@ -190,7 +193,7 @@ extern "C" int dbg_sketch_reads(int k, const uint8_t *packed, const uint64_t *of
   DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sketch<B>, B, smem));
   const uint64_t chunk = sketch_chunk(pk.total_tiles, (uint64_t)std::max(1, per_sm) * sms);
   const int grid = (int)((pk.total_tiles + chunk - 1) / chunk);
-  k_sketch<B><<<grid, B, smem, s>>>(pk, tile_reads, chunk, registers);
+  DBG_TRY(launch_after(k_sketch<B>, grid, B, smem, s, pk, tile_reads, chunk, registers));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
@@ -235,12 +238,12 @@ extern "C" int dbg_sketch_batch(const dbg_sketch_item *items, int n_items, void 
       tiles += (src.n_reads + tile_reads - 1) / tile_reads;
     }
     pk.total_tiles = tiles;
-    k_zero_registers<<<cnt, 256, 0, s>>>(pk);
+    DBG_TRY(launch_after(k_zero_registers, cnt, 256, 0, s, pk));
     DBG_CK(cudaGetLastError());
     if (tiles == 0) continue;
     const uint64_t chunk = sketch_chunk(tiles, (uint64_t)std::max(1, per_sm) * sms);
     const int grid = (int)((tiles + chunk - 1) / chunk);
-    k_sketch_batch<B><<<grid, B, smem, s>>>(pk, tile_reads, chunk);
+    DBG_TRY(launch_after(k_sketch_batch<B>, grid, B, smem, s, pk, tile_reads, chunk));
     DBG_CK(cudaGetLastError());
   }
   return DBG_OK;

@@ -102,6 +102,7 @@ struct DeviceGuard {
 // (status, spilled: if not null, cleared too)
 __global__ void k_table_init(uint4 *t, uint64_t n_vec, uint32_t *status,
                              unsigned long long *spilled) {
+  after_previous();
   if (status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
     *status = 0u;
     *spilled = 0ull;
@@ -116,6 +117,7 @@ __global__ void k_table_init(uint4 *t, uint64_t n_vec, uint32_t *status,
 // Vertices (occupied slots) and edges (sum of counters) of a table.
 // (wide: keys of k > 32 take two words, so the counters sit at byte 16)
 __global__ void k_stats(const Slot *t, uint64_t n_slots, unsigned long long *acc, int wide) {
+  after_previous();
   unsigned long long nv = 0, ne = 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_slots; i += stride) {
@@ -150,8 +152,8 @@ static int table_init(Slot *table, uint64_t n_slots, uint32_t *status, unsigned 
   const uint64_t n_vec = n_slots * 2;
   uint64_t want = (n_vec + 255) / 256;
   const int grid = (int)std::min<uint64_t>(want, (uint64_t)stream_grid(sms, 8));
-  k_table_init<<<std::max(grid, 1), 256, 0, stream>>>(reinterpret_cast<uint4 *>(table), n_vec,
-                                                      status, spilled);
+  DBG_TRY(launch_after(k_table_init, std::max(grid, 1), 256, 0, stream, reinterpret_cast<uint4
+                       *>(table), n_vec, status, spilled));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
@@ -173,7 +175,8 @@ int launch_stats(const Slot *table, uint64_t n_slots, unsigned long long *acc, c
   DBG_CK(cudaMemsetAsync(acc, 0, 2 * sizeof(unsigned long long), stream));
   const uint64_t want = (n_slots + 255) / 256;
   const int grid = (int)std::min<uint64_t>(want, (uint64_t)stream_grid(sms, 8));
-  k_stats<<<std::max(grid, 1), 256, 0, stream>>>(table, n_slots, acc, wide ? 1 : 0);
+  DBG_TRY(launch_after(k_stats, std::max(grid, 1), 256, 0, stream, table, n_slots, acc, wide ? 1 :
+                       0));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }

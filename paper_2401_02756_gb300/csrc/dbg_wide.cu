@@ -30,6 +30,7 @@ namespace {
 // by the number of reads.
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 6) k_insert_wide(ItemDesc it, int tile_reads, const uint32_t *gate) {
+  after_previous();
   if (gate != nullptr && ld_volatile_u32(gate) != 0u) return;
   __shared__ uint64_t s_off[kWideTile + 1];
   __shared__ uint64_t s_pre[kWideTile + 1];
@@ -194,7 +195,8 @@ int launch_insert_wide(const ItemDesc &it, int sm_count, cudaStream_t s, const u
   const uint64_t resident = (uint64_t)std::max(1, per_sm) * std::max(1, sm_count);
   const int tile_reads = std::min(kWideTile, auto_tile_reads(it.n_reads, resident));
   const uint64_t tiles = (it.n_reads + tile_reads - 1) / tile_reads;
-  k_insert_wide<B><<<(int)std::min(tiles, resident), B, 0, s>>>(it, tile_reads, gate);
+  DBG_TRY(launch_after(k_insert_wide<B>, (int)std::min(tiles, resident), B, 0, s, it, tile_reads,
+                       gate));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
