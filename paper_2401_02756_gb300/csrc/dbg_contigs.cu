@@ -22,12 +22,12 @@
 // 32-byte load.  A second pass over the bits emits the start edges.
 //
 // A walk is a chain of dependent loads (about half a microsecond each), so a
-// long contig is cut at splitters: one in kSplit of the single-exit vertices,
+// long contig is cut at splitters: one in kSpacing of the single-exit vertices,
 // chosen by the key's hash.  Every splitter walks to the next one, all in
-// parallel; kLevels rounds of pointer doubling give jumps over up to
-// 2^kLevels segments; a contig walks to its first splitter and jumps on from
-// there, listing a unit of 2^kLevels segments per jump; and a warp per unit
-// writes its segments' bases, a lane each.  A contig that meets a cycle (or a
+// parallel, noting the labels; rounds of pointer doubling give jumps over up to
+// 2^levels segments; a contig walks to its first splitter and jumps on from
+// there, listing a unit of 2^levels segments per jump; and a lane per segment
+// of a unit writes its bases.  A contig that meets a cycle (or a
 // stretch of kMaxWalk steps without a splitter, which only a short cycle is)
 // is walked by one thread instead: Brent's cycle detection (R. P. Brent, "An
 // improved Monte Carlo factorization algorithm", BIT 20, 1980) finds the
@@ -35,11 +35,9 @@
 //
 // Measured against one thread per contig walking by table lookups, with a pass
 // each to clear, mark, count and emit, twice over for the size query: a 50 kb
-// error-free genome (one contig) 43 -> 0.37 ms, a 5 Mbp graph of 31,000
-// contigs (2.75 GB table) 16.4 -> 2.1 ms, of which k_links takes 1.08 (the
-// table read once: 0.41) and segments, lengths, heads and units 0.15 to 0.27
-// each, the latency of their longest chain.  kSplit: 32 against 64 halves that
-// chain; the jumps make the number of segments matter little.
+// error-free genome (one contig) 43 -> 0.25 ms, a 5 Mbp graph of 31,000
+// contigs (2.75 GB table) 16.4 -> 1.6 ms, of which k_links takes 1.05 (the
+// table read once: 0.41), segments 0.15 (5 M random slots: 0.12), units 0.09.
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_scan.cuh>
 
@@ -112,8 +110,8 @@ __global__ void __launch_bounds__(256) k_normalize(uint4 *t, uint64_t n, double 
   }
 }
 
-constexpr uint32_t kSplit = 32;        // one splitter in so many single-exit vertices
-constexpr int kLevels = 5;             // jumps of up to 2^kLevels segments: a lane each
+constexpr uint32_t kSpacing = 4;       // one splitter in so many single-exit vertices (a power of two)
+constexpr uint32_t kLabels = 32;
 constexpr uint32_t kMaxWalk = 2048;    // steps without a splitter before a walk counts as a cycle's
 constexpr uint32_t kEnd = ~0u;         // a segment's successor: the walk ends there
 constexpr uint32_t kCyclic = ~0u - 1;  // it went kMaxWalk steps without meeting a splitter
@@ -124,10 +122,13 @@ constexpr unsigned long long kIsSplitter = 1ull << 63;  // in a slot's link: the
 struct Links {
   uint32_t *marks;                    // a bit per slot: an edge points to its vertex
   uint2 *degree;                      // per 32 slots: bits of one exit, bits of several
-  ulonglong2 *split;                  // a splitter's slot and its successor's slot
-  uint32_t *next, *len;               // [kLevels + 1][cap]: the splitter 2^l segments on, the edges to it
-  uint32_t cap;                       // splitters kept (a vertex past them is an ordinary one)
+  ulonglong2 *split;                  // a splitter's slot (its label in the two top bits), its successor's
+  unsigned long long *labels;         // the first kLabels labels of its segment, two bits each
+  uint32_t *next, *len;               // [levels + 1][kept]: the splitter 2^l segments on, the edges to it
+  uint32_t cap;                       // splitters there is room for (a vertex past them is an ordinary one)
+  uint32_t kept;                      // splitters there are
   unsigned long long *n_split;        // splitters found
+  int levels;                         // jumps of up to 2^levels segments
 };
 
 __device__ __forceinline__ unsigned long long *link_of(Slot *t, uint64_t s) {
@@ -155,47 +156,71 @@ struct SlotWords {
 };
 
 // Every edge marks its target; every single-exit vertex gets its link; the
-// out-degrees as bits.  A warp takes 32 consecutive slots.  Bound by one read
-// of the table, then by the random target lookups.
+// out-degrees as bits.  A warp takes kLinkWords times 32 consecutive slots (once in
+// a table of few CTAs).  Bound by one read of the table, then by the random target lookups.  (Splitters are
+// numbered by the CTA: an atomic per warp on the one counter, at one splitter in 4
+// vertices, took 2.6 ms of a 2.75 GB table where the rest takes 1.05.)
+template <int kLinkWords>
 __global__ void __launch_bounds__(256) k_links(View v, Links k) {
   after_previous();
-  const int lane = threadIdx.x & 31;
-  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  const uint64_t w0 = (((uint64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5;
-  const uint64_t words = (v.n + 31) >> 5;
-  for (uint64_t w = w0; w < words; w += warps) {
-    const uint64_t i = (w << 5) + lane;
-    unsigned long long key = kEmpty;
-    uint32_t exits = 0;
-    if (i < v.n) {
-      const SlotWords sl(v.t, i);
-      key = sl.key();
-      if (key != kEmpty) exits = sl.exits();
-    }
-    uint64_t target = 0;
-    for (uint32_t rest = exits; rest; rest &= rest - 1) {
-      const uint32_t b = (uint32_t)__ffs((int)rest) - 1u;
-      const uint64_t s = find_key(v, ((key << 2) | (uint64_t)b) & v.mask);
-      if (s == kNotFound) {
-        atomicCAS(v.status, 0u, (uint32_t)DBG_ERR_CAPACITY);  // a target is missing
-        continue;
+  __shared__ uint32_t s_picks[2];
+  __shared__ unsigned long long s_at;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const uint64_t words = (v.n + 31) >> 5, step = (uint64_t)warps * kLinkWords;
+  if (threadIdx.x < 2) s_picks[threadIdx.x] = 0u;
+  __syncthreads();
+  int turn = 0;
+  for (uint64_t w0 = blockIdx.x * step; w0 < words; w0 += gridDim.x * step, turn ^= 1) {
+    uint64_t target[kLinkWords];
+    unsigned ones[kLinkWords], picks[kLinkWords];
+    uint32_t at[kLinkWords], label[kLinkWords];
+#pragma unroll
+    for (int u = 0; u < kLinkWords; ++u) {
+      const uint64_t w = w0 + (uint64_t)(u * warps + warp), i = (w << 5) + lane;
+      unsigned long long key = kEmpty;
+      uint32_t exits = 0;
+      if (i < v.n) {
+        const SlotWords sl(v.t, i);
+        key = sl.key();
+        if (key != kEmpty) exits = sl.exits();
       }
-      target = s;
-      atomicOr(&k.marks[s >> 5], 1u << (s & 31));
+      target[u] = 0;
+      for (uint32_t rest = exits; rest; rest &= rest - 1) {
+        const uint32_t b = (uint32_t)__ffs((int)rest) - 1u;
+        const uint64_t s = find_key(v, ((key << 2) | (uint64_t)b) & v.mask);
+        if (s == kNotFound) {
+          atomicCAS(v.status, 0u, (uint32_t)DBG_ERR_CAPACITY);  // a target is missing
+          continue;
+        }
+        target[u] = s;
+        atomicOr(&k.marks[s >> 5], 1u << (s & 31));
+      }
+      label[u] = (uint32_t)__ffs((int)exits) - 1u;  // (of a single-exit vertex)
+      const bool one = exits != 0 && (exits & (exits - 1)) == 0;
+      ones[u] = __ballot_sync(0xffffffffu, one);
+      const unsigned several = __ballot_sync(0xffffffffu, exits != 0 && !one);
+      if (lane == 0 && w < words) k.degree[w] = make_uint2(ones[u], several);
+      picks[u] = __ballot_sync(0xffffffffu,
+                               one && ((uint32_t)key_hash(key) & (kSpacing - 1u)) == 0u);
+      at[u] = 0;
+      if (lane == 0 && picks[u]) at[u] = atomicAdd(&s_picks[turn], (uint32_t)__popc(picks[u]));
     }
-    const bool one = exits != 0 && (exits & (exits - 1)) == 0;
-    const unsigned ones = __ballot_sync(0xffffffffu, one);
-    const unsigned several = __ballot_sync(0xffffffffu, exits != 0 && !one);
-    if (lane == 0) k.degree[w] = make_uint2(ones, several);
-    const bool pick = one && (uint32_t)key_hash(key) % kSplit == 0u;
-    const unsigned picks = __ballot_sync(0xffffffffu, pick);
-    unsigned long long at = 0;
-    if (lane == 0 && picks) at = atomicAdd(k.n_split, (unsigned long long)__popc(picks));
-    at = __shfl_sync(0xffffffffu, at, 0) + __popc(picks & ((1u << lane) - 1u));
-    if (one) {
-      const bool split = pick && at < k.cap;
-      if (split) k.split[at] = make_ulonglong2(i, target);
-      *link_of(v.t, i) = split ? (kIsSplitter | at) : target;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s_at = s_picks[turn] ? atomicAdd(k.n_split, (unsigned long long)s_picks[turn]) : 0ull;
+      s_picks[turn ^ 1] = 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kLinkWords; ++u) {
+      const uint64_t i = ((w0 + (uint64_t)(u * warps + warp)) << 5) + lane;
+      const unsigned long long n = s_at + __shfl_sync(0xffffffffu, at[u], 0) +
+                                   (unsigned)__popc(picks[u] & ((1u << lane) - 1u));
+      if (!(ones[u] >> lane & 1u)) continue;
+      const bool split = (picks[u] >> lane & 1u) && n < k.cap;
+      if (split)
+        k.split[n] = make_ulonglong2(i | ((unsigned long long)label[u] << 62), target[u]);
+      *link_of(v.t, i) = split ? (kIsSplitter | n) : target[u];
     }
   }
 }
@@ -239,12 +264,16 @@ __global__ void __launch_bounds__(256) k_start_edges(View v, Links k, unsigned l
   }
 }
 
-// Every splitter walks to the next splitter or to the end of its chain.
-__global__ void __launch_bounds__(256) k_segments(View v, Links k, uint32_t n_split) {
+// Every splitter walks to the next splitter or to the end of its chain and notes
+// the labels on its way, so that writing the contigs need not walk again (a 5
+// Mbp graph: units 0.30 -> 0.09 ms).
+__global__ void __launch_bounds__(256) k_segments(View v, Links k) {
   after_previous();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_split; i += stride) {
-    uint64_t s = k.split[i].y;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k.kept; i += stride) {
+    const ulonglong2 from = k.split[i];
+    uint64_t s = from.y;
+    unsigned long long labels = from.x >> 62;
     uint32_t edges = 1, next = kCyclic;
     for (; edges <= kMaxWalk; ++edges) {
       const SlotWords sl(v.t, s);
@@ -258,20 +287,22 @@ __global__ void __launch_bounds__(256) k_segments(View v, Links k, uint32_t n_sp
         next = (uint32_t)link;
         break;
       }
+      if (edges < kLabels) labels |= (unsigned long long)(__ffs((int)e) - 1) << (2 * edges);
       s = link;
     }
+    k.labels[i] = labels;
     k.next[i] = next;
     k.len[i] = edges;
   }
 }
 
 // Jumps of level l + 1 from those of level l.
-__global__ void __launch_bounds__(256) k_double(Links k, uint32_t n_split, int l) {
+__global__ void __launch_bounds__(256) k_double(Links k, int l) {
   after_previous();
-  const uint32_t *next = k.next + (size_t)l * k.cap, *len = k.len + (size_t)l * k.cap;
-  uint32_t *next2 = k.next + (size_t)(l + 1) * k.cap, *len2 = k.len + (size_t)(l + 1) * k.cap;
+  const uint32_t *next = k.next + (size_t)l * k.kept, *len = k.len + (size_t)l * k.kept;
+  uint32_t *next2 = k.next + (size_t)(l + 1) * k.kept, *len2 = k.len + (size_t)(l + 1) * k.kept;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_split; i += stride) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k.kept; i += stride) {
     const uint32_t a = next[i];
     const bool on = a < kCyclic;
     next2[i] = on ? next[a] : a;
@@ -331,7 +362,7 @@ __device__ uint64_t contig_edges(const View &v, const Links &k, uint64_t x0, uin
   return 1 + mu + lam;  // the walk arrives at x_mu again after mu + lam steps
 }
 
-// A stretch of up to 2^kLevels segments of a contig, from splitter `split`,
+// A stretch of up to 2^levels segments of a contig, from splitter `split`,
 // `rel` edges into the contig.
 struct Unit {
   uint32_t contig, split;
@@ -350,7 +381,8 @@ __global__ void __launch_bounds__(256)
                      uint64_t guard, Contig *contigs, unsigned long long *len, Unit *units,
                      unsigned long long *n_units, uint64_t units_cap) {
   after_previous();
-  const uint32_t *jump = k.next + (size_t)kLevels * k.cap, *jlen = k.len + (size_t)kLevels * k.cap;
+  const uint32_t *jump = k.next + (size_t)k.levels * k.kept;
+  const uint32_t *jlen = k.len + (size_t)k.levels * k.kept;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_starts; i += stride) {
     const uint64_t x0 = find_key(v, starts[i] & v.mask);
@@ -428,31 +460,35 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// A warp per unit: lane j takes the j-th segment, found by jumps of the bits
-// of j, and writes its bases.
+// A lane per segment of a unit: the j-th is found by jumps of the bits of j, and
+// its bases are written.
 __global__ void __launch_bounds__(256)
     k_contig_units(View v, Links k, const Unit *units, uint64_t n_units, int m,
                    const Contig *contigs, const unsigned long long *off, char *out) {
   after_previous();
-  const int lane = threadIdx.x & 31;
-  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t u = (((uint64_t)blockIdx.x * blockDim.x) + threadIdx.x) >> 5; u < n_units;
-       u += warps) {
-    const Unit un = units[u];
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; g >> k.levels < n_units;
+       g += stride) {
+    const uint32_t j0 = (uint32_t)g & ((1u << k.levels) - 1u);
+    const Unit un = units[g >> k.levels];
     if (!contigs[un.contig].by_units) continue;  // a cycle: written by the contig's own thread
     uint32_t i = un.split;
     unsigned long long rel = un.rel;
-#pragma unroll
-    for (int l = 0; l < kLevels; ++l) {
-      if (((lane >> l) & 1) && i < kCyclic) {
-        rel += k.len[(size_t)l * k.cap + i];
-        i = k.next[(size_t)l * k.cap + i];
+    for (int l = k.levels - 1; l >= 0; --l) {  // (longest first: lanes past the end leave at once)
+      if (((j0 >> l) & 1u) && i < kCyclic) {
+        rel += k.len[(size_t)l * k.kept + i];
+        i = k.next[(size_t)l * k.kept + i];
       }
     }
     if (i >= kCyclic) continue;
     char *o = out + off[un.contig] + m + rel;
     const uint32_t edges = k.len[i];
-    uint64_t s = k.split[i].x;
+    if (edges <= kLabels) {
+      unsigned long long labels = k.labels[i];
+      for (uint32_t j = 0; j < edges; ++j, labels >>= 2) o[j] = letter((uint32_t)labels & 3u);
+      continue;
+    }
+    uint64_t s = k.split[i].x & (~0ull >> 2);
     for (uint32_t j = 0; j < edges; ++j) {
       const SlotWords sl(v.t, s);
       o[j] = letter((uint32_t)__ffs((int)sl.exits()) - 1u);
@@ -476,6 +512,29 @@ struct Guard {
     if (changed) cudaSetDevice(prev);
   }
 };
+
+// The passes that walk -- segments, lengths, heads, units -- take as long as
+// their longest chain of half-microsecond steps: about kSpacing * ln(splitters)
+// for a segment, and a jump per kSpacing * 2^levels edges of the longest contig.
+// Splitters are dense, then, as far as there is room (a splitter takes 24 bytes
+// and 8 a level): for every one of a table of up to 2^20 slots, for one in 32
+// single-exit vertices of a full larger table, which a graph cleaned of its error
+// k-mers seldom reaches.  One in 4 against one in 32: a 50 kb genome 500 -> 360 us
+// with its build, the 31,000 contigs of a 5 Mbp one 2.1 -> 1.8 ms.
+uint64_t room_splitters(uint64_t n_slots) {
+  const uint64_t n = std::max(std::min<uint64_t>(n_slots / kSpacing, 1u << 18), n_slots / 32);
+  return std::min<uint64_t>(n + n / 12 + 1024, 1ull << 30);
+}
+constexpr int kMaxLevels = 10;
+int room_levels(uint64_t n_slots) { return n_slots <= 1ull << 23 ? kMaxLevels : 5; }
+// Levels: jumps over 1024 edges at least, and over a contig's average number of
+// segments, as far as `room` numbers are enough for the arrays.
+int levels_of(uint64_t n_split, uint64_t contigs, uint64_t room) {
+  int levels = 8;
+  static_assert((kSpacing << 8) == 1024, "jumps over 1024 edges");
+  while (levels < kMaxLevels && (n_split / contigs) >> levels) ++levels;
+  return (int)std::min<uint64_t>(levels, room / n_split - 1);
+}
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -538,14 +597,14 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   const int grid = std::max(1, h->sm_count) * 8;
   Scratch scr{s};
   // marks, degrees and splitters by the table's size; a twelfth more splitters
-  // than one vertex in kSplit of a full table gives (when that much memory is
+  // than one vertex in `spacing` of a full table gives (when that much memory is
   // not to be had: none, and every contig is walked by its own thread)
   const uint64_t words = (h->n_slots + 31) >> 5;
-  uint64_t cap = std::min<uint64_t>(h->n_slots / kSplit + h->n_slots / (12 * kSplit) + 1024,
-                                    1ull << 30);
+  uint64_t cap = room_splitters(h->n_slots);
+  const uint64_t rounds = (uint64_t)room_levels(h->n_slots) + 1;
   const size_t mark_bytes = align256(words * 4), bits_bytes = 256 + mark_bytes + align256(words * 8);
-  auto split_bytes = [](uint64_t c) {
-    return align256(c * sizeof(ulonglong2)) + 2 * align256(c * 4 * (kLevels + 1));
+  auto split_bytes = [rounds](uint64_t c) {
+    return align256(c * sizeof(ulonglong2)) + 2 * align256(c * 4 * rounds) + align256(c * 8);
   };
   char *buf = nullptr;
   st = scr.get(reinterpret_cast<void **>(&buf), bits_bytes + split_bytes(cap));
@@ -562,12 +621,18 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   k.split = reinterpret_cast<ulonglong2 *>(buf + bits_bytes);
   k.next = reinterpret_cast<uint32_t *>(buf + bits_bytes + align256(cap * sizeof(ulonglong2)));
   k.len = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(k.next) +
-                                       align256(cap * 4 * (kLevels + 1)));
+                                       align256(cap * 4 * rounds));
+  k.labels = reinterpret_cast<unsigned long long *>(
+      reinterpret_cast<char *>(k.len) + align256(cap * 4 * rounds));
   k.cap = (uint32_t)cap;
   k.n_split = counts + 1;
   DBG_CK(cudaMemsetAsync(buf, 0, 256 + mark_bytes, s));  // counts and marks
-  DBG_TRY(launch_after(k_links, (int)std::min<uint64_t>((words + 7) / 8, (uint64_t)grid), 256, 0, s,
-                       v, k));
+  if (h->n_slots <= 1u << 20)
+    DBG_TRY(launch_after(k_links<1>, (int)std::min<uint64_t>((words + 7) / 8, (uint64_t)grid), 256,
+                         0, s, v, k));
+  else
+    DBG_TRY(launch_after(k_links<2>, (int)std::min<uint64_t>((words + 15) / 16, (uint64_t)grid),
+                         256, 0, s, v, k));
   DBG_CK(cudaGetLastError());
 
   // the start edges into a buffer that holds as many as an ordinary graph has;
@@ -601,10 +666,13 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   }
   if (S > 0xFFFFFFFFull) return DBG_ERR_CAPACITY;  // (contig numbers in a unit are 32-bit)
 
+  k.kept = n_split;
   if (n_split > 0) {
+    k.levels = levels_of(n_split, S, cap * rounds);
     const int sg = (int)std::min<uint64_t>(((uint64_t)n_split + 255) / 256, (uint64_t)grid);
-    DBG_TRY(launch_after(k_segments, sg, 256, 0, s, v, k, n_split));
-    for (int l = 0; l < kLevels; ++l) DBG_TRY(launch_after(k_double, sg, 256, 0, s, k, n_split, l));
+    DBG_TRY(launch_after(k_segments, sg, 256, 0, s, v, k));
+    for (int l = 0; l < k.levels; ++l)
+      DBG_TRY(launch_after(k_double, sg, 256, 0, s, k, l));
     DBG_CK(cudaGetLastError());
   }
   size_t sort_bytes = 0, scan_bytes = 0;
@@ -625,11 +693,11 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   void *temp = buf2 + 3 * eb + cb;
   DBG_CK(cub::DeviceRadixSort::SortKeys(temp, sort_bytes, starts_a, starts_b, (int64_t)S, 0,
                                         2 * m + 2, s));
-  // a unit per jump: one or two a contig, and one in every 2^kLevels splitters
+  // a unit per jump: one or two a contig, and one in every 2^levels splitters
   // (again with as many as were counted when contigs share long tails)
   const uint64_t guard = 4 * h->n_slots + 64;
   const int cg = (int)std::min<uint64_t>((S + 255) / 256, (uint64_t)grid);
-  uint64_t units_cap = n_split > 0 ? 2 * S + (n_split >> (kLevels - 1)) + 1024 : 0;
+  uint64_t units_cap = n_split > 0 ? 2 * S + (n_split >> (k.levels - 1)) + 1024 : 0;
   Unit *units = nullptr;
   unsigned long long B = 0;
   for (;;) {
@@ -656,8 +724,8 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   DBG_TRY(launch_after(k_contig_heads, cg, 256, 0, s, v, k, starts_b, S, m, contigs, off, chars));
   DBG_CK(cudaGetLastError());
   if (got[2] > 0) {
-    DBG_TRY(launch_after(k_contig_units, (int)std::min<uint64_t>((got[2] + 7) / 8, (uint64_t)grid),
-                         256, 0, s, v, k, units, got[2], m, contigs, off, chars));
+    DBG_TRY(launch_after(k_contig_units, (int)std::min<uint64_t>(((got[2] << k.levels) + 255) / 256,
+                         (uint64_t)grid), 256, 0, s, v, k, units, got[2], m, contigs, off, chars));
     DBG_CK(cudaGetLastError());
   }
   DBG_CK(cudaMemcpyAsync(offsets_out, off, (S + 1) * sizeof(uint64_t), cudaMemcpyDefault, s));

@@ -71,3 +71,19 @@ def test_normalize_small_and_large_counts(divisor):
     g.close()
     assert np.array_equal(keys, ref.keys)
     assert np.array_equal(counts, oc.normalize(ref.counts, divisor))
+
+
+# (tables at the edges of the splitters' spacings and of the room for more levels)
+@pytest.mark.parametrize("slots", [1 << 20, (1 << 20) + 1, (1 << 21) + 1, (1 << 22) + 1, 1 << 23,
+                                   (1 << 23) + 1])
+def test_table_sizes(slots):
+    k = 21
+    tail = random_text(9_000, 3)
+    loop = random_text(3000, 8)
+    texts = [random_text(n, 200 + n) for n in (25, 700, 250_000)]
+    texts += [random_text(60, 100 + i) + tail for i in range(20)] + [random_text(500, 9) + loop + loop[:k]]
+    rs = synth.from_strings(texts, k)
+    ref = oracle.build_graph(rs.packed, rs.offsets, k)
+    g = gpu_graph(rs, capacity=slots)
+    assert g.contigs() == oc.find_contigs(ref.keys, ref.counts, k)
+    g.close()
