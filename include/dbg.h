@@ -304,7 +304,9 @@ int dbg_build_batch(const dbg_batch_item *items, int n_items, void *stream);
 
 /* Give back the device memory the library keeps between calls: the batched
  * inserts' buffers and the pool of the exports and of mid-size rebuilds, on every device
- * (each is synchronised first).  Later calls allocate again as needed.
+ * (each is synchronised first), and the 4 KB page of pinned host memory that
+ * results are reported through when no call uses it (calls copy their results
+ * until the next graph is created).  Later calls allocate again as needed.
  * Errors: CUDA. */
 int dbg_release_scratch(void);
 

@@ -554,10 +554,10 @@ struct Scratch {
 };
 
 int read_status(dbg_handle h, cudaStream_t s) {
-  uint32_t st = 0;
-  DBG_CK(cudaMemcpyAsync(&st, h->d_status, sizeof(st), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaStreamSynchronize(s));
-  return (int)st;
+  const DeviceWord status{h->d_status, 4};
+  uint64_t got = 0;
+  DBG_TRY(read_words(&status, 1, &got, s));
+  return (int)got;
 }
 
 }  // namespace
@@ -639,17 +639,15 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   // a second pass when there are more
   uint64_t starts_cap = h->n_slots / 16 + 1024;
   unsigned long long *starts_a = nullptr;
-  unsigned long long got[3] = {0, 0, 0};  // start edges, splitters, units
+  uint64_t got[4] = {0, 0, 0, 0};  // start edges, splitters, units, status
   for (;;) {
     DBG_TRY(scr.get(reinterpret_cast<void **>(&starts_a), starts_cap * sizeof(unsigned long long)));
     DBG_TRY(launch_after(k_start_edges, (int)std::min<uint64_t>((words + 255) / 256,
                          (uint64_t)grid), 256, 0, s, v, k, starts_a, counts, starts_cap));
     DBG_CK(cudaGetLastError());
-    uint32_t status = 0;
-    DBG_CK(cudaMemcpyAsync(got, counts, sizeof(got), cudaMemcpyDeviceToHost, s));
-    DBG_CK(cudaMemcpyAsync(&status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, s));
-    DBG_CK(cudaStreamSynchronize(s));
-    if (status != DBG_OK) return (int)status;
+    const DeviceWord words[] = {{counts, 8}, {counts + 1, 8}, {counts + 2, 8}, {h->d_status, 4}};
+    DBG_TRY(read_words(words, 4, got, s));
+    if (got[3] != DBG_OK) return (int)got[3];
     if (got[0] <= starts_cap) break;
     starts_cap = got[0];
     DBG_CK(cudaMemsetAsync(counts, 0, sizeof(unsigned long long), s));
@@ -707,13 +705,12 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
                          units, counts + 2, units_cap));
     DBG_CK(cudaGetLastError());
     DBG_CK(cub::DeviceScan::ExclusiveSum(temp, scan_bytes, len, off, (int64_t)(S + 1), s));
-    uint32_t status = 0;
-    DBG_CK(cudaMemcpyAsync(&B, off + S, sizeof(B), cudaMemcpyDeviceToHost, s));
-    DBG_CK(cudaMemcpyAsync(&got[2], counts + 2, sizeof(got[2]), cudaMemcpyDeviceToHost, s));
-    DBG_CK(cudaMemcpyAsync(&status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, s));
-    DBG_CK(cudaStreamSynchronize(s));
-    *n_bases = B;
-    if (status != DBG_OK) return (int)status;
+    const DeviceWord words[] = {{counts + 2, 8}, {h->d_status, 4}, {off + S, 8}};
+    uint64_t now[3];
+    DBG_TRY(read_words(words, 3, now, s));
+    got[2] = now[0];
+    *n_bases = B = now[2];
+    if (now[1] != DBG_OK) return (int)now[1];
     if (got[2] <= units_cap) break;
     units_cap = got[2];
     DBG_CK(cudaMemsetAsync(counts + 2, 0, sizeof(unsigned long long), s));

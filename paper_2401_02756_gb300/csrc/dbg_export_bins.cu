@@ -72,6 +72,7 @@ struct Plan {
   uint32_t *first_bin;  // [buckets + 2]
   uint32_t *cursor;     // [buckets + 2][kCursorStride] next free position, or null: the bins' own
   ExportMeta *meta;
+  ExportMeta *report;   // the sort's copy of it in pinned host memory, or null
 };
 
 // Whether the placing and the sort may run: a complete graph, room for it,
@@ -345,6 +346,7 @@ __global__ void __launch_bounds__(kSortBlock, RECORDS && !WIDE ? 6 : 4)
       RECORDS ? reinterpret_cast<unsigned char *>(s_src + kBucketCap)
               : reinterpret_cast<unsigned char *>(s_row + kBucketCap));
   __shared__ uint32_t s_warp[kSortBlock / 32];
+  if (p.report && blockIdx.x == 0 && threadIdx.x == 0) *p.report = *p.meta;
   if (!may_run(p)) return;
   const uint32_t b = blockIdx.x;
   if (b > p.meta->vertices >> p.bucket_log2) return;
@@ -495,6 +497,8 @@ int run(dbg_handle h, const Shape &sh, uint64_t max_rows, void *buf, Slot *rec, 
   p.max_rows = max_rows;
   p.max_placed = rec ? rec_rows : ~0ull;
   p.meta = reinterpret_cast<ExportMeta *>(b);
+  const ReportSlot slot;
+  p.report = reinterpret_cast<ExportMeta *>(slot.p);
   p.bins = reinterpret_cast<uint32_t *>(b + sh.off_bins);
   p.start = reinterpret_cast<uint32_t *>(b + sh.off_start);
   p.first_bin = reinterpret_cast<uint32_t *>(b + sh.off_first);
@@ -535,8 +539,9 @@ int run(dbg_handle h, const Shape &sh, uint64_t max_rows, void *buf, Slot *rec, 
                          counts));
   }
   DBG_CK(cudaGetLastError());
-  DBG_CK(cudaMemcpyAsync(&m, p.meta, sizeof(m), cudaMemcpyDeviceToHost, s));
+  if (!p.report) DBG_CK(cudaMemcpyAsync(&m, p.meta, sizeof(m), cudaMemcpyDeviceToHost, s));
   DBG_CK(cudaStreamSynchronize(s));
+  if (p.report) m = *p.report;
   return DBG_OK;
 }
 

@@ -57,6 +57,71 @@ int scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
   return DBG_OK;
 }
 
+namespace {
+constexpr int kReportSlots = 64;  // (calls in flight at once that report this way)
+std::mutex g_report_mu;
+uint64_t *g_report_page = nullptr;
+uint64_t g_report_used = 0;  // a bit per slot
+
+struct Words {
+  DeviceWord w[kMaxWords];
+};
+__global__ void k_report(Words words, int n, volatile uint64_t *out) {
+  after_previous();
+  const int i = threadIdx.x;
+  if (i < n)
+    out[i] = words.w[i].bytes == 8 ? *static_cast<const volatile uint64_t *>(words.w[i].p)
+                                   : *static_cast<const volatile uint32_t *>(words.w[i].p);
+}
+}  // namespace
+
+ReportSlot::ReportSlot() : p(nullptr) {
+  std::lock_guard<std::mutex> lock(g_report_mu);
+  if (!g_report_page || g_report_used == ~0ull) return;
+  int i = 0;
+  while (g_report_used >> i & 1u) ++i;
+  g_report_used |= 1ull << i;
+  p = g_report_page + i * kMaxWords;
+}
+
+ReportSlot::~ReportSlot() {
+  if (!p) return;
+  std::lock_guard<std::mutex> lock(g_report_mu);
+  g_report_used &= ~(1ull << ((p - g_report_page) / kMaxWords));
+}
+
+void make_report_page() {
+  std::lock_guard<std::mutex> lock(g_report_mu);
+  if (g_report_page) return;
+  void *page = nullptr;
+  if (cudaHostAlloc(&page, kReportSlots * kMaxWords * sizeof(uint64_t), cudaHostAllocPortable) ==
+      cudaSuccess)
+    g_report_page = static_cast<uint64_t *>(page);
+  else
+    cudaGetLastError();
+}
+
+void release_report_page() {
+  std::lock_guard<std::mutex> lock(g_report_mu);
+  if (!g_report_page || g_report_used) return;
+  cudaFreeHost(g_report_page);
+  g_report_page = nullptr;
+}
+
+int read_words(const DeviceWord *words, int n, uint64_t *out, cudaStream_t s) {
+  ReportSlot slot;
+  Words w = {};
+  for (int i = 0; i < n; ++i) {
+    out[i] = 0;
+    w.w[i] = words[i];
+    if (!slot.p) DBG_CK(cudaMemcpyAsync(&out[i], words[i].p, words[i].bytes, cudaMemcpyDeviceToHost, s));
+  }
+  if (slot.p) DBG_TRY(launch_after(k_report, 1, 32, 0, s, w, n, slot.p));
+  DBG_CK(cudaStreamSynchronize(s));
+  for (int i = 0; slot.p && i < n; ++i) out[i] = slot.p[i];
+  return DBG_OK;
+}
+
 uint64_t pool_reserved_bytes(int dev) {
   std::lock_guard<std::mutex> lock(g_pool_mu);
   if (dev < 0 || dev >= 64 || !g_pools[dev]) return 0;
@@ -297,6 +362,7 @@ extern "C" int dbg_create_ex(int k, uint64_t capacity, uint32_t max_probes, dbg_
   do {
     st = device_of(h);
     if (st != DBG_OK) break;
+    dbg::make_report_page();
     cudaError_t e = cudaMalloc(&h->table, capacity * sizeof(dbg::Slot));
     if (e != cudaSuccess) { h->table = nullptr; st = dbg::cuda_fail(e, "cudaMalloc(table)"); break; }
     void *small = nullptr;
@@ -896,6 +962,7 @@ extern "C" uint64_t dbg_scratch_bytes(void) {
 extern "C" int dbg_release_scratch(void) {
   int st = dbg::release_batch_scratch();
   if (st != DBG_OK) return st;
+  dbg::release_report_page();
   return dbg::release_scratch_pools();
 }
 
@@ -908,13 +975,11 @@ extern "C" int dbg_get_status(dbg_handle h, void *stream) {
   DeviceGuard g(h->device);
   if (g.err != cudaSuccess) return dbg::cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  uint32_t st = 0;
-  unsigned long long spilled = 0;
-  DBG_CK(cudaMemcpyAsync(&st, h->d_status, sizeof(st), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaMemcpyAsync(&spilled, h->d_spill_count, sizeof(spilled), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaStreamSynchronize(s));
-  if (st == DBG_OK && spilled > 0) return DBG_ERR_NEEDS_GROW;
-  return (int)st;
+  const dbg::DeviceWord words[] = {{h->d_status, 4}, {h->d_spill_count, 8}};
+  uint64_t got[2];
+  DBG_TRY(dbg::read_words(words, 2, got, s));
+  if (got[0] == DBG_OK && got[1] > 0) return DBG_ERR_NEEDS_GROW;
+  return (int)got[0];
 }
 
 extern "C" int dbg_stats(dbg_handle h, uint64_t *n_vertices, uint64_t *n_edges, void *stream) {
@@ -925,32 +990,27 @@ extern "C" int dbg_stats(dbg_handle h, uint64_t *n_vertices, uint64_t *n_edges, 
   if (h->built_counts) {
     // the graph was last rebuilt on the tiled binned path, which counted its
     // new vertices and its edges: read them unless the build fell back
-    uint32_t head[2] = {0, 0};  // status, counted flag
-    unsigned long long built[2] = {0, 0}, spilled = 0;
-    DBG_CK(cudaMemcpyAsync(head, h->d_status, sizeof(head), cudaMemcpyDeviceToHost, s));
-    DBG_CK(cudaMemcpyAsync(built, dbg::small_built(h->d_status), sizeof(built),
-                           cudaMemcpyDeviceToHost, s));
-    DBG_CK(cudaMemcpyAsync(&spilled, h->d_spill_count, sizeof(spilled), cudaMemcpyDeviceToHost, s));
-    DBG_CK(cudaStreamSynchronize(s));
-    if (head[1] == 1u && head[0] == DBG_OK && spilled == 0) {
-      if (n_vertices) *n_vertices = built[0];
-      if (n_edges) *n_edges = built[1];
+    const unsigned long long *built = dbg::small_built(h->d_status);
+    const dbg::DeviceWord words[] = {{h->d_status, 4}, {dbg::small_counted(h->d_status), 4},
+                                     {h->d_spill_count, 8}, {built, 8}, {built + 1, 8}};
+    uint64_t got[5];
+    DBG_TRY(dbg::read_words(words, 5, got, s));
+    if (got[1] == 1u && got[0] == DBG_OK && got[2] == 0) {
+      if (n_vertices) *n_vertices = got[3];
+      if (n_edges) *n_edges = got[4];
       return DBG_OK;
     }
   }
   int st = dbg::launch_stats(h->table, h->n_slots, h->d_acc, s, h->k > 32);
   if (st != DBG_OK) return st;
-  unsigned long long acc[2] = {0, 0};
-  uint32_t status = 0;
-  unsigned long long spilled = 0;
-  DBG_CK(cudaMemcpyAsync(acc, h->d_acc, sizeof(acc), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaMemcpyAsync(&status, h->d_status, sizeof(status), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaMemcpyAsync(&spilled, h->d_spill_count, sizeof(spilled), cudaMemcpyDeviceToHost, s));
-  DBG_CK(cudaStreamSynchronize(s));
-  if (n_vertices) *n_vertices = acc[0];
-  if (n_edges) *n_edges = acc[1];
-  if (status == DBG_OK && spilled > 0) return DBG_ERR_NEEDS_GROW;
-  return (int)status;
+  const dbg::DeviceWord words[] = {{h->d_acc, 8}, {h->d_acc + 1, 8}, {h->d_status, 4},
+                                   {h->d_spill_count, 8}};
+  uint64_t got[4];
+  DBG_TRY(dbg::read_words(words, 4, got, s));
+  if (n_vertices) *n_vertices = got[0];
+  if (n_edges) *n_edges = got[1];
+  if (got[2] == DBG_OK && got[3] > 0) return DBG_ERR_NEEDS_GROW;
+  return (int)got[2];
 }
 
 // ---------------------------------------------------------------------------
