@@ -389,8 +389,7 @@ uint64_t dbg_export_scratch_bytes(int k, uint64_t n_vertices, uint64_t n_slots);
  * `scratch` is a 256-byte aligned device buffer of at least
  * dbg_export_scratch_bytes(k, n, n_slots) bytes, all owned by the caller.
  * k <= 32 and a table of at most 2^32 slots.  Same result and ordering as
- * dbg_export_sorted (the vertices are counted by the compaction into the
- * outputs); waits for `stream`.  Errors: INVALID_ARG (including too small or
+ * dbg_export_sorted (the vertices are counted on the way); waits for `stream`.  Errors: INVALID_ARG (including too small or
  * misaligned scratch and host outputs), CUDA, BUFFER_TOO_SMALL (a size query
  * with max_n = 0), and the sticky status.  After an error the outputs'
  * contents are unspecified. */

@@ -20,9 +20,9 @@
 //   apply   -- one CTA per tile: a bulk copy brings the tile into shared
 //              memory, the tile's events are applied there with
 //              shared-memory CAS and add, a bulk copy writes it back;
-//   deferred -- the events whose probe left their tile and those of the
-//              overflow area, from their home slot, with the global
-//              find-or-claim.
+//   deferred -- the events whose probe left their tile (from the next tile
+//              on) and those of the overflow area (from their home slot),
+//              with the global find-or-claim.
 // The earlier streaming apply (all CTAs sweep the region-ordered events with
 // global atomics inside an L2-resident window) remains as apply_mode = 1; it
 // needs gap-free region ranges, so it keeps an exact count pass (histogram
@@ -60,7 +60,7 @@ constexpr int kMaxTilesPerRegion = 4096;    // beyond this the streaming apply i
 // 657 M (more parts than fit below 2^19) - / 63 / 41.6 / 40.7.  A chain of
 // tables scatters one table's reads at a time, so it takes four times the
 // regions: 24 tables of 50 kb to 2 Mbp 7.32 / 7.36 / 7.54 / 7.90 ms.
-constexpr int kTiledShiftMin = 18, kTiledShiftMax = 21;
+constexpr int kTiledShiftMin = 18, kTiledShift = 21;
 constexpr uint64_t kTableRegions = 256, kChainRegions = 1024;
 
 // The tiled path's bookkeeping for one chain of items (one or many tables).
@@ -1596,7 +1596,7 @@ int ceil_log2(uint64_t x) {
 namespace {
 
 int tiled_shift(uint64_t n_slots, uint64_t regions) {
-  return std::min(kTiledShiftMax,
+  return std::min(kTiledShift,
                   std::max(kTiledShiftMin, ceil_log2((n_slots + regions - 1) / regions)));
 }
 
