@@ -366,9 +366,8 @@ def run_ours(args):
     if tiled:  # bucket sizing: total + buckets; split: units (tile buckets) + tile scatter
         kernels["bin_count"]["launches_per_step"] = 2
         kernels["bin_split"]["launches_per_step"] = 2
-        # the fall-back span: the gated emptying pass and the gated direct
-        # insert (both return at once when the binned kernels did the work)
-        kernels["direct_fallback"]["launches_per_step"] = 2
+        # (the fall-back span is one launch: the gated direct insert, which
+        # returns at once when the binned kernels did the work)
     kernel_bytes = {
         "direct": touches * SECTOR_RMW_BYTES + in_bytes,
         # (the direct path's build empties the table first: 32 B per slot,
@@ -545,10 +544,9 @@ def run_ours(args):
             "reset": "folded into the build (dbg_build_reads): the tiled apply writes every "
                      "table tile from an EMPTY tile in shared memory",
             "export_ms": export_ms,
-            "export_note": "dbg_export_sorted into device buffers (compaction that counts the "
-                           "vertices, radix sort of (32-bit key prefix, slot) pairs inside the "
-                           "output buffers, gather, runs of equal prefixes put in order); median "
-                           "of 3 after a warm-up",
+            "export_note": "dbg_export_sorted into device buffers (histogram of the keys' top "
+                           "bits, one scattered placing pass, a shared-memory sort per bucket); "
+                           "median of 3 after a warm-up",
             "downstream": downstream,
             "step_ms_p50": float(np.percentile(step_ms, 50)),
             "step_ms_p99": float(np.percentile(step_ms, 99)),
