@@ -13,7 +13,7 @@
 // Only rebuilds from empty (dbg_build_reads) come here: an insert into a held
 // graph stays with the direct kernel.  Bound as the one-word path is, by issue
 // and shared-memory latency, at twice the event bytes: 168 M positions into a
-// table of 110 M slots 12.7 -> 5.2 ms (scatter 1.55, split 1.32, apply 2.19),
+// table of 110 M slots 12.7 -> 5.1 ms (scatter 1.55, split 1.30, apply 2.16),
 // where the direct insert is held by the table's random sectors.
 
 namespace {
