@@ -910,7 +910,7 @@ __device__ __forceinline__ void stage_chunk(uint64_t *stage, const uint64_t *ev,
 
 template <int BLOCK, bool STAGED, bool SMALL>
 __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)  // two CTAs of 512 threads per SM
-    k_tile_scatter(const uint64_t *__restrict__ ev, uint64_t *__restrict__ ev2, uint64_t ev2_cap,
+    k_tile_scatter(const uint64_t *ev, uint64_t *ev2, uint64_t ev2_cap,
                    const unsigned long long *begin, const unsigned long long *counts, TileAux aux,
                    int parts, uint64_t unit, int tpr, uint32_t *status, uint32_t *use_binned) {
   after_previous();
@@ -1246,8 +1246,8 @@ __device__ __forceinline__ void empty_soa_tile(const SoaTile &tile, uint32_t *fp
 
 template <int BLOCK, bool FRESH, int N, bool SMALL>
 __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 threads per SM
-    k_tile_apply(const __grid_constant__ ItemPack<N> pk, const uint64_t *__restrict__ ev2,
-                 uint64_t *ev, const unsigned long long *begin, TileAux aux, int parts,
+    k_tile_apply(const __grid_constant__ ItemPack<N> pk, const uint64_t *ev2, uint64_t *ev,
+                 const unsigned long long *begin, TileAux aux, int parts,
                  int tpr_log2, const uint32_t *use_binned) {
   after_previous();
   if (ld_volatile_u32(use_binned) == 0u) return;
@@ -1532,8 +1532,8 @@ struct ListShare {
 // fresh: a rebuild; without the binned path the tables are emptied here.
 template <int N>
 __global__ void k_tile_deferred(const __grid_constant__ ItemPack<N> pk,
-                                const uint64_t *__restrict__ ev,
-                                const uint64_t *__restrict__ ev2, const unsigned long long *begin,
+                                const uint64_t *ev, const uint64_t *ev2,
+                                const unsigned long long *begin,
                                 TileAux aux, int parts, bool fresh, const uint32_t *use_binned) {
   after_previous();
   if (ld_volatile_u32(use_binned) == 0u) {

@@ -206,7 +206,7 @@ size_t wide_split_smem(int tpr) {
 // As k_tile_scatter: every event of a unit to its tile's bucket, each chunk of
 // kWideFlush events sorted by tile in shared memory.
 __global__ void __launch_bounds__(kWideBlock, 2)
-    k_wide_split(const WideEvent *__restrict__ ev, WideEvent *__restrict__ ev2, uint64_t ev2_cap,
+    k_wide_split(const WideEvent *ev, WideEvent *ev2, uint64_t ev2_cap,
                  const unsigned long long *begin, const unsigned long long *counts, TileAux aux,
                  int parts, uint64_t unit, int tpr, uint32_t *use_binned) {
   after_previous();
@@ -339,7 +339,7 @@ constexpr size_t kWideTileBytes = (size_t)kTileSlots * (8 + 8 + 16) + kFpBytes;
 // As k_tile_apply for fresh tables: every tile of the table starts as EMPTY
 // slots in shared memory, takes its events and is written once.
 __global__ void __launch_bounds__(kWideBlock, 3)
-    k_wide_apply(ItemDesc it, const WideEvent *__restrict__ ev2, WideEvent *ev,
+    k_wide_apply(ItemDesc it, const WideEvent *ev2, WideEvent *ev,
                  const unsigned long long *begin, TileAux aux, int parts, int tpr_log2,
                  const uint32_t *use_binned) {
   after_previous();
@@ -449,8 +449,8 @@ __global__ void __launch_bounds__(kWideBlock, 3)
 
 // As k_tile_deferred: the events that left their tile, then the overflow area,
 // from their home slots.
-__global__ void k_wide_deferred(const __grid_constant__ ItemPack<1> pk, const WideEvent *__restrict__ ev,
-                                const WideEvent *__restrict__ ev2, const unsigned long long *begin,
+__global__ void k_wide_deferred(const __grid_constant__ ItemPack<1> pk, const WideEvent *ev,
+                                const WideEvent *ev2, const unsigned long long *begin,
                                 TileAux aux, int parts, const uint32_t *use_binned) {
   after_previous();
   if (ld_volatile_u32(use_binned) == 0u) {

@@ -212,7 +212,10 @@ __device__ __forceinline__ bool find_or_claim(Slot *table, uint64_t n_slots, uin
 
 // First statement of every kernel that launch_next launches: lets the stream's
 // next kernel take its places on the SMs, then waits until the kernels before
-// this one have ended and their writes are visible.
+// this one have ended and their writes are visible.  Such a kernel's pointers
+// are not __restrict__: for a const one that promises that nobody writes what
+// it points to while the kernel runs, this wait included, and the loads need
+// not stay behind it.
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

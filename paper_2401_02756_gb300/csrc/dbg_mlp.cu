@@ -46,8 +46,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 // registers), and sums over the lanes.
 template <bool TRAIN>
 __global__ void __launch_bounds__(32 * kWarps)
-    k_rows(const float *__restrict__ P, const float *__restrict__ x,
-           const float *__restrict__ target, int B, float *y, Work w) {
+    k_rows(const float *P, const float *x, const float *target, int B, float *y, Work w) {
   after_previous();
   __shared__ float s_h1[kRows][kHid], s_h2[kRows][kHid], s_dh2[kRows][kHid];
   __shared__ float s_part[kRows][kHid], s_dy[kRows];
@@ -158,7 +157,7 @@ constexpr int kGradRows = 256;                  // rows staged at a time
 // quarter of the batch per group of 64 threads; the first CTA of a layer sums
 // its biases too.
 __global__ void __launch_bounds__(256, 2)
-    k_grads(const float *__restrict__ x, const float *__restrict__ target, int B, Work w, Adam ad) {
+    k_grads(const float *x, const float *target, int B, Work w, Adam ad) {
   after_previous();
   __shared__ __align__(16) float s_x[kGradRows][kCols];
   __shared__ float s_red[4][kHid][kCols + 1];
