@@ -1580,6 +1580,7 @@ __global__ void k_tables_init(const __grid_constant__ ItemPack<N> pk) {
   if (i >= pk.n_items) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *pk.d[i].status = 0u;
+    *small_counted(pk.d[i].status) = 0u;
     *pk.d[i].spill_count = 0ull;
   }
   empty_table(pk.d[i], blockIdx.x, gridDim.x);
@@ -2073,6 +2074,7 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
   pk.total_tiles = walk_tiles;
   pk.d[0] = it;
   pk.d[0].region0 = 0;
+  DBG_CK(cudaMemsetAsync(small_counted(h->d_status), 0, 4, s));  // (it counts nothing)
   DBG_CK(cudaMemsetAsync(mv.ctr, 0, 4 * sizeof(unsigned long long), s));
   DBG_CK(cudaMemsetAsync(mv.counts, 0, geo.parts * sizeof(unsigned long long), s));
   mark(1, s);

@@ -86,8 +86,10 @@ __device__ __forceinline__ uint32_t quotient(uint32_t c, double divisor) {
   return q >= 4294967295.0 ? 0xffffffffu : (uint32_t)q;
 }
 
-__global__ void __launch_bounds__(256) k_normalize(uint4 *t, uint64_t n, double divisor, int wide) {
+__global__ void __launch_bounds__(256) k_normalize(uint4 *t, uint64_t n, double divisor, int wide,
+                                                 uint32_t *counted) {
   after_previous();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *counted = 0u;  // (the counters change)
   __shared__ uint32_t s_quot[kQuot];
   for (uint32_t c = threadIdx.x; c < kQuot; c += blockDim.x) s_quot[c] = quotient(c, divisor);
   __syncthreads();
@@ -575,7 +577,7 @@ extern "C" int dbg_normalize(dbg_handle h, double divisor, void *stream) {
   const uint64_t want = (h->n_slots + 255) / 256;
   const int grid = (int)std::min<uint64_t>(want, (uint64_t)std::max(1, h->sm_count) * 8);
   DBG_TRY(launch_after(k_normalize, grid, 256, 0, s, reinterpret_cast<uint4 *>(h->table),
-                       h->n_slots, divisor, h->k > 32 ? 1 : 0));
+                       h->n_slots, divisor, h->k > 32 ? 1 : 0, small_counted(h->d_status)));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }

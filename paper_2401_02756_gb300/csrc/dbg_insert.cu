@@ -93,6 +93,8 @@ __global__ void __launch_bounds__(BLOCK, 2048 / BLOCK)
     k_insert(const __grid_constant__ ItemPack<N> pk, int tile_reads, const uint32_t *gate) {
   after_previous();
   if (gate != nullptr && ld_volatile_u32(gate) != 0u) return;
+  if (blockIdx.x == 0)  // (the graphs grow, uncounted)
+    for (int i = threadIdx.x; i < pk.n_items; i += BLOCK) *small_counted(pk.d[i].status) = 0u;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ volatile uint32_t s_cap_hit;
   InsertVisitor<AGG> vis{&s_cap_hit};

@@ -224,7 +224,8 @@ __device__ __forceinline__ void after_previous() {
 // Every graph's small block of device memory (64 bytes beside its table):
 // the sticky status (u32) at byte 0; a flag at 4 set by a rebuild from empty
 // on the tiled binned path whose vertex and edge counts at 40 and 48 are then
-// exact (cleared when the build falls back to the direct insert); the stats
+// exact, and cleared by every kernel that changes the graph without counting
+// (so it holds for replayed calls too, which the host does not see); the stats
 // accumulators (2 x u64) at 16; the spill count (u64) at 32.  Kernels reach
 // the flag and the counts from an item's status pointer.
 constexpr size_t kSmallCounted = 4, kSmallAcc = 16, kSmallSpill = 32, kSmallBuilt = 40;
@@ -284,9 +285,9 @@ struct dbg_graph {
   // first needs it; batched inserts use the library's own)
   dbg::BinScratch bin;
   uint64_t bin_want = 0;                    // events asked for by dbg_reserve_events (0: default)
-  // the last call that changed the graph was a rebuild on the tiled binned
-  // path, which counts its vertices and edges (see small_counted): dbg_stats
-  // then reads them instead of counting the table
+  // the last call issued that changes the graph was a rebuild on the tiled binned
+  // path, which counts its vertices and edges: dbg_stats then reads them instead
+  // of counting the table, if the device's flag (small_counted) still stands
   bool built_counts = false;
   // optional per-kernel timing of insert calls (dbg_enable_kernel_timing)
   int timer_cap = 0;                        // calls kept

@@ -170,6 +170,7 @@ __global__ void k_table_init(uint4 *t, uint64_t n_vec, uint32_t *status,
   after_previous();
   if (status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
     *status = 0u;
+    *small_counted(status) = 0u;
     *spilled = 0ull;
   }
   const uint4 head = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);
@@ -525,6 +526,7 @@ extern "C" int dbg_grow(dbg_handle h, uint64_t new_capacity, void *stream) {
   h->built_counts = false;
   DeviceGuard g(h->device);
   if (g.err != cudaSuccess) return dbg::cuda_fail(g.err, "cudaSetDevice");
+  DBG_CK(cudaMemsetAsync(dbg::small_counted(h->d_status), 0, 4, static_cast<cudaStream_t>(stream)));
   return dbg::launch_grow(h, new_capacity, static_cast<cudaStream_t>(stream));
 }
 
@@ -988,8 +990,9 @@ extern "C" int dbg_stats(dbg_handle h, uint64_t *n_vertices, uint64_t *n_edges, 
   if (g.err != cudaSuccess) return dbg::cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (h->built_counts) {
-    // the graph was last rebuilt on the tiled binned path, which counted its
-    // new vertices and its edges: read them unless the build fell back
+    // the call issued last was a rebuild on the tiled binned path, which counts its
+    // new vertices and its edges: read them if the device agrees (the build did
+    // not fall back, and no replayed call has changed the graph since)
     const unsigned long long *built = dbg::small_built(h->d_status);
     const dbg::DeviceWord words[] = {{h->d_status, 4}, {dbg::small_counted(h->d_status), 4},
                                      {h->d_spill_count, 8}, {built, 8}, {built + 1, 8}};

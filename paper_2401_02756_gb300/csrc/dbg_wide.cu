@@ -32,6 +32,7 @@ template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 6) k_insert_wide(ItemDesc it, int tile_reads, const uint32_t *gate) {
   after_previous();
   if (gate != nullptr && ld_volatile_u32(gate) != 0u) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *small_counted(it.status) = 0u;  // (it grows, uncounted)
   __shared__ uint64_t s_off[kWideTile + 1];
   __shared__ uint64_t s_pre[kWideTile + 1];
   __shared__ __align__(16) uint64_t s_win[kWideWinBytes / 8 + 4];
