@@ -2218,8 +2218,12 @@ int launch_binned_batch(const ItemDesc *items, const uint64_t *want, int n,
   uint64_t slots = 0;  // (of a chain's worth of tables)
   for (int i = 0; i < n; ++i) slots += items[i].n_slots;
   if (n > kBatchItems) slots = slots / (uint64_t)n * kBatchItems;
-  const int shift = t.region_log2 > 0 ? std::max(t.region_log2, kTileLog2)
-                                      : tiled_shift(slots, kChainRegions);
+  int shift = t.region_log2 > 0 ? std::max(t.region_log2, kTileLog2)
+                                : tiled_shift(slots, kChainRegions);
+  // (the average table can be far below the largest, which takes one chain alone)
+  if (t.region_log2 <= 0)
+    for (int i = 0; i < n; ++i)
+      while (shift < kTiledShift && regions_of(items[i].n_slots, shift) > kBinMaxParts) ++shift;
   const int sms = std::max(1, sm_count);
   int dev = 0;
   DBG_CK(cudaGetDevice(&dev));
