@@ -851,7 +851,7 @@ extern "C" uint64_t dbg_export_scratch_bytes(int k, uint64_t n_vertices, uint64_
   uint64_t a = 0, b = 0, c = 0;
   if (prefix_scratch_bytes(k, D, a) != DBG_OK) return 0;
   if (in_place_scratch_bytes<uint32_t>(D, 2 * (k - 1), b) != DBG_OK) return 0;
-  if (export_bins_scratch(k, D, c) != DBG_OK) return 0;
+  if (export_bins_scratch(k, D, n_slots, c) != DBG_OK) return 0;
   return std::max(a, std::max(b, c));
 }
 
@@ -864,7 +864,7 @@ extern "C" int dbg_export_sorted_with(dbg_handle h, uint64_t *keys_out, uint32_t
   if (g.err != cudaSuccess) return cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint64_t D = 0, need = 0;
-  DBG_TRY(export_bins_scratch(h->k, std::min(max_n, h->n_slots), need));
+  DBG_TRY(export_bins_scratch(h->k, std::min(max_n, h->n_slots), h->n_slots, need));
   bool too_dense = true;
   if (max_n > 0 && scratch && ((uintptr_t)scratch & 255u) == 0 && scratch_bytes >= need &&
       in_place_outputs(keys_out, counts_out)) {

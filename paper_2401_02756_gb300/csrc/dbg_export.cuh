@@ -6,8 +6,8 @@
 
 namespace dbg {
 
-// Device bytes of scratch export_bins needs for outputs of `rows` rows.
-int export_bins_scratch(int k, uint64_t rows, uint64_t &bytes);
+// Device bytes of scratch export_bins needs for outputs of `rows` rows of a table.
+int export_bins_scratch(int k, uint64_t rows, uint64_t n_slots, uint64_t &bytes);
 
 // Sorted keys and counter rows into 16-byte aligned device outputs of
 // `max_rows` rows; *D receives the number of vertices (more than max_rows:
