@@ -362,15 +362,17 @@ int dbg_stats(dbg_handle h, uint64_t *n_vertices, uint64_t *n_edges, void *strea
  * device (up to 4 GiB of it stays cached between calls) and is released to
  * it before return.  When both outputs are 16-byte aligned device buffers
  * the records are sorted inside them, and the temporary memory is the sort's
- * bins (up to about 8 MB, or a byte for every 25 vertices if that is more);
+ * bins (up to about 8 MB, or a byte for every 9 vertices if that is more);
  * a graph built on the binned path places its records in the handle's event
  * buffer first, and one with k > 32 in up to 4 GiB of the pool (32 bytes a
  * vertex).  Pinned host outputs (both, 16-byte aligned) are written by the
  * sort itself, from records in one of those places; others go through
- * temporary outputs (24 bytes a row, 32 for k > 32).  Keys crowded into a few prefixes are left to a radix sort (about
- * 6 bytes a vertex in place, otherwise 40, 80 for k > 32).  Errors:
- * INVALID_ARG, OOM, CUDA, BUFFER_TOO_SMALL, and the sticky status (nothing
- * exported when it is set). */
+ * temporary outputs (24 bytes a row, 32 for k > 32).  Vertices whose keys crowd
+ * into a few prefixes take a radix sort of their own (about 41 bytes each, 57
+ * for k > 32); when that is not to be had, or they are more than a quarter of
+ * the outputs' rows, the whole graph takes one (about 6 bytes a vertex in place,
+ * otherwise 40, 80 for k > 32).  Errors: INVALID_ARG, OOM, CUDA,
+ * BUFFER_TOO_SMALL, and the sticky status (nothing exported when it is set). */
 int dbg_export_sorted(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t max_n,
                       uint64_t *n_out, void *stream);
 

@@ -12,8 +12,9 @@ int export_bins_scratch(int k, uint64_t rows, uint64_t n_slots, uint64_t &bytes)
 // Sorted keys and counter rows into 16-byte aligned device outputs of
 // `max_rows` rows; *D receives the number of vertices (more than max_rows:
 // nothing is written).  `scratch`: caller's device memory (256-byte aligned),
-// or null to take it from the library's pool.  *too_dense: the keys crowd into
-// bins too large for this sort and nothing is written.  Waits for `s`.
+// or null to take it from the library's pool.  *too_dense: more of the
+// keys crowd into a few bins than this sort takes (or has scratch for), and the
+// outputs hold nothing of use.  Waits for `s`.
 // `no_records` (if not null): the outputs are to be written once, in order --
 // pinned host memory --, so the records must have a place of their own; set,
 // with nothing else done, when there is none.  Returns the graph's sticky

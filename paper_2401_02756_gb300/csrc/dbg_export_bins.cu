@@ -28,10 +28,18 @@
 // The placed records go to 32-byte records of scratch when there is room for
 // them -- a full sector per scattered store -- and otherwise straight to the
 // outputs, which the sort then reorders in place (an 8- and a 16-byte store a
-// record, 1.5 times the time, but no memory beyond the bins' is needed).  A
-// table whose keys crowd into one bin (more than a bucket's shared memory
-// holds) is left to the radix sort.
-#include <cub/device/device_scan.cuh>
+// record, 1.5 times the time, but no memory beyond the bins' is needed).
+//
+// Genomes of uneven base composition and repeats fill some bins far beyond the
+// others.  A bucket with more records than its CTA's shared memory holds is
+// skipped by the sort; the records of all such buckets are then sorted together
+// by their whole keys, by a radix sort, and written back (56 bytes of scratch a
+// record at most).  They are few: export of 432 M vertices (2^22 bins) at 50 / 40 /
+// 35 / 30 % GC 23.9 / 23.9 / 24.9 / 29.5 ms, with none, none, 1 % and 11 % of the
+// records in such buckets (a radix sort of all: 35.6 to 41.3).
+// Graphs with a quarter of their records in such buckets are left to the radix
+// sort as a whole.
+#include <cub/device/device_radix_sort.cuh>
 
 #include <algorithm>
 
@@ -44,19 +52,23 @@ namespace {
 constexpr int kSortBlock = 256;
 constexpr int kLocalBits = 11;  // bins of the shared-memory counting sort
 constexpr int kLocalBins = 1 << kLocalBits;
-constexpr int kMaxBinBits = 20;
+constexpr int kBinBits = 20, kBinLog2 = 7;  // bins: up to 2^20, or for 2^7 records each
 constexpr int kPlanBins = 8192;  // up to this many: the plan is one CTA's work
 constexpr int kPlanBlock = 1024;
+constexpr int kChunkBlock = 256, kChunkPer = 16;  // more: a CTA for 4,096 bins
+constexpr uint32_t kChunkBins = kChunkBlock * kChunkPer;
 constexpr int kSlotsPerThread = 4;
 constexpr int kCursorStride = 8;  // a bucket's cursor has a sector of its own
 constexpr uint32_t kCursorBins = 1u << 17;  // in place: bucket cursors above so many bins
 constexpr uint64_t kMaxPooledRecords = 4ull << 30;  // (what the pool keeps between calls)
 
 constexpr uint32_t kBucketCap = 2048;  // records a bucket may hold
+constexpr uint64_t kCrowdedShare = 4;  // at most one record in so many may lie in larger ones
 
 struct ExportMeta {
   unsigned long long spilled;
-  uint32_t vertices, max_bin, status;
+  unsigned long long crowded;  // records in buckets of more than kBucketCap, at most
+  uint32_t vertices, status;
 };
 
 // Everything the kernels share.
@@ -67,6 +79,8 @@ struct Plan {
   uint32_t buckets;     // last entry of the bucket arrays (a graph of more vertices is not placed)
   uint64_t max_rows;    // rows of the outputs
   uint64_t max_placed;  // records the scratch holds (place into 32-byte records)
+  uint64_t max_crowded; // records that may lie in buckets above the cap
+  uint2 *sums;          // [2^B / kChunkBins] records of a chunk of bins, of its last bin
   uint32_t *bins;       // [2^B + 1] histogram, then exclusive prefix, then next free position
   uint32_t *start;      // [buckets + 2] first position of a bucket
   uint32_t *first_bin;  // [buckets + 2]
@@ -76,11 +90,18 @@ struct Plan {
 };
 
 // Whether the placing and the sort may run: a complete graph, room for it,
-// and no bucket above the cap.
+// and few records in buckets above the cap.
 __device__ __forceinline__ bool may_run(const Plan &p) {
   const ExportMeta m = *p.meta;
   return m.status == 0u && m.spilled == 0ull && m.vertices <= p.max_rows &&
-         m.vertices <= p.max_placed && (1u << p.bucket_log2) + m.max_bin <= kBucketCap;
+         m.vertices <= p.max_placed && m.crowded <= p.max_crowded;
+}
+
+// Records a bin of n can put into a bucket above the cap: its own and those of
+// the bins before it in its bucket (fewer than 2^bucket_log2).
+__device__ __forceinline__ unsigned long long crowd(const Plan &p, uint32_t n) {
+  const uint32_t T = 1u << p.bucket_log2;
+  return n > kBucketCap - T ? (unsigned long long)n + T : 0ull;
 }
 
 // A key as one or two words.  aligned(): its leading 64 bits, from the top.
@@ -106,13 +127,24 @@ struct Key<true> {
   __device__ __forceinline__ bool empty() const { return hi == kEmpty; }
 };
 
+// The table goes past the L2 (evict_first), the bins' counters stay in it
+// (evict_last): 2^22 bins of 432 M records 25.1 -> 23.9 ms an export, as 2^21 take.
+__device__ __forceinline__ uint32_t next_place(uint32_t *bin, uint64_t pol) {
+  uint32_t at;
+  asm volatile("atom.relaxed.gpu.global.add.L2::cache_hint.u32 %0, [%1], 1, %2;"
+               : "=r"(at)
+               : "l"(bin), "l"(pol)
+               : "memory");
+  return at;
+}
+
 // A 32-byte slot in one load, and a 32-byte record in one store.
 struct Words {
   uint32_t w[8];
 };
 __device__ __forceinline__ Words ld_slot(const Slot *p) {
   Words v;
-  asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+  asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]),
                  "=r"(v.w[5]), "=r"(v.w[6]), "=r"(v.w[7])
                : "l"(p));
@@ -205,7 +237,7 @@ __device__ __forceinline__ void fill_meta(const Plan &p, uint32_t vertices, cons
   p.meta->spilled = *(const volatile unsigned long long *)spilled;
 }
 
-// The plan of up to kPlanBins bins in one CTA: prefix, buckets, largest bin.
+// The plan of up to kPlanBins bins in one CTA: prefix, buckets, crowded bins.
 __global__ void __launch_bounds__(kPlanBlock)
     k_plan(Plan p, const uint32_t *status, const unsigned long long *spilled) {
   after_previous();
@@ -214,12 +246,13 @@ __global__ void __launch_bounds__(kPlanBlock)
   const uint32_t nbins = 1u << p.bin_bits;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t i0 = threadIdx.x * kPer;
-  uint32_t c[kPer], local = 0, most = 0;
+  uint32_t c[kPer], local = 0;
+  unsigned long long crowded = 0;
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
     c[q] = i0 + q < nbins ? p.bins[i0 + q] : 0u;
     local += c[q];
-    most = max(most, c[q]);
+    crowded += crowd(p, c[q]);
   }
   uint32_t incl = local;
   for (int d = 1; d < 32; d <<= 1) {
@@ -252,34 +285,99 @@ __global__ void __launch_bounds__(kPlanBlock)
     p.bins[nbins] = total;
     open_buckets(p, nbins, nbins, total, before);
   }
-  most = __reduce_max_sync(0xffffffffu, most);
-  if (lane == 0 && most) atomicMax(&p.meta->max_bin, most);
+  if (crowded) atomicAdd(&p.meta->crowded, crowded);
   if (threadIdx.x == 0) fill_meta(p, total, status, spilled);
 }
 
-// The same from a finished prefix (more bins).  (The largest bin by one atomic a
-// CTA, and only from a CTA that would raise it: one a warp on the one address
-// took 24 us for 2^20 bins, now 8.)
-__global__ void __launch_bounds__(256)
+// kChunkPer bins of the calling thread in its CTA's chunk.
+__device__ __forceinline__ void load_bins(const Plan &p, uint32_t (&c)[kChunkPer]) {
+  const uint4 *in = reinterpret_cast<const uint4 *>(p.bins + (size_t)blockIdx.x * kChunkBins) +
+                    threadIdx.x * (kChunkPer / 4);
+#pragma unroll
+  for (int q = 0; q < kChunkPer / 4; ++q) {
+    const uint4 v = in[q];
+    c[4 * q] = v.x;
+    c[4 * q + 1] = v.y;
+    c[4 * q + 2] = v.z;
+    c[4 * q + 3] = v.w;
+  }
+}
+
+// Sum over the CTA (kChunkBlock threads), for every thread.
+__device__ __forceinline__ uint32_t chunk_sum(uint32_t v, uint32_t *s_warp) {
+  v = __reduce_add_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = v;
+  __syncthreads();
+  uint32_t sum = 0;
+#pragma unroll
+  for (int w = 0; w < kChunkBlock / 32; ++w) sum += s_warp[w];
+  __syncthreads();
+  return sum;
+}
+
+// More bins, first pass: the records of every chunk of bins (and of its last
+// bin), and the crowded bins.
+__global__ void __launch_bounds__(kChunkBlock) k_bin_sums(Plan p) {
+  after_previous();
+  __shared__ uint32_t s_warp[kChunkBlock / 32];
+  uint32_t c[kChunkPer], local = 0;
+  unsigned long long crowded = 0;
+  load_bins(p, c);
+#pragma unroll
+  for (int q = 0; q < kChunkPer; ++q) {
+    local += c[q];
+    crowded += crowd(p, c[q]);
+  }
+  if (crowded) atomicAdd(&p.meta->crowded, crowded);
+  const uint32_t sum = chunk_sum(local, s_warp);
+  if (threadIdx.x == kChunkBlock - 1) p.sums[blockIdx.x] = make_uint2(sum, c[kChunkPer - 1]);
+}
+
+// Second pass: every chunk's prefix from the sums of those before it, and the
+// buckets its bins open.
+__global__ void __launch_bounds__(kChunkBlock)
     k_buckets(Plan p, const uint32_t *status, const unsigned long long *spilled) {
   after_previous();
-  __shared__ uint32_t s_most;
-  if (threadIdx.x == 0) s_most = 0u;
-  __syncthreads();
+  __shared__ uint32_t s_warp[kChunkBlock / 32], s_last[kChunkBlock + 1];
   const uint32_t nbins = 1u << p.bin_bits;
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t n = 0;
-  if (i <= nbins) {
-    const uint32_t at = p.bins[i];
-    open_buckets(p, i, nbins, at, i ? p.bins[i - 1] : 0u);
-    if (i < nbins) n = p.bins[i + 1] - at;
-    if (i == nbins) fill_meta(p, at, status, spilled);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t ahead = 0;
+  for (uint32_t j = tid; j < blockIdx.x; j += kChunkBlock) ahead += p.sums[j].x;
+  const uint32_t base = chunk_sum(ahead, s_warp);
+  uint32_t c[kChunkPer], local = 0;
+  load_bins(p, c);
+#pragma unroll
+  for (int q = 0; q < kChunkPer; ++q) local += c[q];
+  uint32_t incl = local;
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t o = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += o;
   }
-  n = __reduce_max_sync(0xffffffffu, n);
-  if ((threadIdx.x & 31) == 0 && n) atomicMax(&s_most, n);
+  if (lane == 31) s_warp[warp] = incl;
   __syncthreads();
-  if (threadIdx.x == 0 && s_most > ld_volatile_u32(&p.meta->max_bin))
-    atomicMax(&p.meta->max_bin, s_most);
+  uint32_t at = base + incl - local;
+  for (int w = 0; w < warp; ++w) at += s_warp[w];
+  s_last[tid + 1] = at + local - c[kChunkPer - 1];  // the thread's last bin starts here
+  if (tid == 0) s_last[0] = base - (blockIdx.x ? p.sums[blockIdx.x - 1].y : 0u);
+  __syncthreads();
+  uint32_t before = s_last[tid], prefix[kChunkPer];
+  const uint32_t i0 = blockIdx.x * kChunkBins + tid * kChunkPer;
+#pragma unroll
+  for (int q = 0; q < kChunkPer; ++q) {
+    prefix[q] = at;
+    open_buckets(p, i0 + q, nbins, at, before);
+    before = at;
+    at += c[q];
+  }
+  uint4 *out = reinterpret_cast<uint4 *>(p.bins + i0);
+#pragma unroll
+  for (int q = 0; q < kChunkPer / 4; ++q)
+    out[q] = make_uint4(prefix[4 * q], prefix[4 * q + 1], prefix[4 * q + 2], prefix[4 * q + 3]);
+  if (i0 + kChunkPer == nbins) {  // the end comes after the last bin
+    p.bins[nbins] = at;
+    open_buckets(p, nbins, nbins, at, before);
+    fill_meta(p, at, status, spilled);
+  }
 }
 
 // Every record to its bin's next place: as a 32-byte record of `rec`, or (null)
@@ -294,6 +392,7 @@ __global__ void __launch_bounds__(256) k_place(const Slot *t, uint64_t n, Plan p
                                                Key<WIDE> *keys, uint4 *counts) {
   after_previous();
   if (!may_run(p)) return;
+  const uint64_t pol = l2_policy_evict_last();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += stride * kSlotsPerThread) {
@@ -314,7 +413,7 @@ __global__ void __launch_bounds__(256) k_place(const Slot *t, uint64_t n, Plan p
       if (k.empty()) continue;
       uint32_t *bin = &p.bins[k.aligned(p.key_bits) >> (64 - p.bin_bits)];
       if (!RECORDS && p.cursor) bin = &p.cursor[(*bin >> p.bucket_log2) * kCursorStride];
-      at[u] = atomicAdd(bin, 1u);
+      at[u] = next_place(bin, pol);
     }
 #pragma unroll
     for (int u = 0; u < kSlotsPerThread; ++u) {
@@ -359,7 +458,7 @@ __global__ void __launch_bounds__(kSortBlock, RECORDS && !WIDE ? 6 : 4)
   const uint32_t b = blockIdx.x;
   if (b > p.meta->vertices >> p.bucket_log2) return;
   const uint32_t s0 = p.start[b], n = p.start[b + 1] - s0;
-  if (n == 0) return;
+  if (n == 0 || n > kBucketCap) return;  // (a larger one: k_crowd_gather's)
   const uint32_t bin0 = p.first_bin[b], span = p.first_bin[b + 1] - bin0;
   const uint64_t low = (uint64_t)bin0 << (64 - p.bin_bits);
   const int width = 64 - p.bin_bits + (span > 1 ? 32 - __clz((int)(span - 1)) : 0);
@@ -455,6 +554,134 @@ __global__ void __launch_bounds__(kSortBlock, RECORDS && !WIDE ? 6 : 4)
   }
 }
 
+// The buckets above the cap.  Their records get consecutive numbers, in the
+// buckets' order: off[b] is the first of bucket b.
+constexpr int kOffBlock = 1024, kOffPer = 8;
+__device__ __forceinline__ uint32_t crowded_in(const Plan &p, uint32_t b) {
+  if (b > p.meta->vertices >> p.bucket_log2) return 0u;
+  const uint32_t n = p.start[b + 1] - p.start[b];
+  return n > kBucketCap ? n : 0u;
+}
+__global__ void __launch_bounds__(kOffBlock) k_crowd_offsets(Plan p, uint32_t *off) {
+  after_previous();
+  __shared__ uint32_t s_warp[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t nb = (p.meta->vertices >> p.bucket_log2) + 1u;
+  uint32_t run = 0;
+  for (uint32_t b0 = 0; b0 < nb; b0 += kOffBlock * kOffPer) {
+    const uint32_t b = b0 + threadIdx.x * kOffPer;
+    uint32_t c[kOffPer], n = 0;
+#pragma unroll
+    for (int q = 0; q < kOffPer; ++q) n += c[q] = crowded_in(p, b + q);
+    uint32_t incl = n;
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t o = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += o;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    uint32_t total = 0, below = 0;
+    for (int w = 0; w < kOffBlock / 32; ++w) {
+      if (w < warp) below += s_warp[w];
+      total += s_warp[w];
+    }
+    uint32_t at = run + below + incl - n;
+#pragma unroll
+    for (int q = 0; q < kOffPer; ++q) {
+      if (b + q < nb) off[b + q] = at;
+      at += c[q];
+    }
+    run += total;
+    __syncthreads();
+  }
+}
+
+// What a record's number leads to: its key's words, its counter row, and for the
+// sort the numbers themselves.
+struct Crowd {
+  uint32_t *off;
+  uint64_t n;  // numbers there are (records, and a few that are none: they sort last)
+  unsigned long long *lo[2], *hi[2];
+  uint32_t *idx[2];
+  uint4 *row;
+};
+
+__global__ void __launch_bounds__(256) k_crowd_none(Crowd c, int wide) {
+  after_previous();
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < c.n; i += stride) {
+    c.idx[0][i] = (uint32_t)i;
+    c.lo[0][i] = ~0ull;
+    if (wide) c.hi[0][i] = ~0ull;
+  }
+}
+
+// A CTA takes kCrowdGroup buckets: f(position, number) for every
+// record of those above the cap.
+constexpr uint32_t kCrowdGroup = 16;
+template <class F>
+__device__ __forceinline__ void each_crowded(const Plan &p, const Crowd &c, F &&f) {
+  __shared__ uint32_t s_n[kCrowdGroup];
+  const uint32_t b0 = blockIdx.x * kCrowdGroup;
+  if (threadIdx.x < kCrowdGroup) s_n[threadIdx.x] = crowded_in(p, b0 + threadIdx.x);
+  __syncthreads();
+  for (uint32_t q = 0; q < kCrowdGroup; ++q) {
+    const uint32_t n = s_n[q];
+    if (n == 0) continue;
+    const uint32_t s0 = p.start[b0 + q], at = c.off[b0 + q];
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) f(s0 + i, at + i);
+  }
+}
+
+template <bool WIDE, bool RECORDS>
+__global__ void __launch_bounds__(256)
+    k_crowd_gather(Plan p, const Slot *rec, const Key<WIDE> *keys, const uint4 *counts, Crowd c) {
+  after_previous();
+  each_crowded(p, c, [&](uint32_t from, uint32_t at) {
+    Key<WIDE> k;
+    if constexpr (RECORDS) {
+      k = ld_record_key<WIDE>(rec + from);
+      c.row[at] = *(reinterpret_cast<const uint4 *>(rec + from) + (WIDE ? 1 : 0));
+    } else {
+      k = keys[from];
+      c.row[at] = counts[from];
+    }
+    if constexpr (WIDE) {
+      c.lo[0][at] = k.lo;
+      c.hi[0][at] = k.hi;
+    } else {
+      c.lo[0][at] = k.w;
+    }
+  });
+}
+
+// hi[1] := hi[0] in the order of the first sort.
+__global__ void __launch_bounds__(256) k_crowd_high(Crowd c) {
+  after_previous();
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < c.n; i += stride)
+    c.hi[1][i] = c.hi[0][c.idx[1][i]];
+}
+
+// The records of those buckets in order (idx: the sorted numbers).
+template <bool WIDE>
+__global__ void __launch_bounds__(256)
+    k_crowd_write(Plan p, Crowd c, const uint32_t *idx, Key<WIDE> *keys, uint4 *counts) {
+  after_previous();
+  each_crowded(p, c, [&](uint32_t to, uint32_t at) {
+    const uint32_t from = idx[at];
+    Key<WIDE> k;
+    if constexpr (WIDE) {
+      k.lo = c.lo[0][from];
+      k.hi = c.hi[0][from];
+    } else {
+      k.w = c.lo[0][from];
+    }
+    keys[to] = k;
+    counts[to] = c.row[from];
+  });
+}
+
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
 int ceil_log2(uint64_t x) {
@@ -465,41 +692,110 @@ int ceil_log2(uint64_t x) {
 
 // Bins and buckets for at most `rows` vertices: buckets of T = 2^10 records
 // or, in a small graph, few enough for about 512 CTAs; bins for 16 records, so
-// that few atomics meet on one counter, and at most 2^20 of them.  Outputs of a
-// sixteenth of the table's slots or less may be too small for its vertices: the
-// bins are then for that many, or the counting would meet on a few counters
-// (57 M vertices counted for outputs of 1,000 rows: 16.8 ms, with the table's
-// bins 0.5).
+// that few atomics meet on one counter, up to 2^20 of them or one for 128 records
+// (more of them cost uniform genomes time: 57 M vertices 2.92 ms, 3.02 with 2^22
+// bins; fewer leave more to the crowded buckets' sort).  Outputs of a quarter of
+// the table's slots or less may be too small for its vertices: the bins are then
+// for that many, or the counting would meet on a few counters (57 M vertices
+// counted for outputs of 1,000 rows: 16.8 ms, with the table's bins 0.6).
 struct Shape {
   int bin_bits, bucket_log2;
   uint32_t nbins, buckets;
-  size_t temp, off_bins, off_start, off_first, off_cursor, off_temp, total;
+  size_t off_bins, off_start, off_first, off_cursor, off_sums, total;
 };
 
-int export_shape(int k, uint64_t rows, uint64_t n_slots, Shape &sh) {
+void export_shape(int k, uint64_t rows, uint64_t n_slots, Shape &sh) {
   const int bits = ceil_log2(std::max<uint64_t>(rows, 2));
   sh.bucket_log2 = std::min(10, std::max(7, bits - 9));
-  sh.bin_bits = std::min(std::min(kMaxBinBits, 2 * (k - 1)),
-                         std::max(1, ceil_log2(std::max<uint64_t>(rows, n_slots / 16)) - 4));
+  const int weight = ceil_log2(std::max<uint64_t>(std::max<uint64_t>(rows, 2), n_slots / 4));
+  sh.bin_bits = std::min(std::min(std::max(kBinBits, weight - kBinLog2), 2 * (k - 1)),
+                         std::max(1, weight - 4));
   sh.nbins = 1u << sh.bin_bits;
   sh.buckets = (uint32_t)(rows >> sh.bucket_log2) + 1u;
-  sh.temp = 0;
-  if (sh.nbins > (uint32_t)kPlanBins)
-    DBG_CK(cub::DeviceScan::ExclusiveSum(nullptr, sh.temp, (uint32_t *)nullptr, (uint32_t *)nullptr,
-                                         (int)sh.nbins + 1, (cudaStream_t)0));
   sh.off_bins = 256;  // (the meta block first: cleared with the histogram)
   sh.off_start = sh.off_bins + al256(((size_t)sh.nbins + 1) * 4);
   sh.off_first = sh.off_start + al256(((size_t)sh.buckets + 2) * 4);
   sh.off_cursor = sh.off_first + al256(((size_t)sh.buckets + 2) * 4);
-  sh.off_temp = sh.off_cursor +
+  sh.off_sums = sh.off_cursor +
                 (sh.nbins > kCursorBins ? al256(((size_t)sh.buckets + 2) * 4 * kCursorStride) : 0);
-  sh.total = sh.off_temp + al256(sh.temp);
+  sh.total = sh.off_sums +
+             (sh.nbins > (uint32_t)kPlanBins ? al256(sh.nbins / kChunkBins * sizeof(uint2)) : 0);
+}
+
+// Scratch for the crowded buckets' records: the arrays of a Crowd of n and the
+// radix sort's.
+struct CrowdLayout {
+  size_t off, lo[2], hi[2], idx[2], row, temp, temp_bytes, total;
+};
+
+int crowd_layout(int k, uint64_t n, uint32_t buckets, CrowdLayout &l) {
+  l.temp_bytes = 0;
+  DBG_CK(cub::DeviceRadixSort::SortPairs(nullptr, l.temp_bytes, (unsigned long long *)nullptr,
+                                         (unsigned long long *)nullptr, (uint32_t *)nullptr,
+                                         (uint32_t *)nullptr, (int64_t)n, 0, 64, (cudaStream_t)0));
+  size_t at = 0;
+  auto take = [&at](size_t bytes) {
+    const size_t here = at;
+    at += al256(bytes);
+    return here;
+  };
+  l.off = take(((size_t)buckets + 2) * 4);
+  for (int i = 0; i < 2; ++i) {
+    l.lo[i] = take(n * 8);
+    l.hi[i] = take(k > 32 ? n * 8 : 0);
+    l.idx[i] = take(n * 4);
+  }
+  l.row = take(n * 16);
+  l.temp = take(l.temp_bytes);
+  l.total = at;
   return DBG_OK;
 }
 
+// Sort the buckets above the cap, `n` numbers for their records, after the others.
 template <bool WIDE>
-int run(dbg_handle h, const Shape &sh, uint64_t max_rows, void *buf, Slot *rec, uint64_t rec_rows,
-        uint64_t *keys_out, uint32_t *counts_out, ExportMeta &m, cudaStream_t s) {
+int sort_crowded(dbg_handle h, const Shape &sh, const Plan &p, uint64_t n, char *b,
+                 const CrowdLayout &l, const Slot *rec, Key<WIDE> *keys, uint4 *counts,
+                 cudaStream_t s) {
+  Crowd c;
+  c.off = reinterpret_cast<uint32_t *>(b + l.off);
+  c.n = n;
+  for (int i = 0; i < 2; ++i) {
+    c.lo[i] = reinterpret_cast<unsigned long long *>(b + l.lo[i]);
+    c.hi[i] = reinterpret_cast<unsigned long long *>(b + l.hi[i]);
+    c.idx[i] = reinterpret_cast<uint32_t *>(b + l.idx[i]);
+  }
+  c.row = reinterpret_cast<uint4 *>(b + l.row);
+  const int grid = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)std::max(1, h->sm_count) * 8);
+  const int groups = (int)((sh.buckets + kCrowdGroup - 1) / kCrowdGroup);
+  DBG_TRY(launch_after(k_crowd_offsets, 1, kOffBlock, 0, s, p, c.off));
+  DBG_TRY(launch_after(k_crowd_none, grid, 256, 0, s, c, WIDE ? 1 : 0));
+  if (rec)
+    DBG_TRY(launch_after(k_crowd_gather<WIDE, true>, groups, 256, 0, s, p, rec, keys, counts, c));
+  else
+    DBG_TRY(launch_after(k_crowd_gather<WIDE, false>, groups, 256, 0, s, p, rec, keys, counts, c));
+  size_t temp = l.temp_bytes;
+  DBG_CK(cub::DeviceRadixSort::SortPairs(b + l.temp, temp, c.lo[0], c.lo[1], c.idx[0], c.idx[1],
+                                         (int64_t)n, 0, std::min(64, p.key_bits), s));
+  const uint32_t *idx = c.idx[1];
+  if (WIDE && p.key_bits > 64) {  // the low words' order is kept among equal high words
+    DBG_TRY(launch_after(k_crowd_high, grid, 256, 0, s, c));
+    DBG_CK(cub::DeviceRadixSort::SortPairs(b + l.temp, temp, c.hi[1], c.lo[1], c.idx[1], c.idx[0],
+                                           (int64_t)n, 0, p.key_bits - 64, s));
+    idx = c.idx[0];
+  }
+  DBG_TRY(launch_after(k_crowd_write<WIDE>, groups, 256, 0, s, p, c, idx, keys, counts));
+  DBG_CK(cudaGetLastError());
+  DBG_CK(cudaStreamSynchronize(s));
+  return DBG_OK;
+}
+
+// (buf_bytes: what there is of `buf`; the crowded buckets' scratch comes from its
+// rest, or from the pool when buf is the pool's.  *too_dense: too many crowded
+// records, or no scratch for them.)
+template <bool WIDE>
+int run(dbg_handle h, const Shape &sh, uint64_t max_rows, void *buf, uint64_t buf_bytes, bool pooled,
+        Slot *rec, uint64_t rec_rows, uint64_t *keys_out, uint32_t *counts_out, ExportMeta &m,
+        bool *too_dense, cudaStream_t s) {
   char *b = static_cast<char *>(buf);
   Plan p;
   p.key_bits = 2 * (h->k - 1);
@@ -508,6 +804,8 @@ int run(dbg_handle h, const Shape &sh, uint64_t max_rows, void *buf, Slot *rec, 
   p.buckets = sh.buckets;
   p.max_rows = max_rows;
   p.max_placed = rec ? rec_rows : ~0ull;
+  p.max_crowded = std::max<uint64_t>(std::min(max_rows, h->n_slots) / kCrowdedShare, 1u << 16);
+  p.sums = reinterpret_cast<uint2 *>(b + sh.off_sums);
   p.meta = reinterpret_cast<ExportMeta *>(b);
   const ReportSlot slot;
   p.report = reinterpret_cast<ExportMeta *>(slot.p);
@@ -528,10 +826,8 @@ int run(dbg_handle h, const Shape &sh, uint64_t max_rows, void *buf, Slot *rec, 
   if (sh.nbins <= (uint32_t)kPlanBins) {
     DBG_TRY(launch_after(k_plan, 1, kPlanBlock, 0, s, p, h->d_status, h->d_spill_count));
   } else {
-    size_t temp = sh.temp;
-    DBG_CK(cub::DeviceScan::ExclusiveSum(b + sh.off_temp, temp, p.bins, p.bins,
-                                         (int)sh.nbins + 1, s));
-    DBG_TRY(launch_after(k_buckets, (sh.nbins + 256) / 256, 256, 0, s, p, h->d_status,
+    DBG_TRY(launch_after(k_bin_sums, sh.nbins / kChunkBins, kChunkBlock, 0, s, p));
+    DBG_TRY(launch_after(k_buckets, sh.nbins / kChunkBins, kChunkBlock, 0, s, p, h->d_status,
                          h->d_spill_count));
   }
   DBG_CK(cudaGetLastError());
@@ -554,14 +850,34 @@ int run(dbg_handle h, const Shape &sh, uint64_t max_rows, void *buf, Slot *rec, 
   if (!p.report) DBG_CK(cudaMemcpyAsync(&m, p.meta, sizeof(m), cudaMemcpyDeviceToHost, s));
   DBG_CK(cudaStreamSynchronize(s));
   if (p.report) m = *p.report;
-  return DBG_OK;
+  *too_dense = m.crowded > p.max_crowded;
+  if (m.crowded == 0 || *too_dense || m.status != DBG_OK || m.spilled > 0 ||
+      m.vertices > p.max_rows || m.vertices > p.max_placed)
+    return DBG_OK;
+  CrowdLayout l;
+  const uint64_t nc = std::min<uint64_t>(m.crowded, m.vertices);
+  DBG_TRY(crowd_layout(h->k, nc, sh.buckets, l));
+  if (!pooled) {
+    *too_dense = buf_bytes - sh.total < l.total;
+    return *too_dense ? DBG_OK : sort_crowded<WIDE>(h, sh, p, nc, b + sh.total, l, rec, keys,
+                                                       counts, s);
+  }
+  char *more = nullptr;
+  if (scratch_alloc(reinterpret_cast<void **>(&more), l.total, s) != DBG_OK) {
+    cudaGetLastError();
+    *too_dense = true;
+    return DBG_OK;
+  }
+  const int st = sort_crowded<WIDE>(h, sh, p, nc, more, l, rec, keys, counts, s);
+  cudaFreeAsync(more, s);
+  return st;
 }
 
 }  // namespace
 
 int export_bins_scratch(int k, uint64_t rows, uint64_t n_slots, uint64_t &bytes) {
   Shape sh{};
-  DBG_TRY(export_shape(k, rows, n_slots, sh));
+  export_shape(k, rows, n_slots, sh);
   bytes = sh.total;
   return DBG_OK;
 }
@@ -573,7 +889,7 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
   if (no_records) *no_records = false;
   const uint64_t rows = std::min(max_rows, h->n_slots);
   Shape sh{};
-  DBG_TRY(export_shape(h->k, rows, h->n_slots, sh));
+  export_shape(h->k, rows, h->n_slots, sh);
   char *buf = static_cast<char *>(scratch);
   if (!scratch) DBG_TRY(scratch_alloc(reinterpret_cast<void **>(&buf), sh.total, s));
   if (scratch && scratch_bytes < sh.total) return DBG_ERR_INVALID_ARG;
@@ -611,8 +927,8 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
       const cudaError_t e = cudaStreamWaitEvent(s, h->bin.done, 0);
       if (e != cudaSuccess) { rc = cuda_fail(e, "cudaStreamWaitEvent"); break; }
     }
-    rc = h->k > 32 ? run<true>(h, sh, max_rows, buf, rec, rec_rows, keys_out, counts_out, m, s)
-                   : run<false>(h, sh, max_rows, buf, rec, rec_rows, keys_out, counts_out, m, s);
+    rc = (h->k > 32 ? run<true> : run<false>)(h, sh, max_rows, buf, scratch_bytes, !scratch, rec,
+                                              rec_rows, keys_out, counts_out, m, too_dense, s);
     if (own && rc == DBG_OK) {
       const cudaError_t e = cudaEventRecord(h->bin.done, s);
       if (e != cudaSuccess) rc = cuda_fail(e, "cudaEventRecord");
@@ -630,7 +946,6 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
   if (m.status != DBG_OK) return (int)m.status;
   if (m.spilled > 0) return DBG_ERR_NEEDS_GROW;
   *D = m.vertices;
-  *too_dense = m.vertices > 0 && (1u << sh.bucket_log2) + m.max_bin > kBucketCap;
   return DBG_OK;
 }
 
