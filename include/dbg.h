@@ -362,7 +362,8 @@ int dbg_stats(dbg_handle h, uint64_t *n_vertices, uint64_t *n_edges, void *strea
  * device (up to 4 GiB of it stays cached between calls) and is released to
  * it before return.  When both outputs are 16-byte aligned device buffers
  * the records are sorted inside them, and the temporary memory is the sort's
- * bins (up to about 8 MB, or a byte for every 9 vertices if that is more);
+ * bins (up to about 8 MB, or a byte for every 9 vertices if that is more) and,
+ * if there is room, a bit per table slot;
  * a graph built on the binned path places its records in the handle's event
  * buffer first, and one with k > 32 in up to 4 GiB of the pool (32 bytes a
  * vertex).  Pinned host outputs (both, 16-byte aligned) are written by the
@@ -377,7 +378,8 @@ int dbg_export_sorted(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, ui
                       uint64_t *n_out, void *stream);
 
 /* Device bytes of scratch dbg_export_sorted_with needs for a graph of
- * n_vertices vertices (k <= 32, a table of at most 2^32 slots): the sort's
+ * n_vertices vertices (k <= 32, a table of at most 2^32 slots; more is used
+ * for a bit per slot and for crowded vertices' sort, if it is there): the sort's
  * bins, and for the radix sort behind it its histograms, one slot index per
  * vertex and the lists of runs of keys that share a prefix.  0 for arguments
  * it does not take.  Needs a device (the sort sizes its work for it). */

@@ -76,3 +76,41 @@ def test_a_sixteenth_of_the_table(k):
         assert np.array_equal(keys.cpu().numpy().view(np.uint64), ref.keys)
         assert np.array_equal(counts.cpu().numpy().view(np.uint32), ref.counts)
         g.close()
+
+
+# (12.5 M slots: a warp takes more slots at a time from there on)
+@pytest.mark.parametrize("slots", [20_001, 3_000_000, 9_961_471, 9_961_472, 12_500_001])
+@pytest.mark.parametrize("k", [25, 51])
+def test_sparse_tables(slots, k):
+    import torch
+    rs = synth.ragged_reads(60, 150, k, 8)
+    ref = oracle.build_graph(rs.packed, rs.offsets, k)
+    D = len(ref.keys)
+    g = dbg.Graph(k, slots)
+    g.set_tuning(insert_path=1)
+    g.insert(*to_device(rs))
+    keys, counts = outputs(D, k)
+    assert g.export_into(keys, counts) == D
+    assert np.array_equal(keys.cpu().numpy().view(np.uint64), ref.keys)
+    assert np.array_equal(counts.cpu().numpy().view(np.uint32), ref.counts)
+    if k <= 32:  # the caller's scratch, with and without room for a bit per slot
+        need = dbg.export_scratch_bytes(k, D, slots)
+        for room in (0, slots // 8 + 512):
+            keys, counts = outputs(D, k)
+            scratch = torch.empty(need + room, dtype=torch.uint8, device="cuda")
+            assert g.export_with(keys, counts, scratch) == D
+            assert np.array_equal(keys.cpu().numpy().view(np.uint64), ref.keys)
+            assert np.array_equal(counts.cpu().numpy().view(np.uint32), ref.counts)
+    g.close()
+
+
+def test_a_sparse_table_is_read_once():
+    # 3.2 GB with a few thousand vertices: the export takes about one pass over
+    # the table, as counting its vertices does
+    rs = synth.ragged_reads(60, 150, 31, 8)
+    g = dbg.Graph(31, 100_000_000)
+    g.set_tuning(insert_path=1)
+    g.insert(*to_device(rs))
+    out = outputs(g.stats()[0], 31)
+    assert seconds(lambda: g.export_into(*out)) < 1.5 * seconds(g.stats)
+    g.close()
