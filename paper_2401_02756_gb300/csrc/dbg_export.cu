@@ -785,10 +785,9 @@ int export_bins_mapped(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, u
 }
 
 // The sort by bins into other outputs (pageable or unaligned memory, or one of
-// the two not asked for): into temporary ones, then copied.
-int export_bins_copied(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t max_n,
-                       uint64_t *D, cudaStream_t s, bool *too_dense) {
-  const uint64_t rows = std::min(max_n, h->n_slots);
+// the two not asked for): into temporary ones of `rows` rows, then copied.
+int export_bins_rows(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t rows,
+                     uint64_t *D, cudaStream_t s, bool *too_dense) {
   const size_t key_bytes = h->k > 32 ? 16 : 8, kb = align256(rows * key_bytes);
   char *buf = nullptr;
   DBG_TRY(scratch_alloc(reinterpret_cast<void **>(&buf), kb + align256(rows * 16), s));
@@ -806,6 +805,21 @@ int export_bins_copied(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, u
   e = cudaStreamSynchronize(s);
   if (rc == DBG_OK && e != cudaSuccess) rc = cuda_fail(e, "cudaStreamSynchronize");
   return rc;
+}
+
+// With as many rows as the outputs or the table could take, so that nothing is
+// counted before; when there is no memory for that, with as many as there are
+// vertices.
+int export_bins_copied(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t max_n,
+                       uint64_t *D, cudaStream_t s, bool *too_dense) {
+  const uint64_t rows = std::min(max_n, h->n_slots);
+  const int st = export_bins_rows(h, keys_out, counts_out, rows, D, s, too_dense);
+  if (st != DBG_ERR_OOM) return st;
+  cudaGetLastError();
+  *too_dense = false;
+  DBG_TRY(dbg_stats(h, D, nullptr, s));
+  if (*D == 0 || *D > max_n) return DBG_OK;
+  return export_bins_rows(h, keys_out, counts_out, *D, D, s, too_dense);
 }
 
 }  // namespace
