@@ -122,6 +122,7 @@ constexpr unsigned long long kIsSplitter = 1ull << 63;  // in a slot's link: the
 // What the passes share.  A slot's link (its 8 bytes of padding), for a
 // single-exit vertex: its successor's slot, or kIsSplitter | number.
 struct Links {
+  uint64_t w0, nw;                    // the words of 32 slots that the bits below are of
   uint32_t *marks;                    // a bit per slot: an edge points to its vertex
   uint2 *degree;                      // per 32 slots: bits of one exit, bits of several
   ulonglong2 *split;                  // a splitter's slot (its label in the two top bits), its successor's
@@ -195,13 +196,13 @@ __global__ void __launch_bounds__(256) k_links(View v, Links k) {
           continue;
         }
         target[u] = s;
-        atomicOr(&k.marks[s >> 5], 1u << (s & 31));
+        if ((s >> 5) - k.w0 < k.nw) atomicOr(&k.marks[(s >> 5) - k.w0], 1u << (s & 31));
       }
       label[u] = (uint32_t)__ffs((int)exits) - 1u;  // (of a single-exit vertex)
       const bool one = exits != 0 && (exits & (exits - 1)) == 0;
       ones[u] = __ballot_sync(0xffffffffu, one);
       const unsigned several = __ballot_sync(0xffffffffu, exits != 0 && !one);
-      if (lane == 0 && w < words) k.degree[w] = make_uint2(ones[u], several);
+      if (lane == 0 && w - k.w0 < k.nw) k.degree[w - k.w0] = make_uint2(ones[u], several);
       picks[u] = __ballot_sync(0xffffffffu,
                                one && ((uint32_t)key_hash(key) & (kSpacing - 1u)) == 0u);
       at[u] = 0;
@@ -235,14 +236,13 @@ __global__ void __launch_bounds__(256) k_start_edges(View v, Links k, unsigned l
                                                      unsigned long long *count, uint64_t cap) {
   after_previous();
   const int lane = threadIdx.x & 31;
-  const uint64_t words = (v.n + 31) >> 5;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t base = (uint64_t)blockIdx.x * blockDim.x; base < words; base += stride) {
-    const uint64_t w = base + threadIdx.x;
+  for (uint64_t base = (uint64_t)blockIdx.x * blockDim.x; base < k.nw; base += stride) {
+    const uint64_t at_word = base + threadIdx.x, w = k.w0 + at_word;
     uint32_t starts = 0, ones = 0, edges = 0;
-    if (w < words) {
-      const uint2 deg = k.degree[w];
-      ones = deg.x & ~k.marks[w];
+    if (at_word < k.nw) {
+      const uint2 deg = k.degree[at_word];
+      ones = deg.x & ~k.marks[at_word];
       starts = ones | deg.y;
       edges = (uint32_t)__popc(ones);
     }
@@ -582,77 +582,83 @@ extern "C" int dbg_normalize(dbg_handle h, double divisor, void *stream) {
   return DBG_OK;
 }
 
-extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_bases,
-                                uint64_t *offsets_out, uint64_t max_contigs, uint64_t *n_contigs,
-                                uint64_t *n_bases, void *stream) {
-  using namespace dbg;
-  if (!h || !n_contigs || !n_bases || h->k > 32) return DBG_ERR_INVALID_ARG;
-  Guard g(h->device);
-  if (g.err != cudaSuccess) return cuda_fail(g.err, "cudaSetDevice");
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int st = dbg_get_status(h, stream);
-  if (st != DBG_OK) return st;
+namespace dbg {
+namespace {
 
+// The contigs of a complete graph.  frugal: with memory for the contigs and a few
+// bits a slot only -- no splitters (every contig is walked by its own thread), the
+// start edges counted before they are listed, and, when a bit of each kind per
+// slot is not to be had, bits for a part of the table and a pass for every part.
+int find_contigs(dbg_handle h, char *bases_out, uint64_t max_bases, uint64_t *offsets_out,
+                 uint64_t max_contigs, uint64_t *n_contigs, uint64_t *n_bases, cudaStream_t s,
+                 bool frugal) {
   const int m = h->k - 1;
   const View v{h->table, h->n_slots, h->max_probes,
                m >= 32 ? ~0ull : ((1ull << (2 * m)) - 1ull), h->d_status};
   const int grid = std::max(1, h->sm_count) * 8;
   Scratch scr{s};
-  // marks, degrees and splitters by the table's size; a twelfth more splitters
-  // than one vertex in `spacing` of a full table gives (when that much memory is
-  // not to be had: none, and every contig is walked by its own thread)
+  // marks, degrees and splitters by the table's size
   const uint64_t words = (h->n_slots + 31) >> 5;
-  uint64_t cap = room_splitters(h->n_slots);
+  const uint64_t cap = frugal ? 0 : room_splitters(h->n_slots);
+  uint64_t nw = words;
   const uint64_t rounds = (uint64_t)room_levels(h->n_slots) + 1;
-  const size_t mark_bytes = align256(words * 4), bits_bytes = 256 + mark_bytes + align256(words * 8);
+  auto bits_bytes = [](uint64_t w) { return 256 + align256(w * 4) + align256(w * 8); };
   auto split_bytes = [rounds](uint64_t c) {
     return align256(c * sizeof(ulonglong2)) + 2 * align256(c * 4 * rounds) + align256(c * 8);
   };
   char *buf = nullptr;
-  st = scr.get(reinterpret_cast<void **>(&buf), bits_bytes + split_bytes(cap));
-  if (st == DBG_ERR_OOM) {
+  for (;; nw = (nw + 1) / 2) {
+    const int st = scr.get(reinterpret_cast<void **>(&buf), bits_bytes(nw) + split_bytes(cap));
+    if (st == DBG_OK) break;
+    if (st != DBG_ERR_OOM || !frugal || nw <= 1024) return st;
     cudaGetLastError();
-    cap = 0;
-    st = scr.get(reinterpret_cast<void **>(&buf), bits_bytes);
   }
-  if (st != DBG_OK) return st;
   unsigned long long *counts = reinterpret_cast<unsigned long long *>(buf);  // [3], see below
+  const size_t mark_bytes = align256(nw * 4);
   Links k{};
   k.marks = reinterpret_cast<uint32_t *>(buf + 256);
   k.degree = reinterpret_cast<uint2 *>(buf + 256 + mark_bytes);
-  k.split = reinterpret_cast<ulonglong2 *>(buf + bits_bytes);
-  k.next = reinterpret_cast<uint32_t *>(buf + bits_bytes + align256(cap * sizeof(ulonglong2)));
+  k.split = reinterpret_cast<ulonglong2 *>(buf + bits_bytes(nw));
+  k.next = reinterpret_cast<uint32_t *>(buf + bits_bytes(nw) + align256(cap * sizeof(ulonglong2)));
   k.len = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(k.next) +
                                        align256(cap * 4 * rounds));
   k.labels = reinterpret_cast<unsigned long long *>(
       reinterpret_cast<char *>(k.len) + align256(cap * 4 * rounds));
   k.cap = (uint32_t)cap;
   k.n_split = counts + 1;
-  DBG_CK(cudaMemsetAsync(buf, 0, 256 + mark_bytes, s));  // counts and marks
-  if (h->n_slots <= 1u << 20)
-    DBG_TRY(launch_after(k_links<1>, (int)std::min<uint64_t>((words + 7) / 8, (uint64_t)grid), 256,
-                         0, s, v, k));
-  else
-    DBG_TRY(launch_after(k_links<2>, (int)std::min<uint64_t>((words + 15) / 16, (uint64_t)grid),
-                         256, 0, s, v, k));
-  DBG_CK(cudaGetLastError());
 
-  // the start edges into a buffer that holds as many as an ordinary graph has;
-  // a second pass when there are more
-  uint64_t starts_cap = h->n_slots / 16 + 1024;
+  // the start edges into a buffer that holds as many as an ordinary graph has; a
+  // second pass when there are more
+  uint64_t starts_cap = frugal ? 0 : h->n_slots / 16 + 1024;
   unsigned long long *starts_a = nullptr;
   uint64_t got[4] = {0, 0, 0, 0};  // start edges, splitters, units, status
-  for (;;) {
-    DBG_TRY(scr.get(reinterpret_cast<void **>(&starts_a), starts_cap * sizeof(unsigned long long)));
-    DBG_TRY(launch_after(k_start_edges, (int)std::min<uint64_t>((words + 255) / 256,
-                         (uint64_t)grid), 256, 0, s, v, k, starts_a, counts, starts_cap));
+  for (bool linked = false;;) {
+    if (starts_cap > 0)
+      DBG_TRY(scr.get(reinterpret_cast<void **>(&starts_a), starts_cap * sizeof(unsigned long long)));
+    // (the start edges of the parts add up; the splitters are numbered anew in each)
+    const size_t kept = nw < words || linked ? sizeof(unsigned long long) : 0;
+    if (kept) DBG_CK(cudaMemsetAsync(counts, 0, kept, s));
+    for (k.w0 = 0; k.w0 < words; k.w0 += nw) {
+      k.nw = std::min(nw, words - k.w0);
+      if (!linked || nw < words) {
+        DBG_CK(cudaMemsetAsync(buf + kept, 0, 256 - kept + mark_bytes, s));  // counts, marks
+        if (h->n_slots <= 1u << 20)
+          DBG_TRY(launch_after(k_links<1>, (int)std::min<uint64_t>((words + 7) / 8, (uint64_t)grid),
+                               256, 0, s, v, k));
+        else
+          DBG_TRY(launch_after(k_links<2>, (int)std::min<uint64_t>((words + 15) / 16,
+                               (uint64_t)grid), 256, 0, s, v, k));
+      }
+      DBG_TRY(launch_after(k_start_edges, (int)std::min<uint64_t>((k.nw + 255) / 256,
+                           (uint64_t)grid), 256, 0, s, v, k, starts_a, counts, starts_cap));
+    }
     DBG_CK(cudaGetLastError());
-    const DeviceWord words[] = {{counts, 8}, {counts + 1, 8}, {counts + 2, 8}, {h->d_status, 4}};
-    DBG_TRY(read_words(words, 4, got, s));
+    const DeviceWord read[] = {{counts, 8}, {counts + 1, 8}, {counts + 2, 8}, {h->d_status, 4}};
+    DBG_TRY(read_words(read, 4, got, s));
     if (got[3] != DBG_OK) return (int)got[3];
     if (got[0] <= starts_cap) break;
     starts_cap = got[0];
-    DBG_CK(cudaMemsetAsync(counts, 0, sizeof(unsigned long long), s));
+    linked = true;
   }
   const uint64_t S = got[0];
   const uint32_t n_split = (uint32_t)std::min<uint64_t>(got[1], cap);
@@ -730,4 +736,25 @@ extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_base
   DBG_CK(cudaMemcpyAsync(offsets_out, off, (S + 1) * sizeof(uint64_t), cudaMemcpyDefault, s));
   DBG_CK(cudaMemcpyAsync(bases_out, chars, B, cudaMemcpyDefault, s));
   return read_status(h, s);
+}
+
+}  // namespace
+}  // namespace dbg
+
+extern "C" int dbg_find_contigs(dbg_handle h, char *bases_out, uint64_t max_bases,
+                                uint64_t *offsets_out, uint64_t max_contigs, uint64_t *n_contigs,
+                                uint64_t *n_bases, void *stream) {
+  using namespace dbg;
+  if (!h || !n_contigs || !n_bases || h->k > 32) return DBG_ERR_INVALID_ARG;
+  Guard g(h->device);
+  if (g.err != cudaSuccess) return cuda_fail(g.err, "cudaSetDevice");
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  DBG_TRY(dbg_get_status(h, stream));  // complete graphs only
+  const int st = find_contigs(h, bases_out, max_bases, offsets_out, max_contigs, n_contigs, n_bases,
+                              s, false);
+  if (st != DBG_ERR_OOM) return st;
+  cudaGetLastError();
+  DBG_CK(cudaStreamSynchronize(s));  // (what the first attempt took is free again)
+  trim_scratch_pool(h->device);
+  return find_contigs(h, bases_out, max_bases, offsets_out, max_contigs, n_contigs, n_bases, s, true);
 }

@@ -315,6 +315,8 @@ int cuda_fail(cudaError_t e, const char *what);
 // Temporary device memory from the library's stream-ordered pool (free it
 // with cudaFreeAsync on a stream).
 int scratch_alloc(void **p, size_t bytes, cudaStream_t s);
+// Give what device `dev`'s pool holds and nobody uses back to the device.
+void trim_scratch_pool(int dev);
 // Give the pools' cached memory back to the device (synchronising each device).
 int release_scratch_pools();
 // Device bytes the pool of device `dev` holds now.

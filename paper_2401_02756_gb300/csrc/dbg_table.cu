@@ -131,6 +131,11 @@ uint64_t pool_reserved_bytes(int dev) {
   return v;
 }
 
+void trim_scratch_pool(int dev) {
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (dev >= 0 && dev < 64 && g_pools[dev]) cudaMemPoolTrimTo(g_pools[dev], 0);
+}
+
 int release_scratch_pools() {
   std::lock_guard<std::mutex> lock(g_pool_mu);
   int prev = 0;

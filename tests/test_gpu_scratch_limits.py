@@ -8,6 +8,7 @@ import pytest
 
 import oracle
 from gpu_util import to_device
+from oracle import contigs as oc
 from paper_2401_02756_gb300 import build, dbg, synth
 
 pytestmark = pytest.mark.gpu
@@ -71,3 +72,39 @@ def test_export_into_more_rows_than_there_is_memory_for(k):
     del taken
     g.close()
     dbg.release_scratch()
+
+
+# 1,100 MB: no room for splitters; 500: nor for a list of the usual number of start
+# edges; 200: nor for bits of the whole table
+@pytest.mark.parametrize("megabytes", [3000, 1100, 500, 200])
+def test_contigs(megabytes):
+    rs = synth.ragged_reads(300, 150, 31, 4)
+    ref = oracle.build_graph(rs.packed, rs.offsets, 31)
+    want = oc.find_contigs(ref.keys, ref.counts, 31)
+    g = graph(rs)
+    taken = all_but(megabytes)
+    got = g.contigs()
+    del taken
+    g.close()
+    dbg.release_scratch()
+    assert got == want
+
+
+def test_many_contigs():
+    # more memory for the contigs than for anything else: their lists and their
+    # text fit, what makes finding them faster does not
+    slots = 80_000_000
+    rs = synth.sample_reads(synth.random_genome(2_000_000, 2), 2_000_000, 100, 0.02, 2, 21, "r")
+    g = dbg.Graph(21, slots)
+    g.set_tuning(insert_path=1)
+    g.insert(*to_device(rs))
+    want = g.contigs()
+    S, B = len(want), sum(map(len, want))
+    need = slots // 32 * 12 + 64 * S + B
+    assert 32 * S > need // 8 + (64 << 20)
+    taken = all_but((need + need // 8 + (64 << 20)) >> 20)
+    got = g.contigs()
+    del taken
+    g.close()
+    dbg.release_scratch()
+    assert got == want
