@@ -370,6 +370,7 @@ struct Unit {
   uint32_t contig, split;
   unsigned long long rel;
 };
+constexpr uint64_t kMaxUnitContigs = 0xFFFFFFFFull;
 // A contig's own thread writes its first `own` edges (all of them when it
 // does not go by splitters).
 struct Contig {
@@ -670,7 +671,8 @@ int find_contigs(dbg_handle h, char *bases_out, uint64_t max_bases, uint64_t *of
     DBG_CK(cudaStreamSynchronize(s));
     return DBG_OK;
   }
-  if (S > 0xFFFFFFFFull) return DBG_ERR_CAPACITY;  // (contig numbers in a unit are 32-bit)
+  // (contig numbers in a unit are 32-bit; the frugal form has no units)
+  if (S > kMaxUnitContigs && !frugal) return DBG_ERR_OOM;
 
   k.kept = n_split;
   if (n_split > 0) {
