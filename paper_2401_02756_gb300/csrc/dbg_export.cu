@@ -16,6 +16,8 @@
 // small histogram space.  Host outputs go through temporary device buffers.
 #include <cub/device/device_radix_sort.cuh>
 
+#include <cuda.h>
+
 #include <algorithm>
 
 #include "dbg_export.cuh"
@@ -749,23 +751,41 @@ int export_radix(dbg_handle h, uint64_t D, uint64_t *keys_out, uint32_t *counts_
   return export_pairs<unsigned long long>(h, D, keys_out, counts_out, s);
 }
 
+// One pinned allocation or registration that [p, p + bytes) lies in?  (Its two
+// ends being pinned does not say so: they may be two registrations with pageable
+// memory between them.)
+bool one_range(const void *p, uint64_t bytes) {
+  using Get = CUresult (*)(void *, CUpointer_attribute, CUdeviceptr);
+  static const Get get = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault,
+                                         &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      return Get(nullptr);
+    }
+    return reinterpret_cast<Get>(f);
+  }();
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  const CUdeviceptr at = (CUdeviceptr)(uintptr_t)p;
+  return get && get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) == CUDA_SUCCESS &&
+         get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) == CUDA_SUCCESS && start <= at &&
+         at - start <= size && bytes <= size - (at - start);
+}
+
 // The device's view of pinned host memory [p, p + bytes), 16-byte aligned, or
 // null.
 void *mapped_host(void *p, uint64_t bytes) {
   if (!p || bytes == 0 || ((uintptr_t)p & 15u)) return nullptr;
-  cudaPointerAttributes a{}, z{};
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
-      cudaPointerGetAttributes(&z, static_cast<char *>(p) + bytes - 1) != cudaSuccess) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
-  const bool host = a.type == cudaMemoryTypeHost && z.type == cudaMemoryTypeHost &&
-                    a.devicePointer && z.devicePointer;
-  // (both ends in one mapping)
-  return host && static_cast<char *>(z.devicePointer) - static_cast<char *>(a.devicePointer) ==
-                     (int64_t)(bytes - 1)
-             ? a.devicePointer
-             : nullptr;
+  return a.type == cudaMemoryTypeHost && a.devicePointer && one_range(p, bytes) ? a.devicePointer
+                                                                                : nullptr;
 }
 
 // The sort by bins into pinned host memory: the bucket sort writes its rows
