@@ -244,11 +244,14 @@ int dbg_insert_reads_host(dbg_handle h, const uint8_t *packed, const uint64_t *o
  * else for 4.25 events per slot or 160 per read, up to 2.3 GB); inside a
  * stream capture, without that memory or with more events than it holds the
  * direct insert does it.  dbg_binned_counters does not tell of such a call.  A
- * rebuild with k from 33 to 63 is binned too, with
- * 16-byte events (tables of 256 MiB or more; default 3 events per slot, 34
- * bytes per event across the two buffers; the direct insert when they would
- * take more than half of the device's free memory).  Errors: as
- * dbg_insert_reads. */
+ * rebuild with k from 33 to 63 is binned too, with 16-byte events (tables of
+ * 256 MiB or more; default 3 events per slot, 34 bytes per event across the two
+ * buffers).  Those buffers belong to the library, one set per device, grown as
+ * needed and kept until dbg_release_scratch or until an allocation of the
+ * library's finds no memory; such rebuilds on one device run one after another
+ * on the GPU.  The direct insert does it inside a stream capture, and when the
+ * buffers would take more than a quarter of the device's memory or half of what
+ * is free.  Errors: as dbg_insert_reads. */
 int dbg_build_reads(dbg_handle h, const uint8_t *packed, const uint64_t *offsets,
                     uint64_t n_reads, void *stream);
 
@@ -302,17 +305,17 @@ int dbg_insert_batch(const dbg_batch_item *items, int n_items, void *stream);
  * launch per group of 128.  Errors: as dbg_insert_batch. */
 int dbg_build_batch(const dbg_batch_item *items, int n_items, void *stream);
 
-/* Give back the device memory the library keeps between calls: the batched
- * inserts' buffers and the pool of the exports and of mid-size rebuilds, on every device
- * (each is synchronised first), and the 4 KB page of pinned host memory that
+/* Give back the device memory the library keeps between calls: the buffers of the
+ * batched inserts and of rebuilds with k > 32, and the pool of the exports and of
+ * mid-size rebuilds, on every device (each is synchronised first), and the 4 KB page of pinned host memory that
  * results are reported through when no call uses it (calls copy their results
  * until the next graph is created).  Later calls allocate again as needed.
  * Errors: CUDA. */
 int dbg_release_scratch(void);
 
 /* Device bytes the library holds between calls on the current device: the
- * batched inserts' buffers and the pool of the exports and of mid-size rebuilds (what
- * dbg_release_scratch gives back).  A caller that keeps a device-memory
+ * buffers of the batched inserts and of rebuilds with k > 32, and the pool of the
+ * exports and of mid-size rebuilds (what dbg_release_scratch gives back).  A caller that keeps a device-memory
  * budget counts them; 0 when there is no device. */
 uint64_t dbg_scratch_bytes(void);
 

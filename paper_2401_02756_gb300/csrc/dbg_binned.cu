@@ -1660,7 +1660,7 @@ uint64_t default_events(uint64_t n_slots) {
 int ensure_events(BinScratch &sc, uint64_t events) {
   if (!sc.meta) {
     void *p = nullptr;
-    cudaError_t e = cudaMalloc(&p, kBinMetaBytes);
+    cudaError_t e = device_malloc(&p, kBinMetaBytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(binned meta)");
     sc.meta = static_cast<unsigned long long *>(p);
   }
@@ -1672,7 +1672,7 @@ int ensure_events(BinScratch &sc, uint64_t events) {
     sc.ev = sc.ev2 = nullptr;
     sc.cap = 0;
     void *p = nullptr;
-    cudaError_t e = cudaMalloc(&p, events * sizeof(uint64_t));
+    cudaError_t e = device_malloc(&p, events * sizeof(uint64_t));
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(binned events)");
     sc.ev = static_cast<uint64_t *>(p);
     sc.cap = events;
@@ -1683,9 +1683,6 @@ int ensure_events(BinScratch &sc, uint64_t events) {
 }  // namespace
 
 uint64_t bin_events_wanted(dbg_handle h) {
-  if (h->k > 32)
-    return 2 * (h->bin_want ? h->bin_want
-                            : std::max(kBinMinEvents, kBinWideEventsPerSlot * h->n_slots));
   return h->bin_want ? h->bin_want : default_events(h->n_slots);
 }
 
@@ -1761,7 +1758,7 @@ bool ensure_tile_scratch(BinScratch &sc, int parts, uint64_t tiles, bool capturi
   if (cudaDeviceSynchronize() != cudaSuccess) return false;  // earlier calls may use them
   if (!sc.ev2) {
     void *p = nullptr;
-    if (cudaMalloc(&p, ev2_capacity(sc.cap) * sizeof(uint64_t)) != cudaSuccess) {
+    if (device_malloc(&p, ev2_capacity(sc.cap) * sizeof(uint64_t)) != cudaSuccess) {
       cudaGetLastError();  // clear the allocation failure
       return false;
     }
@@ -1772,7 +1769,7 @@ bool ensure_tile_scratch(BinScratch &sc, int parts, uint64_t tiles, bool capturi
     sc.aux = nullptr;
     sc.aux_bytes = 0;
     void *p = nullptr;
-    if (cudaMalloc(&p, need) != cudaSuccess) {
+    if (device_malloc(&p, need) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
@@ -2185,6 +2182,10 @@ int launch_binned_pooled(dbg_handle h, const ItemDesc &it, const dbg_tuning &tun
   return st;
 }
 
+namespace {
+constexpr int kMaxDevices = 64;
+}  // namespace
+
 #include "dbg_binned_wide.cuh"
 
 // ---------------------------------------------------------------------------
@@ -2193,7 +2194,6 @@ int launch_binned_pooled(dbg_handle h, const ItemDesc &it, const dbg_tuning &tun
 
 namespace {
 
-constexpr int kMaxDevices = 64;
 std::mutex g_batch_mu;
 BinScratch g_batch[kMaxDevices];
 
@@ -2306,11 +2306,7 @@ uint64_t bin_ev2_bytes(dbg_handle h) {
 uint64_t batch_scratch_bytes(int dev) {
   if (dev < 0 || dev >= kMaxDevices) return 0;
   std::lock_guard<std::mutex> lock(g_batch_mu);
-  const BinScratch &sc = g_batch[dev];
-  uint64_t b = sc.aux_bytes + (sc.meta ? kBinMetaBytes : 0);
-  if (sc.ev) b += sc.cap * sizeof(uint64_t);
-  if (sc.ev2) b += ev2_capacity(sc.cap) * sizeof(uint64_t);
-  return b;
+  return scratch_bytes_of(g_batch[dev]);
 }
 
 int release_batch_scratch() {
@@ -2318,10 +2314,11 @@ int release_batch_scratch() {
   int prev = 0;
   DBG_CK(cudaGetDevice(&prev));
   for (int d = 0; d < kMaxDevices; ++d) {
-    if (!g_batch[d].meta && !g_batch[d].ev) continue;
+    if (!g_batch[d].meta && !g_batch[d].ev && wide_scratch_bytes(d) == 0) continue;
     DBG_CK(cudaSetDevice(d));
     DBG_CK(cudaDeviceSynchronize());
     free_bin_scratch(g_batch[d]);
+    release_wide_scratch(d);
   }
   DBG_CK(cudaSetDevice(prev));
   return DBG_OK;
@@ -2329,6 +2326,18 @@ int release_batch_scratch() {
 
 int binned_counters(dbg_handle h, uint64_t *out) {
   out[0] = out[1] = out[2] = 0;
+  if (h->k > 32) {
+    unsigned long long overflow = 0, deferred = 0;
+    DBG_CK(cudaDeviceSynchronize());
+    DBG_CK(cudaMemcpy(&overflow, small_word(h->d_status, kSmallOverflow), sizeof(overflow),
+                      cudaMemcpyDeviceToHost));
+    DBG_CK(cudaMemcpy(&deferred, small_word(h->d_status, kSmallDeferred), sizeof(deferred),
+                      cudaMemcpyDeviceToHost));
+    out[0] = deferred != 0;
+    out[1] = deferred ? deferred - 1 : 0;
+    out[2] = overflow;
+    return DBG_OK;
+  }
   if (!h->bin.meta) return DBG_OK;  // no binned call yet
   DBG_CK(cudaDeviceSynchronize());
   uint32_t flag = 0;

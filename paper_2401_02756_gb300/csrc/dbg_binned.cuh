@@ -40,9 +40,8 @@ constexpr size_t kBinClearedBytes = (4 + 2 * (size_t)kBatchItems) * 8;
 // most kBinMaxParts of them.
 BinGeometry bin_geometry(uint64_t n_slots, int region_log2);
 
-// The event capacity a handle's binned inserts use, in 8-byte units: what
-// dbg_reserve_events asked for, else the default of 4.25 per table slot (k > 32:
-// two units an event, 3 events per slot by default).
+// The event capacity a handle's binned inserts use (k < 32): what dbg_reserve_events
+// asked for, else the default of 4.25 per table slot.
 uint64_t bin_events_wanted(dbg_handle h);
 
 // Make sure the handle holds an event buffer of at least `events` events
@@ -81,14 +80,12 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
 int launch_binned_pooled(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cudaStream_t s,
                          int call, const InputParts *input, bool *done);
 
-// Rebuild a graph with k from 33 to 63 through 16-byte events (dbg_binned_wide.cuh);
-// the scratch must be there (wide_scratch_ready).
-int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int call);
-
-// Whether a wide rebuild on `s` can have its scratch: made now if it is not
-// there yet, unless the stream is being captured or the device is short of
-// memory.
-bool wide_scratch_ready(dbg_handle h, cudaStream_t s);
+// Rebuild a graph with k from 33 to 63 through 16-byte events (dbg_binned_wide.cuh),
+// with the device's scratch for that.  False in *done: it is not to be had (a
+// captured stream, a device short of memory), nothing was launched.
+int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int call, bool *done);
+// Device bytes of that scratch on device `dev`.
+uint64_t wide_scratch_bytes(int dev);
 
 // Insert many read sets, each into its own table (k <= 31), through binned
 // chains: every chain is one launch of each binned kernel over all of its

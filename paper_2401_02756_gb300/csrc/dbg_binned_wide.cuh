@@ -486,58 +486,78 @@ __global__ void k_wide_deferred(const __grid_constant__ ItemPack<1> pk, const Wi
     atomicAdd(small_built(it.status), (unsigned long long)claimed);
 }
 
+// What dbg_binned_counters tells, kept by the graph: the next graph's call
+// overwrites the scratch's.
+__global__ void k_wide_told(uint32_t *status, const uint32_t *use_binned, TileAux aux) {
+  after_previous();
+  if (threadIdx.x != 0) return;
+  const bool binned = ld_volatile_u32(use_binned) != 0u;
+  *small_word(status, kSmallOverflow) = binned ? *aux.overflow : 0ull;
+  *small_word(status, kSmallDeferred) = binned ? *aux.deferred + 1ull : 0ull;
+}
+
 int wide_shift(dbg_handle h) {
   const int log2 = h->tuning.region_log2 > 0 ? h->tuning.region_log2
                                              : tiled_shift(h->n_slots, kTableRegions);
   return bin_geometry(h->n_slots, std::max(log2, kTileLog2)).shift;
 }
 
-}  // namespace
+// The units of 8 bytes that a graph's rebuild has room for: two an event.
+uint64_t wide_units_wanted(dbg_handle h) {
+  return 2 * (h->bin_want ? h->bin_want
+                          : std::max(kBinMinEvents, kBinWideEventsPerSlot * h->n_slots));
+}
 
-bool wide_scratch_ready(dbg_handle h, cudaStream_t s) {
-  const int shift = wide_shift(h);
-  if ((1 << (shift - kTileLog2)) > kMaxBinsPerThread * kWideBlock) return false;
-  const uint64_t want = bin_events_wanted(h), tiles = table_tiles(h->n_slots, shift);
-  const int parts = regions_of(h->n_slots, shift);
-  if (want / 2 >= kMaxChainEvents) return false;  // (bucket positions are 32-bit)
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) return false;
-  const bool capturing = capture != cudaStreamCaptureStatusNone;
-  if (h->bin.cap != want) {
-    if (capturing) return false;
-    // about 100 bytes a slot by default: only out of memory nobody may need soon
+// The scratch of the wide rebuilds, one a device, shared by its graphs: at about
+// 100 bytes a slot by default it is three times the table, too much for every
+// graph to keep.  The calls that use it follow one another on the GPU.  No
+// captured call uses it (a replay would find it replaced or given back).
+struct WideScratch {
+  std::mutex mu;
+  BinScratch sc;
+};
+WideScratch g_wide[kMaxDevices];
+thread_local bool t_in_wide = false;  // (this thread holds a WideScratch's lock)
+
+uint64_t scratch_bytes_of(const BinScratch &sc) {
+  return sc.aux_bytes + (sc.meta ? kBinMetaBytes : 0) + (sc.ev ? sc.cap * sizeof(uint64_t) : 0) +
+         (sc.ev2 ? ev2_capacity(sc.cap) * sizeof(uint64_t) : 0);
+}
+
+// Room for `want` 8-byte units, taken when there is not: no more than a quarter of the
+// device's memory, and half of what is free beside the scratch's own.
+bool ensure_wide(BinScratch &sc, uint64_t want, int parts, uint64_t tiles) {
+  if (sc.cap < want) {
     size_t free_bytes = 0, all = 0;
-    if (cudaMemGetInfo(&free_bytes, &all) != cudaSuccess ||
-        (want + ev2_capacity(want)) * sizeof(uint64_t) + kBinMetaBytes > free_bytes / 2 ||
-        ensure_events(h->bin, want) != DBG_OK) {
+    const uint64_t need = (want + ev2_capacity(want)) * sizeof(uint64_t) + kBinMetaBytes;
+    if (cudaMemGetInfo(&free_bytes, &all) != cudaSuccess || need > all / 4 ||
+        need > (free_bytes + scratch_bytes_of(sc)) / 2) {
       cudaGetLastError();
       return false;
     }
   }
-  return ensure_tile_scratch(h->bin, parts, tiles, capturing);
+  if ((sc.cap >= want || ensure_events(sc, want) == DBG_OK) &&
+      ensure_tile_scratch(sc, parts, tiles, false))
+    return true;
+  cudaGetLastError();
+  if (cudaDeviceSynchronize() == cudaSuccess) free_bin_scratch(sc);
+  return false;
 }
 
-int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int call) {
-  BinScratch &sc = h->bin;
-  const int shift = wide_shift(h), parts = regions_of(h->n_slots, shift);
+int wide_chain(dbg_handle h, const ItemDesc &it, BinScratch &sc, uint64_t want, int shift, int parts,
+               uint64_t tiles, cudaStream_t s, int call) {
   const int tpr = 1 << (shift - kTileLog2), sms = std::max(1, h->sm_count);
-  const uint64_t tiles = table_tiles(h->n_slots, shift);
   const bool overlap = tiles <= kOverlapTiles;
-  const uint64_t cap = sc.cap / 2, cap2 = ev2_capacity(sc.cap) / 2;  // events
+  const uint64_t cap = want / 2, cap2 = ev2_capacity(want) / 2;  // events
   const Marks mark{h, call};
   const MetaView mv = meta_view(sc);
   const TileAux aux = tile_aux(sc, parts, tiles);
   WideEvent *ev = reinterpret_cast<WideEvent *>(sc.ev);
   WideEvent *ev2 = reinterpret_cast<WideEvent *>(sc.ev2);
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  DBG_CK(cudaStreamIsCapturing(s, &capture));
-  const bool capturing = capture != cudaStreamCaptureStatusNone;
-  if (!capturing) DBG_CK(cudaStreamWaitEvent(s, sc.done, 0));
   ItemPack<1> pk{};
   pk.n_items = 1;
   pk.d[0] = it;
   pk.d[0].region0 = 0;
-  sc.counters = aux.overflow;
   DBG_CK(cudaMemsetAsync(mv.ctr, 0, kBinClearedBytes, s));
   mark(1, s);
   const int gx = (int)std::max<uint64_t>((uint64_t)sms * 4,
@@ -593,7 +613,50 @@ int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int cal
   mark(7, s);
   DBG_TRY(launch_insert_wide(it, h->sm_count, s, mv.flag));
   mark(8, s);
-  h->built_counts = true;  // (unless it fell back: see small_counted)
-  if (!capturing) DBG_CK(cudaEventRecord(sc.done, s));
-  return DBG_OK;
+  return launch_next(overlap, k_wide_told, 1, 32, 0, s, it.status, mv.flag, aux);
+}
+
+}  // namespace
+
+int launch_binned_wide(dbg_handle h, const ItemDesc &it, cudaStream_t s, int call, bool *done) {
+  *done = false;
+  const int shift = wide_shift(h), parts = regions_of(h->n_slots, shift);
+  const uint64_t want = wide_units_wanted(h), tiles = table_tiles(h->n_slots, shift);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  DBG_CK(cudaStreamIsCapturing(s, &capture));
+  if (capture != cudaStreamCaptureStatusNone ||
+      (1 << (shift - kTileLog2)) > kMaxBinsPerThread * kWideBlock ||
+      want / 2 >= kMaxChainEvents ||  // (bucket positions are 32-bit)
+      h->device >= kMaxDevices)
+    return DBG_OK;
+  WideScratch &w = g_wide[h->device];
+  std::lock_guard<std::mutex> lock(w.mu);
+  t_in_wide = true;
+  int st = DBG_OK;
+  if (ensure_wide(w.sc, want, parts, tiles)) {
+    *done = true;
+    cudaError_t e = cudaStreamWaitEvent(s, w.sc.done, 0);
+    if (e == cudaSuccess) st = wide_chain(h, it, w.sc, want, shift, parts, tiles, s, call);
+    if (e == cudaSuccess) e = cudaEventRecord(w.sc.done, s);  // (after an error, too)
+    if (st == DBG_OK && e != cudaSuccess) st = cuda_fail(e, "wide scratch");
+    h->built_counts = st == DBG_OK;  // (unless it fell back: see small_counted)
+  }
+  t_in_wide = false;
+  return st;
+}
+
+uint64_t wide_scratch_bytes(int dev) {
+  if (dev < 0 || dev >= kMaxDevices) return 0;
+  std::lock_guard<std::mutex> lock(g_wide[dev].mu);
+  return scratch_bytes_of(g_wide[dev].sc);
+}
+
+uint64_t release_wide_scratch(int dev) {
+  if (dev < 0 || dev >= kMaxDevices || t_in_wide) return 0;
+  std::lock_guard<std::mutex> lock(g_wide[dev].mu);
+  BinScratch &sc = g_wide[dev].sc;
+  const uint64_t held = scratch_bytes_of(sc);
+  if (held == 0 || cudaDeviceSynchronize() != cudaSuccess) return 0;
+  free_bin_scratch(sc);
+  return held;
 }

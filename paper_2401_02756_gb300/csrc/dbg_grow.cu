@@ -61,7 +61,7 @@ int launch_grow(dbg_handle h, uint64_t new_capacity, cudaStream_t s) {
   if (new_capacity > (~0ull / sizeof(Slot))) return DBG_ERR_INVALID_ARG;
 
   Slot *nt = nullptr;
-  cudaError_t e = cudaMalloc(&nt, new_capacity * sizeof(Slot));
+  cudaError_t e = device_malloc(reinterpret_cast<void **>(&nt), new_capacity * sizeof(Slot));
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(grown table)");
   int st = launch_table_init(nt, new_capacity, s);
   // a failure flag of its own, so a too-small new table leaves the graph as it was

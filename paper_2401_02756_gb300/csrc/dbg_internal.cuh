@@ -226,9 +226,15 @@ __device__ __forceinline__ void after_previous() {
 // on the tiled binned path whose vertex and edge counts at 40 and 48 are then
 // exact, and cleared by every kernel that changes the graph without counting
 // (so it holds for replayed calls too, which the host does not see); the stats
-// accumulators (2 x u64) at 16; the spill count (u64) at 32.  Kernels reach
-// the flag and the counts from an item's status pointer.
-constexpr size_t kSmallCounted = 4, kSmallAcc = 16, kSmallSpill = 32, kSmallBuilt = 40;
+// accumulators (2 x u64) at 16; the spill count (u64) at 32; and of a wide
+// rebuild that was binned the overflow count (u64) at 8 and the deferred count
+// plus one at 56.  Kernels reach the flag and the counts from an item's status
+// pointer.
+constexpr size_t kSmallCounted = 4, kSmallOverflow = 8, kSmallAcc = 16, kSmallSpill = 32,
+                 kSmallBuilt = 40, kSmallDeferred = 56;
+__host__ __device__ inline unsigned long long *small_word(uint32_t *status, size_t at) {
+  return reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(status) + at);
+}
 __host__ __device__ inline uint32_t *small_counted(uint32_t *status) {
   return reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(status) + kSmallCounted);
 }
@@ -312,6 +318,11 @@ void timer_mark(dbg_handle h, int call, int m, cudaStream_t s);
 
 // Error plumbing shared by the entry points (host side).
 int cuda_fail(cudaError_t e, const char *what);
+// cudaMalloc, with the wide rebuilds' scratch given back when there is no memory.
+cudaError_t device_malloc(void **p, size_t bytes);
+// Give back that scratch on device `dev`, the current one (nothing while this
+// thread uses it); returns its bytes.
+uint64_t release_wide_scratch(int dev);
 // Temporary device memory from the library's stream-ordered pool (free it
 // with cudaFreeAsync on a stream).
 int scratch_alloc(void **p, size_t bytes, cudaStream_t s);

@@ -35,6 +35,16 @@ std::mutex g_pool_mu;
 cudaMemPool_t g_pools[64] = {};
 }  // namespace
 
+cudaError_t device_malloc(void **p, size_t bytes) {
+  const cudaError_t e = cudaMalloc(p, bytes);
+  int dev = 0;
+  if (e != cudaErrorMemoryAllocation || cudaGetDevice(&dev) != cudaSuccess ||
+      release_wide_scratch(dev) == 0)
+    return e;
+  cudaGetLastError();
+  return cudaMalloc(p, bytes);
+}
+
 int scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
   int dev = 0;
   DBG_CK(cudaGetDevice(&dev));
@@ -53,7 +63,12 @@ int scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
     }
     pool = g_pools[dev];
   }
-  DBG_CK(cudaMallocFromPoolAsync(p, bytes, pool, s));
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  if (e == cudaErrorMemoryAllocation && release_wide_scratch(dev) > 0) {
+    cudaGetLastError();
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "cudaMallocFromPoolAsync");
   return DBG_OK;
 }
 
@@ -369,7 +384,8 @@ extern "C" int dbg_create_ex(int k, uint64_t capacity, uint32_t max_probes, dbg_
     st = device_of(h);
     if (st != DBG_OK) break;
     dbg::make_report_page();
-    cudaError_t e = cudaMalloc(&h->table, capacity * sizeof(dbg::Slot));
+    cudaError_t e = dbg::device_malloc(reinterpret_cast<void **>(&h->table),
+                                       capacity * sizeof(dbg::Slot));
     if (e != cudaSuccess) { h->table = nullptr; st = dbg::cuda_fail(e, "cudaMalloc(table)"); break; }
     void *small = nullptr;
     e = cudaMalloc(&small, kSmallBytes);
@@ -500,7 +516,7 @@ extern "C" int dbg_get_info(dbg_handle h, dbg_info *out) {
   out->table_bytes = h->n_slots * sizeof(dbg::Slot);
   out->max_probes = h->max_probes;
   out->device = h->device;
-  out->event_capacity = h->bin.cap ? h->bin.cap / (h->k > 32 ? 2 : 1) : h->bin_want;
+  out->event_capacity = h->bin.cap ? h->bin.cap : h->bin_want;
   out->spill_capacity = h->spill_cap;
   return DBG_OK;
 }
@@ -519,7 +535,7 @@ extern "C" int dbg_set_spill(dbg_handle h, uint64_t records) {
   h->spill_cap = 0;
   if (records == 0) return DBG_OK;
   void *p = nullptr;
-  cudaError_t e = cudaMalloc(&p, records * sizeof(dbg::SpillRecord));
+  cudaError_t e = dbg::device_malloc(&p, records * sizeof(dbg::SpillRecord));
   if (e != cudaSuccess) return dbg::cuda_fail(e, "cudaMalloc(spill)");
   h->d_spill = static_cast<dbg::SpillRecord *>(p);
   h->spill_cap = records;
@@ -635,9 +651,11 @@ int insert_one(dbg_handle h, const dbg::ItemDesc &it, cudaStream_t s, bool fresh
                const dbg::InputParts *input = nullptr) {
   h->built_counts = false;  // (set again by a rebuild on the tiled binned path)
   const int call = dbg::timer_begin_call(h);
-  if (h->k > 32 && fresh && want_binned(h) && dbg::wide_scratch_ready(h, s)) {
+  if (h->k > 32 && fresh && want_binned(h)) {
     DBG_TRY(dbg::wait_input(input, s));
-    return dbg::launch_binned_wide(h, it, s, call);
+    bool done = false;
+    const int st = dbg::launch_binned_wide(h, it, s, call, &done);
+    if (done || st != DBG_OK) return st;
   }
   const bool binned = h->k <= 32 && want_binned(h) &&
                       (h->bin.cap == dbg::bin_events_wanted(h) ||
@@ -712,7 +730,7 @@ int grow_stage(dbg_handle h, uint64_t bytes, uint64_t reads) {
     }
     h->stage_packed_bytes = 0;
     for (int i = 0; i < 2; ++i) {
-      cudaError_t e = cudaMalloc(&h->stage_packed[i], bytes);
+      cudaError_t e = dbg::device_malloc(reinterpret_cast<void **>(&h->stage_packed[i]), bytes);
       if (e != cudaSuccess) return dbg::cuda_fail(e, "cudaMalloc(staging)");
     }
     h->stage_packed_bytes = bytes;
@@ -725,7 +743,8 @@ int grow_stage(dbg_handle h, uint64_t bytes, uint64_t reads) {
     }
     h->stage_offsets_count = 0;
     for (int i = 0; i < 2; ++i) {
-      cudaError_t e = cudaMalloc(&h->stage_offsets[i], (reads + 1) * sizeof(uint64_t));
+      cudaError_t e = dbg::device_malloc(reinterpret_cast<void **>(&h->stage_offsets[i]),
+                                         (reads + 1) * sizeof(uint64_t));
       if (e != cudaSuccess) return dbg::cuda_fail(e, "cudaMalloc(staging)");
     }
     h->stage_offsets_count = reads + 1;
@@ -963,7 +982,8 @@ extern "C" int dbg_build_batch(const dbg_batch_item *items, int n_items, void *s
 extern "C" uint64_t dbg_scratch_bytes(void) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  return dbg::batch_scratch_bytes(dev) + dbg::pool_reserved_bytes(dev);
+  return dbg::batch_scratch_bytes(dev) + dbg::wide_scratch_bytes(dev) +
+         dbg::pool_reserved_bytes(dev);
 }
 
 extern "C" int dbg_release_scratch(void) {
