@@ -45,6 +45,7 @@ struct SketchVisitor {
   // rho counts zeros in: a key for which they are above `lim` has rho <= floor
   // (a floor of 0 drops nothing; from 22 on, any set bit among them does).
   uint32_t lim = kLead;
+  bool first = true;  // before the item's first tile
   static constexpr uint32_t kLead = (1u << 22) - 1u;
   __device__ void set_floor() {  // (the calling warp's; the minimum of all registers)
     uint32_t m = ~0u;
@@ -53,24 +54,35 @@ struct SketchVisitor {
     m = __reduce_min_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0) *s_floor = m;
   }
-  // A read set's first tile: what its other CTAs know already.
-  __device__ void item_begin(uint32_t *g) {
+  // A read set's first tile: what its other CTAs know already.  (A CTA of the
+  // first wave starts with the others: they know nothing yet, and asking would
+  // be 2 us of a small read set's 34.)
+  __device__ void item_begin(uint32_t *g, bool first_wave) {
     g_reg = g;
-    for (int j = threadIdx.x; j < kSketchRegs; j += blockDim.x) s_reg[j] = ld_volatile_u32(g + j);
+    first = true;
+    for (int j = threadIdx.x; j < kSketchRegs; j += blockDim.x)
+      s_reg[j] = first_wave ? 0u : ld_volatile_u32(g + j);
+    if (threadIdx.x == 0) *s_floor = 0u;
     __syncthreads();
+    if (first_wave) return;
     if (threadIdx.x < 32) set_floor();
     __syncthreads();
   }
-  // Its last tile: what this CTA knows.
-  __device__ void item_end() {
+  // Its last tile: what this CTA knows.  (ask: others have merged theirs by now,
+  // and most registers need no atomic)
+  __device__ void item_end(bool ask) {
     __syncthreads();
     for (int j = threadIdx.x; j < kSketchRegs; j += blockDim.x)
-      if (s_reg[j] > ld_volatile_u32(g_reg + j)) atomicMax(&g_reg[j], s_reg[j]);
+      if (s_reg[j] > (ask ? ld_volatile_u32(g_reg + j) : 0u)) atomicMax(&g_reg[j], s_reg[j]);
     __syncthreads();
   }
   __device__ void tile_begin() {
     const uint32_t f = *s_floor;
     lim = f < 22u ? kLead >> f : 0u;
+    if (first) {  // (the registers are as item_begin left them)
+      first = false;
+      return;
+    }
     for (int j = threadIdx.x; j < kSketchRegs; j += blockDim.x) {
       const uint32_t own = s_reg[j], all = ld_volatile_u32(g_reg + j);
       if (own > all)
@@ -84,16 +96,14 @@ struct SketchVisitor {
   __device__ void round_end() {}
   __device__ void vertex(bool valid, uint64_t key, bool, uint32_t, int, int, const VertexCtx &) {
     if (!valid) return;
-    // fmix64(key ^ salt) up to its second product, whose high word is the
-    // hash's (the last shift by 33 leaves it alone): the low word is only
-    // needed for the few keys that the test lets through
-    uint64_t x = key ^ kSketchSalt;
-    x = (x ^ (x >> 33)) * 0xff51afd7ed558ccdull;
-    x ^= x >> 33;
-    const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
-    const uint32_t h_hi = __umulhi(lo, 0x1a85ec53u) + lo * 0xc4ceb9feu + hi * 0x1a85ec53u;
-    if ((h_hi & kLead) > lim) return;  // 1 + clz(rest) <= floor: no register can rise
-    uint64_t h = x * 0xc4ceb9fe1a85ec53ull;
+    // fmix64(key ^ salt) up to its last shift, which leaves the hash's high word
+    // alone.  (The product's high word by itself first, the whole for the few keys
+    // that pass, is more instructions: 64 samples 1.29 -> 1.25 ms, two tiles of
+    // 10 kb reads, of which most keys pass, 1.36 -> 1.26.)
+    uint64_t h = key ^ kSketchSalt;
+    h = (h ^ (h >> 33)) * 0xff51afd7ed558ccdull;
+    h = (h ^ (h >> 33)) * 0xc4ceb9fe1a85ec53ull;
+    if (((uint32_t)(h >> 32) & kLead) > lim) return;  // 1 + clz(rest) <= floor: no register can rise
     h ^= h >> 33;
     const uint64_t rest = h << 10;
     const uint32_t idx = (uint32_t)(h >> 54);
@@ -104,16 +114,17 @@ struct SketchVisitor {
 
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, kSketchCtas)
-    k_sketch(const __grid_constant__ ItemPack<1> pk, int tile_reads, uint64_t chunk, uint32_t *regs) {
+    k_sketch(const __grid_constant__ ItemPack<1> pk, int tile_reads, uint64_t chunk,
+             uint32_t first_wave, uint32_t *regs) {
   after_previous();
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t *s_reg = reinterpret_cast<uint32_t *>(smem + tile_smem_bytes(tile_reads));
   __shared__ uint32_t s_floor;
   SketchVisitor vis{s_reg, nullptr, &s_floor};
-  vis.item_begin(regs);
+  vis.item_begin(regs, blockIdx.x < first_wave);
   for_each_vertex<BLOCK, 1, kSketchRun>(pk, tile_reads, smem, vis, blockIdx.x * chunk,
                                         (blockIdx.x + 1) * chunk, 1);
-  vis.item_end();
+  vis.item_end(gridDim.x > first_wave);
 }
 
 // Many read sets per launch.  Each CTA takes a contiguous range of tiles, so
@@ -123,7 +134,7 @@ __global__ void __launch_bounds__(BLOCK, kSketchCtas)
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, kSketchCtas)
     k_sketch_batch(const __grid_constant__ ItemPack<kSketchItems> pk, int tile_reads,
-                   uint64_t chunk) {
+                   uint64_t chunk, uint32_t first_wave) {
   after_previous();
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t *s_reg = reinterpret_cast<uint32_t *>(smem + tile_smem_bytes(tile_reads));
@@ -134,9 +145,9 @@ __global__ void __launch_bounds__(BLOCK, kSketchCtas)
     const int it = find_item(pk, t);
     const uint64_t end = it + 1 < pk.n_items ? pk.d[it + 1].tile_begin : pk.total_tiles;
     const uint64_t tb = min(t1, end);
-    vis.item_begin(reinterpret_cast<uint32_t *>(pk.d[it].table));
+    vis.item_begin(reinterpret_cast<uint32_t *>(pk.d[it].table), blockIdx.x < first_wave);
     for_each_vertex<BLOCK, kSketchItems, kSketchRun>(pk, tile_reads, smem, vis, t, tb, 1);
-    vis.item_end();
+    vis.item_end(gridDim.x > first_wave);
     t = tb;
   }
 }
@@ -146,6 +157,7 @@ __global__ void __launch_bounds__(BLOCK, kSketchCtas)
 // 30 % of the warps' time unused; 64 samples 1.47 ms at one, 1.40 at two, 1.41
 // at four, 1.56 at eight).
 constexpr uint64_t kSketchWaves = 2;
+constexpr uint64_t kSketchMinReads = 8;  // reads a tile (dbg_sketch_reads)
 
 uint64_t sketch_chunk(uint64_t tiles, uint64_t resident) {
   return std::max<uint64_t>(1, (tiles + kSketchWaves * resident - 1) / (kSketchWaves * resident));
@@ -171,7 +183,16 @@ extern "C" int dbg_sketch_reads(int k, const uint8_t *packed, const uint64_t *of
   DBG_CK(cudaMemsetAsync(registers, 0, (kSketchRegs + 1) * sizeof(uint32_t), s));
   if (n_reads == 0) return DBG_OK;
   constexpr int B = 256;
-  const int tile_reads = B;
+  int dev = 0, sms = 0, per_sm = 0;
+  DBG_CK(cudaGetDevice(&dev));
+  DBG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &per_sm, k_sketch<B>, B, tile_smem_bytes(B) + kSketchRegs * sizeof(uint32_t)));
+  const uint32_t resident = (uint32_t)(std::max(1, per_sm) * sms);
+  // (a read set of few tiles is cut into one for every fourth resident CTA, as each
+  // merges 1,024 registers: 500 reads of 10 kb ran on two CTAs, 1.33 -> 0.07 ms)
+  const int tile_reads = (int)std::min<uint64_t>(
+      B, std::max<uint64_t>(kSketchMinReads, (4 * n_reads + resident - 1) / resident));
   ItemPack<1> pk{};
   pk.n_items = 1;
   pk.total_tiles = (n_reads + tile_reads - 1) / tile_reads;
@@ -187,13 +208,9 @@ extern "C" int dbg_sketch_reads(int k, const uint8_t *packed, const uint64_t *of
   it.k = k;
   it.vec_ok = ((uintptr_t)packed & 15u) == 0 ? 1 : 0;
   const size_t smem = tile_smem_bytes(tile_reads) + kSketchRegs * sizeof(uint32_t);
-  int dev = 0, sms = 0, per_sm = 0;
-  DBG_CK(cudaGetDevice(&dev));
-  DBG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sketch<B>, B, smem));
-  const uint64_t chunk = sketch_chunk(pk.total_tiles, (uint64_t)std::max(1, per_sm) * sms);
+  const uint64_t chunk = sketch_chunk(pk.total_tiles, resident);
   const int grid = (int)((pk.total_tiles + chunk - 1) / chunk);
-  DBG_TRY(launch_after(k_sketch<B>, grid, B, smem, s, pk, tile_reads, chunk, registers));
+  DBG_TRY(launch_after(k_sketch<B>, grid, B, smem, s, pk, tile_reads, chunk, resident, registers));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
@@ -241,9 +258,10 @@ extern "C" int dbg_sketch_batch(const dbg_sketch_item *items, int n_items, void 
     DBG_TRY(launch_after(k_zero_registers, cnt, 256, 0, s, pk));
     DBG_CK(cudaGetLastError());
     if (tiles == 0) continue;
-    const uint64_t chunk = sketch_chunk(tiles, (uint64_t)std::max(1, per_sm) * sms);
+    const uint32_t resident = (uint32_t)(std::max(1, per_sm) * sms);
+    const uint64_t chunk = sketch_chunk(tiles, resident);
     const int grid = (int)((tiles + chunk - 1) / chunk);
-    DBG_TRY(launch_after(k_sketch_batch<B>, grid, B, smem, s, pk, tile_reads, chunk));
+    DBG_TRY(launch_after(k_sketch_batch<B>, grid, B, smem, s, pk, tile_reads, chunk, resident));
     DBG_CK(cudaGetLastError());
   }
   return DBG_OK;
