@@ -196,8 +196,9 @@ int launch_insert_wide(const ItemDesc &it, int sm_count, cudaStream_t s, const u
   const uint64_t resident = (uint64_t)std::max(1, per_sm) * std::max(1, sm_count);
   const int tile_reads = std::min(kWideTile, auto_tile_reads(it.n_reads, resident));
   const uint64_t tiles = (it.n_reads + tile_reads - 1) / tile_reads;
-  DBG_TRY(launch_after(k_insert_wide<B>, (int)std::min(tiles, resident), B, 0, s, it, tile_reads,
-                       gate));
+  // (plainly behind a binned chain, see the one-word insert's launch)
+  DBG_TRY(launch_next(gate == nullptr, k_insert_wide<B>, (int)std::min(tiles, resident), B, 0, s,
+                      it, tile_reads, gate));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
