@@ -1575,7 +1575,7 @@ __global__ void k_tile_deferred(const __grid_constant__ ItemPack<N> pk,
 // its sticky status and spill count.
 template <int N>
 __global__ void k_tables_init(const __grid_constant__ ItemPack<N> pk) {
-  after_previous();
+  wait_previous();
   const int i = blockIdx.y;
   if (i >= pk.n_items) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1584,6 +1584,7 @@ __global__ void k_tables_init(const __grid_constant__ ItemPack<N> pk) {
     *pk.d[i].spill_count = 0ull;
   }
   empty_table(pk.d[i], blockIdx.x, gridDim.x);
+  let_next();
 }
 
 int ceil_log2(uint64_t x) {

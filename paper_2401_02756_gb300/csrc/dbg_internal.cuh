@@ -216,10 +216,21 @@ __device__ __forceinline__ bool find_or_claim(Slot *table, uint64_t n_slots, uin
 // are not __restrict__: for a const one that promises that nobody writes what
 // it points to while the kernel runs, this wait included, and the loads need
 // not stay behind it.
-__device__ __forceinline__ void after_previous() {
+__device__ __forceinline__ void let_next() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+__device__ __forceinline__ void after_previous() {
+  let_next();
+  wait_previous();
+}
+// (A kernel that fills the device and has an insert behind it waits at its start
+// and calls let_next at its end instead: CTAs that take their places as it ends,
+// one SM after another, fill the first SMs that are free and stay there -- 402
+// reads of 10 kb, k = 51, on 201 CTAs: 0.69 ms behind the emptying of the table,
+// 0.40 alone.)
 
 // Every graph's small block of device memory (64 bytes beside its table):
 // the sticky status (u32) at byte 0; a flag at 4 set by a rebuild from empty

@@ -187,7 +187,7 @@ struct DeviceGuard {
 // (status, spilled: if not null, cleared too)
 __global__ void k_table_init(uint4 *t, uint64_t n_vec, uint32_t *status,
                              unsigned long long *spilled) {
-  after_previous();
+  wait_previous();
   if (status != nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
     *status = 0u;
     *small_counted(status) = 0u;
@@ -198,6 +198,7 @@ __global__ void k_table_init(uint4 *t, uint64_t n_vec, uint32_t *status,
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += stride)
     t[i] = (i & 1) ? tail : head;
+  let_next();
 }
 
 // Vertices (occupied slots) and edges (sum of counters) of a table.

@@ -8,6 +8,7 @@ import glob
 import os
 import re
 
+WAITS = ("after_previous();", "wait_previous();")
 CSRC = os.path.join(os.path.dirname(__file__), "..", "paper_2401_02756_gb300", "csrc")
 
 
@@ -57,11 +58,11 @@ def test_every_overlapped_kernel_waits_first():
     kernels = _kernels()
     names = _overlapped()
     assert len(names) > 25 and names <= set(kernels)
-    late = [n for n in names if not kernels[n][1].startswith("after_previous();")]
+    late = [n for n in names if not kernels[n][1].startswith(WAITS)]
     assert not late, late
 
 
 def test_no_restrict_parameter_where_the_launch_overlaps():
     promised = [n for n, (params, body) in _kernels().items()
-                if body.startswith("after_previous();") and "__restrict__" in params]
+                if body.startswith(WAITS) and "__restrict__" in params]
     assert not promised, promised
