@@ -27,9 +27,13 @@ namespace {
 // L2): 168 M positions into a 3.5 GB table 14.7 -> 12.5 ms (1.43 probes each,
 // 241 M sector reads and as many sectors made dirty as positions), by one
 // 128-bit load a probe, a warp-scanned prefix, 16-byte staging and tiles cut
-// by the number of reads.
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 6) k_insert_wide(ItemDesc it, int tile_reads, const uint32_t *gate) {
+// by the number of reads.  (CTAS: per SM.  A table that the L2 holds is bound by
+// the probes' latency: 32 registers for 64 warps an SM, 4 M positions of 75-base
+// reads into 80 MB 128 us at 40 registers -> 117, 4 M of 1 kb reads 158 -> 145; the
+// 3.5 GB table is better off with 40, 12.5 ms against 12.9.)
+template <int BLOCK, int CTAS>
+__global__ void __launch_bounds__(BLOCK, CTAS)
+    k_insert_wide(ItemDesc it, int tile_reads, const uint32_t *gate) {
   after_previous();
   if (gate != nullptr && ld_volatile_u32(gate) != 0u) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) *small_counted(it.status) = 0u;  // (it grows, uncounted)
@@ -191,14 +195,17 @@ size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 int launch_insert_wide(const ItemDesc &it, int sm_count, cudaStream_t s, const uint32_t *gate) {
   if (it.n_reads == 0) return DBG_OK;
   constexpr int B = 256;
+  constexpr uint64_t kL2Bytes = 128ull << 20;
+  const auto kern = it.n_slots * sizeof(WideSlot) <= kL2Bytes ? k_insert_wide<B, 8>
+                                                              : k_insert_wide<B, 6>;
   int per_sm = 0;
-  DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_insert_wide<B>, B, 0));
+  DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, B, 0));
   const uint64_t resident = (uint64_t)std::max(1, per_sm) * std::max(1, sm_count);
   const int tile_reads = std::min(kWideTile, auto_tile_reads(it.n_reads, resident));
   const uint64_t tiles = (it.n_reads + tile_reads - 1) / tile_reads;
   // (plainly behind a binned chain, see the one-word insert's launch)
-  DBG_TRY(launch_next(gate == nullptr, k_insert_wide<B>, (int)std::min(tiles, resident), B, 0, s,
-                      it, tile_reads, gate));
+  DBG_TRY(launch_next(gate == nullptr, kern, (int)std::min(tiles, resident), B, 0, s, it,
+                      tile_reads, gate));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }

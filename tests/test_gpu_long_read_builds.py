@@ -20,14 +20,18 @@ def _lib():
     dbg.load()
 
 
-def sampled(genome, n, length, seed):
+def sampled(genome, n, length, seed, err=0.0):
     """(packed, offsets) of n reads of a genome, made on the GPU."""
     import torch
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed)
     text = torch.randint(0, 4, (genome,), dtype=torch.uint8, device="cuda", generator=gen)
     starts = torch.randint(0, genome - length + 1, (n, 1), device="cuda", generator=gen)
-    reads = text[starts + torch.arange(length, device="cuda")].view(-1, 4)
+    reads = text[starts + torch.arange(length, device="cuda")].view(-1)
+    if err:
+        wrong = torch.rand(reads.numel(), device="cuda", generator=gen) < err
+        reads = (reads + wrong.to(torch.uint8)) & 3
+    reads = reads.view(-1, 4)
     packed = reads[:, 0] | (reads[:, 1] << 2) | (reads[:, 2] << 4) | (reads[:, 3] << 6)
     return packed, torch.arange(n + 1, device="cuda") * length
 
@@ -60,7 +64,7 @@ def test_few_long_reads(k):
 
 def test_a_rebuild_of_more_events_than_its_scratch_holds():
     # given to the direct insert after the binned chain's kernels
-    dev = sampled(2_000_000, 65_000, 5000, 9)
+    dev = sampled(2_000_000, 65_000, 5000, 9, err=0.0005)
     g = dbg.Graph(31, 4_000_000)
     g.reserve_events(17_000_000)
     rebuild = seconds(lambda: g.build(*dev))
