@@ -82,15 +82,44 @@ struct InsertVisitor {
   }
 };
 
+// Reads per tile when the tuning leaves it open.  A tile is a CTA's unit of
+// work, and a thread holds one position in flight, so a read set of few tiles
+// leaves the chip idle: 1,000 reads in tiles of 256 ran on 4 CTAs (276 us;
+// now 17).  The reads are cut into whole waves of the resident CTAs with at
+// most kAutoTileReads reads a tile (20,000 reads on 1,216 CTAs: 94 us as one
+// wave of 17, 109 as a wave of 16 and its rest), and at least kMinTileReads:
+// a tile of one read would leave most of a CTA's threads idle.  That suits reads
+// of 100 bases and more.  Tiles of 20 shorter ones hold too few positions for a
+// CTA's threads and barriers, and only the device knows: a large read set's tiles
+// take up to kShortTileReads of them, for kTilePositions positions (571,000 reads
+// of 36 bases, k = 31: 174 us with tiles of 20, 112 with 109; 182,000 of 50: 110 ->
+// 102).  Many read sets in one launch take up to kAutoTileReadsMany (128 sets of 36-base
+// reads 0.67 ms with 20, 0.50 with 48 as with 256; of 150 bases 0.57 and 0.56).
+constexpr int kMinTileReads = 2, kAutoTileReads = 20, kAutoTileReadsMany = 48;
+constexpr int kShortTileReads = 128;
+constexpr uint64_t kTilePositions = 768;
+constexpr uint64_t kAdaptReads = 12;  // reads per resident CTA from which the device is asked
+
+__device__ __forceinline__ int short_tile_reads(const ItemDesc &it, int tile_reads) {
+  const uint64_t bases = it.offsets[it.n_reads] - it.offsets[0];  // (decreasing: any size will do)
+  const uint64_t length = bases / it.n_reads;
+  const uint64_t positions = length + 2 > (uint64_t)it.k ? length + 2 - (uint64_t)it.k : 1ull;
+  const uint64_t reads = kTilePositions / positions;
+  return max(tile_reads, (int)min(reads, (uint64_t)kShortTileReads));
+}
+
 // Bound by the latency of dependent L2 round trips: a warp waits for its
 // longest probe chain (about four loads and a CAS over its 32 positions), so
 // the kernel is held to 32 registers for 64 warps an SM (a few words spill):
 // 9.2 M positions into a 56 MB table 270 us at 48 registers -> 231 us.  A run
 // of four positions per thread with their probes in flight together took
 // 335 us: twice the instructions, at 13 active lanes instead of 19.
+// (adapt, one read set: a tile may take up to kShortTileReads reads, when they are
+// short -- see short_tile_reads)
 template <int BLOCK, bool AGG, int N>
 __global__ void __launch_bounds__(BLOCK, 2048 / BLOCK)
-    k_insert(const __grid_constant__ ItemPack<N> pk, int tile_reads, const uint32_t *gate) {
+    k_insert(const __grid_constant__ ItemPack<N> pk, int tile_reads, bool adapt,
+             const uint32_t *gate) {
   after_previous();
   if (gate != nullptr && ld_volatile_u32(gate) != 0u) return;
   if (blockIdx.x == 0)  // (the graphs grow, uncounted)
@@ -98,18 +127,13 @@ __global__ void __launch_bounds__(BLOCK, 2048 / BLOCK)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ volatile uint32_t s_cap_hit;
   InsertVisitor<AGG> vis{&s_cap_hit};
-  for_each_vertex<BLOCK, N, 1>(pk, tile_reads, smem_raw, vis, blockIdx.x, pk.total_tiles,
-                               gridDim.x);
+  uint64_t tiles = pk.total_tiles;
+  if (N == 1 && adapt) {
+    tile_reads = short_tile_reads(pk.d[0], tile_reads);
+    tiles = (pk.d[0].n_reads + (uint64_t)tile_reads - 1) / (uint64_t)tile_reads;
+  }
+  for_each_vertex<BLOCK, N, 1>(pk, tile_reads, smem_raw, vis, blockIdx.x, tiles, gridDim.x);
 }
-
-// Reads per tile when the tuning leaves it open.  A tile is a CTA's unit of
-// work, and a thread holds one position in flight, so a read set of few tiles
-// leaves the chip idle: 1,000 reads in tiles of 256 ran on 4 CTAs (276 us;
-// now 17).  The reads are cut into whole waves of the resident CTAs with at
-// most kAutoTileReads reads a tile (20,000 reads on 1,216 CTAs: 94 us as one
-// wave of 17, 109 as a wave of 16 and its rest), and at least kMinTileReads:
-// a tile of one read would leave most of a CTA's threads idle.
-constexpr int kMinTileReads = 2, kAutoTileReads = 20;
 
 // Number the items' tiles and launch.
 template <int BLOCK, bool AGG, int N>
@@ -117,16 +141,19 @@ int launch_one(ItemPack<N> &pk, int tile_reads, int grid_ctas, int sm_count, cud
                const uint32_t *gate) {
   auto kern = k_insert<BLOCK, AGG, N>;
   int per_sm = 0;
-  size_t smem = tile_smem_bytes(tile_reads > 0 ? tile_reads : kAutoTileReads);
+  size_t smem = tile_smem_bytes(tile_reads > 0 ? tile_reads : kShortTileReads);
   if (smem > 48 * 1024)
     DBG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BLOCK, smem));
   const int resident = std::max(1, per_sm) * std::max(1, sm_count);
+  bool adapt = false;
   if (tile_reads <= 0) {
     uint64_t reads = 0;
     for (int i = 0; i < pk.n_items; ++i) reads += pk.d[i].n_reads;
-    tile_reads = auto_tile_reads(reads, (uint64_t)resident);
-    smem = tile_smem_bytes(tile_reads);
+    tile_reads = auto_tile_reads(reads, (uint64_t)resident,
+                                 N == 1 ? kAutoTileReads : kAutoTileReadsMany);
+    adapt = N == 1 && reads > kAdaptReads * (uint64_t)resident;
+    if (!adapt) smem = tile_smem_bytes(tile_reads);
   }
   pk.total_tiles = 0;
   for (int i = 0; i < pk.n_items; ++i) {
@@ -136,10 +163,12 @@ int launch_one(ItemPack<N> &pk, int tile_reads, int grid_ctas, int sm_count, cud
   if (pk.total_tiles == 0) return DBG_OK;
   int grid = grid_ctas > 0 ? grid_ctas : resident;
   if ((uint64_t)grid > pk.total_tiles) grid = (int)pk.total_tiles;
-  // (a gated insert plainly: its CTAs stay on their SMs to the end, and those that
-  // are placed while the binned chain's last kernel still runs get that kernel's
-  // shared memory, too little for as many as fit: 323 M events 19.8 ms, not 13.0)
-  DBG_TRY(launch_next(gate == nullptr, kern, grid, BLOCK, smem, stream, pk, tile_reads, gate));
+  // (a gated insert plainly: its CTAs stay on their SMs to the end, so they are not
+  // to be placed while the binned chain's last kernel still runs.  323 M events of
+  // 65,000 reads 5.7 ms, 5.7 to 6.5 launched over it; into a table that fills up on
+  // the way 14.1 against 19.8)
+  DBG_TRY(launch_next(gate == nullptr, kern, grid, BLOCK, smem, stream, pk, tile_reads, adapt,
+                      gate));
   DBG_CK(cudaGetLastError());
   return DBG_OK;
 }
@@ -165,9 +194,9 @@ int launch_pack(const ItemDesc *items, int n_items, int tile_reads, const dbg_tu
 
 }  // namespace
 
-int auto_tile_reads(uint64_t reads, uint64_t resident) {
-  const uint64_t waves = std::max<uint64_t>(1, (reads + resident * kAutoTileReads - 1) /
-                                                   (resident * kAutoTileReads));
+int auto_tile_reads(uint64_t reads, uint64_t resident, int most) {
+  if (most <= 0) most = kAutoTileReads;
+  const uint64_t waves = std::max<uint64_t>(1, (reads + resident * most - 1) / (resident * most));
   const uint64_t ctas = resident * waves;
   return (int)std::max<uint64_t>(kMinTileReads, (reads + ctas - 1) / ctas);
 }

@@ -444,8 +444,8 @@ int launch_insert(const ItemDesc *items, int n_items, const dbg_tuning &tuning, 
                   cudaStream_t stream, const uint32_t *gate = nullptr);
 
 // Reads per tile of a direct insert of `reads` reads by `resident` CTAs, when
-// the tuning leaves it open.
-int auto_tile_reads(uint64_t reads, uint64_t resident);
+// the tuning leaves it open (most: 0 for the usual limit).
+int auto_tile_reads(uint64_t reads, uint64_t resident, int most = 0);
 
 // Resolved tuning (defaults filled in).
 dbg_tuning resolve_tuning(const dbg_tuning &t);

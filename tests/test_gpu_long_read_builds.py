@@ -64,7 +64,7 @@ def test_few_long_reads(k):
 
 def test_a_rebuild_of_more_events_than_its_scratch_holds():
     # given to the direct insert after the binned chain's kernels
-    dev = sampled(2_000_000, 65_000, 5000, 9, err=0.0005)
+    dev = sampled(2_000_000, 65_000, 5000, 9, err=0.0001)
     g = dbg.Graph(31, 4_000_000)
     g.reserve_events(17_000_000)
     rebuild = seconds(lambda: g.build(*dev))
