@@ -238,8 +238,8 @@ int dbg_insert_reads_host(dbg_handle h, const uint8_t *packed, const uint64_t *o
  * no other call may use the handle from another stream meanwhile.  The
  * sticky status and pending spill records are cleared first.  n_reads == 0
  * only empties the table.  A rebuild (k <= 31) of a table of 16 MiB to 256 MiB
- * is binned too when about 4 million events or more are to be expected -- the
- * size dbg_reserve_events gave, else 64 a read -- with buffers that the
+ * is binned too when about 8 million events or more are to be expected -- the
+ * size dbg_reserve_events gave, else 8 a read -- with buffers that the
  * library's pool lends for the call (17 bytes per event for the reserved size,
  * else for 4.25 events per slot or 160 per read, up to 2.3 GB); inside a
  * stream capture, without that memory or with more events than it holds the

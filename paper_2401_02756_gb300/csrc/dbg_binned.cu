@@ -2124,10 +2124,13 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
 // table, and the graph may be one of many).  The direct insert is bound by its
 // requests to L2 (a probe and a counter add an event, 2.6e10 events/s); the
 // binned kernels take a third of that time an event and 0.15 ms for themselves.
-// Reads of 150 bases, direct and binned: 3.6 M events 0.18 / 0.14 ms, 8.5 M 0.34 /
-// 0.20, 24 M 0.92 / 0.45; 2.4 M are even, and below kBinPooledMinEvents the kernels'
-// own time decides.  Under 16 MiB (256 tiles for 456 CTAs of the apply) the gain
-// is a third (48 M events 2.1 / 1.4 ms), not worth a scratch 50 times the table.
+// Builds, direct and binned: 3 M events 0.09 ms each, 5 M 0.12 to 0.16 / 0.16 to
+// 0.18, 8 M 0.18 to 0.21 / 0.19 to 0.20, 16 M 0.33 to 0.38 / 0.30 to 0.31; below
+// kBinPooledMinEvents the kernels' own time decides.  Without a reserved size a
+// read counts as kBinPooledPerRead events, since short ones have no more: 571,000
+// of 36 bases, k = 31, are 4 M events, 0.12 ms direct and 0.17 binned.  Under 16 MiB
+// (256 tiles for 456 CTAs of the apply) the gain is a third (48 M events 2.1 / 1.4
+// ms), not worth a scratch 50 times the table.
 // The events the scratch has room for: what was reserved, else as for a held buffer
 // 4.25 a slot, or 160 a read (what reads of 150 bases and their buckets' margins
 // need, whatever their coverage); more than that and the direct insert does it.
@@ -2139,7 +2142,7 @@ int launch_binned_pooled(dbg_handle h, const ItemDesc &it, const dbg_tuning &tun
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   DBG_CK(cudaStreamIsCapturing(s, &capture));
   if (capture != cudaStreamCaptureStatusNone || t.apply_mode == 1) return DBG_OK;
-  if ((h->bin_want ? h->bin_want : 64 * it.n_reads) < kBinPooledMinEvents ||
+  if ((h->bin_want ? h->bin_want : kBinPooledPerRead * it.n_reads) < kBinPooledMinEvents ||
       h->bin_want > kMaxPooledEvents)
     return DBG_OK;
   const BinGeometry geo = bin_geometry(

@@ -8,7 +8,8 @@ namespace dbg {
 constexpr int kBinMaxParts = 2048;           // regions of one chain (one or many tables), at most
 constexpr uint64_t kBinMinTableBytes = 256ull << 20;  // auto mode: tables at least this big
 constexpr uint64_t kBinPooledMinTableBytes = 16ull << 20;  // auto mode, rebuilds: with scratch from
-constexpr uint64_t kBinPooledMinEvents = 4000000;          // the pool (see launch_binned_pooled)
+constexpr uint64_t kBinPooledMinEvents = 8000000;          // the pool (see launch_binned_pooled)
+constexpr uint64_t kBinPooledPerRead = 8;                  // events taken for granted, a read
 constexpr uint64_t kBinMinEvents = 16ull << 20;       // smallest event buffer
 constexpr uint64_t kBinEventsPerSlot = 4;             // default event buffer: 4.25 events per slot
                                                       // (4 + 1/4, the buckets' margin included)
