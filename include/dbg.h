@@ -68,10 +68,11 @@ typedef struct dbg_graph *dbg_handle;
  * The built graph does not depend on these values: only the speed does. */
 typedef struct dbg_tuning {
   int block_threads;  /* threads per CTA, a multiple of 32 in [64, 1024] (default 256) */
-  int tile_reads;     /* reads staged per tile, in [1, block_threads] (default: by the number of reads) */
+  int tile_reads;     /* reads staged per tile, in [1, block_threads] (default: by the number
+                         and the length of the reads) */
   int grid_ctas;      /* CTAs in the persistent grid (default: SMs x resident CTAs per SM) */
   int warp_aggregate; /* direct insert: 1 merges a warp's equal keys with __match_any_sync,
-                         0 does not, -1: default (1) */
+                         0 (a new handle's) does not, -1: as 1 */
   int insert_path;    /* 0: automatic; 1: direct; 2: binned (k <= 31, and rebuilds with
                          k from 33 to 63; see dbg_insert_reads) */
   int apply_unroll;   /* binned apply: probe slots per thread, 2, 4 or 8 (0: default 4) */
@@ -279,7 +280,7 @@ typedef struct dbg_batch_item {
  * the scatter takes (item, read tile) work units of every read set, the
  * regions of all tables share one event buffer, the split and the tiled
  * apply take every table's regions and tiles.  A chain holds up to 128
- * graphs, 2048 table regions (2^21 slots each, by default) and 3.8e9 events;
+ * graphs, 2048 table regions (2^18 to 2^21 slots each, by default) and 3.8e9 events;
  * its event buffer holds the sum of its graphs' dbg_reserve_events sizes (or
  * defaults), and if the events do not fit it, the direct insert does that
  * chain's work (decided on the device).  The chains' buffers belong to the
@@ -307,16 +308,17 @@ int dbg_build_batch(const dbg_batch_item *items, int n_items, void *stream);
 
 /* Give back the device memory the library keeps between calls: the buffers of the
  * batched inserts and of rebuilds with k > 32, and the pool of the exports and of
- * mid-size rebuilds, on every device (each is synchronised first), and the 4 KB page of pinned host memory that
- * results are reported through when no call uses it (calls copy their results
- * until the next graph is created).  Later calls allocate again as needed.
- * Errors: CUDA. */
+ * mid-size rebuilds, on every device (each is synchronised first), and the 4 KB
+ * page of pinned host memory that results are reported through when no call uses
+ * it (calls copy their results until the next graph is created).  Later calls
+ * allocate again as needed.  Errors: CUDA. */
 int dbg_release_scratch(void);
 
 /* Device bytes the library holds between calls on the current device: the
  * buffers of the batched inserts and of rebuilds with k > 32, and the pool of the
- * exports and of mid-size rebuilds (what dbg_release_scratch gives back).  A caller that keeps a device-memory
- * budget counts them; 0 when there is no device. */
+ * exports and of mid-size rebuilds (what dbg_release_scratch gives back).  A
+ * caller that keeps a device-memory budget counts them; 0 when there is no
+ * device. */
 uint64_t dbg_scratch_bytes(void);
 
 /* Grow-and-rebuild.  dbg_set_spill gives the graph a buffer of `records`
@@ -396,10 +398,10 @@ uint64_t dbg_export_scratch_bytes(int k, uint64_t n_vertices, uint64_t n_slots);
  * `scratch` is a 256-byte aligned device buffer of at least
  * dbg_export_scratch_bytes(k, n, n_slots) bytes, all owned by the caller.
  * k <= 32 and a table of at most 2^32 slots.  Same result and ordering as
- * dbg_export_sorted (the vertices are counted on the way); waits for `stream`.  Errors: INVALID_ARG (including too small or
- * misaligned scratch and host outputs), CUDA, BUFFER_TOO_SMALL (a size query
- * with max_n = 0), and the sticky status.  After an error the outputs'
- * contents are unspecified. */
+ * dbg_export_sorted (the vertices are counted on the way); waits for `stream`.
+ * Errors: INVALID_ARG (including too small or misaligned scratch and host
+ * outputs), CUDA, BUFFER_TOO_SMALL (a size query with max_n = 0), and the sticky
+ * status.  After an error the outputs' contents are unspecified. */
 int dbg_export_sorted_with(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out,
                            uint64_t max_n, uint64_t *n_out, void *scratch,
                            uint64_t scratch_bytes, void *stream);

@@ -53,8 +53,9 @@ constexpr int kTileSlots = 1 << kTileLog2;  // 2048 slots: 64 KB as 32-byte slot
 constexpr int kMaxTilesPerRegion = 4096;    // beyond this the streaming apply is used
 
 // Automatic regions of the tiled path: 2^18 to 2^21 slots, so that a table has
-// at most 256 of them (few regions: long runs in the scatter) and no larger
-// ones than that takes (few tiles per region: long runs in the split).  A
+// at most 256 of them (few regions: long runs in the scatter; more above 2^29
+// slots, where regions stay at 2^21) and no larger ones than that takes (few
+// tiles per region: long runs in the split).  A
 // build at 2^18 / 2^19 / 2^20 / 2^21 slots: 9.9 M slots 0.72 / 0.73 / 0.75 /
 // 0.80 ms, 86 M 3.65 / 3.61 / 3.66 / 3.77, 131 M 7.93 / 7.82 / 7.88 / 8.15,
 // 657 M (more parts than fit below 2^19) - / 63 / 41.6 / 40.7.  A chain of
@@ -1429,10 +1430,11 @@ __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 thr
 }
 
 // find_or_claim from slot s, `probed` slots past the home that are known to hold
-// other keys, with the keys of kAhead slots loaded at a time: the events
-// that are left for the global pass are those with long probes, and each step
-// was a trip to memory (29,000 events of a 5 Mbp build: 39 -> 25 us).  (A slot seen taken by another key stays that key's; one
-// seen empty is claimed or refused by the CAS.)
+// other keys, with the keys of kAhead slots loaded at a time: the events that
+// are left for the global pass are those with long probes, and each step was a
+// trip to memory (29,000 events of a 5 Mbp build: 39 -> 25 us).  (A slot seen
+// taken by another key stays that key's; one seen empty is claimed or refused by
+// the CAS.)
 __device__ __forceinline__ bool find_or_claim_ahead(Slot *table, uint64_t n_slots,
                                                     uint32_t max_probes, uint64_t key, uint64_t s,
                                                     uint32_t probed, uint64_t &slot_out,
@@ -1912,10 +1914,10 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
     // read-modify-write of partly written sectors)
     constexpr int BS = 512;
     const size_t smem = scatter_smem<BS>(scatter_reads, parts);
-    DBG_CK(cudaFuncSetAttribute(k_bin_scatter<BS, N, SMALL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem));
+    const auto kern = k_bin_scatter<BS, N, SMALL, true>;
+    DBG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bin_scatter<BS, N, SMALL, true>, BS, smem));
+    DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BS, smem));
     // one launch over every read tile, or (input arriving in parts) one per
     // part, each after its part's copy: tiles [cut[c], cut[c + 1]) hold reads
     // that have all arrived (a tile split by a cut goes to the later part)
@@ -1965,10 +1967,10 @@ int tiled_chain_of(BinScratch &sc, const ItemDesc *items, int n, int shift, int 
   }
   mark(5, s);
   {
-    // 512 threads: three such CTAs (66 KB of shared memory each, or 50 KB
-    // for a rebuild's split tile, with the fingerprints; registers allow
-    // three) fill an SM with 48 warps, enough to hide the dependent hash and
-    // probe latencies
+    // 512 threads: three such CTAs (66 KB of shared memory each, or 58 KB for a
+    // rebuild's split tile and its warps' queues, with the fingerprints;
+    // registers allow three) fill an SM with 48 warps, enough to hide the
+    // dependent hash and probe latencies
     constexpr int BA = 512;
     const size_t smem = (fresh ? kSoaTileBytes + (BA / 32) * kTileQueue * sizeof(uint64_t)
                                : (size_t)kTileSlots * sizeof(Slot)) +
@@ -2095,10 +2097,10 @@ int launch_binned(dbg_handle h, const ItemDesc &it, const dbg_tuning &tuning, cu
   {
     constexpr int BS = 512;
     const size_t smem = scatter_smem<BS>(tile_reads, geo.parts);
-    DBG_CK(cudaFuncSetAttribute(k_bin_scatter<BS, 1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem));
+    const auto kern = k_bin_scatter<BS, 1, false, false>;
+    DBG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bin_scatter<BS, 1, false, false>, BS, smem));
+    DBG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BS, smem));
     const int grid = (int)std::min<uint64_t>(slices, (uint64_t)std::max(1, per_sm) * sms);
     k_bin_scatter<BS, 1, false, false><<<grid, BS, smem, s>>>(pk, tile_reads, geo.shift, geo.parts, 0,
                                                 walk_tiles, slices, mv.hist, mv.cursor, h->bin.ev,

@@ -77,8 +77,9 @@ __device__ __forceinline__ uint64_t find_key(const View &v, uint64_t key) {
 // The double-precision division is slow here (each slot's took 8.2 ms of a
 // 2.6 GB table), so the CTA divides the counts below kQuot once, into a table
 // in shared memory -- the same expression, so the same integers -- and only
-// larger counts are divided one by one: 0.76 ms, 6.6 TB/s.  (wide: k > 32, the
-// counters are the slot's second half)
+// larger counts are divided one by one: 0.76 ms, the table read and its taken
+// slots written at about 6 TB/s.  (wide: k > 32, the counters are the slot's
+// second half)
 constexpr uint32_t kQuot = 1024;
 
 __device__ __forceinline__ uint32_t quotient(uint32_t c, double divisor) {
@@ -125,10 +126,10 @@ struct Links {
   uint64_t w0, nw;                    // the words of 32 slots that the bits below are of
   uint32_t *marks;                    // a bit per slot: an edge points to its vertex
   uint2 *degree;                      // per 32 slots: bits of one exit, bits of several
-  ulonglong2 *split;                  // a splitter's slot (its label in the two top bits), its successor's
+  ulonglong2 *split;                  // a splitter's slot (label in the two top bits), successor's
   unsigned long long *labels;         // the first kLabels labels of its segment, two bits each
-  uint32_t *next, *len;               // [levels + 1][kept]: the splitter 2^l segments on, the edges to it
-  uint32_t cap;                       // splitters there is room for (a vertex past them is an ordinary one)
+  uint32_t *next, *len;               // [levels + 1][kept]: the splitter 2^l segments on, the edges
+  uint32_t cap;                       // splitters there is room for (the rest are ordinary vertices)
   uint32_t kept;                      // splitters there are
   unsigned long long *n_split;        // splitters found
   int levels;                         // jumps of up to 2^levels segments
@@ -160,9 +161,10 @@ struct SlotWords {
 
 // Every edge marks its target; every single-exit vertex gets its link; the
 // out-degrees as bits.  A warp takes kLinkWords times 32 consecutive slots (once in
-// a table of few CTAs).  Bound by one read of the table, then by the random target lookups.  (Splitters are
-// numbered by the CTA: an atomic per warp on the one counter, at one splitter in 4
-// vertices, took 2.6 ms of a 2.75 GB table where the rest takes 1.05.)
+// a table of few CTAs).  Bound by one read of the table, then by the random target
+// lookups.  (Splitters are numbered by the CTA: an atomic per warp on the one
+// counter, at one splitter in 4 vertices, took 2.6 ms of a 2.75 GB table where the
+// rest takes 1.05.)
 template <int kLinkWords>
 __global__ void __launch_bounds__(256) k_links(View v, Links k) {
   after_previous();

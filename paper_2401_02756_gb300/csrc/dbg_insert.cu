@@ -13,10 +13,10 @@
 // for a key can count at once: no allocate/retry/free loop (Alg. 3's
 // do-while) is needed, and the result is independent of thread order.
 //
-// Warp aggregation (__match_any_sync; on unless the tuning turns it off):
-// lanes of a warp holding the same key probe once (the lowest lane), and
-// lanes adding to the same (slot, label) counter issue one atomicAdd of the
-// group size.
+// Warp aggregation (__match_any_sync; off in a new handle, whose tuning is all
+// zeros; on where the tuning says 1 or leaves it to this file with -1): lanes of
+// a warp holding the same key probe once (the lowest lane), and lanes adding to
+// the same (slot, label) counter issue one atomicAdd of the group size.
 //
 // Probing is bounded by max_probes; a vertex that finds neither its key nor
 // an empty slot sets the sticky DBG_ERR_CAPACITY and the CTA stops, and later
@@ -92,9 +92,9 @@ struct InsertVisitor {
 // of 100 bases and more.  Tiles of 20 shorter ones hold too few positions for a
 // CTA's threads and barriers, and only the device knows: a large read set's tiles
 // take up to kShortTileReads of them, for kTilePositions positions (571,000 reads
-// of 36 bases, k = 31: 174 us with tiles of 20, 112 with 109; 182,000 of 50: 110 ->
-// 102).  Many read sets in one launch take up to kAutoTileReadsMany (128 sets of 36-base
-// reads 0.67 ms with 20, 0.50 with 48 as with 256; of 150 bases 0.57 and 0.56).
+// of 36 bases, k = 31: 174 us with tiles of 20, 110 with 109; 182,000 of 50: 110 ->
+// 105).  Many read sets in one launch take up to kAutoTileReadsMany (128 sets of
+// 36-base reads 0.67 ms with 20, 0.50 with 48 as with 256; of 150 bases 0.57, 0.56).
 constexpr int kMinTileReads = 2, kAutoTileReads = 20, kAutoTileReadsMany = 48;
 constexpr int kShortTileReads = 128;
 constexpr uint64_t kTilePositions = 768;
@@ -205,9 +205,9 @@ dbg_tuning resolve_tuning(const dbg_tuning &t) {
   dbg_tuning r = t;
   if (r.block_threads <= 0) r.block_threads = 256;
   if (r.tile_reads <= 0 || r.tile_reads > r.block_threads) r.tile_reads = r.block_threads;
-  // warp aggregation on by default: it costs nothing where a warp's keys
-  // differ (100 Mbp direct insert: 155.9 ms either way) and merges repeats
-  // (microsatellite reads: 0.85 -> 0.18 ms)
+  // warp aggregation left to us (-1): on, as it merges repeats (microsatellite
+  // reads: 0.85 -> 0.18 ms) and costs nothing where the table's sectors are the
+  // bound (100 Mbp direct insert: 155.9 ms either way)
   if (r.warp_aggregate < 0) r.warp_aggregate = 1;
   if (r.apply_unroll <= 0) r.apply_unroll = 4;
   if (r.apply_chunk <= 0) r.apply_chunk = 8;

@@ -26,9 +26,10 @@ int cuda_fail(cudaError_t e, const char *what) {
 // pool per device, owned by the library, that keeps up to kScratchKeep
 // bytes across synchronisations (the default pool would give every byte
 // back at each one, so a loop of exports would map and unmap memory each
-// time).  Anything above that is released as usual.  4 GiB covers the
-// export of a graph of about 900 million vertices into device buffers (4
-// bytes a vertex plus the sort's histograms).
+// time).  Anything above that is released as usual.  4 GiB covers an export's
+// bins and its records (at most 4 GiB of them come from here), or the scratch of
+// a mid-size rebuild (at most 2.3 GB); a radix export of a graph of up to about 700
+// million vertices into device buffers (6 bytes a vertex).
 namespace {
 constexpr uint64_t kScratchKeep = 4ull << 30;
 std::mutex g_pool_mu;

@@ -29,8 +29,8 @@ Overflow is handled exactly: a table whose status reports that it ran out of
 room is rebuilt at twice the capacity from the request's resident inputs.
 
 Footprint admitted = packed bytes + offsets bytes + registers + table bytes
-+ the export's device buffers (24 bytes a vertex) and the library's sort
-scratch (4 bytes a vertex) for the vertices the table is sized for, held
++ the export's device buffers (24 bytes a vertex) and its sort's scratch
+(``dbg_export_scratch_bytes``) for the vertices the table is sized for, held
 under ``budget_bytes`` together with the buffers the library keeps for the
 binned chains (``dbg_scratch_bytes``; they grow to the largest batch and
 stay): a batch is cut short when the growth it needs does not fit.  Every
@@ -358,7 +358,7 @@ class BuildServer:
             j.graph.set_tuning(insert_path=1)  # (alone: the direct insert, no chain buffers)
             j.graph.build(j.packed, j.offsets, stream=s)
         # the sorted export: into device buffers from the allocator (the sort
-        # then runs inside them, with 4 bytes a vertex of library scratch),
+        # then runs inside them, with dbg_export_scratch_bytes beside them),
         # accounted against the budget while they live, then to pinned host
         # memory.  Only the export workers release memory, so this takes its
         # room even past the budget rather than wait (the peak shows it).
