@@ -970,7 +970,7 @@ int export_bins(dbg_handle h, uint64_t *keys_out, uint32_t *counts_out, uint64_t
       const cudaError_t e = cudaEventRecord(h->bin.done, s);
       if (e != cudaSuccess) rc = cuda_fail(e, "cudaEventRecord");
     }
-    if (rc != DBG_OK || !rec || m.vertices <= rec_rows) break;
+    if (rc != DBG_OK || !rec || m.vertices <= rec_rows || m.vertices > max_rows) break;
     rec = nullptr;  // more vertices than the event buffer holds: into the outputs
     own = false;
   }
