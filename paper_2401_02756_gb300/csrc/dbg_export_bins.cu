@@ -130,7 +130,8 @@ struct Key<true> {
 };
 
 // The table goes past the L2 (evict_first), the bins' counters stay in it
-// (evict_last): 2^22 bins of 432 M records 25.1 -> 23.9 ms an export, as 2^21 take.
+// (evict_last): 2^22 bins of 432 M records 25.1 -> 23.9 ms an export, as 2^21 take
+// (with four slots a thread in flight).
 __device__ __forceinline__ uint32_t next_place(uint32_t *bin, uint64_t pol) {
   uint32_t at;
   asm volatile("atom.relaxed.gpu.global.add.L2::cache_hint.u32 %0, [%1], 1, %2;"
@@ -400,12 +401,15 @@ __global__ void __launch_bounds__(kChunkBlock)
 // records: place 3.26 -> 2.19 ms, sort 1.22 -> 1.30 ms).  A warp takes `run` words
 // of 32 slots at a time and reads the slots whose bits are set (0.5 M
 // vertices in 300 M slots: export 2.79 ms with every slot read again, 1.86 with a word
-// a warp and load, 1.55 with 32; the table read once takes 1.34).
+// a warp and load, 1.55 with 32; the table read once takes 1.34).  Eight slots a
+// thread in flight for records, four in place (432 M records 23.9 -> 22.9 ms an
+// export; 57 M in place 3.9 and 4.1).
 template <bool WIDE, bool RECORDS>
 __global__ void __launch_bounds__(256) k_place(const Slot *t, uint64_t n, uint32_t run, Plan p,
                                                Slot *rec, Key<WIDE> *keys, uint4 *counts) {
   after_previous();
   if (!may_run(p)) return;
+  constexpr int kPer = RECORDS ? 8 : 4;
   const uint64_t pol = l2_policy_evict_last();
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t words = (n + 31) >> 5, warps = (uint64_t)gridDim.x * blockDim.x >> 5;
@@ -416,10 +420,10 @@ __global__ void __launch_bounds__(256) k_place(const Slot *t, uint64_t n, uint32
       taken = p.taken ? p.taken[w0 + lane] : ~0u;
     uint32_t left = __ballot_sync(0xffffffffu, taken != 0u);
     while (left) {
-      Words v[kSlotsPerThread];
-      uint32_t at[kSlotsPerThread];
+      Words v[kPer];
+      uint32_t at[kPer];
 #pragma unroll
-      for (int u = 0; u < kSlotsPerThread; ++u) {
+      for (int u = 0; u < kPer; ++u) {
         const uint32_t w = (uint32_t)__ffs((int)left) - 1u;  // (none: the slots of no word)
         const uint32_t m = __shfl_sync(0xffffffffu, taken, (int)(w & 31u));
         const uint64_t j = ((w0 + w) << 5) + lane;
@@ -430,7 +434,7 @@ __global__ void __launch_bounds__(256) k_place(const Slot *t, uint64_t n, uint32
         left &= left - 1u;
       }
 #pragma unroll
-      for (int u = 0; u < kSlotsPerThread; ++u) {
+      for (int u = 0; u < kPer; ++u) {
         const Key<WIDE> k = key_of<WIDE>(v[u]);
         at[u] = ~0u;
         if (k.empty()) continue;
@@ -439,7 +443,7 @@ __global__ void __launch_bounds__(256) k_place(const Slot *t, uint64_t n, uint32
         at[u] = next_place(bin, pol);
       }
 #pragma unroll
-      for (int u = 0; u < kSlotsPerThread; ++u) {
+      for (int u = 0; u < kPer; ++u) {
         if (at[u] == ~0u) continue;
         if constexpr (RECORDS) {
           st_record(rec + at[u], record_of<WIDE>(v[u]));
