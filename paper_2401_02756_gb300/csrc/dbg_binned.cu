@@ -1373,9 +1373,14 @@ __global__ void __launch_bounds__(BLOCK, 1536 / BLOCK)  // three CTAs of 512 thr
       for (uint32_t base = 0;;) {
 #pragma unroll
         for (int r = 0; r < kBatch; ++r) {
-          if constexpr (!FRESH) {  // (a held graph's lot leaves a tile few events:
-            // 0.18 ms a lot of 12 M events, 0.187 with the queue)
+          if constexpr (!FRESH) {
+            // (no queue: three CTAs' tiles and queues do not fit an SM.  A tile of many
+            // events brings its lanes together again after each: left apart by their
+            // probes they went on at 11 of 32, 16,000 events a tile 2.32 ms a batch of
+            // 60 graphs, 1.96 so; a lot of 1,900 is better off without, 2.075 and 2.09
+            // ms for four)
             if (is_event(e[r])) probe.finish(e[r], it, p, ev, begin, aux.deferred_n);
+            if (n > (uint32_t)(BLOCK * kBatch)) __syncwarp();
             continue;
           }
           const bool keep = is_event(e[r]) && (!step || probe.first_step(e[r]));
