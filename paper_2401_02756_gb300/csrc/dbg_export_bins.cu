@@ -16,8 +16,8 @@
 // (32-bit prefix, slot index) pairs this replaces moved 16 bytes a record four
 // times, gathered a random slot per vertex and put runs of equal prefixes in
 // order in two more passes.  Export of 422.6 M vertices of a 20.8 GB table
-// 35.4 -> 22 ms (histogram 4.0, place 10.8 to 12.3 from card to card, sort 6.5;
-// 7.7 with the counters at the slot's byte 8, two loads a row), of 57 M 5.1 ->
+// 35.4 -> 22.6 ms (histogram 4.1, place 12 to 12.9 from card to card, sort 5.9;
+// 1.2 more with the counters at the slot's byte 8, two loads a row), of 57 M 5.1 ->
 // 2.8 ms; k = 51, 75 M vertices (two 64-bit radix sorts before) 19.7 -> 4.2 ms.
 //
 // The place pass is at the rate of its stores.  A store to a sector that is
@@ -36,7 +36,7 @@
 // skipped by the sort; the records of all such buckets are then sorted together
 // by their whole keys, by a radix sort, and written back (56 bytes of scratch a
 // record at most).  They are few: export of 432 M vertices (2^22 bins) at 50 / 40 /
-// 35 / 30 % GC 23.9 / 23.9 / 24.9 / 29.5 ms, with none, none, 1 % and 11 % of the
+// 35 / 30 % GC 22.9 / 22.9 / 23.8 / 28.7 ms, with none, none, 1 % and 11 % of the
 // records in such buckets (a radix sort of all: 35.6 to 41.3).
 // Graphs with a quarter of their records in such buckets are left to the radix
 // sort as a whole.
